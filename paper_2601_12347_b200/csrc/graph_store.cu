@@ -163,6 +163,70 @@ __global__ void k_expand_copy(ripple_update* ups, int32_t* op_seq, Ctl* ctl, Sid
     }
 }
 
+// The batch from where the caller has it (pinned host memory, read over PCIe by the kernel itself, or device memory)
+// into the library's own buffers, which every later kernel of the chain reads; and the control block's reset.  One
+// launch in place of up to four copy operations (sizes, operations, weights, payload rows): a copy in front of a
+// kernel costs the chain about 2 us each, whatever its size.
+struct StageArgs {
+    Ctl* ctl;
+    StageIn in;
+    ripple_update* ups;
+    float* opw;
+    float* feat;
+    int d0;
+};
+
+__device__ __forceinline__ bool d_aligned16(const void* a, const void* b) {
+    return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
+}
+
+// Every thread takes one piece of each of the three arrays per round and asks for all three before it stores any: a
+// read of host memory takes over a microsecond, and the grid gives a batch of any size a single round.
+__device__ __forceinline__ void d_stage_in(const StageArgs& a, long long tid, long long nthreads) {
+    const uint32_t* src[3] = {reinterpret_cast<const uint32_t*>(a.in.ups), reinterpret_cast<const uint32_t*>(a.in.opw),
+                              reinterpret_cast<const uint32_t*>(a.in.rows)};
+    uint32_t* dst[3] = {reinterpret_cast<uint32_t*>(a.ups), reinterpret_cast<uint32_t*>(a.opw), reinterpret_cast<uint32_t*>(a.feat)};
+    const long long words[3] = {3ll * a.in.n_ops, a.in.opw ? a.in.n_ops : 0, (long long)a.in.n_rows * a.d0};
+    long long most = 0;
+    bool wide[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        wide[k] = d_aligned16(src[k], dst[k]);
+        most = max(most, wide[k] ? (words[k] + 3) >> 2 : words[k]);
+    }
+    for (long long i = tid; i < most; i += nthreads) {
+        uint4 x[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (wide[k] && 4 * i + 3 < words[k]) x[k] = reinterpret_cast<const uint4*>(src[k])[i];
+            else if (!wide[k] && i < words[k]) x[k].x = src[k][i];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (wide[k] && 4 * i + 3 < words[k]) reinterpret_cast<uint4*>(dst[k])[i] = x[k];
+            else if (!wide[k] && i < words[k]) dst[k][i] = x[k].x;
+            else if (wide[k] && 4 * i < words[k])
+                for (long long j = 4 * i; j < words[k]; ++j) dst[k][j] = src[k][j];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256) k_stage_in(const __grid_constant__ StageArgs a) {
+    pdl_enter();
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+    if (a.in.ups) d_stage_in(a, tid, nt);
+    if (tid == nt - 1) d_ctl_reset(a.ctl, a.in.n_ops, a.in.n_rows);
+}
+
+static StageArgs stage_args(const Ctx* c) { return StageArgs{c->ctl, c->stage_in, c->ups_dev, c->opw_dev, c->feat_dev, c->d[0]}; }
+
+static int stage_grid(const Ctx* c) {   // one 16-byte piece of the larger array per thread, up to eight blocks per SM
+    const long long words = std::max<long long>(3ll * c->stage_in.n_ops, (long long)c->stage_in.n_rows * c->d[0]);
+    return c->stage_in.ups ? (int)std::min<long long>(words / 1024 + 1, c->n_sm * 8) : 1;
+}
+
+void graph_batch_stage_in(Ctx* c) { RP_LAUNCH(c, k_stage_in, stage_grid(c), 256, 0, stage_args(c)); }
+
 __device__ __forceinline__ void d_classify(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_seq, int N,
                                            Ctl* ctl, unsigned long long* hkeys, unsigned long long* hwin, int hmask,
                                            int32_t* op_slot, int32_t* feat_last, int32_t* vdel_seq, int no_vertex_ops) {
@@ -661,7 +725,7 @@ __global__ void k_commit_degrees(Ctl* ctl, const Rec* __restrict__ rec, Side out
 }
 
 // ... and all of them in one block, a barrier between the phases, for the batches that are replayed
-// from a captured chain (up to RP_GRAPH_MAX_BATCH operations: a few hundred records at most, which one
+// from a captured chain (up to RP_ONE_BLOCK_BATCH operations: a few hundred records at most, which one
 // block handles in a single sweep per phase).  Small batches are bound by the number of launches.
 __global__ void __launch_bounds__(1024)
 k_mutate_small(Ctl* ctl, Rec* rec, Side out, Side in, const int32_t* __restrict__ grow_out,
@@ -688,45 +752,74 @@ k_mutate_small(Ctl* ctl, Rec* rec, Side out, Side in, const int32_t* __restrict_
 // update, the list A_0 (sorted in shared memory from the winning feature operations: no sweep of the
 // frontier bitmap), the feature rows with their old values or deltas, and the sender list of hop 1 with its
 // out-degree prefix -- nine launches of the general chain -- in one block with barriers in between.
+struct ApplySmallArgs {
+    StageArgs st;
+    const int32_t* op_seq;
+    int N;
+    unsigned long long *hkeys, *hwin;
+    int hmask;
+    int32_t *op_slot, *feat_last, *vdel_seq;
+    Side out, in;
+    Rec* rec;
+    uint32_t* bitmap;
+    int32_t *grow[2], *shrink[2];
+    int64_t* moved_start;
+    int32_t* moved_cap;
+    int32_t* deg_out_old;
+    float* H0;
+    int ld;
+    float* D;
+    int keep_old;
+    int32_t* A0;
+    int build_senders;
+    int32_t *senders, *posmap;
+    int64_t* coff;
+};
+
 __global__ void __launch_bounds__(1024)
-k_apply_small(Ctl* ctl, const int* params, const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_seq, int N,
-              unsigned long long* hkeys, unsigned long long* hwin, int hmask, int32_t* op_slot, int32_t* feat_last,
-              int32_t* vdel_seq, Side out, Side in, Rec* rec, uint32_t* bitmap, const float* __restrict__ op_w,
-              int32_t* grow_out, int32_t* grow_in, int32_t* shrink_out, int32_t* shrink_in, int64_t* moved_start,
-              int32_t* moved_cap, int32_t* deg_out_old, const float* __restrict__ feat, int d0, float* H0, int ld,
-              float* D, int keep_old, int32_t* A0, int build_senders, int32_t* senders, int32_t* posmap, int64_t* coff) {
+k_apply_small(const __grid_constant__ ApplySmallArgs a) {
     pdl_enter();
     __shared__ int s_ids[RP_TINY_BATCH];
     __shared__ int s_n;
-    if (threadIdx.x == 0) { d_ctl_reset(ctl, params); s_n = 0; }
+    Ctl* ctl = a.st.ctl;
+    const StageIn& src_in = a.st.in;
+    if (threadIdx.x == 0) { d_ctl_reset(ctl, src_in.n_ops, src_in.n_rows); s_n = 0; }
+    if (src_in.ups) {   // (the payload rows are read where they lie)
+        if ((int)threadIdx.x < 3 * src_in.n_ops)
+            reinterpret_cast<uint32_t*>(a.st.ups)[threadIdx.x] = reinterpret_cast<const uint32_t*>(src_in.ups)[threadIdx.x];
+        if (src_in.opw && (int)threadIdx.x < src_in.n_ops) a.st.opw[threadIdx.x] = src_in.opw[threadIdx.x];
+    }
+    const ripple_update* ups = a.st.ups;
+    const float* op_w = src_in.opw ? a.st.opw : nullptr;
+    const float* feat = src_in.ups ? src_in.rows : a.st.feat;
     __syncthreads();
-    d_classify(ups, op_seq, N, ctl, hkeys, hwin, hmask, op_slot, feat_last, vdel_seq, 0);
+    d_classify(ups, a.op_seq, a.N, ctl, a.hkeys, a.hwin, a.hmask, a.op_slot, a.feat_last, a.vdel_seq, 0);
     __syncthreads();
-    d_resolve(ups, op_seq, ctl, hwin, op_slot, feat_last, vdel_seq, out, in, rec, bitmap, op_w, grow_out, grow_in,
-              shrink_out, shrink_in, nullptr);
+    d_resolve(ups, a.op_seq, ctl, a.hwin, a.op_slot, a.feat_last, a.vdel_seq, a.out, a.in, a.rec, a.bitmap, op_w, a.grow[0],
+              a.grow[1], a.shrink[0], a.shrink[1], nullptr);
     __syncthreads();
-    d_del_mark(ctl, rec, out, in);
+    d_del_mark(ctl, a.rec, a.out, a.in);
     __syncthreads();
-    d_del_tail_read(ctl, rec, out, in);
+    d_del_tail_read(ctl, a.rec, a.out, a.in);
     __syncthreads();
-    d_del_tail_pack(ctl, rec, out, in);
+    d_del_tail_pack(ctl, a.rec, a.out, a.in);
     __syncthreads();
-    d_del_fill(ctl, rec, out, in);
+    d_del_fill(ctl, a.rec, a.out, a.in);
     __syncthreads();
-    d_grow_rows(ctl, out, in, grow_out, grow_in, shrink_out, shrink_in, moved_start, moved_cap);
+    d_grow_rows(ctl, a.out, a.in, a.grow[0], a.grow[1], a.shrink[0], a.shrink[1], a.moved_start, a.moved_cap);
     __syncthreads();
-    d_add_write(ctl, rec, out, in);
+    d_add_write(ctl, a.rec, a.out, a.in);
     __syncthreads();
-    d_commit_degrees(ctl, rec, out, in, deg_out_old, moved_start, moved_cap);
+    d_commit_degrees(ctl, a.rec, a.out, a.in, a.deg_out_old, a.moved_start, a.moved_cap);
     __syncthreads();
     if (ctl->abort) return;
     // A_0: the vertices whose last feature operation this is, ascending
     const int n = ctl->n_ops;
     if ((int)threadIdx.x < n) {
         const ripple_update op = ups[threadIdx.x];
-        if (op.op == RIPPLE_OP_SET_FEATURE && feat_last[op.u] == (int)threadIdx.x) {
+        if (op.op == RIPPLE_OP_SET_FEATURE && a.feat_last[op.u] == (int)threadIdx.x) {
             s_ids[atomicAdd(&s_n, 1)] = op.u;
-            atomicAnd(&bitmap[op.u >> 5], ~(1u << (op.u & 31)));   // (resolution marked it for the general chain's sweep)
+            atomicAnd(&a.bitmap[op.u >> 5], ~(1u << (op.u & 31)));   // (resolution marked it for the general chain's sweep)
         }
     }
     __syncthreads();
@@ -737,47 +830,74 @@ k_apply_small(Ctl* ctl, const int* params, const ripple_update* __restrict__ ups
         for (int k = 0; k < na; ++k) rank += s_ids[k] < mine;
     }
     __syncthreads();
-    if (mine >= 0) { s_ids[rank] = mine; A0[rank] = mine; }
-    if (threadIdx.x == 0) { ctl->nA[0] = na; if (build_senders) ctl->nC[0] = na; }
+    if (mine >= 0) { s_ids[rank] = mine; a.A0[rank] = mine; }
+    if (threadIdx.x == 0) { ctl->nA[0] = na; if (a.build_senders) ctl->nC[0] = na; }
     __syncthreads();
     // feature rows: one warp per vertex of A_0
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = warp; i < na; i += (int)(blockDim.x >> 5)) {
         const int v = s_ids[i];
-        const float* src = feat + (size_t)ups[feat_last[v]].v * d0;
-        for (int k = lane; k < ld; k += 32) {
-            const float x = k < d0 ? src[k] : 0.f;
-            const float o = H0[(size_t)v * ld + k];
-            D[(size_t)i * ld + k] = keep_old ? o : x - o;
-            H0[(size_t)v * ld + k] = x;
+        const float* src = feat + (size_t)ups[a.feat_last[v]].v * a.st.d0;
+        for (int k = lane; k < a.ld; k += 32) {
+            const float x = k < a.st.d0 ? src[k] : 0.f;
+            const float o = a.H0[(size_t)v * a.ld + k];
+            a.D[(size_t)i * a.ld + k] = a.keep_old ? o : x - o;
+            a.H0[(size_t)v * a.ld + k] = x;
         }
     }
     // senders of hop 1 = A_0, with the prefix of their out-degrees (max / min aggregation lists its own: the rows
     // of A_0 whose values really changed)
-    if (build_senders && threadIdx.x == 0) {
+    if (a.build_senders && threadIdx.x == 0) {
         int64_t sum = 0;
         for (int i = 0; i < na; ++i) {
             const int v = s_ids[i];
-            senders[i] = v;
-            posmap[v] = i;
-            coff[i] = sum;
-            sum += out.deg[v];
+            a.senders[i] = v;
+            a.posmap[v] = i;
+            a.coff[i] = sum;
+            sum += a.out.deg[v];
         }
-        coff[na] = sum;
+        a.coff[na] = sum;
         ctl->E[1] = (unsigned long long)sum;
     }
 }
 
-void graph_batch_apply_small(Ctx* c, int n) {
-    (void)n;
-    Side& o = c->side[0];
-    Side& i = c->side[1];
-    RP_LAUNCH(c, k_apply_small, 1, 1024, 0, c->ctl, (const int*)c->params_dev, (const ripple_update*)c->ups_dev,
-              (const int32_t*)c->op_seq, c->N, c->hkeys, c->hwin, c->hsize - 1, c->op_slot, c->feat_last, c->vdel_seq, o, i,
-              c->rec, c->bitmap, (const float*)(c->has_opw ? c->opw_dev : nullptr), c->grow_list[0], c->grow_list[1],
-              c->shrink_list[0], c->shrink_list[1], c->moved_start, c->moved_cap, c->deg_out_old,
-              (const float*)c->feat_dev, c->d[0], c->H[0], c->ld[0], c->D[0], (int)(c->attention || rp_monotonic(c->agg)),
-              c->A[0], (int)!rp_monotonic(c->agg), c->Clist[0], c->posmap, c->coff);
+static ApplySmallArgs apply_small_args(const Ctx* c) {
+    ApplySmallArgs a{};
+    a.st = stage_args(c);
+    a.op_seq = c->op_seq; a.N = c->N; a.hkeys = c->hkeys; a.hwin = c->hwin; a.hmask = c->hsize - 1; a.op_slot = c->op_slot;
+    a.feat_last = c->feat_last; a.vdel_seq = c->vdel_seq; a.out = c->side[0]; a.in = c->side[1]; a.rec = c->rec;
+    a.bitmap = c->bitmap;
+    for (int s = 0; s < 2; ++s) { a.grow[s] = c->grow_list[s]; a.shrink[s] = c->shrink_list[s]; }
+    a.moved_start = c->moved_start; a.moved_cap = c->moved_cap; a.deg_out_old = c->deg_out_old;
+    a.H0 = c->H[0]; a.ld = c->ld[0]; a.D = c->D[0]; a.keep_old = c->attention || rp_monotonic(c->agg);
+    a.A0 = c->A[0]; a.build_senders = !rp_monotonic(c->agg);
+    a.senders = c->Clist[0]; a.posmap = c->posmap; a.coff = c->coff;
+    return a;
+}
+
+bool batch_is_tiny(const Ctx* c, int n) { return n >= 1 && n <= RP_TINY_APPLY && !c->may_expand && !c->src_norm; }
+
+void graph_batch_apply_small(Ctx* c) { RP_LAUNCH(c, k_apply_small, 1, 1024, 0, apply_small_args(c)); }
+
+// The root of a captured chain is told where this batch lies: the one thing that differs between two replays.
+cudaError_t graph_batch_retarget(Ctx* c, int n, cudaGraphExec_t exec, cudaGraphNode_t root) {
+    cudaKernelNodeParams p{};
+    StageArgs st;
+    ApplySmallArgs ap;
+    void* args[1];
+    if (batch_is_tiny(c, n)) {
+        ap = apply_small_args(c);
+        args[0] = &ap;
+        p.func = reinterpret_cast<void*>(k_apply_small);
+        p.gridDim = dim3(1); p.blockDim = dim3(1024);
+    } else {
+        st = stage_args(c);
+        args[0] = &st;
+        p.func = reinterpret_cast<void*>(k_stage_in);
+        p.gridDim = dim3((unsigned)stage_grid(c)); p.blockDim = dim3(256);
+    }
+    p.kernelParams = args;
+    return cudaGraphExecKernelNodeSetParams(exec, root, &p);
 }
 
 void graph_batch_mutate(Ctx* c, int n) {
@@ -786,7 +906,7 @@ void graph_batch_mutate(Ctx* c, int n) {
     int grid = std::min(div_up(2 * n, T), c->n_sm * 8);
     Side& o = c->side[0];
     Side& i = c->side[1];
-    if (n <= RP_GRAPH_MAX_BATCH) {
+    if (n <= RP_ONE_BLOCK_BATCH) {
         RP_LAUNCH(c, k_mutate_small, 1, 1024, 0, c->ctl, c->rec, o, i, c->grow_list[0], c->grow_list[1],
                   c->shrink_list[0], c->shrink_list[1], c->moved_start, c->moved_cap, c->deg_out_old);
         return;
@@ -807,10 +927,19 @@ void graph_batch_mutate(Ctx* c, int n) {
 __global__ void k_cleanup(const ripple_update* __restrict__ ups, int N, Ctl* ctl,
                           const Rec* __restrict__ rec, Side out, Side in, unsigned long long* hkeys,
                           unsigned long long* hwin, const int32_t* __restrict__ op_slot, int32_t* feat_last,
-                          int32_t* vdel_seq, int32_t* deg_out_old, uint32_t* bitmap) {
+                          int32_t* vdel_seq, int32_t* deg_out_old, uint32_t* bitmap, Ctl* ctl_host) {
     pdl_enter();
     const int n_rec = ctl->n_rec, n = ops_total(ctl);
-    if (blockIdx.x == 0 && threadIdx.x == 0 && !ctl->abort) ctl->num_edges += ctl->n_add - ctl->n_del;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0 && !ctl->abort) ctl->num_edges += ctl->n_add - ctl->n_del;
+        __syncthreads();
+        // the last kernel of the chain: the control block goes to the host's pinned copy from here (a copy operation
+        // behind the chain costs about 4 us; the stores are visible to the host once the stream has been waited for)
+        static_assert(sizeof(Ctl) % 4 == 0, "copied in words");
+        if (ctl_host)
+            for (int i = threadIdx.x; i < (int)(sizeof(Ctl) / 4); i += blockDim.x)
+                reinterpret_cast<volatile uint32_t*>(ctl_host)[i] = reinterpret_cast<const uint32_t*>(ctl)[i];
+    }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < max(n, n_rec); i += gridDim.x * blockDim.x) {
         if (i < n) {
             ripple_update op = ups[i];
@@ -836,7 +965,7 @@ void graph_batch_cleanup(Ctx* c, int n) {
     const int T = 256;
     RP_LAUNCH(c, k_cleanup, std::min(div_up(n, T), c->n_sm * 8), T, 0, c->ups_dev, c->N, c->ctl, c->rec,
               c->side[0], c->side[1], c->hkeys, c->hwin, c->op_slot, c->feat_last, c->vdel_seq, c->deg_out_old,
-              c->bitmap);
+              c->bitmap, c->ctl_host);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -41,11 +41,9 @@ static cudaError_t dev_alloc(T** p, size_t count, int fill_byte = -2) {
     return e;
 }
 
-// params[0] = number of ops, params[1] = number of payload rows (device memory, so that a captured
-// launch chain can be replayed for batches that differ in them)
-__global__ void k_ctl_reset(Ctl* ctl, const int* params) {
+__global__ void k_ctl_reset(Ctl* ctl, int n_ops, int n_rows) {
     pdl_enter();
-    d_ctl_reset(ctl, params);
+    d_ctl_reset(ctl, n_ops, n_rows);
 }
 
 static void destroy_ctx(Ctx* c) {
@@ -74,11 +72,9 @@ static void destroy_ctx(Ctx* c) {
     cudaFree(c->op_slot); cudaFree(c->rec); cudaFree(c->tile_sums); cudaFree(c->scan_done); cudaFree(c->ctl);
     cudaFree(c->moved_start); cudaFree(c->moved_cap);
     if (c->ctl_host) cudaFreeHost(c->ctl_host);
-    if (c->params_host) cudaFreeHost(c->params_host);
     if (c->stage_host) cudaFreeHost(c->stage_host);
-    cudaFree(c->stage_dev);
-    cudaFree(c->params_dev);
     for (auto& g : c->graph_exec) if (g) cudaGraphExecDestroy(g);
+    for (auto& g : c->graph) if (g) cudaGraphDestroy(g);
     for (auto& e : c->ev) if (e) cudaEventDestroy(e);
     for (auto& e : c->ev_sc) if (e) cudaEventDestroy(e);
     for (auto& e : c->ev_rg) if (e) cudaEventDestroy(e);
@@ -111,9 +107,7 @@ static void full_layer(Ctx* c, int l) {
 static ripple_status run_full(Ctx* c) {
     c->launches = 0;
     c->debug_tc_withhold = 0;
-    c->params_host[0] = 0; c->params_host[1] = 0;
-    cudaMemcpyAsync(c->params_dev, c->params_host, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream);
-    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
     if (c->timing) cudaEventRecord(c->ev[0], c->stream);
     for (int l = 1; l <= c->L; ++l) full_layer(c, l);
     if (c->timing) cudaEventRecord(c->ev[1], c->stream);
@@ -123,6 +117,8 @@ static ripple_status run_full(Ctx* c) {
     c->stats.gpu_launches = c->launches;
     return RIPPLE_OK;
 }
+
+static size_t coff_items(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / RP_ANEW_CHUNK) + 64; }
 
 static std::vector<float> padded_matrix(const float* src, int rows, int cols, int rows_p, int cols_p) {
     std::vector<float> m((size_t)rows_p * cols_p, 0.f);
@@ -205,11 +201,10 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         c->attention = layers[0].kind == RIPPLE_LAYER_GAT;
         c->n_local = o.n_local;
         CK(dev_alloc(&c->ctl, 1, 0));
-        CK(dev_alloc(&c->params_dev, 2, 0));
-        CK(cudaMallocHost(&c->params_host, 2 * sizeof(int)));
-        c->stage_bytes = 64 + (size_t)RP_GRAPH_MAX_BATCH * (sizeof(ripple_update) + sizeof(float) + sizeof(float) * (size_t)layers[0].d_in);
+        // room for a batch that arrives in pageable memory: a couple of thousand operations, half a megabyte of rows
+        c->stage_bytes = 64 + (size_t)std::min<int64_t>(o.max_batch, 2048) * (sizeof(ripple_update) + sizeof(float)) +
+                         std::max<size_t>((size_t)512 << 10, 512 * sizeof(float) * (size_t)layers[0].d_in);
         CK(cudaMallocHost(&c->stage_host, c->stage_bytes));
-        CK(dev_alloc(&c->stage_dev, c->stage_bytes));
         c->no_graphs = o.no_graphs;
         {
             const char* e = getenv("RIPPLE_NO_PDL");
@@ -381,8 +376,9 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         CK(dev_alloc(&c->moved_start, (size_t)4 * o.max_batch));
         CK(dev_alloc(&c->moved_cap, (size_t)4 * o.max_batch));
         // degree prefix of a sender list; also the (vertex, chunk) work items of long in-lists during a
-        // gather: a row of more than 256 entries gives at most 2 items per 256 of them
-        CK(dev_alloc(&c->coff, std::max((size_t)N + 2, (size_t)(c->side[1].col_size / 128) + 64), 0));
+        // gather: a row of more than 256 entries gives at most 2 items per 256 of them, a row gathered anew by the
+        // fold one per RP_ANEW_CHUNK and one more
+        CK(dev_alloc(&c->coff, coff_items(c, (size_t)N), 0));
         CK(dev_alloc(&c->bitmap, (size_t)c->n_words + 256, 0));
         if (rp_monotonic(agg)) {
             CK(dev_alloc(&c->bitmap2, (size_t)c->n_words + 256, 0));
@@ -446,12 +442,12 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
     // A handful of updates: the whole of Apply and the hop-0 sender list in one block (the chain of a small batch
     // is bound by the number of dependent steps, not by their work); also the merged frontier kernel below.
     const bool tiny = nb >= 1 && nb <= RP_TINY_BATCH && !c->may_expand && !c->src_norm && !rp_monotonic(c->agg);
-    if (nb >= 1 && nb <= RP_TINY_APPLY && !c->may_expand && !c->src_norm) {
+    if (batch_is_tiny(c, nb)) {
         STAMP();  // 0
-        graph_batch_apply_small(c, nb);
+        graph_batch_apply_small(c);
         if (rp_monotonic(c->agg)) max_senders_build(c, 0);
     } else {
-        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+        graph_batch_stage_in(c);
         STAMP();  // 0
         // Apply (Sec. 3.3): normalise the batch, mutate both adjacency directions, replace features
         graph_batch_classify(c, nb);
@@ -551,18 +547,26 @@ static void arm_rebuild(Ctx* c, int nb) {
     }
 }
 
-// Small batches are launch-bound (about fifty short kernels): their chain is captured once per
-// batch size into a CUDA graph and replayed.  Returns false if this batch must take the direct path.
-static bool launch_batch_graph(Ctx* c, int nb) {
-    if (c->no_graphs || c->timing || nb < 1 || nb > RP_GRAPH_MAX_BATCH) return false;
+// Number of operations the launches of a batch are sized for: the next power of two (from 4).  Every kernel strides
+// over the counts it reads from the control block, so any size at least the batch's is correct; batches of
+// similar size share one captured chain.
+static int chain_size(const Ctx* c, int nb) {
+    int n = RP_TINY_APPLY;
+    while (n < nb) n <<= 1;
+    return (int)std::max<int64_t>(nb, std::min<int64_t>(n, c->max_batch));
+}
+
+// The chain (twenty to fifty mostly short kernels) is captured once per launch geometry into a CUDA graph and replayed:
+// a launch of its own costs the host 2.3 us, more than many of the kernels take, a node of a replayed chain 0.9 us
+// (both measured on empty kernels).  Returns false if this batch must take the direct path.
+static bool launch_batch_graph(Ctx* c, int ng) {
+    if (c->no_graphs || c->timing || ng < 1 || c->debug_tc_withhold) return false;
     // the captured chain differs with the expansion kernels and with the hops whose rebuilding form is enqueued
-    int key = 4 * nb + (c->may_expand ? 1 : 0) + (c->has_opw ? 2 : 0);
-    key = 2 * key + (c->tc_armed ? 1 : 0);
-    key = 2 * key + (c->packed_now ? 1 : 0);   // (the chain holds the addresses its kernels read the batch from)
+    uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->tc_armed ? 4 : 0);
     for (int l = 1; l <= c->L; ++l) key = 4 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0);
     int slot = -1;
     for (int i = 0; i < RP_GRAPH_SLOTS; ++i)
-        if (c->graph_exec[i] && c->graph_n[i] == key) slot = i;
+        if (c->graph_exec[i] && c->graph_key[i] == key) slot = i;
     if (slot < 0) {
         // Capturing costs a millisecond or more: only a chain that keeps coming back is worth it.  A
         // stream whose batch sizes never repeat is launched kernel by kernel.
@@ -580,13 +584,20 @@ static bool launch_batch_graph(Ctx* c, int nb) {
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { c->no_graphs = 1; return false; }
         c->launches = 0;
-        enqueue_batch(c, nb, false);
+        enqueue_batch(c, ng, false);
         cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+        size_t roots = 1;
+        if (e == cudaSuccess) e = cudaGraphGetRootNodes(g, &c->graph_root[slot], &roots);
+        if (e == cudaSuccess && roots != 1) e = cudaErrorUnknown;
         if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_exec[slot], g, 0);
-        if (g) cudaGraphDestroy(g);
+        if (c->graph[slot]) cudaGraphDestroy(c->graph[slot]);
+        c->graph[slot] = g;   // (its root node names the node of the executable chain)
         if (e != cudaSuccess) { cudaGetLastError(); c->graph_exec[slot] = nullptr; c->no_graphs = 1; return false; }
-        c->graph_n[slot] = key;
+        c->graph_key[slot] = key;
         c->graph_launches[slot] = c->launches;
+    } else if (graph_batch_retarget(c, ng, c->graph_exec[slot], c->graph_root[slot]) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
     }
     c->launches = c->graph_launches[slot];
     return cudaGraphLaunch(c->graph_exec[slot], c->stream) == cudaSuccess;
@@ -625,10 +636,6 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
         s.ms_total = s.ms_graph = 0.f;
         return RIPPLE_OK;
     }
-    float* own_feat = c->feat_dev;
-    ripple_update* own_ups = c->ups_dev;
-    float* own_opw = c->opw_dev;
-    int* own_params = c->params_dev;
     c->launches = 0;
     int evi = 0;
     // A vertex deletion becomes one edge deletion per incident edge on the device.  Launches are
@@ -638,57 +645,59 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
     bool wide = false;
     if (mem == RIPPLE_MEM_HOST)
         for (int i = 0; i < nb && !wide; ++i) wide = ups[i].op == RIPPLE_OP_DEL_VERTEX;
-    const int ng = wide ? (int)c->max_batch : nb;
+    const int ng = wide ? (int)c->max_batch : chain_size(c, nb);
     c->may_expand = wide || mem != RIPPLE_MEM_HOST;
     {   // diagnostic: a wait that nothing ends, to exercise the time-out path without faulting the device
         const char* e = getenv("RIPPLE_DEBUG_TC_WITHHOLD");
         c->debug_tc_withhold = e && e[0] == '1';
     }
     arm_rebuild(c, nb);
-    const bool try_graph = !wide && !c->no_graphs && !c->timing && nb >= 1 && nb <= RP_GRAPH_MAX_BATCH;
-    const cudaMemcpyKind kind = mem == RIPPLE_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     c->has_opw = c->weighted && edge_weights && nb;
-    // A small host batch without vertex deletions travels in one copy: sizes, operations, weights and payload
-    // rows are packed into pinned memory at offsets that depend on the number of operations alone (a captured
-    // chain holds them), and the kernels read them where they land.
-    const bool packed = mem == RIPPLE_MEM_HOST && !wide && nb >= 1 && nb <= RP_GRAPH_MAX_BATCH && nr <= RP_GRAPH_MAX_BATCH;
-    c->packed_now = packed;
-    c->few_rows_form = nb <= 128;
-    if (packed) {
+    c->few_rows_form = ng <= 128;
+    // The first kernel of the chain fetches the batch itself, from device memory or from pinned host memory: the caller's
+    // if it is pinned, else a packed copy in the library's own staging area.  Pageable batches that do not fit there
+    // are copied ahead of the chain.
+    c->stage_in = StageIn{ups, c->has_opw ? edge_weights : nullptr, feat_rows, nb, nr};
+    if (mem == RIPPLE_MEM_HOST) {
         auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
-        const size_t off_ups = 16, off_w = off_ups + pad16(sizeof(ripple_update) * (size_t)nb);
-        const size_t off_rows = off_w + (c->weighted ? pad16(sizeof(float) * (size_t)nb) : 0);
-        const size_t total = off_rows + sizeof(float) * (size_t)nr * c->d[0];
-        int* head = reinterpret_cast<int*>(c->stage_host);
-        head[0] = nb; head[1] = nr;
-        memcpy(c->stage_host + off_ups, ups, sizeof(ripple_update) * (size_t)nb);
-        if (c->has_opw) memcpy(c->stage_host + off_w, edge_weights, sizeof(float) * (size_t)nb);
-        if (nr) memcpy(c->stage_host + off_rows, feat_rows, sizeof(float) * (size_t)nr * c->d[0]);
-        CK(cudaMemcpyAsync(c->stage_dev, c->stage_host, total, cudaMemcpyHostToDevice, c->stream));
-        c->params_dev = reinterpret_cast<int*>(c->stage_dev);
-        c->ups_dev = reinterpret_cast<ripple_update*>(c->stage_dev + off_ups);
-        c->opw_dev = reinterpret_cast<float*>(c->stage_dev + off_w);
-        c->feat_dev = reinterpret_cast<float*>(c->stage_dev + off_rows);
-    } else {
-        // operations are always staged: generated edge deletions are appended behind them
-        if (nb) CK(cudaMemcpyAsync(c->ups_dev, ups, sizeof(ripple_update) * (size_t)nb, kind, c->stream));
-        if (c->has_opw) CK(cudaMemcpyAsync(c->opw_dev, edge_weights, sizeof(float) * (size_t)nb, kind, c->stream));
-        if (mem == RIPPLE_MEM_HOST || try_graph) {
-            // a replayed graph reads the library's own staging buffers, so device payload rows are copied too
-            if (nr) CK(cudaMemcpyAsync(c->feat_dev, feat_rows, sizeof(float) * (size_t)nr * c->d[0], kind, c->stream));
+        const size_t b_ups = sizeof(ripple_update) * (size_t)nb, b_w = c->has_opw ? sizeof(float) * (size_t)nb : 0;
+        const size_t b_rows = sizeof(float) * (size_t)nr * c->d[0];
+        auto on_device = [](const void* p) -> const void* {   // the device's address of pinned host memory, or null
+            cudaPointerAttributes at;
+            if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+            return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+        };
+        // (packing this much takes less time than the look-up and the device's first sight of pages it has not read before)
+        const bool small = pad16(b_ups) + pad16(b_w) + b_rows <= (64u << 10);
+        const void *pu = nullptr, *pw = nullptr, *pr = nullptr;
+        if (!small && (pu = on_device(ups)) && (!nr || (pr = on_device(feat_rows))) && (!b_w || (pw = on_device(edge_weights)))) {
+            c->stage_in.ups = static_cast<const ripple_update*>(pu);
+            c->stage_in.opw = static_cast<const float*>(pw);
+            c->stage_in.rows = static_cast<const float*>(pr);
+        } else if (pad16(b_ups) + pad16(b_w) + b_rows <= c->stage_bytes) {
+            char* at = c->stage_host;
+            memcpy(at, ups, b_ups);
+            c->stage_in.ups = reinterpret_cast<const ripple_update*>(at);
+            at += pad16(b_ups);
+            if (b_w) { memcpy(at, edge_weights, b_w); c->stage_in.opw = reinterpret_cast<const float*>(at); }
+            at += pad16(b_w);
+            if (nr) { memcpy(at, feat_rows, b_rows); c->stage_in.rows = reinterpret_cast<const float*>(at); }
         } else {
-            c->feat_dev = const_cast<float*>(feat_rows);   // device payload rows are read in place
+            CK(cudaMemcpyAsync(c->ups_dev, ups, b_ups, cudaMemcpyHostToDevice, c->stream));
+            if (b_w) CK(cudaMemcpyAsync(c->opw_dev, edge_weights, b_w, cudaMemcpyHostToDevice, c->stream));
+            if (nr) CK(cudaMemcpyAsync(c->feat_dev, feat_rows, b_rows, cudaMemcpyHostToDevice, c->stream));
+            c->stage_in.ups = nullptr;
         }
-        c->params_host[0] = nb; c->params_host[1] = nr;
-        CK(cudaMemcpyAsync(c->params_dev, c->params_host, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     }
-    if (!try_graph || !launch_batch_graph(c, nb)) {
+    if (!launch_batch_graph(c, ng)) {
         c->launches = 0;
         evi = enqueue_batch(c, ng, c->timing != 0);
     }
-    c->feat_dev = own_feat; c->ups_dev = own_ups; c->opw_dev = own_opw; c->params_dev = own_params;
-    st = sync_and_fetch_ctl(c);
-    if (st) return st;
+    {   // (the chain's last kernel has put the control block into ctl_host)
+        cudaError_t e = cudaStreamSynchronize(c->stream);
+        if (!e) e = cudaGetLastError();
+        if (e) { set_err(c, "CUDA error while running the batch: %s", cudaGetErrorString(e)); return RIPPLE_ERR_CUDA; }
+    }
     {
         const Ctl& h = *c->ctl_host;
         ripple_stats& s = c->stats;
@@ -740,7 +749,6 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
     }
     return RIPPLE_OK;
 fail:
-    c->feat_dev = own_feat; c->ups_dev = own_ups; c->opw_dev = own_opw; c->params_dev = own_params;
     return st;
 }
 
@@ -858,7 +866,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
     for (int l = 1; l <= L; ++l) if (c->layer[l].kind == RIPPLE_LAYER_GIN) max_hid = std::max(max_hid, c->layer[l].ld_hid);
     CK(cudaStreamSynchronize(c->stream));
     for (auto& g : c->graph_exec) if (g) { cudaGraphExecDestroy(g); g = nullptr; }   // captured chains hold the old addresses
-    memset(c->graph_n, 0, sizeof(c->graph_n));
+    memset(c->graph_key, 0, sizeof(c->graph_key));
     memset(c->seen_key, 0, sizeof(c->seen_key));
     memset(c->seen_count, 0, sizeof(c->seen_count));
     for (int l = 0; l <= L; ++l) {
@@ -885,8 +893,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
     CK(grow_array(&c->att_so, N0 + 32, N1 + 32, 0));
     if (c->att_items) CK(grow_array(&c->att_items, N0 + (size_t)(c->side[1].col_size / RP_ATT_CHUNK) + 64, N1 + (size_t)(c->side[1].col_size / RP_ATT_CHUNK) + 64, 0));
     {
-        const size_t other = (size_t)(c->side[1].col_size / 128) + 64;
-        CK(grow_array(&c->coff, std::max(N0 + 2, other), std::max(N1 + 2, other), 0));
+        CK(grow_array(&c->coff, coff_items(c, N0), coff_items(c, N1), 0));
     }
     {
         const size_t w0 = (size_t)c->n_words + 256, w1 = (N1 + 31) / 32 + 256;
@@ -921,16 +928,14 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
         c->debug_tc_withhold = 0;
         c->tc_armed = 1;
         c->few_rows_form = count <= 256;
-        c->params_host[0] = 0; c->params_host[1] = 0;
-        cudaMemcpyAsync(c->params_dev, c->params_host, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream);
-        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
         k_list_new_vertices<<<std::min(div_up(count, 256), c->n_sm * 4), 256, 0, c->stream>>>(c->ctl, L, first, count, lists_dev, (int)lists.size());
         for (int l = 1; l <= L && !c->attention; ++l) {   // (attention: an isolated vertex outputs zeros and its logit halves are zero)
             if (c->pre[l]) sender_transform(c, l);
             self_project(c, l, false);
             update_rows(c, l, false);
         }
-        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
         st = sync_and_fetch_ctl(c);
         cudaFree(lists_dev);
         if (st) return st;
@@ -1124,9 +1129,7 @@ extern "C" ripple_status ripple_part_bootstrap_layer(ripple_ctx* ctx, int32_t l)
     if (ripple_status ps = peers_known(c)) return ps;
     cudaSetDevice(c->device);
     c->launches = 0;
-    c->params_host[0] = 0; c->params_host[1] = 0;
-    cudaMemcpyAsync(c->params_dev, c->params_host, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream);
-    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
     part_fetch_halo_rows(c, l - 1);
     full_layer(c, l);
     c->stats.num_layers = c->L;
@@ -1164,12 +1167,10 @@ extern "C" ripple_status ripple_part_begin(ripple_ctx* ctx, const ripple_update*
     if (c->has_silent) cudaMemcpyAsync(c->silent_dev, no_compute, (size_t)nb, kind, c->stream);
     if (c->has_opw) cudaMemcpyAsync(c->opw_dev, edge_weights, sizeof(float) * (size_t)nb, kind, c->stream);
     if (nr) cudaMemcpyAsync(c->feat_dev, feat_rows, sizeof(float) * (size_t)nr * c->d[0], kind, c->stream);
-    c->params_host[0] = nb; c->params_host[1] = nr;
-    cudaMemcpyAsync(c->params_dev, c->params_host, 2 * sizeof(int), cudaMemcpyHostToDevice, c->stream);
     cudaMemsetAsync(c->rows_sent, 0, sizeof(unsigned long long) * (RP_MAXL + 1), c->stream);
     // launch geometry for at least one operation: a worker with an empty share still takes part in every hop
     c->part_nb = std::max(nb, 1);
-    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, c->params_dev);
+    RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, nb, nr);
     graph_batch_classify(c, c->part_nb);
     graph_batch_mutate(c, c->part_nb);
     frontier_seed_features(c, c->part_nb);

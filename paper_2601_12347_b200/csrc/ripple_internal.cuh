@@ -16,12 +16,13 @@
 
 #define RP_MAXL RIPPLE_MAX_LAYERS
 #define RP_TOMB (-1)
-#define RP_GRAPH_MAX_BATCH 512   // batches up to this size replay a captured launch chain
-#define RP_GRAPH_SLOTS 8
+#define RP_ONE_BLOCK_BATCH 512   // batches up to this size have their row updates done by one block
+#define RP_GRAPH_SLOTS 16
 #define RP_GRAPH_SEEN 32    // recently seen chain keys: a chain is captured at its second appearance
 #define RP_POOL_CLASSES 32          // block size classes of the adjacency store: class k holds blocks of 2^k entries
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
+#define RP_ANEW_CHUNK 32            // in-list entries per work item of a row gathered anew by the fold (sizes the item buffer)
 #define RP_ATT_CHUNK 128            // attention: in-list entries per work item of a recomputation (sizes the item buffer)
 #define RP_TINY_BATCH 32            // batches up to this size list their frontiers and senders in one block each
 #define RP_TINY_APPLY 4             // ... and up to this size run the whole of Apply in one block (operations are resolved one after the other there)
@@ -71,9 +72,8 @@ struct Ctl {
     int work_counter[8];              // dynamic work distribution tickets (reset by the consumer)
 };
 
-// Start of a batch: everything back to zero except what lives across batches; params[0] = number of
-// operations, params[1] = number of payload rows.
-__device__ __forceinline__ void d_ctl_reset(Ctl* ctl, const int* params) {
+// Start of a batch: everything back to zero except what lives across batches.
+__device__ __forceinline__ void d_ctl_reset(Ctl* ctl, int n_ops, int n_rows) {
     Ctl z;
     memset(&z, 0, sizeof(Ctl));
     for (int s = 0; s < 2; ++s) {
@@ -82,8 +82,8 @@ __device__ __forceinline__ void d_ctl_reset(Ctl* ctl, const int* params) {
         z.pool_lost[s] = ctl->pool_lost[s];
     }
     z.num_edges = ctl->num_edges;
-    z.n_ops = params[0];
-    z.n_rows = params[1];
+    z.n_ops = n_ops;
+    z.n_rows = n_rows;
     *ctl = z;
 }
 
@@ -129,6 +129,14 @@ struct TcW {
     float* hi;
     float* lo;
     int k_pad, n_pad;
+};
+
+// Where a batch lies: pinned host memory or device memory, in either case read by the first kernel of its chain.
+struct StageIn {
+    const ripple_update* ups;   // null: the copies into the library's own buffers are already enqueued
+    const float* opw;           // weight per operation, or null
+    const float* rows;          // payload rows
+    int n_ops, n_rows;
 };
 
 struct LayerDev {
@@ -244,19 +252,18 @@ struct Ctx {
     int64_t* tile_sums;
     int n_tile_sums;
     int* scan_done;    // blocks of a scan's first kernel that have finished (zero between scans)
-    char* stage_host;  // pinned: sizes, operations, weights and payload rows of a small host batch, packed for one copy
-    char* stage_dev;
+    char* stage_host;  // pinned: operations, weights and payload rows of a batch that arrives in pageable memory
     size_t stage_bytes;
-    int packed_now;    // the batch being applied arrived through the packed staging buffer
+    StageIn stage_in;  // the batch being applied
     int few_rows_form; // the batch being applied is small: its row updates carry the few-row form (see k_update_rows)
-    int* params_dev;   // {n_ops, n_rows} of the batch being applied
-    int* params_host;  // pinned
     int no_graphs;
+    cudaGraph_t graph[RP_GRAPH_SLOTS];
     cudaGraphExec_t graph_exec[RP_GRAPH_SLOTS];
-    int graph_n[RP_GRAPH_SLOTS];
+    cudaGraphNode_t graph_root[RP_GRAPH_SLOTS];   // the chain's first kernel: its argument says where the batch lies
+    uint64_t graph_key[RP_GRAPH_SLOTS];
     int64_t graph_launches[RP_GRAPH_SLOTS];
     int graph_next;
-    int seen_key[RP_GRAPH_SEEN];
+    uint64_t seen_key[RP_GRAPH_SEEN];
     int seen_count[RP_GRAPH_SEEN];
     int seen_next;
     Ctl* ctl;        // device
@@ -307,7 +314,10 @@ inline int pad4(int x) { return (x + 3) & ~3; }
 cudaError_t graph_build(Ctx* c, const int32_t* src_dev, const int32_t* dst_dev, const float* w_dev, int64_t E,
                         double slack, int64_t pool_edges);
 void graph_batch_classify(Ctx* c, int n);   // validate, dedupe, find net changes, plan
-void graph_batch_apply_small(Ctx* c, int n);            // a handful of updates: control block reset, Apply and the hop-0 senders in one block
+bool batch_is_tiny(const Ctx* c, int n);                // a handful of updates: Apply runs in one block
+void graph_batch_stage_in(Ctx* c);                      // first kernel of a chain: the batch into the library's buffers, control block reset
+void graph_batch_apply_small(Ctx* c);                   // first kernel of a tiny batch's chain: the same, all of Apply and the hop-0 senders, in one block
+cudaError_t graph_batch_retarget(Ctx* c, int n, cudaGraphExec_t exec, cudaGraphNode_t root);   // a captured chain reads this batch
 void graph_batch_mutate(Ctx* c, int n);                 // apply the net changes to both directions
 void graph_batch_cleanup(Ctx* c, int n);                // reset per-batch scratch
 cudaError_t graph_export(Ctx* c, int64_t* rowptr, int32_t* col, float* weight, int64_t col_capacity, int64_t* n_edges);

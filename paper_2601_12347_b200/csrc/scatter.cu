@@ -40,6 +40,9 @@ __device__ __forceinline__ void add4(float4& a, const float4& x, float c) {
 // single warp busy for 0.7 ms, longer than everything else of a hop on the sparse graph.
 constexpr int SPMM_HUB_DEGREE = 256;
 constexpr int SPMM_HUB_CHUNK = 256;
+// ... and the few rows that the fold sends back to be gathered anew in shorter ones: there is one warp for every
+// chunk, and the chain waits for the longest (ten rows of the weighted sum on the sparse graph: 63 us in chunks of 256)
+constexpr int SPMM_ANEW_CHUNK = RP_ANEW_CHUNK;
 
 // acc += sum over in-list entries [j_begin, j_end) of row v of c_u * M_u; LPR lanes hold one row
 // (NV float4 slots each), a warp works on 32 / LPR neighbours per step, four steps in flight.
@@ -140,7 +143,7 @@ k_spmm_pull(int N, Side in, const int32_t* __restrict__ deg_out, int src_norm,
 
 // The chunks of the long in-lists, one warp per 256-entry chunk; chunk sums are added to the row,
 // which the kernel that queued the chunks has zeroed.
-template <int NV, int LPR>
+template <int NV, int LPR, int CHUNK = SPMM_HUB_CHUNK>
 __global__ void __launch_bounds__(256)
 k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const float* __restrict__ M, int ld,
             float* S, const int2* __restrict__ items, const int* __restrict__ n_items) {
@@ -155,7 +158,7 @@ k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const fl
         float4 acc[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        spmm_accumulate<NV, LPR>(acc, in, w.x, w.y * SPMM_HUB_CHUNK, min(deg, (w.y + 1) * SPMM_HUB_CHUNK), deg_out,
+        spmm_accumulate<NV, LPR>(acc, in, w.x, w.y * CHUNK, min(deg, (w.y + 1) * CHUNK), deg_out,
                                  src_norm, M, ld);
         if (sub == 0) {
 #pragma unroll
@@ -792,7 +795,7 @@ k_fold_deltas(Ctl* ctl, int l, const int32_t* __restrict__ A, int ld, float* S, 
         __syncwarp();
         for (int q = lane; q < nq; q += 32) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
         const int deg = deg_in[v];
-        const int nch = (deg + SPMM_HUB_CHUNK - 1) / SPMM_HUB_CHUNK;
+        const int nch = (deg + SPMM_ANEW_CHUNK - 1) / SPMM_ANEW_CHUNK;
         int first = 0;
         if (lane == 0) {
             if (nch) first = atomicAdd(&ctl->rebuild_items[l], nch);
@@ -813,7 +816,7 @@ void fold_deltas(Ctx* c, int l) {
               c->rebuild_tau2, c->side[1].deg, items);
     if (!c->Eb[l]) return;
 #define HUBS(NV, LPR)                                                                                              \
-    RP_LAUNCH(c, (k_spmm_hubs<NV, LPR>), c->n_sm * 8, 256, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld, \
+    RP_LAUNCH(c, (k_spmm_hubs<NV, LPR, SPMM_ANEW_CHUNK>), c->n_sm * 8, 256, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld, \
               c->S[l], items, &c->ctl->rebuild_items[l])
     RP_WIDTH_DISPATCH(ld, HUBS);
 #undef HUBS

@@ -192,8 +192,30 @@ class _DevArray:
         self._owner = owner
 
 
+def _addr(a: np.ndarray) -> int:
+    return a.__array_interface__["data"][0]   # (a.ctypes.data builds an object first)
+
+
 def _is_torch_cuda(x) -> bool:
     return hasattr(x, "is_cuda") and bool(x.is_cuda)
+
+
+class _Handle:
+    """Owns the library's context: views of its buffers keep it alive, whatever becomes of the `Ripple` object."""
+
+    def __init__(self, lib, h, stream):
+        self.lib, self.h, self.stream = lib, h, stream
+
+    def close(self):
+        if self.h.value:
+            self.lib.ripple_destroy(self.h)
+            self.h.value = None
+
+    def __del__(self):
+        try:
+            self.close()
+        except Exception:
+            pass
 
 
 class Ripple:
@@ -219,6 +241,8 @@ class Ripple:
         self.L = len(model.layers)
         self.dims = [model.layers[0].d_in] + [l.d_out for l in model.layers]
         self.h = ctypes.c_void_p(None)
+        self._views = {}       # tensors over the library's buffers, by name: their addresses change only in reserve_vertices
+        self._handle = _Handle(self.lib, self.h, None)
         keep = []
         g = _Graph()
         g.num_vertices = self.n
@@ -271,25 +295,19 @@ class Ripple:
         opt.device = torch.cuda.current_device()
         self._stream = stream if stream is not None else torch.cuda.Stream()
         opt.stream = self._stream.cuda_stream
+        self._handle.stream = self._stream
         torch.cuda.current_stream().synchronize()
         st = self.lib.ripple_create(ctypes.byref(g), fptr, fmem, layers, self.L, int(model.agg),
                                     ctypes.byref(opt), ctypes.byref(self.h))
         if st != OK:
             msg = self.lib.ripple_last_error(None).decode()
-            self.h = ctypes.c_void_p(None)
+            self.h.value = None
             raise RippleError(st, msg)
 
     # ---- lifetime ------------------------------------------------------------------------
     def close(self):
-        if getattr(self, "h", None) and self.h.value:
-            self.lib.ripple_destroy(self.h)
-            self.h = ctypes.c_void_p(None)
-
-    def __del__(self):
-        try:
-            self.close()
-        except Exception:
-            pass
+        self._views.clear()
+        self._handle.close()
 
     def _check(self, st: int):
         if st != OK:
@@ -317,7 +335,7 @@ class Ripple:
                 n, uptr = ups.shape[0], ups.data_ptr()
             else:
                 ups = np.ascontiguousarray(ups, dtype=UPDATE_DTYPE)
-                n, uptr = ups.size, ups.ctypes.data
+                n, uptr = ups.size, _addr(ups)
             mem = MEM_HOST
             if feat_rows is None:
                 nr, fptr = 0, None
@@ -325,7 +343,7 @@ class Ripple:
                 nr, fptr = feat_rows.shape[0], feat_rows.data_ptr()
             else:
                 feat_rows = np.ascontiguousarray(feat_rows, dtype=np.float32)
-                nr, fptr = feat_rows.shape[0], feat_rows.ctypes.data
+                nr, fptr = feat_rows.shape[0], _addr(feat_rows)
         if op_weights is None:
             self._check(self.lib.ripple_apply_batch(self.h, uptr, n, fptr, nr, mem))
             return
@@ -336,7 +354,7 @@ class Ripple:
             wptr = op_weights.data_ptr()
         else:
             op_weights = np.ascontiguousarray(op_weights, dtype=np.float32)
-            wptr = op_weights.ctypes.data
+            wptr = _addr(op_weights)
         assert op_weights.shape[0] == n
         self._check(self.lib.ripple_apply_batch_weighted(self.h, uptr, n, fptr, nr, wptr, mem))
 
@@ -346,6 +364,7 @@ class Ripple:
     def reserve_vertices(self, n: int) -> None:
         """Raises the id capacity to n: the new ids are isolated vertices with zero features.  Views
         obtained earlier (embeddings, aggregate, affected, degrees) are invalid afterwards."""
+        self._views.clear()
         self._check(self.lib.ripple_reserve_vertices(self.h, int(n)))
         self.n = int(n)
 
@@ -353,14 +372,21 @@ class Ripple:
         self._check(self.lib.ripple_recompute_full(self.h))
 
     # ---- read-out (borrowed device memory, valid until the next apply / recompute / close) ----
-    def _matrix(self, fn, layer: int, width: int):
+    # Wrapping device memory as a tensor takes several microseconds, a good part of the smallest batches' time, so
+    # each buffer is wrapped once; callers get aliases.
+    def _view(self, key, make):
+        t = self._views.get(key)
+        if t is None:
+            t = self._views[key] = self._torch.as_tensor(make(), device="cuda")
+        return t.detach()
+
+    def _make_matrix(self, fn, layer: int, width: int):
         ptr, ld = ctypes.c_void_p(), ctypes.c_int64()
         self._check(fn(self.h, layer, ctypes.byref(ptr), ctypes.byref(ld)))
-        arr = _DevArray(ptr.value, (self.n, width), "<f4", strides=(4 * ld.value, 4), owner=self)
-        return self._torch.as_tensor(arr, device="cuda")
+        return _DevArray(ptr.value, (self.n, width), "<f4", strides=(4 * ld.value, 4), owner=self._handle)
 
     def embeddings(self, layer: int):
-        return self._matrix(self.lib.ripple_get_embeddings, layer, self.dims[layer])
+        return self._view(("H", layer), lambda: self._make_matrix(self.lib.ripple_get_embeddings, layer, self.dims[layer]))
 
     def aggregate(self, layer: int):
         """(tensor view N x width, transformed): the cached aggregate of `layer`; if transformed,
@@ -369,21 +395,20 @@ class Ripple:
         width, tr = ctypes.c_int32(), ctypes.c_int32()
         self._check(self.lib.ripple_get_aggregate(self.h, layer, ctypes.byref(ptr), ctypes.byref(ld),
                                                   ctypes.byref(width), ctypes.byref(tr)))
-        arr = _DevArray(ptr.value, (self.n, width.value), "<f4", strides=(4 * ld.value, 4), owner=self)
+        arr = _DevArray(ptr.value, (self.n, width.value), "<f4", strides=(4 * ld.value, 4), owner=self._handle)
         return self._torch.as_tensor(arr, device="cuda"), bool(tr.value)
 
     def affected(self, layer: int):
         ptr, cnt = ctypes.c_void_p(), ctypes.c_int64()
         self._check(self.lib.ripple_get_affected(self.h, layer, ctypes.byref(ptr), ctypes.byref(cnt)))
-        if cnt.value == 0:
-            return self._torch.zeros(0, dtype=self._torch.int32, device="cuda")
-        return self._torch.as_tensor(_DevArray(ptr.value, (cnt.value,), "<i4", owner=self), device="cuda")
+        return self._view(("A", layer), lambda: _DevArray(ptr.value, (self.n,), "<i4", owner=self._handle))[: cnt.value]
 
     def degrees(self):
-        po, pi = ctypes.c_void_p(), ctypes.c_void_p()
-        self._check(self.lib.ripple_get_degrees(self.h, ctypes.byref(po), ctypes.byref(pi)))
-        mk = lambda p: self._torch.as_tensor(_DevArray(p.value, (self.n,), "<i4", owner=self), device="cuda")
-        return mk(po), mk(pi)
+        def make(which):
+            po, pi = ctypes.c_void_p(), ctypes.c_void_p()
+            self._check(self.lib.ripple_get_degrees(self.h, ctypes.byref(po), ctypes.byref(pi)))
+            return _DevArray((po, pi)[which].value, (self.n,), "<i4", owner=self._handle)
+        return self._view("deg_out", lambda: make(0)), self._view("deg_in", lambda: make(1))
 
     def export_graph(self) -> Tuple[np.ndarray, np.ndarray]:
         """Canonical CSR over out-edges (host arrays): rowptr[N+1], col ascending per row."""
