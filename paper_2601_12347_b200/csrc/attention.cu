@@ -79,13 +79,14 @@ k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* 
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2, nqh = ld_h >> 2;
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
     const int qden = d >> 2, cden = d & 3;   // the denominator's place in the row
-    for (int64_t e0 = (int64_t)warp * ATT_CHUNK; e0 < E; e0 += (int64_t)nwarps * ATT_CHUNK) {
-        const int64_t e1 = min(e0 + ATT_CHUNK, E);
+    TicketWalk walk(&ctl->walk_ticket[l], E, ATT_CHUNK, 4 * ATT_CHUNK);
+    for (; walk.has(); walk.advance()) {
+        const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
+        walk.take();
         int i = upper_row(coff, nC, e0);
         int64_t e = e0;
         while (e < e1) {
@@ -304,13 +305,14 @@ k_att_gather(Ctl* ctl, int l, const int2* __restrict__ items, Side in, const flo
     pdl_enter();
     if (ctl->abort) return;
     const int n = ctl->rebuild_items[l];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2, nqh = ld_h >> 2;
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
     const int qden = d >> 2, cden = d & 3;
-    for (int it = warp; it < n; it += nwarps) {
-        const int v = items[it].x, ch = items[it].y;
+    TicketWalk walk(&ctl->hub_ticket[l], n, 1, 1);
+    for (; walk.has(); walk.advance()) {
+        const int v = items[walk.at].x, ch = items[walk.at].y;
+        walk.take();
         const int deg = in.deg[v];
         const int j_begin = ch * ATT_GATHER, j_end = min(deg, j_begin + ATT_GATHER);
         const int64_t base = in.start[v];

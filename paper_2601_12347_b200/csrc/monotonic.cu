@@ -343,13 +343,14 @@ k_max_messages(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int32
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
     const unsigned group = LPR == 32 ? FULL : (((1u << LPR) - 1u) << (sub * LPR));
-    for (int64_t e0 = (int64_t)warp * MAX_CHUNK; e0 < E; e0 += (int64_t)nwarps * MAX_CHUNK) {
-        const int64_t e1 = min(e0 + MAX_CHUNK, E);
+    TicketWalk walk(&ctl->walk_ticket[l], E, MAX_CHUNK, 4 * MAX_CHUNK);
+    for (; walk.has(); walk.advance()) {
+        const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
+        walk.take();
         int i = upper_row(coff, nC, e0);
         int64_t e = e0;
         while (e < e1) {

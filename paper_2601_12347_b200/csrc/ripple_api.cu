@@ -46,6 +46,14 @@ __global__ void k_ctl_reset(Ctl* ctl, int n_ops, int n_rows) {
     d_ctl_reset(ctl, n_ops, n_rows);
 }
 
+// The device's first access to a page of host memory takes tens of microseconds: taken here, at creation, for the staging
+// area and the control block's copy, instead of in the first batch.
+__global__ void k_touch_host(const char* stage, size_t bytes, volatile int* ctl_host) {
+    int x = 0;
+    for (size_t i = (size_t)threadIdx.x * 4096; i < bytes; i += (size_t)blockDim.x * 4096) x |= *(volatile const char*)(stage + i);
+    if (threadIdx.x == 0) *ctl_host = x & 0;
+}
+
 static void destroy_ctx(Ctx* c) {
     if (!c) return;
     cudaSetDevice(c->device);
@@ -222,6 +230,8 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         max_prepare();
         CK(cudaMallocHost(&c->ctl_host, sizeof(Ctl)));
         memset(c->ctl_host, 0, sizeof(Ctl));
+        memset(c->stage_host, 0, c->stage_bytes);
+        k_touch_host<<<1, 256, 0, c->stream>>>(c->stage_host, c->stage_bytes, reinterpret_cast<volatile int*>(c->ctl_host));
         c->n_words = (N + 31) / 32;
         c->n_tile_sums = std::max(div_up(N, 1024) + 2, div_up(c->n_words, 256) + 2);
         CK(dev_alloc(&c->tile_sums, (size_t)c->n_tile_sums, 0));

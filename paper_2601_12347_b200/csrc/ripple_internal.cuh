@@ -64,6 +64,8 @@ struct Ctl {
     int n_rebuilt[RP_MAXL + 1];       // aggregate rows of hop l gathered anew because their rounding budget ran out
     int rebuild_items[RP_MAXL + 1];   // (vertex, chunk) work items of the long rows among them
     int max_items[RP_MAXL + 1];       // max / min: (long row, chunk) work items of hop l's recomputation
+    int walk_ticket[RP_MAXL + 1];     // walk of the senders' out-lists: next unassigned chunk (see OutWalk)
+    int hub_ticket[RP_MAXL + 1];      // chunks of long in-lists: next unassigned work item
     int regather_ticket[RP_MAXL + 1]; // rebuilding form: next unassigned position of A_l
     int gather_ticket[RP_MAXL + 1];   // gathering form of the delta scatter: next unassigned position of A_l
     int gather_long_ticket[RP_MAXL + 1];  // ... and next unassigned work item of the long in-lists

@@ -146,14 +146,16 @@ k_spmm_pull(int N, Side in, const int32_t* __restrict__ deg_out, int src_norm,
 template <int NV, int LPR, int CHUNK = SPMM_HUB_CHUNK>
 __global__ void __launch_bounds__(256)
 k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const float* __restrict__ M, int ld,
-            float* S, const int2* __restrict__ items, const int* __restrict__ n_items) {
+            float* S, const int2* __restrict__ items, const int* __restrict__ n_items, int* ticket) {
     pdl_enter();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
     const int sub = lane / LPR, ql = lane % LPR;
     const int n = *n_items;
-    for (int it = warp; it < n; it += nwarps) {
-        const int2 w = items[it];
+    if (n == 0) return;
+    TicketWalk walk(ticket, n, 1, 1);
+    for (; walk.has(); walk.advance()) {
+        const int2 w = items[walk.at];
+        walk.take();
         const int deg = in.deg[w.x];
         float4 acc[NV];
 #pragma unroll
@@ -186,7 +188,7 @@ void spmm_full(Ctx* c, int l) {
         RP_LAUNCH(c, (k_spmm_pull<NV, LPR>), grid, T, 0, c->N, c->side[1], c->side[0].deg, (int)c->src_norm, M,   \
                   ld, c->S[l], items, n_items, &c->ctl->regather_ticket[l]);                                      \
         RP_LAUNCH(c, (k_spmm_hubs<NV, LPR>), grid, T, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld,     \
-                  c->S[l], items, n_items);                                                                        \
+                  c->S[l], items, n_items, &c->ctl->hub_ticket[l]);                                                \
     } while (0)
     RP_WIDTH_DISPATCH(ld, SPMM);
 #undef SPMM
@@ -195,7 +197,7 @@ void spmm_full(Ctx* c, int l) {
 // ---------------------------------------------------------------------------------------------
 // push scatter
 // ---------------------------------------------------------------------------------------------
-constexpr int PUSH_CHUNK = 64;  // edges per warp work item
+constexpr int PUSH_CHUNK = 64, PUSH_CHUNK_LARGE = 256;  // edges per warp work item
 
 template <int NV, int LPR>
 __global__ void __launch_bounds__(256)
@@ -206,12 +208,13 @@ k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
-    for (int64_t e0 = (int64_t)warp * PUSH_CHUNK; e0 < E; e0 += (int64_t)nwarps * PUSH_CHUNK) {
-        const int64_t e1 = min(e0 + PUSH_CHUNK, E);
+    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE);
+    for (; walk.has(); walk.advance()) {
+        const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
+        walk.take();
         int i = upper_row(coff, nC, e0);
         int64_t e = e0;
         while (e < e1) {
@@ -274,13 +277,14 @@ k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, cons
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id();
     int msg_of[NI], slot_of[NI];
 #pragma unroll
     for (int i = 0; i < NI; ++i) { msg_of[i] = (32 * i + lane) / NQ; slot_of[i] = (32 * i + lane) % NQ; }
-    for (int64_t e0 = (int64_t)warp * PUSH_CHUNK; e0 < E; e0 += (int64_t)nwarps * PUSH_CHUNK) {
-        const int64_t e1 = min(e0 + PUSH_CHUNK, E);
+    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE);
+    for (; walk.has(); walk.advance()) {
+        const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
+        walk.take();
         int i = upper_row(coff, nC, e0);
         int64_t e = e0;
         while (e < e1) {
@@ -817,7 +821,7 @@ void fold_deltas(Ctx* c, int l) {
     if (!c->Eb[l]) return;
 #define HUBS(NV, LPR)                                                                                              \
     RP_LAUNCH(c, (k_spmm_hubs<NV, LPR, SPMM_ANEW_CHUNK>), c->n_sm * 8, 256, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld, \
-              c->S[l], items, &c->ctl->rebuild_items[l])
+              c->S[l], items, &c->ctl->rebuild_items[l], &c->ctl->hub_ticket[l])
     RP_WIDTH_DISPATCH(ld, HUBS);
 #undef HUBS
 }
@@ -899,7 +903,7 @@ void regather_layer(Ctx* c, int l) {
         RP_LAUNCH(c, (k_regather<NV, LPR>), grid, T, 0, c->ctl, l, c->A[l], c->side[1], c->side[0].deg,           \
                   (int)c->src_norm, M, ld, c->S[l], items, n_items, c->Eb[l]);                                     \
         RP_LAUNCH(c, (k_spmm_hubs<NV, LPR>), grid, T, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld,     \
-                  c->S[l], items, n_items);                                                                        \
+                  c->S[l], items, n_items, &c->ctl->hub_ticket[l]);                                                \
     } while (0)
     RP_WIDTH_DISPATCH(ld, REGATHER);
 #undef REGATHER
