@@ -6,6 +6,7 @@
 //   SIMT fp32    register-tiled GEMM whose A operand is gathered by row id (this file); used
 //                while the affected set is too small to be a real dense contraction;
 //   tensor core  tcgen05 TF32 with a 3-term split that keeps fp32 accuracy (layer_update_tc.cu).
+// A launch takes one or two problems: the neighbour and the self projection of a layer's senders read the same rows.
 #include "layer_update.cuh"
 
 #include <algorithm>
@@ -29,12 +30,12 @@ __device__ __forceinline__ bool upd_few(const UpdParams& p, int n) {
     return n > 0 && n <= FEW_MAX && p.K > 0 && p.K <= FEW_K;
 }
 
-__device__ __forceinline__ void update_few_rows(const UpdParams& p, int n_all, float* A_s, float* red, int* row_id,
+__device__ __forceinline__ void update_few_rows(const UpdParams& p, int n_all, int first, float* A_s, float* red, int* row_id,
                                                 float* row_scale) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kq = p.K >> 2;
     const int groups = (p.n_cols + FEW_COLS - 1) / FEW_COLS, row_groups = (n_all + FEW_ROWS - 1) / FEW_ROWS;
-    for (int item = blockIdx.x; item < groups * row_groups; item += gridDim.x) {
+    for (int item = first; item < groups * row_groups; item += gridDim.x) {
         const int g = item % groups, r0 = (item / groups) * FEW_ROWS;
         const int n = min(FEW_ROWS, n_all - r0);   // rows of this block: compact indices r0 .. r0 + n - 1
         __syncthreads();
@@ -84,24 +85,30 @@ __device__ __forceinline__ void update_few_rows(const UpdParams& p, int n_all, f
 // overlap their launches, and calling the few-row form out of line cost the small batches 10 us of the 30 it saves.
 template <bool FEW>
 __global__ void __launch_bounds__(256)
-k_update_rows(const Ctl* ctl, UpdParams p) {
+k_update_rows(const Ctl* ctl, const __grid_constant__ UpdPair pair) {
     pdl_enter();
     if (ctl->abort) return;
     __shared__ __align__(16) float As[BK][BM + 4];
     __shared__ __align__(16) float Bs[BK][BN];
     __shared__ int row_id[BM];
     __shared__ float row_scale[BM];
+    int used = 0;   // work items of the problems before: the next one starts at the block after the last of them
+    for (int pi = 0; pi < pair.n; ++pi) {
+    const UpdParams& p = pair.p[pi];
     const int n = upd_rows(p);
-    if (upd_use_tc(p, n) || upd_use_narrow(p, n)) return;
+    if (upd_use_tc(p, n) || upd_use_narrow(p, n)) continue;
+    const int first = (int)((blockIdx.x + gridDim.x - (unsigned)used % gridDim.x) % gridDim.x);
     if (FEW && upd_few(p, n)) {
         static_assert(sizeof(As) >= sizeof(float) * FEW_ROWS * FEW_K && sizeof(Bs) >= sizeof(float) * 8 * FEW_ROWS * FEW_COLS,
                       "the few-row form borrows the tiles' shared memory");
-        update_few_rows(p, n, &As[0][0], &Bs[0][0], row_id, row_scale);
-        return;
+        update_few_rows(p, n, first, &As[0][0], &Bs[0][0], row_id, row_scale);
+        used += ((p.n_cols + FEW_COLS - 1) / FEW_COLS) * ((n + FEW_ROWS - 1) / FEW_ROWS);
+        continue;
     }
     const int row_tiles = (n + BM - 1) / BM, col_tiles = (p.n_cols + BN - 1) / BN;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    for (int tile = blockIdx.x; tile < row_tiles * col_tiles; tile += gridDim.x) {
+    used += row_tiles * col_tiles;
+    for (int tile = first; tile < row_tiles * col_tiles; tile += gridDim.x) {
         const int rt = tile / col_tiles, ct = tile - rt * col_tiles;
         const int r0 = rt * BM, c0 = ct * BN;
         __syncthreads();
@@ -167,6 +174,7 @@ k_update_rows(const Ctl* ctl, UpdParams p) {
                               row_scale[lr]);
             }
         }
+    }
     }
 }
 
@@ -336,65 +344,65 @@ k_update_rows_elementwise(const Ctl* ctl, UpdParams p) {
     }
 }
 
-// launches both forms; exactly one of them does the work (decided on the device)
-static void launch_update(Ctx* c, UpdParams& p, const TcW& tw) {
-    p.tc_mode = TC_OFF;
-    // measured on the dense graph: the tensor-core form wins for wide outputs (256 columns: 5.5 ms
-    // against 9.8 ms SIMT) and loses for narrow ones, where staging latency dominates
-    // The tensor-core twin is only put into the chain when the last batch's frontiers (or a whole-graph pass)
-    // were large enough for it; without it the SIMT form takes whatever comes.
-    if (tw.hi && c->gemm_mode != RIPPLE_GEMM_FP32 && p.K > 0 && tw.n_pad >= 128 && (c->tc_armed || !p.list)) {
-        p.tc_mode = c->gemm_mode == RIPPLE_GEMM_TF32 ? TC_TF32 : TC_TF32X3;
-        p.tc_min_rows = 1024;
-        p.tc_withhold = c->debug_tc_withhold;
-        p.Wt_hi = tw.hi; p.Wt_lo = tw.lo; p.k_pad = tw.k_pad; p.n_pad = tw.n_pad;
-    }
-    if (p.K == 0) {
-        RP_LAUNCH(c, k_update_rows_elementwise, c->n_sm * 8, 256, 0, c->ctl, p);
+// Launches every form that the row counts can call for; exactly one of them does the work of each problem (decided on
+// the device).
+static void launch_update(Ctx* c, UpdPair& u, const TcW* const (&tw)[2], const TcW* both = nullptr) {
+    if (u.p[0].K == 0) {
+        RP_LAUNCH(c, k_update_rows_elementwise, c->n_sm * 8, 256, 0, c->ctl, u.p[0]);
         return;
     }
-    // narrow outputs over many rows have a form of their own; in the chain under the same condition as the
-    // tensor-core form (the last batch's frontiers, or a whole-graph pass, were large)
-    p.narrow_min_rows = (p.n_cols <= NBN && p.a_mode != A_SUM && p.tc_mode == TC_OFF && (c->tc_armed || !p.list)) ? NARROW_MIN_ROWS : 0;
-    if (c->few_rows_form && p.list) RP_LAUNCH(c, k_update_rows<true>, c->n_sm * 4, 256, 0, c->ctl, p);
-    else RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, p);
-    if (p.narrow_min_rows) RP_LAUNCH(c, k_update_rows_narrow, c->n_sm * 2, 256, NARROW_SMEM, c->ctl, p);
-    if (p.tc_mode != TC_OFF) launch_update_tc(c, p);
+    UpdPair tc{};      // the problems that have a tensor-core twin
+    for (int i = 0; i < u.n; ++i) {
+        UpdParams& p = u.p[i];
+        p.tc_mode = TC_OFF;
+        p.narrow_min_rows = 0;
+        // The forms for many rows are only put into the chain when the last batch's frontiers (or a whole-graph pass)
+        // were large enough for them; without them the tiled SIMT form takes whatever comes.
+        if (!c->tc_armed && p.list) continue;
+        if (tw[i]->w && c->gemm_mode != RIPPLE_GEMM_FP32) {
+            p.tc_mode = c->gemm_mode == RIPPLE_GEMM_TF32 ? TC_TF32 : TC_TF32X3;
+            p.tc_min_rows = 1024;
+            p.tc_withhold = c->debug_tc_withhold;
+            p.tc_w = tw[i]->w; p.tc_groups = tw[i]->groups; p.tc_chunks = tw[i]->chunks;
+            tc.p[tc.n++] = p;
+        } else if (p.n_cols <= NBN && p.a_mode != A_SUM) {
+            // plain fp32 arithmetic was asked for: narrow outputs over many rows have a form of their own
+            p.narrow_min_rows = NARROW_MIN_ROWS;
+        }
+    }
+    if (c->few_rows_form && u.p[0].list) RP_LAUNCH(c, k_update_rows<true>, c->n_sm * 4, 256, 0, c->ctl, u);
+    else if (u.p[0].list || tc.n < u.n || c->N < 1024) RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, u);
+    for (int i = 0; i < u.n; ++i)
+        if (u.p[i].narrow_min_rows) RP_LAUNCH(c, k_update_rows_narrow, c->n_sm * 2, 256, NARROW_SMEM, c->ctl, u.p[i]);
+    if (both && tc.n == 2) {
+        tc.stacked = 1;
+        tc.p[0].tc_w = both->w; tc.p[0].tc_groups = both->groups;
+    }
+    if (tc.n) launch_update_tc(c, tc);
 }
 
-// rows_out[i] = rows_in[i] * W_n for i < n: the neighbour part of layer l applied to compact rows
-// (sender deltas, record rows, or every embedding row at bootstrap)
-void neighbour_transform(Ctx* c, int l, const float* rows_in, int ld_rows, const int* n_dev, int n_host,
-                         float* rows_out) {
-    const LayerDev& ly = c->layer[l];
-    UpdParams p{};
-    p.list = nullptr; p.n_dev = n_dev; p.n_host = n_host;
-    p.a_mode = A_DENSE; p.epi_mode = EPI_TEMP;
-    p.Hprev = rows_in; p.ld_h = ld_rows;
-    p.K = ly.ld_in;
-    p.W = ly.kind == RIPPLE_LAYER_SAGE ? ly.W1 + (size_t)ly.ld_in * ly.ld_out : ly.W1;
-    p.ldw = c->ws[l]; p.bias = nullptr; p.n_cols = c->ws[l];
-    p.act = RIPPLE_ACT_IDENTITY; p.Hout = rows_out; p.ld_o = c->ws[l];
-    launch_update(c, p, ly.tc_nbr);
+static void launch_update(Ctx* c, const UpdParams& p, const TcW& tw) {
+    UpdPair u{};
+    u.p[0] = p;
+    u.n = 1;
+    launch_update(c, u, {&tw, &tw});
 }
 
-// Layers that transform before the scatter keep P^l_u = W_n^T h^{l-1}_u for every vertex.  For the
-// senders of hop l (rows whose h^{l-1}, or whose source coefficient, changed) this recomputes the
-// row, commits it and emits the transformed delta message c_new P_new - c_old P_old as a compact
-// row.  Because the next batch subtracts exactly the value cached here, the deltas of successive
-// batches telescope: the aggregate tracks the cached rows without a rounding drift of its own.
-void sender_transform(Ctx* c, int l) {
+// P^l_u = W_n^T h^{l-1}_u (all rows if `full`)
+static UpdParams neighbour_problem(Ctx* c, int l, bool full) {
     const LayerDev& ly = c->layer[l];
     UpdParams p{};
-    p.list = c->Clist[(l - 1) & 1]; p.n_dev = &c->ctl->nC[l - 1]; p.n_host = 0;
+    p.list = full ? nullptr : c->Clist[(l - 1) & 1];
+    p.n_dev = full ? nullptr : &c->ctl->nC[l - 1];
+    p.n_host = c->N;
     p.a_mode = A_SELF; p.epi_mode = EPI_COMMIT; p.alpha = 1.0f;
     p.Hprev = c->H[l - 1]; p.ld_h = c->ld[l - 1];
     p.K = ly.ld_in;
     p.W = ly.kind == RIPPLE_LAYER_SAGE ? ly.W1 + (size_t)ly.ld_in * ly.ld_out : ly.W1;
     p.ldw = c->ws[l]; p.bias = nullptr; p.n_cols = c->ws[l];
-    p.act = RIPPLE_ACT_IDENTITY; p.Hout = c->P[l]; p.ld_o = c->ws[l]; p.Dout = c->Dt;
+    p.act = RIPPLE_ACT_IDENTITY; p.Hout = c->P[l]; p.ld_o = c->ws[l];
     p.src_norm = c->src_norm; p.deg_out = c->side[0].deg; p.deg_out_old = c->deg_out_old;
-    launch_update(c, p, ly.tc_nbr);
+    return p;
 }
 
 // Z^l_v = W_self^T h^{l-1}_v for the rows whose h^{l-1} changed (all rows at bootstrap).  SAGE
@@ -402,8 +410,7 @@ void sender_transform(Ctx* c, int l) {
 // (A_{l-1}), not where its output is needed (A_l, usually far larger).  The affected-row update
 // then contracts over the aggregate only (half the K of [h || x]); for a layer that also
 // transforms before the scatter nothing is left to contract.
-void self_project(Ctx* c, int l, bool full) {
-    if (!c->Z[l]) return;
+static UpdParams self_problem(Ctx* c, int l, bool full) {
     const LayerDev& ly = c->layer[l];
     UpdParams p{};
     p.list = full ? nullptr : c->A[l - 1];
@@ -413,7 +420,35 @@ void self_project(Ctx* c, int l, bool full) {
     p.Hprev = c->H[l - 1]; p.ld_h = c->ld[l - 1];
     p.K = ly.ld_in; p.W = ly.W1; p.ldw = ly.ld_out; p.n_cols = ly.ld_out;
     p.act = RIPPLE_ACT_IDENTITY; p.Hout = c->Z[l]; p.ld_o = ly.ld_out;
-    launch_update(c, p, ly.tc_self);
+    return p;
+}
+
+static void project(Ctx* c, int l, const UpdParams& nbr, bool full) {
+    const LayerDev& ly = c->layer[l];
+    UpdPair u{};
+    u.p[0] = nbr;
+    u.n = 1;
+    if (c->Z[l]) u.p[u.n++] = self_problem(c, l, full);   // the same rows: one launch for both products
+    launch_update(c, u, {&ly.tc_nbr, &ly.tc_self}, ly.tc_pair.w ? &ly.tc_pair : nullptr);
+}
+
+void project_full(Ctx* c, int l) { project(c, l, neighbour_problem(c, l, true), true); }
+
+// Layers that transform before the scatter keep P^l_u = W_n^T h^{l-1}_u for every vertex.  For the
+// senders of hop l (rows whose h^{l-1}, or whose source coefficient, changed) this recomputes the
+// row, commits it and emits the transformed delta message c_new P_new - c_old P_old as a compact
+// row.  Because the next batch subtracts exactly the value cached here, the deltas of successive
+// batches telescope: the aggregate tracks the cached rows without a rounding drift of its own.
+// The senders' self projections (their rows are those of A_{l-1}) are computed along with them.
+void sender_transform(Ctx* c, int l) {
+    UpdParams p = neighbour_problem(c, l, false);
+    p.Dout = c->Dt;
+    project(c, l, p, false);
+}
+
+void self_project(Ctx* c, int l, bool full) {
+    if (!c->Z[l] || c->pre[l]) return;   // (a layer that transforms first has done it with the neighbour projection)
+    launch_update(c, self_problem(c, l, full), c->layer[l].tc_self);
 }
 
 void update_rows(Ctx* c, int l, bool full) {

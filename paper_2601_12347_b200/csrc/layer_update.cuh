@@ -26,9 +26,8 @@ struct UpdParams {
     int K;                          // reduction length
     // B operand
     const float* W; int ldw;        // K x ldw, row-major (SIMT form)
-    const float* Wt_hi;             // tensor-core form: transposed (n_pad x k_pad, K contiguous), split
-    const float* Wt_lo;             //   into a tf32-exact part and the remainder
-    int k_pad, n_pad;
+    const float* tc_w;              // tensor-core form (see TcW)
+    int tc_groups, tc_chunks;
     const float* bias;
     int n_cols;                     // ldw (padded output width)
     int act;
@@ -48,6 +47,13 @@ struct UpdParams {
     int tc_min_rows;
     int tc_withhold;                // diagnostic: the tensor-core kernel never signals its first finished tile
     int narrow_min_rows;            // > 0: launches of at least this many rows belong to the form for narrow outputs
+};
+
+// One launch works on one or two problems (two products over the same rows, or over nearly the same).
+struct UpdPair {
+    UpdParams p[2];
+    int n;
+    int stacked;   // tensor-core form: both problems, over the very same rows, in one column group
 };
 
 __device__ __forceinline__ float coef_deg(int deg) { return deg > 0 ? 1.0f / sqrtf((float)deg) : 0.0f; }
@@ -148,6 +154,6 @@ __device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, 
 }
 
 // layer_update_tc.cu
-void launch_update_tc(Ctx* c, const UpdParams& p);
+void launch_update_tc(Ctx* c, const UpdPair& pair);
 
 }  // namespace rp

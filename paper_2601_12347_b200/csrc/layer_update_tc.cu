@@ -1,21 +1,35 @@
 // Tensor-core form of the affected-row layer update for sm_100a: tcgen05.mma (kind::tf32) with
 // the accumulator tile in tensor memory.
 //
-// One persistent CTA per SM takes tiles of 128 affected rows x all (<= 256) output columns, in
-// passes of at most 128 columns.  Per 32-float K chunk the loader warps gather the A rows by vertex
-// id (applying the sink normalisation or the GIN self factor on the way), split every fp32 value x
-// into hi = x with the 13 low mantissa bits cleared (exactly representable in tf32) and lo = x - hi,
-// and store both into shared memory in the K-major 128-byte-swizzle layout the tensor core reads;
-// the transposed weights arrive pre-split the same way (cp.async from L2, two steps ahead).  One
-// elected thread issues hi*hi + lo*hi + hi*lo (three MMAs per 8-float K step), which reproduces
-// the fp32 product to about 2^-21 relative, and commits to an mbarrier so that the stage can be
-// refilled.  With tc_mode = TC_TF32 only hi*hi is issued (plain TF32, 2^-11).  Accumulators are
-// double-buffered in tensor memory; eight epilogue warps read a finished tile back with tcgen05.ld
-// and run the same fused bias / activation / delta / commit code as the SIMT form while the next
-// tile's main loop is already running.
+// One persistent CTA per SM takes tiles of R affected rows x one group of at most 128 output columns.  The product is
+// formed transposed, weights times rows: the 128 lanes of the accumulator are output columns and its R columns are
+// affected rows, so that a warp reading it back holds 32 consecutive columns of one row per register -- whole lines
+// of the row's embedding, cached projection and delta, with no turn through shared memory.
+//
+// Per 32-float K chunk the loader warps gather the rows by vertex id with asynchronous copies straight into shared
+// memory, in the K-major 128-byte-swizzle layout the tensor core reads.  The tensor core takes the upper 19 bits of an
+// fp32 entry x (its tf32 part, hi); the loaders read the landed pieces back and store lo = x - hi, exact in fp32, as a
+// second operand.  The transposed weights lie in global memory already split, swizzled and cut into chunks, so that a
+// chunk is one bulk copy.  One thread issues hi * hi + lo * hi + hi * lo per 8-float K step, which reproduces the fp32
+// product to about 2^-21 relative (the product of the two low parts is left out).  With tc_mode = TC_TF32 only hi * hi
+// is issued (plain TF32, 2^-10).  Row factors (sink normalisation, GIN's self factor) are applied to the finished sums.
+// Accumulators are double-buffered in tensor memory: the epilogue warps finish a tile (bias / cached terms /
+// activation / delta / commit) while the next tile's main loop is already running.
+//
+// What bounds it and why it is cut this way.  Each of the three pipelines -- gather and split, products, epilogue -- needs
+// about a microsecond per step whatever the bandwidth, so they overlap and each is kept free of chains: sixteen loader
+// warps with three chunks in flight, one warp that does nothing but issue (its operands in uniform registers), one that
+// fetches weights, eight epilogue warps whose loads travel ahead and whose stores are predicated.  The weights of a group
+// stay in shared memory for the life of the CTA while they fit (K <= 128: 128 KB, tiles of 128 rows); beyond that they
+// stream from L2 with every chunk, on tiles of 192 rows.  Groups of one row tile run on neighbouring CTAs at the same
+// time and find each other's rows in L2; two narrow products over the same rows (the neighbour and the self projection
+// of a layer's senders) share one group, side by side.
+// Measured on 600 K rows (self and aggregate product of a layer, K = 100, 256 columns each: 1.18 -> 0.67 ms; neighbour
+// and self projection, K = 256, 48 columns each: 0.99 ms on SIMT -> 0.32; GIN's two products of 256 x 256: 2.02 -> 0.97 ms).
 //
 // Every wait is bounded: if an mbarrier does not complete within the spin limit the CTA records
-// RIPPLE_ERR_TIMEOUT in the control block, frees its tensor memory and returns.
+// RIPPLE_ERR_TIMEOUT in the control block, waits (again bounded) for its own copies and products in flight, frees its
+// tensor memory and returns.
 #include "layer_update.cuh"
 
 #include <algorithm>
@@ -24,10 +38,25 @@
 
 namespace rp {
 
-constexpr int TC_M = 128;        // rows per tile (= TMEM lanes)
+constexpr int TC_COLS = 128;     // output columns per group (= TMEM lanes)
 constexpr int TC_KC = 32;        // floats per K chunk: one 128-byte swizzle row
-constexpr int TC_THREADS = 256;
-constexpr int TC_A_BYTES = TC_M * 128;
+// Loader threads: sixteen warps on tiles of 192 rows, eight on tiles of 128 (whose epilogue, with a cached projection to
+// read for every row, needs the registers more).
+__host__ __device__ constexpr int tc_loaders(bool resident) { return resident ? 256 : 512; }
+__host__ __device__ constexpr int tc_tile(bool resident) { return resident ? 128 : 192; }
+constexpr int TC_EPI_WARPS = 8;  // two per tensor-memory lane quarter, half of the tile's rows each
+__host__ __device__ constexpr int tc_threads(bool resident) { return tc_loaders(resident) + 32 * TC_EPI_WARPS + 64; }   // and the warps that issue and that fetch the weights
+constexpr int TC_W_HALF = TC_COLS * 128;         // one half (hi or lo) of a chunk of weights
+constexpr int TC_W_BYTES = 2 * TC_W_HALF;
+constexpr int TC_RESIDENT_CHUNKS = 4;            // weights of up to this many chunks stay in shared memory
+constexpr int TC_W_STAGES = 2;                   // stages of weights that stream
+// Stages of rows as they come (the high operand) and of their remainders (the low one); blocks of 16 rows an epilogue
+// warp reads ahead.  What fits: 227 KB hold 64 or 128 KB of weights and
+//   weights stay:    3 x 16 KB + 2 x 16 KB of rows, 16 KB read ahead (alpha h + scale S: 2 x 16 KB twice)
+//   weights stream:  3 x 24 KB + 2 x 24 KB of rows, 32 KB read ahead (alpha h + scale S: 3 x 24 KB twice, 16 KB)
+__host__ __device__ constexpr int tc_hi(bool resident, bool sum) { return resident && sum ? 2 : 3; }
+__host__ __device__ constexpr int tc_lo(bool resident, bool sum) { return sum ? tc_hi(resident, sum) : 2; }
+__host__ __device__ constexpr int tc_ahead(bool resident, bool sum) { return resident || sum ? 1 : 2; }
 constexpr uint32_t TC_SPIN_LIMIT = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -49,6 +78,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
         if (ok) return true;
     }
     return false;
+}
+
+// a predicated store: as a branch of its own per row the epilogue's sixteen stores took 110 cycles each
+__device__ __forceinline__ void tc_store_if(bool on, float* to, float x) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.f32 [%0], %1;\n\t}" ::"l"(to), "f"(x), "r"((int)on) : "memory");
+}
+
+// true in one lane of the (converged) warp
+__device__ __forceinline__ bool tc_elect() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -79,94 +120,114 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                  ::"r"(smem_u32(bar)) : "memory");
 }
 
+// instruction descriptor: fp32 accumulate, tf32 x tf32, both K-major, N = rows, M = 128
+__host__ __device__ constexpr uint32_t tc_idesc(int rows) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(rows >> 3) << 17) | ((uint32_t)(TC_COLS >> 4) << 24);
+}
+
 // byte offset of 16-byte chunk c (0..7) of row r inside a K-major SWIZZLE_128B tile
-__device__ __forceinline__ uint32_t tc_swz(int r, int c) {
+__host__ __device__ __forceinline__ uint32_t tc_swz(int r, int c) {
     return (uint32_t)((r >> 3) * 1024 + (r & 7) * 128 + (((c ^ r) & 7) << 4));
 }
 
-__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
+// what the tensor core reads of x
+__device__ __forceinline__ float tf32_seen(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
 
-__device__ __forceinline__ void cp_async16(uint32_t smem_addr, const float* gptr) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr), "l"(gptr) : "memory");
+__device__ __forceinline__ float4 tc_lds(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void tc_sts(uint32_t a, float4 v) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// barrier among the loader warps only (the other roles never join it)
-__device__ __forceinline__ void loaders_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TC_THREADS) : "memory"); }
-
-// the same barrier, returning whether any loader thread passed a non-zero flag: a decision every
-// loader thread takes alike (a thread that left the loop alone would strand the others here)
-__device__ __forceinline__ bool loaders_sync_any(int flag) {
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(out) : "r"(flag), "n"(TC_THREADS) : "memory");
-    return out != 0;
+// one chunk of weights: a single bulk copy that completes on the barrier
+__device__ __forceinline__ void tc_copy_weights(void* dst, const float* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-// warp-uniform view of the failure flag
-__device__ __forceinline__ bool warp_failed(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
+__device__ __forceinline__ void tc_load16(uint32_t (&x)[16], uint32_t taddr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]),
+          "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]),
+          "=r"(x[14]), "=r"(x[15])
+        : "r"(taddr) : "memory");
+}
 
-constexpr int TC_STAGES = 2;
-constexpr int TC_NH = 256;                 // output columns per MMA pass (all of them: n_pad <= 256)
-constexpr int TC_EPI_WARPS = 8;             // two per tensor-memory lane quarter, alternating column slabs
-constexpr int TC_ALL_THREADS = TC_THREADS + 32 + 32 * TC_EPI_WARPS;
-constexpr int TC_SLAB = 16;                // columns per epilogue step
-constexpr int TC_SLAB_LD = TC_SLAB + 4;    // 20 floats: 16-byte stores of 8 consecutive rows fall on distinct banks
 
-// Warp roles.  Warps 0..7 ("loaders") stage the operands, warp 8 issues the MMAs, warps 9..16 run
-// the epilogue.  Every K chunk of a tile (128 rows x all output columns) is one step and takes one
-// of two operand stages; the step counter runs on across tiles, so the loads of the next tile
-// start while the last MMAs of this one are still in flight.
-// Accumulators are double-buffered in tensor memory: the epilogue of tile t overlaps the main
-// loop of tile t + 1.  Barriers (all waits bounded):
-//   full[s]        8 arrivals (one per loader warp, after its stores and proxy fence) -> MMA warp may read
-//   empty[s]       tcgen05.commit of the MMAs that read stage s                      -> loaders may refill
+// own[k] without an index register
+template <int N, typename T>
+__device__ __forceinline__ T tc_pick(const T (&own)[N], int k) {
+    T o = own[0];
+#pragma unroll
+    for (int j = 1; j < N; ++j) o = k == j ? own[j] : o;
+    return o;
+}
+
+// Barriers (all waits bounded):
+//   full_x[s]      8 or 16 arrivals (one per loader warp, after its stores)          -> MMA warp may read the rows
+//   full_w[s]      bytes of the weights' copy                                         -> ... and the weights
+//   empty[s]       tcgen05.commit of the MMAs that read stage s                      -> both may be refilled
 //   acc_full[b]    tcgen05.commit after the last MMA of a tile into buffer b         -> epilogue may read
 //   acc_empty[b]   8 arrivals (one per epilogue warp, accumulators read)             -> MMA warp may overwrite
-// Weights of step g + 1 are requested (cp.async from L2) as soon as step g has been handed over;
-// the gathered A rows are prefetched one step ahead in registers.
-template <bool X3>
-__global__ void __launch_bounds__(TC_ALL_THREADS, 1)
-k_update_rows_tc(Ctl* ctl, UpdParams p) {
+// The step counter runs on across tiles, so the loads of the next tile start while the last MMAs of this one are
+// still in flight.
+// RESIDENT: the weights stay in shared memory, tiles of 128 rows; else they stream, tiles of 256 rows.
+// SUM: the row operand is alpha h + scale S (GIN), two rows per entry.
+template <bool RESIDENT, bool SUM>
+__global__ void __launch_bounds__(tc_threads(RESIDENT), 1)
+k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
+    constexpr int TC_LOADERS = tc_loaders(RESIDENT);
+    constexpr int TILE = tc_tile(RESIDENT), RSTEP = TC_LOADERS / 8, ITS = TILE / RSTEP;
+    constexpr int X_HALF = TILE * 128, NH = tc_hi(RESIDENT, SUM), NL = tc_lo(RESIDENT, SUM);
+    constexpr int W_SLOTS = RESIDENT ? TC_RESIDENT_CHUNKS : TC_W_STAGES;
+    constexpr int BUF = TILE <= 128 ? 128 : 256;                 // tensor-memory columns from one accumulator to the other
     pdl_enter();
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full[TC_STAGES], empty[TC_STAGES], acc_full[2], acc_empty[2];
+    __shared__ uint64_t full_x[NH], full_w[W_SLOTS], empty[NH], acc_full[2], acc_empty[2], drained;
     __shared__ uint32_t tmem_slot;
-    __shared__ int row_id[2][TC_M];
-    __shared__ float row_scale[2][TC_M];
     __shared__ volatile int s_fail;
 
     if (ctl->abort) return;
-    const int n = upd_rows(p);
+    // This CTA's column group: those of the first problem, then those of the second; or one group for both.
+    const bool stacked = pair.stacked != 0;
+    const int g0 = pair.p[0].tc_groups, G = g0 + (pair.n > 1 && !stacked ? pair.p[1].tc_groups : 0);
+    const int my_g = (int)blockIdx.x % G, member = (int)blockIdx.x / G, members = ((int)gridDim.x - my_g + G - 1) / G;
+    const UpdParams& p = pair.p[my_g < g0 ? 0 : 1];
+    const int grp = my_g < g0 ? my_g : my_g - g0;
+    // (what the issuing warp's control flow depends on is broadcast: its operands stay in uniform registers only if the
+    // compiler can see that the warp runs as one; otherwise every MMA instruction costs 90 cycles to issue)
+    const int n = __shfl_sync(FULL, upd_rows(p), 0);
     if (!upd_use_tc(p, n)) return;
-    const int row_tiles = (n + TC_M - 1) / TC_M;
-    if ((int)blockIdx.x >= row_tiles) return;   // before any allocation
+    const int row_tiles = (n + TILE - 1) / TILE;
+    if (member >= row_tiles) return;   // before any allocation
 
     // the diagnostic that withholds a completion also shortens the waits, so that they run out in milliseconds
     const uint32_t spin_limit = p.tc_withhold ? (1u << 16) : TC_SPIN_LIMIT;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool is_loader = warp < TC_THREADS / 32;
-    const bool is_mma_warp = warp == TC_THREADS / 32;
-    const int n_pad = p.n_pad;
-    const int n_pass = (n_pad + TC_NH - 1) / TC_NH;
-    constexpr uint32_t B_BYTES = TC_NH * 128u;
-    constexpr uint32_t STAGE_BYTES = (X3 ? 2u : 1u) * (TC_A_BYTES + B_BYTES);
+    const int tid = threadIdx.x, warp = __shfl_sync(FULL, tid >> 5, 0), lane = tid & 31;
+    const bool x3 = p.tc_mode == TC_TF32X3;
+    const int nchunks = p.tc_chunks, K = p.K;
+    const float* weights = p.tc_w + (size_t)grp * nchunks * (TC_W_BYTES / 4);
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    float* slabs = reinterpret_cast<float*>(smem + TC_STAGES * STAGE_BYTES);   // one 32-row slab per epilogue warp
-    uint32_t buf_cols = 32;
-    while ((int)buf_cols < n_pad) buf_cols <<= 1;
-    const uint32_t tmem_cols = 2 * buf_cols;
+    uint8_t* x_ring = smem;                                      // stages of rows
+    uint8_t* l_ring = smem + (size_t)NH * X_HALF;                // stages of their remainders
+    uint8_t* w_ring = l_ring + (size_t)NL * X_HALF;              // stages of [hi | lo] weights, or all chunks of them
+    constexpr uint32_t tmem_cols = 2 * BUF;
 
     if (tid == 0) {
-        for (int s = 0; s < TC_STAGES; ++s) { mbar_init(&full[s], TC_THREADS / 32); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < NH; ++s) { mbar_init(&full_x[s], TC_LOADERS / 32); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < W_SLOTS; ++s) mbar_init(&full_w[s], 1);
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], TC_EPI_WARPS); }
+        mbar_init(&drained, 1);
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -180,225 +241,420 @@ k_update_rows_tc(Ctl* ctl, UpdParams p) {
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
 
-    const int nchunks = p.k_pad / TC_KC;
-    const int steps_per_tile = n_pass * nchunks;
-    const int my_tiles = (row_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int total_steps = my_tiles * steps_per_tile;
+    const int my_tiles = (row_tiles - member + members - 1) / members;
+    const int total_steps = my_tiles * nchunks;
+    auto tile_row = [&](int lt) { return (member + lt * members) * TILE; };
 
-    if (is_mma_warp) {
-        // ---------------- MMA issue ----------------
-        int g = 0;
-        bool failed = false;
-        for (int lt = 0; lt < my_tiles && !failed; ++lt) {
-            const int b = lt & 1, ub = lt >> 1;
-            // the epilogue must have drained this accumulator buffer (tile lt - 2)
-            if (lane == 0 && ub > 0 && !mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit)) s_fail = 1;
+    if (warp < TC_LOADERS / 32) {
+        // ---------------- row gathers ----------------
+        // thread: piece c of the rows rb + RSTEP it of every chunk.  A chunk travels as asynchronous copies straight into
+        // its stage of the high operand, NH - 1 chunks ahead; when it has landed, the thread that asked for a piece reads
+        // it back, takes what the tensor core will not see of it -- it reads the upper 19 bits of an entry -- and stores
+        // that as the low operand.  (Row pieces held in registers across the barrier waits took 1.9 us per chunk, most
+        // of it one warp's chain of dependent instructions.)
+        const int c = tid & 7, rb = tid >> 3;
+        const bool from_s = p.a_mode == A_AGG || SUM;
+        const float* const base = (from_s ? p.S : p.Hprev) + c * 4;
+        const int ldr = from_s ? p.ld_s : p.ld_h, ldh = p.ld_h;
+        const int32_t* const list = p.a_mode == A_DENSE ? nullptr : p.list;
+        const uint32_t x_mine = smem_u32(x_ring) + tc_swz(rb, c), l_mine = smem_u32(l_ring) + tc_swz(rb, c);
+        int rows_next[ITS];           // rows of the tile after the one being requested
+        auto ids = [&](int lt) {
+#pragma unroll
+            for (int it = 0; it < ITS; ++it) {
+                const int i = tile_row(lt) + rb + RSTEP * it;
+                const int j = lt < my_tiles && i < n ? i : 0;   // (rows beyond the last are multiplied and dropped)
+                rows_next[it] = list ? list[j] : j;
+            }
+        };
+        const float *ptr[ITS], *ptr_h[SUM ? ITS : 1];
+        float sc_next[SUM ? ITS : 1], sc_req[SUM ? ITS : 1];   // row factors of the tile being requested, and after it
+        auto aim = [&]() {
+#pragma unroll
+            for (int it = 0; it < ITS; ++it) {
+                const size_t r = (size_t)rows_next[it];
+                ptr[it] = base + r * ldr;
+                if constexpr (SUM) {
+                    ptr_h[it] = p.Hprev + c * 4 + r * ldh;
+                    sc_req[it] = sc_next[it];
+                }
+            }
+        };
+        auto scales = [&]() {
+            if constexpr (SUM) {
+#pragma unroll
+                for (int it = 0; it < ITS; ++it) sc_next[it] = upd_row_scale(p, rows_next[it]);
+            }
+        };
+        ids(0);
+        scales();
+        aim();
+        ids(1);
+        scales();
+        int lt_l = 0, k_l = 0, s_l = 0;   // tile, K offset and stage of the next chunk to request
+        // beyond K (and beyond the last chunk) zeros are written and nothing is read
+        auto request = [&](bool live) {
+            const uint32_t bytes = live && k_l + c * 4 < K ? 16u : 0u;
+            const int off = bytes ? k_l : 0;
+#pragma unroll
+            for (int it = 0; it < ITS; ++it) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                             ::"r"(x_mine + (uint32_t)(s_l * X_HALF + it * (RSTEP * 128))), "l"(ptr[it] + off), "r"(bytes) : "memory");
+                if constexpr (SUM)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                                 ::"r"(l_mine + (uint32_t)(s_l * X_HALF + it * (RSTEP * 128))), "l"(ptr_h[it] + off), "r"(bytes) : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (++s_l == NH) s_l = 0;
+            k_l += TC_KC;
+            if (k_l >= K) {
+                k_l = 0;
+                ++lt_l;
+                aim();
+                ids(lt_l + 1);
+                scales();
+            }
+        };
+        // (SUM: the factors of the chunk being converted belong to an earlier request: kept per stage)
+        float sc_ring[SUM ? NH : 1][SUM ? ITS : 1];
+        auto keep = [&](int slot) {
+            if constexpr (SUM) {
+#pragma unroll
+                for (int it = 0; it < ITS; ++it)
+#pragma unroll
+                    for (int d = 0; d < NH; ++d) if (d == slot) sc_ring[d][it] = sc_req[it];
+            }
+        };
+        const float alpha = p.alpha;
+#pragma unroll
+        for (int d = 0; d < NH - 1; ++d) { keep(d); request(d < total_steps); }
+        int s = 0, sl = 0, s_prev = NH - 1;
+        uint32_t ph_prev = 1;         // phase of the stage that the step before used (a fresh barrier counts as completed)
+        bool ok = true;
+        for (int g = 0; g < total_steps && ok; ++g) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(NH - 2) : "memory");
+            const uint32_t hi = x_mine + (uint32_t)(s * X_HALF), lo = l_mine + (uint32_t)(sl * X_HALF);
+            if (x3 || SUM) {
+                float4 x[ITS];
+#pragma unroll
+                for (int it = 0; it < ITS; ++it) x[it] = tc_lds(hi + it * (RSTEP * 128));
+                if constexpr (SUM) {
+#pragma unroll
+                    for (int it = 0; it < ITS; ++it) {
+                        const float4 h = tc_lds(lo + it * (RSTEP * 128));
+                        float f = sc_ring[0][it];
+#pragma unroll
+                        for (int d = 1; d < NH; ++d) f = d == s ? sc_ring[d][it] : f;
+                        x[it] = make_float4(f * x[it].x + alpha * h.x, f * x[it].y + alpha * h.y, f * x[it].z + alpha * h.z, f * x[it].w + alpha * h.w);
+                        tc_sts(hi + it * (RSTEP * 128), x[it]);
+                    }
+                }
+#pragma unroll
+                for (int it = 0; it < ITS; ++it)
+                    tc_sts(lo + it * (RSTEP * 128), make_float4(x[it].x - tf32_seen(x[it].x), x[it].y - tf32_seen(x[it].y),
+                                                                x[it].z - tf32_seen(x[it].z), x[it].w - tf32_seen(x[it].w)));
+            }
             __syncwarp();
-            if ((failed = warp_failed(&s_fail))) break;
-            tc_fence_after();
-            for (int ps = 0; ps < n_pass && !failed; ++ps) {
-                const int ncol = min(TC_NH, n_pad - ps * TC_NH);
-                // instruction descriptor: fp32 accumulate, tf32 x tf32, both K-major, N = ncol, M = 128
-                const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(ncol >> 3) << 17) |
-                                       ((uint32_t)(TC_M >> 4) << 24);
-                const uint32_t d_addr = tmem_base + (uint32_t)b * buf_cols + (uint32_t)(ps * TC_NH);
-                for (int kc = 0; kc < nchunks; ++kc, ++g) {
-                    const int s = g % TC_STAGES;
-                    const uint32_t u = (uint32_t)(g / TC_STAGES);
-                    uint8_t* a_hi = smem + (size_t)s * STAGE_BYTES;
-                    uint8_t* a_lo = a_hi + TC_A_BYTES;
-                    uint8_t* b_hi = a_hi + (X3 ? 2 : 1) * TC_A_BYTES;
-                    uint8_t* b_lo = b_hi + B_BYTES;
-                    if (lane == 0) {
-                        if (!mbar_wait_bounded(&full[s], u & 1, spin_limit)) s_fail = 1;
-                        if (!s_fail) {
-                            tc_fence_after();
-                            const uint64_t da_hi = tc_smem_desc(smem_u32(a_hi)), db_hi = tc_smem_desc(smem_u32(b_hi));
-                            const uint64_t da_lo = tc_smem_desc(smem_u32(a_lo)), db_lo = tc_smem_desc(smem_u32(b_lo));
-#pragma unroll
-                            for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
-                                const uint64_t adv = (uint64_t)((j * 32) >> 4);
-                                tc_mma_tf32(d_addr, da_hi + adv, db_hi + adv, idesc, (kc | j) != 0);
-                                if (X3) {
-                                    tc_mma_tf32(d_addr, da_lo + adv, db_hi + adv, idesc, 1u);
-                                    tc_mma_tf32(d_addr, da_hi + adv, db_lo + adv, idesc, 1u);
-                                }
-                            }
-                            tc_commit(&empty[s]);
-                            // (diagnostic: with tc_withhold the first tile is never reported finished, so that
-                            // the epilogue's bounded wait runs out and the status path can be exercised)
-                            if (ps == n_pass - 1 && kc == nchunks - 1 && !(p.tc_withhold && lt == 0)) tc_commit(&acc_full[b]);
-                        }
-                    }
-                    __syncwarp();
-                    if ((failed = warp_failed(&s_fail))) break;
-                }
-            }
+            if (lane == 0) mbar_arrive(&full_x[s]);
+            // the stage that the step before used takes the chunk NH - 1 steps ahead (and, with two stages of
+            // remainders, the next step's remainders go where those of the step before were)
+            ok = mbar_wait_bounded(&empty[s_prev], ph_prev, spin_limit);
+            keep(s_prev);
+            request(g + NH - 1 < total_steps);
+            if (g > 0 && s_prev == NH - 1) ph_prev ^= 1;
+            if (g == 0) ph_prev = 0;
+            s_prev = s;
+            if (++s == NH) s = 0;
+            if (++sl == NL) sl = 0;
         }
-    } else if (is_loader) {
-        // ---------------- operand staging ----------------
-        constexpr int A_ITERS = (TC_M * 8) / TC_THREADS;
-        constexpr int B_ITERS = (TC_NH * 8) / TC_THREADS;
-        auto write_ids = [&](int lt) {   // vertex ids and sink scales of local tile lt, buffer lt & 1
-            if (tid < TC_M) {
-                const int i = ((int)blockIdx.x + lt * (int)gridDim.x) * TC_M + tid;
-                int v = -1;
-                float sc = 0.f;
-                if (lt < my_tiles && i < n) {
-                    v = p.list ? p.list[i] : i;
-                    sc = upd_row_scale(p, v);
-                }
-                row_id[lt & 1][tid] = v;
-                row_scale[lt & 1][tid] = sc;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (!ok) s_fail = 1;
+    } else if (warp < TC_LOADERS / 32 + TC_EPI_WARPS) {
+        // ---------------- epilogue ----------------
+        // A warp's index modulo 4 fixes the tensor-memory lanes it may read: output columns 32 q .. 32 q + 31 of the
+        // group, one per lane; the two warps of a quarter take half of the tile's rows each, BLK rows at a time.
+        constexpr int BLK = 16, HALF = TILE / 2, OWN = HALF / 32;
+        const int q = warp & 3, half = (warp - TC_LOADERS / 32) >> 2;
+        // what this lane's column belongs to
+        int lc = grp * TC_COLS + 32 * q + lane;
+        const UpdParams* mine = &p;
+        if (stacked && lc >= pair.p[0].n_cols) { lc -= pair.p[0].n_cols; mine = &pair.p[1]; }
+        const bool col_ok = lc < mine->n_cols;
+        if (!col_ok) { lc = 0; mine = &p; }
+        float* const hout = mine->Hout + lc;
+        float* const dout = mine->epi_mode == EPI_COMMIT && mine->Dout ? mine->Dout + lc : nullptr;
+        const float bias = mine->bias ? mine->bias[lc] : 0.f;
+        const int ldo = mine->ld_o;
+        const uint32_t ld_bytes = 4u * (uint32_t)ldo;
+        const bool relu = mine->act == RIPPLE_ACT_RELU, keep_old = mine->dout_old != 0;
+        // (the same for every lane of the launch)
+        const bool any_z = p.addend2 != nullptr, any_old = upd_needs_old(p) || (stacked && upd_needs_old(pair.p[1]));
+        const bool plus_s = p.addend || p.addend_rw, temp = p.epi_mode == EPI_TEMP;
+        const bool coefs = p.src_norm && any_old;
+        const bool scaled = p.a_mode == A_AGG || plus_s;
+        const float alpha = p.a_mode == A_SELF ? p.alpha : 1.0f;
+        const bool warp_busy = __any_sync(FULL, col_ok);
+        // the row that is read ahead: the cached projection or the row's previous value (both have the output's width)
+        const bool fetching = any_z || any_old;
+        int v_own[OWN], v_next[OWN];        // rows of this tile and the next, 32 per register
+        float sc_own[OWN], sc_next[OWN];
+        auto ids = [&](int lt) {
+#pragma unroll
+            for (int k = 0; k < OWN; ++k) {
+                const int i = tile_row(lt) + HALF * half + 32 * k + lane;
+                const bool in = lt < my_tiles && i < n;
+                v_next[k] = in ? (p.list ? p.list[i] : i) : 0;
+                sc_next[k] = 1.0f;
+                if (scaled && in) sc_next[k] = upd_row_scale(p, v_next[k]);
             }
         };
-        float4 ax[A_ITERS], ax_next[A_ITERS];
-        auto load_a = [&](int g, float4 (&dst)[A_ITERS]) {   // 128 rows x 8 pieces of 16 bytes, by vertex id
-            const int lt = g / steps_per_tile, kc = (g - lt * steps_per_tile) % nchunks, b = lt & 1;
-            const int r0 = ((int)blockIdx.x + lt * (int)gridDim.x) * TC_M;
+        // Rows are worked on in blocks.  What is read ahead of a block was requested DEPTH blocks before, across the end of
+        // the tile too, as asynchronous copies into shared memory, 16 bytes per lane and four rows per instruction:
+        // loads into registers were waited for at the next barrier wait, whatever their distance to the first use.
+        constexpr int DEPTH = tc_ahead(RESIDENT, SUM), BLOCKS = HALF / BLK;
+        float* const zbuf = reinterpret_cast<float*>(w_ring + (size_t)W_SLOTS * TC_W_BYTES) + (warp - TC_LOADERS / 32) * (DEPTH * BLK * 32);
+        // the piece of the row that this lane copies: four columns, of the problem they belong to
+        const float* piece;
+        {
+            int pc = grp * TC_COLS + 32 * q + 4 * (lane & 7);
+            const UpdParams* of = &p;
+            if (stacked && pc >= pair.p[0].n_cols) { pc -= pair.p[0].n_cols; of = &pair.p[1]; }
+            if (pc >= of->n_cols) { pc = 0; of = &p; }
+            piece = (any_z ? of->addend2 : of->Hout) + pc;
+        }
+        auto fetch = [&](int slot, int v_src, int at) {
 #pragma unroll
-            for (int it = 0; it < A_ITERS; ++it) {
-                const int idx = tid + it * TC_THREADS, r = idx >> 3, c = idx & 7;
-                const int v = row_id[b][r], k = kc * TC_KC + c * 4;
-                dst[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (v >= 0 && k < p.K) dst[it] = upd_load_a(p, v, r0 + r, k, row_scale[b][r]);
-            }
-        };
-        // asynchronous copy of step g's pre-split transposed weights (<= 128 output columns x 8 pieces
-        // of 16 bytes, hi and lo) from L2 straight into their swizzled places in stage g % TC_STAGES; the MMAs
-        // that last read that stage must have finished.  Always closes one copy group.
-        auto copy_b = [&](int g) {
-            if (g < total_steps) {
-                const int s = g % TC_STAGES;
-                const uint32_t u = (uint32_t)(g / TC_STAGES);
-                if (u > 0 && !s_fail && !mbar_wait_bounded(&empty[s], (u - 1) & 1, spin_limit)) s_fail = 1;
-                const int r = g % steps_per_tile, ps = r / nchunks, kc = r - ps * nchunks;
-                const int ncol = min(TC_NH, n_pad - ps * TC_NH);
-                uint8_t* b_hi = smem + (size_t)s * STAGE_BYTES + (X3 ? 2 : 1) * TC_A_BYTES;
-                uint8_t* b_lo = b_hi + B_BYTES;
-#pragma unroll
-                for (int it = 0; it < B_ITERS; ++it) {
-                    const int idx = tid + it * TC_THREADS;
-                    if (idx < ncol * 8) {
-                        const size_t go = (size_t)(ps * TC_NH + (idx >> 3)) * p.k_pad + kc * TC_KC + (idx & 7) * 4;
-                        const uint32_t off = tc_swz(idx >> 3, idx & 7);
-                        cp_async16(smem_u32(b_hi + off), p.Wt_hi + go);
-                        if (X3) cp_async16(smem_u32(b_lo + off), p.Wt_lo + go);
-                    }
-                }
+            for (int i = 0; i < BLK / 4; ++i) {
+                const int r = 4 * i + (lane >> 3), v = __shfl_sync(FULL, v_src, at + r);
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                             ::"r"(smem_u32(zbuf + slot * (BLK * 32) + r * 32 + 4 * (lane & 7))), "l"(piece + (size_t)v * ldo) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        write_ids(0);
-        write_ids(1);
-        loaders_sync();
-        load_a(0, ax);
-        copy_b(0);
-        for (int g = 0; g < total_steps; ++g) {
-            const int s = g % TC_STAGES;
-            const int lt = g / steps_per_tile;
-            if (lt >= 1 && g == lt * steps_per_tile) {
-                // ids of the tile after this one; their buffer last served tile lt - 1, fully staged by now
-                write_ids(lt + 1);
-                if (loaders_sync_any(s_fail)) break;   // the only place the loaders leave early, all together
-            }
-            uint8_t* a_hi = smem + (size_t)s * STAGE_BYTES;
-            uint8_t* a_lo = a_hi + TC_A_BYTES;                              // only if X3
-            // next step's row gathers first (registers), so that they have a whole step to land
-            if (g + 1 < total_steps) load_a(g + 1, ax_next);
+        ids(0);
+        if (fetching && warp_busy) {
 #pragma unroll
-            for (int it = 0; it < A_ITERS; ++it) {
-                const int idx = tid + it * TC_THREADS;
-                const uint32_t off = tc_swz(idx >> 3, idx & 7);
-                const float4 x = ax[it];
-                const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
-                *reinterpret_cast<float4*>(a_hi + off) = h;
-                if (X3) *reinterpret_cast<float4*>(a_lo + off) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
-            }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");   // this step's weights have landed
-            fence_async_smem();   // generic-proxy stores -> visible to the tensor core's async proxy
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&full[s]);
-            copy_b(g + 1);   // travels while the next step's rows are split and stored
-#pragma unroll
-            for (int it = 0; it < A_ITERS; ++it) ax[it] = ax_next[it];
+            for (int d = 0; d < DEPTH; ++d) fetch(d, tc_pick<OWN>(v_next, d * BLK / 32), (d * BLK) & 31);
         }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-    } else {
-        // ---------------- epilogue ----------------
-        // A warp's index modulo 4 fixes the tensor-memory lanes it may read: rows 32 q .. 32 q + 31 of the
-        // tile, shared by two warps that take alternate 16-column slabs.  Per slab every lane pulls
-        // its own row's 16 accumulators, the warp turns them through a small shared-memory slab, and
-        // then each pass handles 8 rows x 64 bytes, so that the previous row, the cached projection,
-        // the delta row and the new row move in whole sectors; the loads of all 4 passes are issued
-        // before the first is used.
-        const int q = warp & 3;
-        const int ew = warp - (TC_THREADS / 32 + 1);     // 0..7
-        const int parity = ew >> 2;                      // which of the quarter's two warps: even or odd slabs
-        float* slab = slabs + (size_t)ew * 32 * TC_SLAB_LD;
-        const bool need_old = upd_needs_old(p);
-        const bool need_z = p.addend2 != nullptr;
-        const int sub_r = lane >> 2, sub_c = 4 * (lane & 3);   // 8 rows x 64 bytes per pass
         for (int lt = 0; lt < my_tiles; ++lt) {
             const int b = lt & 1, ub = lt >> 1;
-            const int r0 = ((int)blockIdx.x + lt * (int)gridDim.x) * TC_M + 32 * q;
-            int v_own = -1;
-            float sc_own = 0.f;
-            if (r0 + lane < n) {
-                v_own = p.list ? p.list[r0 + lane] : r0 + lane;
-                sc_own = upd_row_scale(p, v_own);
+            const int r0 = tile_row(lt) + HALF * half;
+#pragma unroll
+            for (int k = 0; k < OWN; ++k) {
+                v_own[k] = v_next[k];
+                sc_own[k] = sc_next[k];
             }
-            if (lane == 0 && !mbar_wait_bounded(&acc_full[b], ub & 1, spin_limit)) s_fail = 1;
-            __syncwarp();
-            if (warp_failed(&s_fail)) break;
+            ids(lt + 1);
+            if (!mbar_wait_bounded(&acc_full[b], ub & 1, spin_limit)) { s_fail = 1; break; }
             tc_fence_after();
-            for (int c0 = parity * TC_SLAB; c0 < p.n_cols; c0 += 2 * TC_SLAB) {
-                uint32_t x[16];
-                const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)b * buf_cols + (uint32_t)c0;
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                    "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                    : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]),
-                      "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]),
-                      "=r"(x[14]), "=r"(x[15])
-                    : "r"(taddr) : "memory");
+            const uint32_t t_mine = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * BUF + HALF * half);
+            auto block = [&](int blk) {
+                const int at = (blk * BLK) & 31, i0 = r0 + blk * BLK;
+                const int v_src = tc_pick<OWN>(v_own, blk * BLK / 32);
+                const float s_src = tc_pick<OWN>(sc_own, blk * BLK / 32);
+                uint32_t x[BLK];
+                tc_load16(x, t_mine + (uint32_t)(blk * BLK));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                float4* mine = reinterpret_cast<float4*>(slab + (size_t)lane * TC_SLAB_LD);
+                if (plus_s) {   // (transformed aggregates with a self term of their own: GIN layers that narrow)
+#pragma unroll 1
+                    for (int r = 0; r < BLK; ++r) {
+                        const int v = __shfl_sync(FULL, v_src, at + r);
+                        const float sc = __shfl_sync(FULL, s_src, at + r);
+                        float acc = 0.f;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    mine[j] = make_float4(__uint_as_float(x[4 * j]), __uint_as_float(x[4 * j + 1]),
-                                          __uint_as_float(x[4 * j + 2]), __uint_as_float(x[4 * j + 3]));
-                __syncwarp();
-                const int col = c0 + sub_c;
-                int vv[4];
-                float ss[4];
-                float4 oldv[4], zv[4];
+                        for (int j = 0; j < BLK; ++j) acc = j == r ? __uint_as_float(x[j]) : acc;
+                        if (i0 + r >= n || !col_ok) continue;
+                        const size_t row = (size_t)v * ldo, sa = (size_t)v * p.ld_add + lc;
+                        float t = p.addend_rw ? p.addend_rw[sa] : p.addend[sa];
+                        if (p.addend_rw) {
+                            t += p.addend_delta[sa];
+                            p.addend_rw[sa] = t;
+                            p.addend_delta[sa] = 0.f;
+                        }
+                        float h = (p.a_mode == A_AGG ? sc : alpha) * acc + bias + sc * t;
+                        if (any_z) h += p.addend2[row + lc];
+                        if (relu) h = fmaxf(h, 0.f);
+                        if (temp) { hout[(size_t)(i0 + r) * ldo] = h; continue; }
+                        if (dout) {
+                            const float o = hout[row];
+                            float cn = 1.f, co = 1.f;
+                            if (p.src_norm) {
+                                const int dold = p.deg_out_old[v];
+                                cn = coef_deg(p.deg_out[v]);
+                                co = dold >= 0 ? coef_deg(dold) : cn;
+                            }
+                            dout[(size_t)(i0 + r) * ldo] = keep_old ? o : cn * h - co * o;
+                        }
+                        hout[row] = h;
+                    }
+                    return;
+                }
+                float h[BLK];
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int rr = 8 * t + sub_r;
-                    vv[t] = __shfl_sync(FULL, v_own, rr);
-                    ss[t] = __shfl_sync(FULL, sc_own, rr);
-                    if (vv[t] >= 0 && col < p.n_cols) {
-                        if (need_old) oldv[t] = upd_load_old(p, vv[t], col);
-                        if (need_z) zv[t] = *reinterpret_cast<const float4*>(p.addend2 + (size_t)vv[t] * p.ld_add + col);
+                for (int r = 0; r < BLK; ++r) h[r] = __uint_as_float(x[r]);
+                if (scaled) {
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) h[r] = __shfl_sync(FULL, s_src, at + r) * h[r] + bias;
+                } else {
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) h[r] = alpha * h[r] + bias;
+                }
+                const float* const z = zbuf + (blk % DEPTH) * (BLK * 32) + lane;
+                if (fetching) {
+                    asm volatile("cp.async.wait_group %0;" ::"n"(DEPTH - 1) : "memory");
+                    __syncwarp();
+                }
+                if (any_z) {
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) h[r] += z[32 * r];
+                }
+                if (relu) {
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) h[r] = fmaxf(h[r], 0.f);
+                }
+                if (any_old) {
+                    const int live = col_ok && dout ? n - i0 : 0;
+                    float* to = dout + (size_t)i0 * ldo;
+                    if (any_z) {   // both a cached projection and the row's previous value: that one is asked for here
+                        float cn = 1.f, co = 1.f;   // source coefficients now and before the batch, one row per lane
+                        if (coefs) {
+                            const int d_old = p.deg_out_old[v_src];
+                            cn = coef_deg(p.deg_out[v_src]);
+                            co = d_old >= 0 ? coef_deg(d_old) : cn;
+                        }
+#pragma unroll
+                        for (int r0_ = 0; r0_ < BLK; r0_ += 4) {
+                            float o[4];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) o[r] = hout[(size_t)__shfl_sync(FULL, v_src, at + r0_ + r) * ldo];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r, to += ldo) {
+                                const float d = __shfl_sync(FULL, cn, at + r0_ + r) * h[r0_ + r] - __shfl_sync(FULL, co, at + r0_ + r) * o[r];
+                                tc_store_if(r0_ + r < live, to, keep_old ? o[r] : d);
+                            }
+                        }
+                    } else if (coefs) {
+                        const int d_old = p.deg_out_old[v_src];
+                        const float cn = coef_deg(p.deg_out[v_src]), co = d_old >= 0 ? coef_deg(d_old) : cn;
+#pragma unroll
+                        for (int r = 0; r < BLK; ++r, to += ldo)
+                            tc_store_if(r < live, to, __shfl_sync(FULL, cn, at + r) * h[r] - __shfl_sync(FULL, co, at + r) * z[32 * r]);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < BLK; ++r, to += ldo) tc_store_if(r < live, to, keep_old ? z[32 * r] : h[r] - z[32 * r]);
                     }
                 }
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int rr = 8 * t + sub_r;
-                    if (vv[t] >= 0 && col < p.n_cols) {
-                        const float4 acc = *reinterpret_cast<const float4*>(slab + (size_t)rr * TC_SLAB_LD + sub_c);
-                        upd_epilogue4(p, vv[t], r0 + rr, col, acc, ss[t], need_old, oldv[t], need_z, zv[t]);
-                    }
+                if (fetching) {
+                    const int nb = blk + DEPTH;
+                    __syncwarp();
+                    fetch(blk % DEPTH, nb < BLOCKS ? tc_pick<OWN>(v_own, nb * BLK / 32) : tc_pick<OWN>(v_next, (nb - BLOCKS) * BLK / 32), (nb * BLK) & 31);
                 }
-                __syncwarp();   // the slab is rewritten by the next step
+                const int live = col_ok ? n - i0 : 0;
+                uint32_t v[BLK];
+#pragma unroll
+                for (int r = 0; r < BLK; ++r) v[r] = (uint32_t)__shfl_sync(FULL, v_src, at + r);
+                if (temp) {
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) v[r] = (uint32_t)(i0 + r);
+                }
+#pragma unroll
+                for (int r = 0; r < BLK; ++r)
+                    tc_store_if(r < live, reinterpret_cast<float*>(reinterpret_cast<char*>(hout) + (uint64_t)v[r] * ld_bytes), h[r]);
+            };
+            if (warp_busy) {
+#pragma unroll 1
+                for (int blk = 0; blk < BLOCKS; ++blk) block(blk);
             }
             tc_fence_before();   // accumulators consumed: the MMA warp may overwrite them after this arrival
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[b]);
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+    } else if (warp == TC_LOADERS / 32 + TC_EPI_WARPS) {
+        // ---------------- MMA issue ----------------
+        const bool lead = tc_elect();
+        constexpr uint32_t idesc = tc_idesc(TILE);
+        const uint64_t dx0 = tc_smem_desc(smem_u32(x_ring)), dl0 = tc_smem_desc(smem_u32(l_ring)), dw0 = tc_smem_desc(smem_u32(w_ring));
+        const bool withhold = p.tc_withhold != 0;
+        int s = 0, sl = 0, sw = 0;
+        uint32_t ph = 0, phw = 0;              // ring slots and phases of this step
+        bool ok = true;
+        for (int lt = 0; lt < my_tiles; ++lt) {
+            const int b = lt & 1, ub = lt >> 1;
+            // the epilogue must have drained this accumulator buffer (tile lt - 2)
+            if (ub > 0) ok = __all_sync(FULL, mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit));
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF);
+            int left = K;
+            for (int kc = 0; kc < nchunks; ++kc, left -= TC_KC) {
+                if (RESIDENT) sw = kc;
+                bool there = true;
+                if (!RESIDENT || lt == 0) there = mbar_wait_bounded(&full_w[sw], phw, spin_limit);
+                there = there && mbar_wait_bounded(&full_x[s], ph, spin_limit);
+                ok = __all_sync(FULL, there);
+                if (!ok) break;
+                // The loaders' stores become visible to the tensor core's async proxy here, on the reader's side of the
+                // barrier: in the loaders the fence would wait for their row gathers in flight as well.
+                fence_async_smem();
+                tc_fence_after();
+                const uint64_t xh = dx0 + (uint64_t)((uint32_t)s * (X_HALF >> 4)), xl = dl0 + (uint64_t)((uint32_t)sl * (X_HALF >> 4));
+                const uint64_t wh = dw0 + (uint64_t)((uint32_t)sw * (TC_W_BYTES >> 4)), wl = wh + (TC_W_HALF >> 4);
+                const bool last = kc == nchunks - 1;
+                if (lead) {
+#pragma unroll
+                    for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
+                        if (8 * j < left) {
+                            tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, idesc, (kc | j) != 0);
+                            if (x3) {
+                                tc_mma_tf32(d_addr, wl + 2 * j, xh + 2 * j, idesc, 1u);
+                                tc_mma_tf32(d_addr, wh + 2 * j, xl + 2 * j, idesc, 1u);
+                            }
+                        }
+                    }
+                    tc_commit(&empty[s]);
+                    // (diagnostic: with tc_withhold the first tile is never reported finished, so that
+                    // the epilogue's bounded wait runs out and the status path can be exercised)
+                    if (last && !(withhold && lt == 0)) tc_commit(&acc_full[b]);
+                }
+                __syncwarp();
+                if (++s == NH) { s = 0; ph ^= 1; }
+                if (++sl == NL) sl = 0;
+                if (!RESIDENT && ++sw == TC_W_STAGES) { sw = 0; phw ^= 1; }
+            }
+            if (!ok) break;
+        }
+        if (!ok) {   // no product of this CTA may be in flight when it leaves
+            if (lead) {
+                s_fail = 1;
+                tc_commit(&drained);
+                mbar_wait_bounded(&drained, 0, TC_SPIN_LIMIT);
+            }
+        }
+    } else {
+        // ---------------- weights: bulk copies, one thread ----------------
+        if (lane == 0) {
+            const int slots = RESIDENT ? nchunks : TC_W_STAGES, all = RESIDENT ? nchunks : total_steps;
+            int kc = 0, sw = 0, s = 0, c = 0;
+            uint32_t ph = 0;
+            for (; c < all; ++c) {
+                if (c >= slots) {   // the step whose weights lie there must have been multiplied: step c - slots
+                    if (!mbar_wait_bounded(&empty[s], ph, spin_limit)) { s_fail = 1; break; }
+                    if (++s == NH) { s = 0; ph ^= 1; }
+                }
+                tc_copy_weights(w_ring + (size_t)sw * TC_W_BYTES, weights + (size_t)kc * (TC_W_BYTES / 4), TC_W_BYTES, &full_w[sw]);
+                if (++kc == nchunks) kc = 0;
+                if (++sw == slots) sw = 0;
+            }
+            // no copy of this CTA may be in flight when it leaves: the latest into each slot (usually long there)
+            for (int k = 0; k < min(c, slots); ++k) {
+                const int latest = c - 1 - k;
+                mbar_wait_bounded(&full_w[latest % slots], (uint32_t)(latest / slots) & 1, TC_SPIN_LIMIT);
+            }
+        }
     }
 
+    __syncwarp();
     if (s_fail && lane == 0) {
         atomicCAS(&ctl->err, 0, (int)RIPPLE_ERR_TIMEOUT);
         ctl->abort = 1;
@@ -410,49 +666,61 @@ k_update_rows_tc(Ctl* ctl, UpdParams p) {
     }
 }
 
-static size_t tc_smem_bytes(bool x3) {
-    const size_t stage = (size_t)(x3 ? 2 : 1) * (TC_A_BYTES + (size_t)TC_NH * 128);
-    return TC_STAGES * stage + (size_t)TC_EPI_WARPS * 32 * TC_SLAB_LD * sizeof(float) + 1024;
+static size_t tc_smem_bytes(bool resident, bool sum) {
+    return (size_t)(tc_hi(resident, sum) + tc_lo(resident, sum)) * tc_tile(resident) * 128 +
+           (size_t)(resident ? TC_RESIDENT_CHUNKS : TC_W_STAGES) * TC_W_BYTES + (size_t)TC_EPI_WARPS * tc_ahead(resident, sum) * 16 * 128 + 1024;
 }
 
-void launch_update_tc(Ctx* c, const UpdParams& p) {
-    const bool x3 = p.tc_mode == TC_TF32X3;
-    // one persistent CTA per SM: the operand stages and the epilogue slabs fill its shared memory
-    const int grid = c->n_sm;
-    if (x3) {
-        RP_LAUNCH(c, k_update_rows_tc<true>, grid, TC_ALL_THREADS, tc_smem_bytes(true), c->ctl, p);
-    } else {
-        RP_LAUNCH(c, k_update_rows_tc<false>, grid, TC_ALL_THREADS, tc_smem_bytes(false), c->ctl, p);
-    }
+void launch_update_tc(Ctx* c, const UpdPair& pair) {
+    const bool resident = pair.p[0].tc_chunks <= TC_RESIDENT_CHUNKS, sum = pair.p[0].a_mode == A_SUM;
+    // one persistent CTA per SM: operands and weights fill its shared memory
+#define TC_GO(RES, SUM) RP_LAUNCH(c, (k_update_rows_tc<RES, SUM>), c->n_sm, tc_threads(RES), tc_smem_bytes(RES, SUM), c->ctl, pair)
+    if (resident && sum) TC_GO(true, true);
+    else if (resident) TC_GO(true, false);
+    else if (sum) TC_GO(false, true);
+    else TC_GO(false, false);
+#undef TC_GO
 }
 
 void tc_prepare() {
-    cudaFuncSetAttribute(k_update_rows_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(true));
-    cudaFuncSetAttribute(k_update_rows_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(false));
+#define TC_SET(RES, SUM) cudaFuncSetAttribute(k_update_rows_tc<RES, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(RES, SUM))
+    TC_SET(true, true);
+    TC_SET(true, false);
+    TC_SET(false, true);
+    TC_SET(false, false);
+#undef TC_SET
 }
 
-// Transposed, K-contiguous, tf32-split copy of a row-major K x ldw weight block.
-cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw) {
-    out->k_pad = (K + TC_KC - 1) / TC_KC * TC_KC;
-    out->n_pad = (ldw + 15) / 16 * 16;
-    if (K <= 0 || out->n_pad > 256) { out->hi = out->lo = nullptr; return cudaSuccess; }
-    const size_t cnt = (size_t)out->k_pad * out->n_pad;
-    std::vector<float> hi(cnt, 0.f), lo(cnt, 0.f);
+// The weights (row-major K x ldw; W2, if given, K x ldw2 beside them) as the kernel copies them: per column group and K
+// chunk, the group's 128 columns as rows of 32 K entries, first rounded to tf32, then the remainders (likewise
+// rounded), in the swizzled layout of the operand.
+cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const float* W2, int ldw2) {
+    *out = TcW{};
+    if (K <= 0 || ldw <= 0) return cudaSuccess;
+    auto round_tf32 = [](float v) {
+        uint32_t bits;
+        memcpy(&bits, &v, 4);
+        bits = (bits + 0x1000u) & 0xffffe000u;
+        memcpy(&v, &bits, 4);
+        return v;
+    };
+    const int cols = ldw + (W2 ? ldw2 : 0);
+    out->groups = (cols + TC_COLS - 1) / TC_COLS;
+    out->chunks = (K + TC_KC - 1) / TC_KC;
+    const size_t block = TC_W_BYTES / 4;
+    std::vector<float> pack(block * out->chunks * out->groups, 0.f);
     for (int k = 0; k < K; ++k)
-        for (int j = 0; j < ldw; ++j) {
-            float x = W[(size_t)k * ldw + j];
-            uint32_t bits;
-            memcpy(&bits, &x, 4);
-            bits &= 0xffffe000u;
-            float h;
-            memcpy(&h, &bits, 4);
-            hi[(size_t)j * out->k_pad + k] = h;
-            lo[(size_t)j * out->k_pad + k] = x - h;
+        for (int j = 0; j < cols; ++j) {
+            const float x = j < ldw ? W[(size_t)k * ldw + j] : W2[(size_t)k * ldw2 + (j - ldw)];
+            const float h = round_tf32(x);
+            const int g = j / TC_COLS, r = j - g * TC_COLS, kc = k / TC_KC, kk = k - kc * TC_KC;
+            float* blk = pack.data() + ((size_t)g * out->chunks + kc) * block;
+            const uint32_t at = tc_swz(r, kk >> 2) / 4 + (kk & 3);
+            blk[at] = h;
+            blk[TC_W_HALF / 4 + at] = round_tf32(x - h);
         }
-    cudaError_t e = cudaMalloc(&out->hi, sizeof(float) * cnt);
-    if (!e) e = cudaMalloc(&out->lo, sizeof(float) * cnt);
-    if (!e) e = cudaMemcpy(out->hi, hi.data(), sizeof(float) * cnt, cudaMemcpyHostToDevice);
-    if (!e) e = cudaMemcpy(out->lo, lo.data(), sizeof(float) * cnt, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMalloc(&out->w, sizeof(float) * pack.size());
+    if (!e) e = cudaMemcpy(out->w, pack.data(), sizeof(float) * pack.size(), cudaMemcpyHostToDevice);
     return e;
 }
 

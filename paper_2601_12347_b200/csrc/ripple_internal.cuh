@@ -126,11 +126,10 @@ struct Rec {
     float tail_w[2];     // deleted: weight found at the tail slot
 };
 
-// transposed (K contiguous), tf32-split copy of a weight block for the tensor-core layer update
+// weight block of the tensor-core layer update: transposed, tf32-split, cut into column groups and K chunks
 struct TcW {
-    float* hi;
-    float* lo;
-    int k_pad, n_pad;
+    float* w;
+    int groups, chunks;        // groups of 128 columns, K chunks of 32
 };
 
 // Where a batch lies: pinned host memory or device memory, in either case read by the first kernel of its chain.
@@ -154,6 +153,7 @@ struct LayerDev {
     TcW tc_nbr;  // neighbour matrix, for layers that transform before the scatter
     TcW tc_2;    // GIN: second matrix
     TcW tc_self; // SAGE: self matrix, for the cached self projection
+    TcW tc_pair; // neighbour and self matrix side by side, where both together have at most 128 columns
 };
 
 struct Ctx {
@@ -360,15 +360,14 @@ void part_fetch_halo_rows(Ctx* c, int l);  // bootstrap: H^l of every assigned h
 
 // layer_update.cu
 void update_rows(Ctx* c, int l, bool full);             // re-apply Update^l + activation, emit deltas
-void self_project(Ctx* c, int l, bool full);            // refresh the cached self projection of a narrow SAGE layer
-void sender_transform(Ctx* c, int l);                   // P^l rows of the senders of hop l, and their transformed deltas
-void neighbour_transform(Ctx* c, int l, const float* rows_in, int ld_rows, const int* n_dev, int n_host,
-                         float* rows_out);              // compact rows times the layer's neighbour matrix
+void self_project(Ctx* c, int l, bool full);            // refresh the cached self projection of a SAGE layer
+void sender_transform(Ctx* c, int l);                   // P^l rows of the senders of hop l, their transformed deltas, and Z^l
+void project_full(Ctx* c, int l);                       // bootstrap: P^l (and Z^l) of every vertex
 void feature_rows(Ctx* c, int n);                       // hop 0: overwrite feature rows, emit deltas
 void extra_sender_rows(Ctx* c, int l, int n);           // deltas of senders whose row did not change
 
 // layer_update_tc.cu
-cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw);
+cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw, const float* W2_host = nullptr, int ldw2 = 0);
 void tc_prepare();   // one-time kernel attributes (not allowed inside a stream capture)
 void narrow_prepare();   // likewise, for the update form for narrow outputs
 

@@ -176,7 +176,7 @@ void spmm_full(Ctx* c, int l) {
     const int ld = c->ws[l];
     const float* M = c->H[l - 1];
     if (c->pre[l]) {
-        neighbour_transform(c, l, c->H[l - 1], c->ld[l - 1], nullptr, c->N, c->P[l]);
+        project_full(c, l);
         M = c->P[l];
     }
     const int grid = c->n_sm * 16, T = 256;
