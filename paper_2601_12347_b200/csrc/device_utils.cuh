@@ -97,7 +97,12 @@ struct TicketWalk {
     __device__ __forceinline__ TicketWalk(int* t, long long n, int small, int large) : total(n), ticket(t) {
         const long long warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
         chunk = small;
-        if (n <= nwarps * small) { ticket = nullptr; at = warp * small; return; }
+        if (n <= nwarps * small) {   // (as many warps as there are units for, an eighth of the small chunk at least)
+            ticket = nullptr;
+            chunk = max(max(small >> 3, 1), (int)((n + nwarps - 1) / nwarps));
+            at = warp * chunk;
+            return;
+        }
         if (n > nwarps * large * 2) chunk = large;
         take();
         advance();

@@ -323,8 +323,8 @@ __device__ __forceinline__ void d_plan_growth(Ctl* ctl, const Rec* __restrict__ 
 __device__ __forceinline__ void d_plan_check(Ctl* ctl, Side out, Side in);
 
 // One block per op: winners are compared with the stored graph and become records or no-ops.
-// The last block to finish then plans the row moves (which rows need a new block, and whether the
-// blocks exist): no launch of its own for that.
+// In batches of up to a few hundred operations the last block to finish then plans the row moves (which rows need a new
+// block, and whether the blocks exist): no launch of its own for that.
 // An explicit edge operation that precedes the deletion of one of its endpoints is superseded by
 // it (for stored edges the generated deletion already wins the slot; for pairs that are not stored
 // nothing was generated, hence the explicit test).  Only the caller's operations are counted.
@@ -333,7 +333,7 @@ d_resolve(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_
           const unsigned long long* __restrict__ hwin, const int32_t* __restrict__ op_slot,
           const int32_t* __restrict__ feat_last, const int32_t* __restrict__ vdel_seq, Side out, Side in,
           Rec* rec, uint32_t* bitmap, const float* __restrict__ op_w, int32_t* grow_out, int32_t* grow_in,
-          int32_t* shrink_out, int32_t* shrink_in, const uint8_t* __restrict__ silent) {
+          int32_t* shrink_out, int32_t* shrink_in, const uint8_t* __restrict__ silent, int plan) {
     __shared__ int s_found;
     __shared__ int s_last;
     if (ctl->abort) return;
@@ -379,6 +379,7 @@ d_resolve(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_
             rec[r] = x;
         }
     }
+    if (!plan) return;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -390,7 +391,7 @@ d_resolve(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_
     d_plan_growth(ctl, rec, out, in, grow_out, grow_in, shrink_out, shrink_in, threadIdx.x, blockDim.x);
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) d_plan_check(ctl, out, in);
+    if (threadIdx.x < 32) d_plan_check(ctl, out, in);
 }
 
 __global__ void __launch_bounds__(256)
@@ -398,10 +399,10 @@ k_resolve(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_
           const unsigned long long* __restrict__ hwin, const int32_t* __restrict__ op_slot,
           const int32_t* __restrict__ feat_last, const int32_t* __restrict__ vdel_seq, Side out, Side in,
           Rec* rec, uint32_t* bitmap, const float* __restrict__ op_w, int32_t* grow_out, int32_t* grow_in,
-          int32_t* shrink_out, int32_t* shrink_in, const uint8_t* __restrict__ silent) {
+          int32_t* shrink_out, int32_t* shrink_in, const uint8_t* __restrict__ silent, int plan) {
     pdl_enter();
     d_resolve(ups, op_seq, ctl, hwin, op_slot, feat_last, vdel_seq, out, in, rec, bitmap, op_w, grow_out, grow_in,
-              shrink_out, shrink_in, silent);
+              shrink_out, shrink_in, silent, plan);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -468,22 +469,43 @@ __device__ __forceinline__ void d_plan_growth(Ctl* ctl, const Rec* __restrict__ 
     }
 }
 
-// what the growing rows cannot take from the free lists must fit into the never-used tail
+// what the growing rows cannot take from the free lists must fit into the never-used tail; one warp, a lane per class
 __device__ __forceinline__ void d_plan_check(Ctl* ctl, Side out, Side in) {
     if (ctl->abort) return;
+    const int k = lane_id();
+    static_assert(RP_POOL_CLASSES <= 32, "a lane per size class");
     for (int s = 0; s < 2; ++s) {
         const Side& sd = s ? in : out;
-        unsigned long long need = 0;
-        for (int k = RP_POOL_MIN_CLASS; k < RP_POOL_CLASSES; ++k) {
-            const int short_of = ctl->grow_demand[s][k] - sd.free_cnt[k];
-            if (short_of > 0) need += (unsigned long long)short_of << k;
-        }
-        ctl->pool_need[s] = need;
-        if (ctl->pool_next[s] + need > (unsigned long long)sd.col_size) {
-            ctl->err = (int)RIPPLE_ERR_CAPACITY;
-            ctl->abort = 1;
+        const int short_of = k >= RP_POOL_MIN_CLASS && k < RP_POOL_CLASSES ? ctl->grow_demand[s][k] - sd.free_cnt[k] : 0;
+        const unsigned long long need = warp_sum(short_of > 0 ? (unsigned long long)short_of << k : 0ull);
+        if (k == 0) {
+            ctl->pool_need[s] = need;
+            if (ctl->pool_next[s] + need > (unsigned long long)sd.col_size) {
+                ctl->err = (int)RIPPLE_ERR_CAPACITY;
+                ctl->abort = 1;
+            }
         }
     }
+}
+
+// The planning of a batch of more than a few hundred operations: in the last block of the resolve kernel its records
+// would be gone through eight per thread, one dependent chain after the other.
+__global__ void __launch_bounds__(256)
+k_plan(Ctl* ctl, const Rec* __restrict__ rec, Side out, Side in, int32_t* grow_out, int32_t* grow_in, int32_t* shrink_out,
+       int32_t* shrink_in) {
+    pdl_enter();
+    __shared__ int s_last;
+    if (ctl->abort) return;
+    d_plan_growth(ctl, rec, out, in, grow_out, grow_in, shrink_out, shrink_in, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&ctl->plan_done, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x < 32) d_plan_check(ctl, out, in);
 }
 
 // n sizes the launches (the number of operations given, or the batch capacity if vertex deletions
@@ -504,7 +526,10 @@ void graph_batch_classify(Ctx* c, int n) {
     RP_LAUNCH(c, k_resolve, grid, T, 0, c->ups_dev, c->op_seq, c->ctl, c->hwin, c->op_slot, c->feat_last,
               c->vdel_seq, c->side[0], c->side[1], c->rec, c->bitmap,
               (const float*)(c->has_opw ? c->opw_dev : nullptr), c->grow_list[0], c->grow_list[1],
-              c->shrink_list[0], c->shrink_list[1], (const uint8_t*)(c->has_silent ? c->silent_dev : nullptr));
+              c->shrink_list[0], c->shrink_list[1], (const uint8_t*)(c->has_silent ? c->silent_dev : nullptr), (int)(n <= RP_ONE_BLOCK_BATCH));
+    if (n > RP_ONE_BLOCK_BATCH)
+        RP_LAUNCH(c, k_plan, std::min(div_up(2 * n, T), c->n_sm), T, 0, c->ctl, (const Rec*)c->rec, c->side[0], c->side[1],
+                  c->grow_list[0], c->grow_list[1], c->shrink_list[0], c->shrink_list[1]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -796,7 +821,7 @@ k_apply_small(const __grid_constant__ ApplySmallArgs a) {
     d_classify(ups, a.op_seq, a.N, ctl, a.hkeys, a.hwin, a.hmask, a.op_slot, a.feat_last, a.vdel_seq, 0);
     __syncthreads();
     d_resolve(ups, a.op_seq, ctl, a.hwin, a.op_slot, a.feat_last, a.vdel_seq, a.out, a.in, a.rec, a.bitmap, op_w, a.grow[0],
-              a.grow[1], a.shrink[0], a.shrink[1], nullptr);
+              a.grow[1], a.shrink[0], a.shrink[1], nullptr, 1);
     __syncthreads();
     d_del_mark(ctl, a.rec, a.out, a.in);
     __syncthreads();

@@ -328,19 +328,82 @@ void narrow_prepare() {
     cudaFuncSetAttribute(k_update_rows_narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NARROW_SMEM);
 }
 
-// K = 0: the layer's self projection and transformed aggregate are both cached, so the update is
-// elementwise (bias + cached terms + activation); one thread per 16-byte piece of a row
+// K = 0: the layer's self projection and transformed aggregate are both cached, so the update is elementwise (bias +
+// cached terms + activation).  HBM bound: per row of d floats it reads S, its pending sums and Z and writes S, zeros and h
+// (24 d bytes; 12 d where the aggregate was gathered anew and nothing is pending).  A thread takes one 16-byte piece of a
+// row, two pieces per round with all their loads asked for before either is used; pieces are numbered through the rows,
+// so that any width keeps every lane busy.
+constexpr int EW_U = 2;
+
 __global__ void __launch_bounds__(256)
-k_update_rows_elementwise(const Ctl* ctl, UpdParams p) {
+k_update_rows_elementwise(const Ctl* ctl, const __grid_constant__ UpdParams p) {
     pdl_enter();
     if (ctl->abort) return;
-    const int n = upd_rows(p), nq = p.n_cols >> 2;
-    const long long total = (long long)n * nq;
-    for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < total;
-         it += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(it / nq), q = (int)(it - (long long)i * nq);
-        const int v = p.list ? p.list[i] : i;
-        upd_epilogue4(p, v, i, 4 * q, make_float4(0.f, 0.f, 0.f, 0.f), upd_row_scale(p, v));
+    const unsigned n = (unsigned)upd_rows(p), nq = (unsigned)p.n_cols >> 2, inv = 0xffffffffu / nq + 1u;   // x / nq = umulhi(x, inv), x small
+    const bool fold = p.addend_rw && !(p.rebuilt && *p.rebuilt);
+    const float* const srows = p.addend_rw ? p.addend_rw : p.addend;
+    constexpr unsigned PER = 256 * EW_U;
+    const unsigned long long step = (unsigned long long)gridDim.x * PER, first = (unsigned long long)blockIdx.x * PER;
+    const unsigned step_row = (unsigned)(step / nq), step_rem = (unsigned)(step - (unsigned long long)step_row * nq);
+    unsigned long long row0 = first / nq;
+    unsigned rem0 = (unsigned)(first - row0 * nq);
+    for (; row0 < n; row0 += step_row, rem0 += step_rem) {
+        if (rem0 >= nq) {
+            rem0 -= nq;
+            if (++row0 >= n) break;
+        }
+        unsigned i[EW_U], col[EW_U];
+        int v[EW_U];
+        bool on[EW_U];
+#pragma unroll
+        for (int u = 0; u < EW_U; ++u) {
+            const unsigned off = rem0 + 256u * u + threadIdx.x, dr = nq == 1 ? off : __umulhi(off, inv);
+            i[u] = (unsigned)row0 + dr;
+            col[u] = 4u * (off - dr * nq);
+            on[u] = row0 + dr < n;
+            v[u] = on[u] ? (p.list ? p.list[i[u]] : (int)i[u]) : 0;
+        }
+        float sc[EW_U];
+        float4 s[EW_U], d[EW_U], z[EW_U], o[EW_U];
+#pragma unroll
+        for (int u = 0; u < EW_U; ++u) {
+            // (pieces beyond the last read row 0 and are dropped)
+            s[u] = d[u] = z[u] = o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            sc[u] = upd_row_scale(p, v[u]);
+            const size_t at = (size_t)v[u] * p.ld_add + col[u];
+            if (srows) s[u] = *reinterpret_cast<const float4*>(srows + at);
+            if (fold) d[u] = *reinterpret_cast<const float4*>(p.addend_delta + at);
+            if (p.addend2) z[u] = *reinterpret_cast<const float4*>(p.addend2 + at);
+            if (p.Dout) o[u] = upd_load_old(p, v[u], col[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < EW_U; ++u) {
+            if (!on[u]) continue;
+            const size_t at = (size_t)v[u] * p.ld_add + col[u];
+            float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p.bias) h = __ldg(reinterpret_cast<const float4*>(p.bias + col[u]));
+            if (fold) {
+                s[u].x += d[u].x; s[u].y += d[u].y; s[u].z += d[u].z; s[u].w += d[u].w;
+                *reinterpret_cast<float4*>(p.addend_rw + at) = s[u];
+                *reinterpret_cast<float4*>(p.addend_delta + at) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            h.x += sc[u] * s[u].x; h.y += sc[u] * s[u].y; h.z += sc[u] * s[u].z; h.w += sc[u] * s[u].w;
+            h.x += z[u].x; h.y += z[u].y; h.z += z[u].z; h.w += z[u].w;
+            if (p.act == RIPPLE_ACT_RELU) {
+                h.x = fmaxf(h.x, 0.f); h.y = fmaxf(h.y, 0.f); h.z = fmaxf(h.z, 0.f); h.w = fmaxf(h.w, 0.f);
+            }
+            if (p.Dout) {
+                float cn = 1.f, co = 1.f;
+                if (p.src_norm) {
+                    const int dold = p.deg_out_old[v[u]];
+                    cn = coef_deg(p.deg_out[v[u]]);
+                    co = dold >= 0 ? coef_deg(dold) : cn;
+                }
+                *reinterpret_cast<float4*>(p.Dout + (size_t)i[u] * p.ld_o + col[u]) =
+                    p.dout_old ? o[u] : make_float4(cn * h.x - co * o[u].x, cn * h.y - co * o[u].y, cn * h.z - co * o[u].z, cn * h.w - co * o[u].w);
+            }
+            *reinterpret_cast<float4*>(p.Hout + (size_t)v[u] * p.ld_o + col[u]) = h;
+        }
     }
 }
 
@@ -468,9 +531,11 @@ void update_rows(Ctx* c, int l, bool full) {
     p.deg_out_old = c->deg_out_old;
     if (pre) {
         p.addend = c->S[l]; p.ld_add = c->ws[l];
-        if (!full && c->fused_fold[l]) { p.addend_rw = c->S[l]; p.addend_delta = c->dS[l]; }   // fold_deltas is skipped for these layers
+        if (!full && c->fused_fold[l]) { p.addend_rw = c->S[l]; p.addend_delta = c->dS[l]; p.rebuilt = &c->ctl->regather[l]; }   // fold_deltas is skipped for these layers
     }
-    float* dout = (full || l == c->L) ? nullptr : c->D[l & 1];  // the last hop sends nothing
+    // the last hop sends nothing, and a layer that transforms first makes its messages from the projections it keeps
+    // (P_new - P_old): it never looks at delta rows, nor does anyone need the row's previous value then
+    float* dout = (full || l == c->L || c->pre[l + 1]) ? nullptr : c->D[l & 1];
     p.dout_old = rp_monotonic(c->agg);
     if (ly.kind == RIPPLE_LAYER_GIN) {
         // hidden = relu(W1^T ((1 + eps) h + x) + b1), kept as compact rows
@@ -556,14 +621,15 @@ __global__ void k_extra_senders(Ctl* ctl, int l, const Rec* __restrict__ rec, in
         if (lane_id() == 0) idx = atomicAdd(&ctl->nC[l], 1);
         idx = __shfl_sync(FULL, idx, 0);
         const float dc = coef_deg(deg_out[x.u]) - coef_deg(x.deg_out_old);
-        for (int k = lane_id(); k < ld; k += 32) D[(size_t)idx * ld + k] = dc * H[(size_t)x.u * ld + k];
+        if (D)
+            for (int k = lane_id(); k < ld; k += 32) D[(size_t)idx * ld + k] = dc * H[(size_t)x.u * ld + k];
         if (lane_id() == 0) { senders[idx] = x.u; posmap[x.u] = idx; }
     }
 }
 
 void extra_sender_rows(Ctx* c, int l, int n) {
     RP_LAUNCH(c, k_extra_senders, std::min(div_up(n, 8), c->n_sm * 8), 256, 0, c->ctl, l, c->rec,
-              c->Clist[l & 1], c->posmap, c->side[0].deg, c->H[l], c->ld[l], c->D[l & 1]);
+              c->Clist[l & 1], c->posmap, c->side[0].deg, c->H[l], c->ld[l], c->pre[l + 1] ? (float*)nullptr : c->D[l & 1]);
 }
 
 }  // namespace rp

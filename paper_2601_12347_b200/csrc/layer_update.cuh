@@ -38,6 +38,7 @@ struct UpdParams {
     const float* addend2;           // rows by id added as they are, same leading dimension (may be null)
     float* addend_rw;               // if set: addend with its pending per-batch sums folded in on the way
     float* addend_delta;            //   (addend_rw += addend_delta, addend_delta = 0); replaces addend
+    const int* rebuilt;             // if set and not zero: the aggregate was gathered anew, nothing is pending (elementwise form)
     int dout_old;                   // Dout receives the row's previous value instead of a delta (monotonic aggregation)
     int src_norm;
     const int32_t* deg_out;

@@ -147,10 +147,14 @@ k_max_rows(Ctl* ctl, int l, int mode, const int32_t* __restrict__ list, const in
     pdl_enter();
     if (ctl->abort) return;
     const int n = n_dev ? *n_dev : n_host;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
     const int sub = lane / LPR, ql = lane % LPR;
-    for (int i = warp; i < n; i += nwarps) {
+    if (n == 0) return;
+    TicketWalk walk(&ctl->regather_ticket[l], n, 1, mode ? 1 : 8);   // (in-lists differ in length)
+    for (; walk.has(); walk.advance()) {
+        const int i0 = (int)walk.at, i1 = min(i0 + walk.chunk, n);
+        walk.take();
+    for (int i = i0; i < i1; ++i) {
         const int v = list ? list[i] : i;
         const int deg = in.deg[v];
         if (deg > (mode ? MAX_HUB_DEGREE : MAX_FULL_PASS_DEGREE)) {
@@ -211,7 +215,7 @@ k_max_rows(Ctl* ctl, int l, int mode, const int32_t* __restrict__ list, const in
         }
         if (mode && __any_sync(FULL, differs) && lane == 0) mark_bit(bitmapA, v);
     }
-    (void)l;
+    }
 }
 
 // Long rows, in three steps so that a hub's in-list is spread over the whole device instead of one block

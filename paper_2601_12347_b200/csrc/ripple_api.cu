@@ -126,7 +126,7 @@ static ripple_status run_full(Ctx* c) {
     return RIPPLE_OK;
 }
 
-static size_t coff_items(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / RP_ANEW_CHUNK) + 64; }
+static size_t coff_items(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / (RP_ANEW_CHUNK / 2)) + 64; }
 
 static std::vector<float> padded_matrix(const float* src, int rows, int cols, int rows_p, int cols_p) {
     std::vector<float> m((size_t)rows_p * cols_p, 0.f);

@@ -40,10 +40,6 @@ __device__ __forceinline__ void add4(float4& a, const float4& x, float c) {
 // single warp busy for 0.7 ms, longer than everything else of a hop on the sparse graph.
 constexpr int SPMM_HUB_DEGREE = 256;
 constexpr int SPMM_HUB_CHUNK = 256;
-// ... and the few rows that the fold sends back to be gathered anew in shorter ones: there is one warp for every
-// chunk, and the chain waits for the longest (ten rows of the weighted sum on the sparse graph: 63 us in chunks of 256)
-constexpr int SPMM_ANEW_CHUNK = RP_ANEW_CHUNK;
-
 // acc += sum over in-list entries [j_begin, j_end) of row v of c_u * M_u; LPR lanes hold one row
 // (NV float4 slots each), a warp works on 32 / LPR neighbours per step, four steps in flight.
 template <int NV, int LPR>
@@ -143,7 +139,7 @@ k_spmm_pull(int N, Side in, const int32_t* __restrict__ deg_out, int src_norm,
 
 // The chunks of the long in-lists, one warp per 256-entry chunk; chunk sums are added to the row,
 // which the kernel that queued the chunks has zeroed.
-template <int NV, int LPR, int CHUNK = SPMM_HUB_CHUNK>
+template <int NV, int LPR>
 __global__ void __launch_bounds__(256)
 k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const float* __restrict__ M, int ld,
             float* S, const int2* __restrict__ items, const int* __restrict__ n_items, int* ticket) {
@@ -160,7 +156,7 @@ k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const fl
         float4 acc[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        spmm_accumulate<NV, LPR>(acc, in, w.x, w.y * CHUNK, min(deg, (w.y + 1) * CHUNK), deg_out,
+        spmm_accumulate<NV, LPR>(acc, in, w.x, w.y * SPMM_HUB_CHUNK, min(deg, (w.y + 1) * SPMM_HUB_CHUNK), deg_out,
                                  src_norm, M, ld);
         if (sub == 0) {
 #pragma unroll
@@ -168,6 +164,43 @@ k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const fl
                 int q = ql + LPR * k;
                 if (q < nq) red_add_v4(S + (size_t)w.x * ld + 4 * q, acc[k]);
             }
+        }
+    }
+}
+
+// The few rows that the fold sends back to be gathered anew.  The chain waits for the longest chunk, so a whole block takes
+// one, 32 entries per warp, and adds its warps' sums up in shared memory before they reach the row (which the fold has
+// zeroed): ten rows of the weighted sum on the sparse graph 63 us with a warp per 256 entries, 10 us so; a hub of 26 000
+// entries, whose row 800 separate additions would queue for, 45 -> 15 us.
+template <int NV, int LPR>
+__global__ void __launch_bounds__(256)
+k_spmm_anew(Side in, const int32_t* __restrict__ deg_out, int src_norm, const float* __restrict__ M, int ld, float* S,
+            const int2* __restrict__ items, const int* __restrict__ n_items) {
+    pdl_enter();
+    extern __shared__ __align__(16) float part[];   // [8][ld]
+    const int n = *n_items, warp = threadIdx.x >> 5, lane = lane_id(), nq = ld >> 2;
+    const int sub = lane / LPR, ql = lane % LPR;
+    constexpr int PER_WARP = RP_ANEW_CHUNK / 8;
+    for (int it = blockIdx.x; it < n; it += gridDim.x) {
+        const int2 w = items[it];
+        const int deg = in.deg[w.x], j0 = w.y * RP_ANEW_CHUNK + warp * PER_WARP;
+        float4 acc[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        spmm_accumulate<NV, LPR>(acc, in, w.x, j0, min(deg, j0 + PER_WARP), deg_out, src_norm, M, ld);
+        __syncthreads();   // the sums of the item before have been read
+        if (sub == 0) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const int q = ql + LPR * k;
+                if (q < nq) *reinterpret_cast<float4*>(part + warp * ld + 4 * q) = acc[k];
+            }
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < nq; q += blockDim.x) {
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < 8; ++k) add4(t, *reinterpret_cast<const float4*>(part + k * ld + 4 * q), 1.0f);
+            red_add_v4(S + (size_t)w.x * ld + 4 * q, t);
         }
     }
 }
@@ -759,7 +792,7 @@ __global__ void k_choose_direction(Ctl* ctl, int l, int mode, int gather, float 
 // (Sec. 3.2's scoped recomputation, for this one row) and the budget starts again.  tau^2 is
 // scaled per vertex by a fixed factor in [0.5, 1), so that rows touched by every batch do not all
 // come due in the same batch.  A row that comes due is zeroed and its in-list queued, in chunks,
-// for k_spmm_hubs.
+// for k_spmm_anew.
 __global__ void __launch_bounds__(256)
 k_fold_deltas(Ctl* ctl, int l, const int32_t* __restrict__ A, int ld, float* S, float* dS, float* budget,
               float tau2, const int32_t* __restrict__ deg_in, int2* items) {
@@ -795,11 +828,11 @@ k_fold_deltas(Ctl* ctl, int l, const int32_t* __restrict__ A, int ld, float* S, 
             if (lane == 0) budget[v] = spent;
             continue;
         }
-        // the row comes due: zero it and queue its in-list, in chunks, for k_spmm_hubs
+        // the row comes due: zero it and queue its in-list, in chunks, for k_spmm_anew
         __syncwarp();
         for (int q = lane; q < nq; q += 32) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
         const int deg = deg_in[v];
-        const int nch = (deg + SPMM_ANEW_CHUNK - 1) / SPMM_ANEW_CHUNK;
+        const int nch = (deg + RP_ANEW_CHUNK - 1) / RP_ANEW_CHUNK;
         int first = 0;
         if (lane == 0) {
             if (nch) first = atomicAdd(&ctl->rebuild_items[l], nch);
@@ -820,8 +853,8 @@ void fold_deltas(Ctx* c, int l) {
               c->rebuild_tau2, c->side[1].deg, items);
     if (!c->Eb[l]) return;
 #define HUBS(NV, LPR)                                                                                              \
-    RP_LAUNCH(c, (k_spmm_hubs<NV, LPR, SPMM_ANEW_CHUNK>), c->n_sm * 8, 256, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld, \
-              c->S[l], items, &c->ctl->rebuild_items[l], &c->ctl->hub_ticket[l])
+    RP_LAUNCH(c, (k_spmm_anew<NV, LPR>), c->n_sm * 4, 256, sizeof(float) * 8 * (size_t)ld, c->side[1], c->side[0].deg, \
+              (int)c->src_norm, M, ld, c->S[l], (const int2*)items, (const int*)&c->ctl->rebuild_items[l])
     RP_WIDTH_DISPATCH(ld, HUBS);
 #undef HUBS
 }
