@@ -65,6 +65,28 @@ k_att_scalars(Ctl* ctl, const int32_t* __restrict__ list, const int* n_dev, int 
     }
 }
 
+// Edge records.  Added edge (u, v): plus the term of u as it was before this hop's changes (the walk
+// brings the difference to the new one if u is a sender).  Deleted edge: minus that
+// term.  A sink that recomputes takes neither.  One warp per record, from the far end of the grid.
+__device__ __forceinline__ void d_att_records(const Ctl* ctl, const Rec* __restrict__ rec, const int32_t* __restrict__ posmap,
+                                              const float* __restrict__ Hprev, const float* __restrict__ Old, int ld_h,
+                                              const float* __restrict__ s_old, const float* __restrict__ att_s,
+                                              const float* __restrict__ att_t, float slope, int d, int ld, float* dS) {
+    const int n = ctl->n_rec;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5, warp = nwarps - 1 - (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = lane_id();
+    for (int r = warp; r < n; r += nwarps) {
+        const int u = rec[r].u, v = rec[r].v;
+        if (posmap[v] >= 0) continue;
+        const int p = posmap[u];
+        const float* row = p >= 0 ? Old + (size_t)p * ld_h : Hprev + (size_t)u * ld_h;
+        const float s = p >= 0 ? s_old[p] : att_s[u];
+        const float e = (rec[r].sign > 0 ? 1.f : -1.f) * att_weight(s, att_t[v], slope);
+        float* dst = dS + (size_t)v * ld;
+        for (int k = lane; k <= d; k += 32) atomicAdd(dst + k, k < d ? e * row[k] : e);
+    }
+}
+
 // Messages along the current out-edges of the senders (the rows of A_{l-1}): e_new h_new - e_old h_old
 // into the accumulator row of every sink that is not itself a sender (those recompute).  An edge added
 // by this batch is walked like any other; its record then adds e_old h_old, which leaves the new term.
@@ -73,9 +95,17 @@ __global__ void __launch_bounds__(256)
 k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff, Side out,
            const int32_t* __restrict__ posmap, const float* __restrict__ Hprev, const float* __restrict__ Old, int ld_h,
            const float* __restrict__ s_old, const float* __restrict__ att_s, const float* __restrict__ att_t,
-           float slope, int d, int ld, float* dS, uint32_t* bitmap) {
+           float slope, int d, int ld, float* dS, uint32_t* bitmap, const Rec* __restrict__ rec) {
     pdl_enter();
     if (ctl->abort) return;
+    {   // the members of A_l that the walk does not find: sinks of edge changes, and A_{l-1} (the senders)
+        const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsize = gridDim.x * blockDim.x;
+        for (int i = gtid; i < ctl->n_rec + ctl->nC[l - 1]; i += gsize) {
+            const int v = i < ctl->n_rec ? rec[i].v : senders[i - ctl->n_rec];
+            atomicOr(&bitmap[v >> 5], 1u << (v & 31));
+        }
+    }
+    d_att_records(ctl, rec, posmap, Hprev, Old, ld_h, s_old, att_s, att_t, slope, d, ld, dS);
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
@@ -141,35 +171,11 @@ k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* 
     }
 }
 
-// Edge records.  Added edge (u, v): plus the term of u as it was before this hop's changes (the walk
-// above has already brought the difference to the new one if u is a sender).  Deleted edge: minus that
-// term.  A sink that recomputes takes neither.  One warp per record.
-__global__ void k_att_records(Ctl* ctl, const Rec* __restrict__ rec, const int32_t* __restrict__ posmap,
-                              const float* __restrict__ Hprev, const float* __restrict__ Old, int ld_h,
-                              const float* __restrict__ s_old, const float* __restrict__ att_s,
-                              const float* __restrict__ att_t, float slope, int d, int ld, float* dS) {
-    pdl_enter();
-    if (ctl->abort) return;
-    const int n = ctl->n_rec;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int lane = lane_id();
-    for (int r = warp; r < n; r += nwarps) {
-        const int u = rec[r].u, v = rec[r].v;
-        if (posmap[v] >= 0) continue;
-        const int p = posmap[u];
-        const float* row = p >= 0 ? Old + (size_t)p * ld_h : Hprev + (size_t)u * ld_h;
-        const float s = p >= 0 ? s_old[p] : att_s[u];
-        const float e = (rec[r].sign > 0 ? 1.f : -1.f) * att_weight(s, att_t[v], slope);
-        float* dst = dS + (size_t)v * ld;
-        for (int k = lane; k <= d; k += 32) atomicAdd(dst + k, k < d ? e * row[k] : e);
-    }
-}
-
 // Per hop-l vertex (or per vertex, `all`): either fold the accumulated messages into the cached row,
 // keeping the row's rounding budget, and write the new embedding row at once; or -- the vertex is a
 // sender (its own h^{l-1} changed), the budget has run out, no in-neighbour is left, or `all` -- zero
 // the row, queue its in-list, in chunks, for k_att_gather and flag the vertex for k_att_update.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_att_fold(Ctl* ctl, int l, const int32_t* __restrict__ A, const int* n_dev, int n_host, int all, int ld, float* S,
            float* dS, float* budget, float tau2, const int32_t* __restrict__ deg_in,
            const int32_t* __restrict__ posmap, int2* items, int d, int act, float* H, int ld_h, float* Old,
@@ -179,21 +185,33 @@ k_att_fold(Ctl* ctl, int l, const int32_t* __restrict__ A, const int* n_dev, int
     const int n = n_dev ? *n_dev : n_host;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
+    const bool fast = !all && nq <= 32 && (ld_h & 3) == 0;
+    // (the fast form asks for the row together with the two words that decide whether it is used, and for the next row
+    // before it works on this one: a warp's rows follow one another, each a round trip to memory)
+    float4 x_nx = make_float4(0.f, 0.f, 0.f, 0.f), y_nx = x_nx, hold_nx = x_nx;
+    float spent_nx = 0.f;
+    int pos_nx = 0, deg_nx = 0, v_nx = 0;
+    auto fetch = [&](int i) {
+        v_nx = A ? A[i] : i;
+        if (lane < nq) {
+            x_nx = reinterpret_cast<const float4*>(S + (size_t)v_nx * ld)[lane];
+            y_nx = reinterpret_cast<const float4*>(dS + (size_t)v_nx * ld)[lane];
+        }
+        if (lane < (ld_h >> 2)) hold_nx = reinterpret_cast<const float4*>(H + (size_t)v_nx * ld_h)[lane];
+        if (budget) spent_nx = budget[v_nx];
+        pos_nx = posmap[v_nx];
+        deg_nx = deg_in[v_nx];
+    };
+    if (fast && warp < n) fetch(warp);
     for (int i = warp; i < n; i += nwarps) {
-        const int v = A ? A[i] : i;
+        const float4 x0 = x_nx, y0 = y_nx, hold0 = hold_nx;
+        const float spent0 = spent_nx;
+        const int v = fast ? v_nx : A ? A[i] : i;
         const size_t off = (size_t)v * ld;
         float4* s = reinterpret_cast<float4*>(S + off);
         float4* dd = reinterpret_cast<float4*>(dS + off);
-        const bool fast = !all && nq <= 32 && (ld_h & 3) == 0;
-        // (the fast form asks for the row together with the two words that decide whether it is used)
-        float4 x0 = make_float4(0.f, 0.f, 0.f, 0.f), y0 = x0, hold0 = x0;
-        float spent0 = 0.f;
-        if (fast) {
-            if (lane < nq) { x0 = s[lane]; y0 = dd[lane]; }
-            if (lane < (ld_h >> 2)) hold0 = reinterpret_cast<const float4*>(H + (size_t)v * ld_h)[lane];
-            if (budget) spent0 = budget[v];
-        }
-        bool anew = all || posmap[v] >= 0 || deg_in[v] == 0;   // (no in-neighbour left: exact zeros)
+        bool anew = all || (fast ? pos_nx >= 0 || deg_nx == 0 : posmap[v] >= 0 || deg_in[v] == 0);   // (no in-neighbour left: exact zeros)
+        if (fast && i + nwarps < n) fetch(i + nwarps);
         bool on_budget = false;
         if (!anew && fast) {
             // Rows of up to 128 floats: one 16-byte piece per lane, so the row, its accumulator, its budget and the
@@ -383,8 +401,10 @@ k_att_gather(Ctl* ctl, int l, const int2* __restrict__ items, Side in, const flo
 __global__ void __launch_bounds__(256)
 k_att_update(Ctl* ctl, const int32_t* __restrict__ list, const int* n_dev, int n_host, const float* __restrict__ S,
              int ld, int d, const int32_t* __restrict__ deg_in, int act, float* H, int ld_h, float* Old,
-             uint32_t* gathered) {
+             uint32_t* gathered, const int32_t* __restrict__ senders, const int* n_senders, int32_t* posmap) {
     pdl_enter();
+    if (senders)   // nobody looks up the hop's senders any more
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < *n_senders; i += gridDim.x * blockDim.x) posmap[senders[i]] = -1;
     if (ctl->abort) return;
     const int n = n_dev ? *n_dev : n_host;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -423,7 +443,8 @@ void att_update(Ctx* c, int l, bool full) {
     float* old_rows = (full || l == c->L) ? nullptr : c->D[l & 1];   // the last hop sends nothing
     RP_LAUNCH(c, k_att_update, c->n_sm * 8, 256, 0, c->ctl, full ? (const int32_t*)nullptr : c->A[l],
               full ? (const int*)nullptr : &c->ctl->nA[l], c->N, c->S[l], c->ws[l], ly.d_in, c->side[1].deg, ly.act,
-              c->H[l], c->ld[l], old_rows, full ? (uint32_t*)nullptr : c->bitmap);
+              c->H[l], c->ld[l], old_rows, full ? (uint32_t*)nullptr : c->bitmap,
+              full ? (const int32_t*)nullptr : sender_list(c, l - 1), full ? (const int*)nullptr : &c->ctl->nC[l - 1], c->posmap);
 }
 
 // bootstrap: logit halves, cached rows and outputs of every vertex
@@ -442,27 +463,23 @@ void att_full(Ctx* c, int l) {
 void att_hop(Ctx* c, int l, int n, bool small) {
     const LayerDev& ly = c->layer[l];
     const int ld = c->ws[l], T = 256;
-    const int32_t* senders = c->Clist[(l - 1) & 1];   // = A_{l-1}, entered in the position map
+    const int32_t* senders = sender_list(c, l - 1);   // = A_{l-1}, entered in the position map
     const float* Old = c->D[(l - 1) & 1];             // their rows before this batch, in list order
     RP_LAUNCH(c, k_att_scalars, c->n_sm * 4, T, 0, c->ctl, senders, (const int*)&c->ctl->nC[l - 1], 0, c->H[l - 1],
               c->ld[l - 1], ly.W1, c->att_s[l], c->att_t[l], c->att_so);
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l], c->stream);
-#define PUSH(NV, LPR) RP_LAUNCH(c, (k_att_push<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, senders, c->coff, c->side[0], c->posmap, c->H[l - 1], Old, c->ld[l - 1], c->att_so, c->att_s[l], c->att_t[l], ly.eps, ly.d_in, ld, c->dS[l], c->bitmap)
+#define PUSH(NV, LPR) RP_LAUNCH(c, (k_att_push<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, senders, c->coff, c->side[0], c->posmap, c->H[l - 1], Old, c->ld[l - 1], c->att_so, c->att_s[l], c->att_t[l], ly.eps, ly.d_in, ld, c->dS[l], c->bitmap, (const Rec*)c->rec)
     RP_WIDTH_DISPATCH(ld, PUSH);
 #undef PUSH
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l + 1], c->stream);
-    if (n > 0)
-        RP_LAUNCH(c, k_att_records, std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, c->rec, c->posmap,
-                  c->H[l - 1], Old, c->ld[l - 1], c->att_so, c->att_s[l], c->att_t[l], ly.eps, ly.d_in, ld, c->dS[l]);
-    // the list A_l: the message walk has marked the sinks it reached, the rest is marked here
-    frontier_mark_extras(c, l);
-    if (small) frontier_compact_small(c, l);   // (a handful of updates on a graph whose bitmap one block can sweep)
+    (void)n;
+    // the list A_l: the message walk has marked it
+    if (small) frontier_compact_small(c, l, false);   // (a handful of updates on a graph whose bitmap one block can sweep)
     else frontier_compact(c, l);
     RP_LAUNCH(c, k_att_fold, c->n_sm * 8, T, 0, c->ctl, l, c->A[l], (const int*)&c->ctl->nA[l], 0, 0, ld, c->S[l],
               c->dS[l], c->Eb[l], c->rebuild_tau2, c->side[1].deg, c->posmap, c->att_items, ly.d_in, ly.act, c->H[l],
               c->ld[l], l == c->L ? (float*)nullptr : c->D[l & 1], c->bitmap);   // (the bitmap is free between two hops' markings)
     launch_gather(c, l);
-    senders_release(c, l - 1);
 }
 
 }  // namespace rp

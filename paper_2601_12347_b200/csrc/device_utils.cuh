@@ -99,7 +99,7 @@ struct TicketWalk {
         chunk = small;
         if (n <= nwarps * small) {   // (as many warps as there are units for, an eighth of the small chunk at least)
             ticket = nullptr;
-            chunk = max(max(small >> 3, 1), (int)((n + nwarps - 1) / nwarps));
+            chunk = max(max(small >> 3, 1), (int)(((unsigned)n + (unsigned)nwarps - 1u) / (unsigned)nwarps));
             at = warp * chunk;
             return;
         }

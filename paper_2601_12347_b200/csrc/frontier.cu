@@ -26,19 +26,17 @@ __device__ __forceinline__ int scan_count(const int* n_dev, int n_host) { return
 
 // Tile sums; the last block to finish turns them into exclusive tile prefixes and writes the total
 // (one launch instead of two: the chain of a small batch is bound by the number of launches).
-// If `senders` is given the listed vertices are, in the same pass, copied there and entered into the
-// position map, and their number into *n_senders: the sender list of a hop whose senders are exactly
-// the affected vertices (no launch of its own for that).
+// If `posmap` is given the listed vertices are, in the same pass, entered into the position map, and their number into
+// *n_senders: the senders of a hop are exactly the affected vertices (no launch of its own for that).
 __global__ void k_scan_tiles(const int32_t* __restrict__ list, const int* n_dev, int n_host,
                              const int32_t* __restrict__ deg, int64_t* tile_sums, int64_t* out,
-                             unsigned long long* total_dev, int* done, int32_t* senders, int32_t* posmap,
-                             int* n_senders) {
+                             unsigned long long* total_dev, int* done, int32_t* posmap, int* n_senders) {
     pdl_enter();
     __shared__ int64_t scratch[33];
     __shared__ int s_last;
     int n = scan_count(n_dev, n_host);
     int n_tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (senders && blockIdx.x == 0 && threadIdx.x == 0) *n_senders = n;
+    if (posmap && blockIdx.x == 0 && threadIdx.x == 0) *n_senders = n;
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         int64_t s = 0;
 #pragma unroll
@@ -47,7 +45,7 @@ __global__ void k_scan_tiles(const int32_t* __restrict__ list, const int* n_dev,
             if (i < n) {
                 const int v = list ? list[i] : i;
                 s += deg[v];
-                if (senders) { senders[i] = v; posmap[v] = i; }
+                if (posmap) posmap[v] = i;
             }
         }
         int64_t total;
@@ -107,18 +105,18 @@ __global__ void k_scan_write(const int32_t* __restrict__ list, const int* n_dev,
     }
 }
 
-static void scan_degrees_and_copy(Ctx* c, const int32_t* list, const int* n_dev, int n_host, const int32_t* deg,
-                                  int64_t* out, unsigned long long* total_dev, int32_t* senders, int* n_senders) {
+static void scan_degrees_and_enter(Ctx* c, const int32_t* list, const int* n_dev, int n_host, const int32_t* deg,
+                                   int64_t* out, unsigned long long* total_dev, int32_t* posmap, int* n_senders) {
     int max_tiles = std::max(1, div_up(c->N, SCAN_TILE));
     int grid = std::min(max_tiles, c->n_sm * 8);
     RP_LAUNCH(c, k_scan_tiles, grid, SCAN_T, 0, list, n_dev, n_host, deg, c->tile_sums, out, total_dev, c->scan_done,
-              senders, c->posmap, n_senders);
+              posmap, n_senders);
     RP_LAUNCH(c, k_scan_write, grid, SCAN_T, 0, list, n_dev, n_host, deg, c->tile_sums, out);
 }
 
 void scan_degrees(Ctx* c, const int32_t* list, const int* n_dev, int n_host, const int32_t* deg,
                   int64_t* out, unsigned long long* total_dev) {
-    scan_degrees_and_copy(c, list, n_dev, n_host, deg, out, total_dev, nullptr, nullptr);
+    scan_degrees_and_enter(c, list, n_dev, n_host, deg, out, total_dev, nullptr, nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -126,40 +124,76 @@ void scan_degrees(Ctx* c, const int32_t* list, const int* n_dev, int n_host, con
 // ---------------------------------------------------------------------------------------------
 constexpr int CMP_T = 256;  // one word per thread
 
-__global__ void k_bitmap_tile_counts(const uint32_t* __restrict__ bitmap, int n_words, int* tile_cnt) {
+// SENDERS: the listed vertices are also the next hop's senders, so the passes that turn the bitmap into the list make
+// their out-degree prefix and position entries as well (two launches of the chain less).
+template <bool SENDERS>
+__global__ void k_bitmap_tile_counts(const uint32_t* __restrict__ bitmap, int n_words, int* tile_cnt,
+                                     const int32_t* __restrict__ deg_out, int64_t* tile_deg) {
     pdl_enter();
     __shared__ int scratch[33];
+    __shared__ int64_t scratch_l[33];
     int w = blockIdx.x * CMP_T + threadIdx.x;
-    int pc = w < n_words ? __popc(bitmap[w]) : 0;
+    uint32_t bits = w < n_words ? bitmap[w] : 0u;
+    int pc = __popc(bits);
     int total;
     block_exclusive_scan<int>(pc, scratch, total);
     if (threadIdx.x == 0) tile_cnt[blockIdx.x] = total;
+    if (SENDERS) {
+        int64_t d = 0, sum;
+        if (total) {
+            while (bits) {
+                d += deg_out[(w << 5) + __ffs(bits) - 1];
+                bits &= bits - 1;
+            }
+        }
+        block_exclusive_scan<int64_t>(d, scratch_l, sum);
+        if (threadIdx.x == 0) tile_deg[blockIdx.x] = sum;
+    }
 }
 
+template <bool SENDERS>
 __global__ void k_bitmap_compact(uint32_t* bitmap, int n_words, const int* __restrict__ tile_cnt,
                                  int32_t* list, int* count_out, const int32_t* __restrict__ deg_in,
-                                 unsigned long long* pull_work) {
+                                 unsigned long long* pull_work, const int32_t* __restrict__ deg_out,
+                                 const int64_t* __restrict__ tile_deg, int32_t* posmap, int64_t* coff, int* n_senders,
+                                 unsigned long long* messages) {
     pdl_enter();
     __shared__ int scratch[33];
-    __shared__ int tile_base;
+    __shared__ int64_t scratch_l[33];
     __shared__ unsigned long long work;
     // base of this tile: sum of the counts of the tiles before it
     int part = 0;
-    for (int t = threadIdx.x; t < (int)blockIdx.x; t += CMP_T) part += tile_cnt[t];
-    int total;
-    block_exclusive_scan<int>(part, scratch, total);
-    if (threadIdx.x == 0) { tile_base = total; work = 0ull; }
-    __syncthreads();
+    int64_t part_d = 0;
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += CMP_T) {
+        part += tile_cnt[t];
+        if (SENDERS) part_d += tile_deg[t];
+    }
+    int tile_base, total;
+    int64_t deg_base = 0, deg_total = 0;
+    block_exclusive_scan<int>(part, scratch, tile_base);
+    if (SENDERS) block_exclusive_scan<int64_t>(part_d, scratch_l, deg_base);
+    if (threadIdx.x == 0) work = 0ull;
     int w = blockIdx.x * CMP_T + threadIdx.x;
     uint32_t bits = w < n_words ? bitmap[w] : 0u;
     if (bits) bitmap[w] = 0u;
     int pc = __popc(bits);
     int off = tile_base + block_exclusive_scan<int>(pc, scratch, total);
+    int64_t at = 0;
+    if (SENDERS) {
+        int64_t d = 0;
+        for (uint32_t b = bits; b; b &= b - 1) d += deg_out[(w << 5) + __ffs(b) - 1];
+        at = deg_base + block_exclusive_scan<int64_t>(d, scratch_l, deg_total);
+    }
     unsigned long long my_work = 0;
     while (bits) {
         int b = __ffs(bits) - 1;
         bits &= bits - 1;
         int v = (w << 5) + b;
+        if (SENDERS) {
+            posmap[v] = off;
+            coff[off] = at;
+            at += deg_out[v];
+        }
         list[off++] = v;
         if (deg_in) my_work += (unsigned long long)deg_in[v];
     }
@@ -169,15 +203,33 @@ __global__ void k_bitmap_compact(uint32_t* bitmap, int n_words, const int* __res
         __syncthreads();
         if (threadIdx.x == 0 && work) atomicAdd(pull_work, work);
     }
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count_out = tile_base + total;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        *count_out = tile_base + total;
+        if (SENDERS) {
+            *n_senders = tile_base + total;
+            *messages = (unsigned long long)(deg_base + deg_total);
+            coff[tile_base + total] = deg_base + deg_total;
+        }
+    }
 }
 
 void bitmap_to_list_from(Ctx* c, uint32_t* bitmap, int32_t* list, int* count_dev, unsigned long long* pull_work) {
     int tiles = div_up(c->n_words, CMP_T);
     int* tile_cnt = reinterpret_cast<int*>(c->tile_sums);  // scan scratch is free here
-    RP_LAUNCH(c, k_bitmap_tile_counts, tiles, CMP_T, 0, bitmap, c->n_words, tile_cnt);
-    RP_LAUNCH(c, k_bitmap_compact, tiles, CMP_T, 0, bitmap, c->n_words, tile_cnt, list, count_dev,
-              pull_work ? c->side[1].deg : nullptr, pull_work);
+    RP_LAUNCH(c, k_bitmap_tile_counts<false>, tiles, CMP_T, 0, bitmap, c->n_words, tile_cnt, (const int32_t*)nullptr, (int64_t*)nullptr);
+    RP_LAUNCH(c, k_bitmap_compact<false>, tiles, CMP_T, 0, bitmap, c->n_words, tile_cnt, list, count_dev,
+              pull_work ? c->side[1].deg : nullptr, pull_work, (const int32_t*)nullptr, (const int64_t*)nullptr, (int32_t*)nullptr,
+              (int64_t*)nullptr, (int*)nullptr, (unsigned long long*)nullptr);
+}
+
+void frontier_compact_senders(Ctx* c, int l) {
+    int tiles = div_up(c->n_words, CMP_T);
+    int64_t* tile_deg = c->tile_sums;
+    int* tile_cnt = reinterpret_cast<int*>(c->tile_sums + tiles);
+    RP_LAUNCH(c, k_bitmap_tile_counts<true>, tiles, CMP_T, 0, c->bitmap, c->n_words, tile_cnt, (const int32_t*)c->side[0].deg, tile_deg);
+    RP_LAUNCH(c, k_bitmap_compact<true>, tiles, CMP_T, 0, c->bitmap, c->n_words, tile_cnt, c->A[l], &c->ctl->nA[l],
+              (const int32_t*)c->side[1].deg, &c->ctl->pull_work[l], (const int32_t*)c->side[0].deg, (const int64_t*)tile_deg,
+              c->posmap, c->coff, &c->ctl->nC[l], &c->ctl->E[l + 1]);
 }
 
 static void bitmap_to_list(Ctx* c, int32_t* list, int* count_dev, unsigned long long* pull_work) {
@@ -219,7 +271,19 @@ __global__ void k_mark_frontier(Ctl* ctl, int l, int self_term, int walk, const 
             if (row_end <= e) { ++i; continue; }
             int64_t seg_end = min(e1, row_end);
             int64_t base = out.start[senders[i]] + (e - coff[i]);
-            for (int64_t j = lane; j < seg_end - e; j += 32) set_bit(bitmap, out.col[base + j]);
+            // four sinks per lane and round, their ids and then their words of the bitmap asked for together
+            const int cnt = (int)(seg_end - e);
+            for (int j = lane; j < cnt; j += 128) {
+                int v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = out.col[base + (j + 32 * k < cnt ? j + 32 * k : j)];
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) w[k] = bitmap[v[k] >> 5];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (!(w[k] & (1u << (v[k] & 31)))) atomicOr(&bitmap[v[k] >> 5], 1u << (v[k] & 31));
+            }
             e = seg_end;
             ++i;
         }
@@ -293,7 +357,7 @@ void frontier_mark(Ctx* c, int l, bool walk, int n) {
     // along with the last kernel of the hop's delta form; an empty batch has nothing to mark
     if (walk)
         RP_LAUNCH(c, k_mark_frontier, c->n_sm * 8, 256, 0, c->ctl, l, (int)c->self_term,
-                  (int)walk, c->Clist[(l - 1) & 1], c->coff, c->side[0], c->rec, c->A[l - 1], c->bitmap);
+                  (int)walk, sender_list(c, l - 1), c->coff, c->side[0], c->rec, c->A[l - 1], c->bitmap);
     (void)n;
     if (!c->rebuild_armed[l]) return;
     // the list A_l is not built yet: its buffer holds the queue of undecided long rows
@@ -304,21 +368,32 @@ void frontier_mark(Ctx* c, int l, bool walk, int n) {
 }
 
 // The frontier of a hop in one block: words of the bitmap are dealt out in contiguous runs, one per thread, so
-// that a block scan of the popcounts places every id.  For batches of a handful of updates on graphs whose
-// bitmap one block can sweep (two launches of the general chain otherwise).
+// that a block scan of the popcounts places every id; and (senders) the next hop's senders, which are the same
+// vertices, with their position entries and the prefix of their out-degrees.  For batches of a handful of updates on
+// graphs whose bitmap one block can sweep (four launches of the general chain otherwise).
 __global__ void __launch_bounds__(1024)
-k_frontier_small(Ctl* ctl, int l, uint32_t* bitmap, int n_words, int32_t* list, const int32_t* __restrict__ deg_in) {
+k_frontier_small(Ctl* ctl, int l, uint32_t* bitmap, int n_words, int32_t* list, const int32_t* __restrict__ deg_in,
+                 int build_senders, const int32_t* __restrict__ deg_out, int32_t* posmap, int64_t* coff) {
     pdl_enter();
     __shared__ int scratch_i[33];
+    __shared__ int64_t scratch_l[33];
     __shared__ unsigned long long s_work;
     if (ctl->abort) return;
     if (threadIdx.x == 0) s_work = 0ull;
     const int per = (n_words + (int)blockDim.x - 1) / (int)blockDim.x;
     const int w0 = min(n_words, (int)threadIdx.x * per), w1 = min(n_words, w0 + per);
     int pc = 0;
-    for (int w = w0; w < w1; ++w) pc += __popc(bitmap[w]);
+    int64_t deg = 0;
+    for (int w = w0; w < w1; ++w) {
+        const uint32_t bits = bitmap[w];
+        pc += __popc(bits);
+        if (build_senders)
+            for (uint32_t b = bits; b; b &= b - 1) deg += deg_out[(w << 5) + __ffs(b) - 1];
+    }
     int total;
     int off = block_exclusive_scan<int>(pc, scratch_i, total);
+    int64_t at = 0, deg_total = 0;
+    if (build_senders) at = block_exclusive_scan<int64_t>(deg, scratch_l, deg_total);
     unsigned long long work = 0;
     for (int w = w0; w < w1; ++w) {
         uint32_t bits = bitmap[w];
@@ -327,6 +402,11 @@ k_frontier_small(Ctl* ctl, int l, uint32_t* bitmap, int n_words, int32_t* list, 
         while (bits) {
             const int v = (w << 5) + __ffs(bits) - 1;
             bits &= bits - 1;
+            if (build_senders) {
+                posmap[v] = off;
+                coff[off] = at;
+                at += deg_out[v];
+            }
             list[off++] = v;
             work += (unsigned long long)deg_in[v];
         }
@@ -334,48 +414,26 @@ k_frontier_small(Ctl* ctl, int l, uint32_t* bitmap, int n_words, int32_t* list, 
     work = warp_sum(work);
     if (lane_id() == 0 && work) atomicAdd(&s_work, work);
     __syncthreads();
-    if (threadIdx.x == 0) { ctl->nA[l] = total; ctl->pull_work[l] = s_work; }
-}
-
-// ... and the sender list made from it (C_l = A_l) with the prefix of the out-degrees, likewise in one block
-__global__ void __launch_bounds__(1024)
-k_senders_small(Ctl* ctl, int l, const int32_t* __restrict__ list, const int32_t* __restrict__ deg_out, int32_t* senders,
-                int32_t* posmap, int64_t* coff) {
-    pdl_enter();
-    __shared__ int64_t scratch_l[33];
-    if (ctl->abort) return;
-    const int total = ctl->nA[l];
-    int64_t carry = 0;
-    for (int i0 = 0; i0 < total; i0 += (int)blockDim.x) {
-        const int i = i0 + (int)threadIdx.x;
-        int v = -1;
-        int64_t d = 0;
-        if (i < total) { v = list[i]; d = deg_out[v]; }
-        int64_t sum;
-        const int64_t ex = block_exclusive_scan<int64_t>(d, scratch_l, sum);
-        if (i < total) { senders[i] = v; posmap[v] = i; coff[i] = carry + ex; }
-        carry += sum;
-    }
     if (threadIdx.x == 0) {
-        coff[total] = carry;
-        ctl->E[l + 1] = (unsigned long long)carry;
-        ctl->nC[l] = total;
+        ctl->nA[l] = total;
+        ctl->pull_work[l] = s_work;
+        if (build_senders) {
+            ctl->nC[l] = total;
+            ctl->E[l + 1] = (unsigned long long)deg_total;
+            coff[total] = deg_total;
+        }
     }
 }
 
 // the members of A_l that no walk of out-lists finds: sinks of edge changes, A_{l-1} for models with a self term
 void frontier_mark_extras(Ctx* c, int l) {
-    RP_LAUNCH(c, k_mark_frontier, c->n_sm * 2, 256, 0, c->ctl, l, (int)c->self_term, 0, c->Clist[(l - 1) & 1], c->coff,
+    RP_LAUNCH(c, k_mark_frontier, c->n_sm * 2, 256, 0, c->ctl, l, (int)c->self_term, 0, sender_list(c, l - 1), c->coff,
               c->side[0], c->rec, c->A[l - 1], c->bitmap);
 }
 
-void frontier_compact_small(Ctx* c, int l) {
-    RP_LAUNCH(c, k_frontier_small, 1, 1024, 0, c->ctl, l, c->bitmap, c->n_words, c->A[l], (const int32_t*)c->side[1].deg);
-}
-
-void senders_build_small(Ctx* c, int l) {
-    RP_LAUNCH(c, k_senders_small, 1, 1024, 0, c->ctl, l, (const int32_t*)c->A[l], (const int32_t*)c->side[0].deg,
-              c->Clist[l & 1], c->posmap, c->coff);
+void frontier_compact_small(Ctx* c, int l, bool senders) {
+    RP_LAUNCH(c, k_frontier_small, 1, 1024, 0, c->ctl, l, c->bitmap, c->n_words, c->A[l], (const int32_t*)c->side[1].deg,
+              (int)senders, (const int32_t*)c->side[0].deg, c->posmap, c->coff);
 }
 
 void frontier_compact(Ctx* c, int l) {
@@ -408,10 +466,10 @@ __global__ void k_senders_release(Ctl* ctl, int l, const int32_t* __restrict__ s
 void senders_build(Ctx* c, int l, int n) {
     int32_t* senders = c->Clist[l & 1];
     if (!c->src_norm) {
-        // the senders are exactly the affected vertices: listed while their out-degrees are summed
+        // the senders are exactly the affected vertices: entered while their out-degrees are summed
         // (after a rejected batch every list is empty, so nothing needs the abort flag here)
-        scan_degrees_and_copy(c, c->A[l], &c->ctl->nA[l], 0, c->side[0].deg, c->coff, &c->ctl->E[l + 1], senders,
-                              &c->ctl->nC[l]);
+        scan_degrees_and_enter(c, c->A[l], &c->ctl->nA[l], 0, c->side[0].deg, c->coff, &c->ctl->E[l + 1], c->posmap,
+                               &c->ctl->nC[l]);
         return;
     }
     RP_LAUNCH(c, k_senders_from_affected, c->n_sm * 4, 256, 0, c->ctl, l, c->A[l], senders, c->posmap);
@@ -420,7 +478,7 @@ void senders_build(Ctx* c, int l, int n) {
 }
 
 void senders_release(Ctx* c, int l) {
-    RP_LAUNCH(c, k_senders_release, c->n_sm * 4, 256, 0, c->ctl, l, c->Clist[l & 1], c->posmap);
+    RP_LAUNCH(c, k_senders_release, c->n_sm * 4, 256, 0, c->ctl, l, (const int32_t*)sender_list(c, l), c->posmap);
 }
 
 }  // namespace rp

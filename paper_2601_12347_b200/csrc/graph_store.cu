@@ -218,6 +218,14 @@ __global__ void __launch_bounds__(256) k_stage_in(const __grid_constant__ StageA
     if (tid == nt - 1) d_ctl_reset(a.ctl, a.in.n_ops, a.in.n_rows);
 }
 
+struct ClassifyArgs {
+    const int32_t* op_seq;
+    int N;
+    unsigned long long *hkeys, *hwin;
+    int hmask;
+    int32_t *op_slot, *feat_last, *vdel_seq;
+};
+
 static StageArgs stage_args(const Ctx* c) { return StageArgs{c->ctl, c->stage_in, c->ups_dev, c->opw_dev, c->feat_dev, c->d[0]}; }
 
 static int stage_grid(const Ctx* c) {   // one 16-byte piece of the larger array per thread, up to eight blocks per SM
@@ -225,7 +233,27 @@ static int stage_grid(const Ctx* c) {   // one 16-byte piece of the larger array
     return c->stage_in.ups ? (int)std::min<long long>(words / 1024 + 1, c->n_sm * 8) : 1;
 }
 
-void graph_batch_stage_in(Ctx* c) { RP_LAUNCH(c, k_stage_in, stage_grid(c), 256, 0, stage_args(c)); }
+__device__ __forceinline__ void d_classify(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_seq, int N,
+                                           Ctl* ctl, unsigned long long* hkeys, unsigned long long* hwin, int hmask,
+                                           int32_t* op_slot, int32_t* feat_last, int32_t* vdel_seq, int no_vertex_ops);
+
+// staging and classification of a small batch in one block, one launch instead of two
+__global__ void __launch_bounds__(1024) k_stage_classify(const __grid_constant__ StageArgs a, const __grid_constant__ ClassifyArgs b) {
+    pdl_enter();
+    if (a.in.ups) d_stage_in(a, threadIdx.x, blockDim.x);
+    if (threadIdx.x == blockDim.x - 1) d_ctl_reset(a.ctl, a.in.n_ops, a.in.n_rows);
+    __syncthreads();
+    d_classify(a.ups, b.op_seq, b.N, a.ctl, b.hkeys, b.hwin, b.hmask, b.op_slot, b.feat_last, b.vdel_seq, 0);
+}
+
+static ClassifyArgs classify_args(const Ctx* c) {
+    return ClassifyArgs{c->op_seq, c->N, c->hkeys, c->hwin, c->hsize - 1, c->op_slot, c->feat_last, c->vdel_seq};
+}
+
+void graph_batch_stage_in(Ctx* c) {
+    if (c->front_one_block) RP_LAUNCH(c, k_stage_classify, 1, 1024, 0, stage_args(c), classify_args(c));
+    else RP_LAUNCH(c, k_stage_in, stage_grid(c), 256, 0, stage_args(c));
+}
 
 __device__ __forceinline__ void d_classify(const ripple_update* __restrict__ ups, const int32_t* __restrict__ op_seq, int N,
                                            Ctl* ctl, unsigned long long* hkeys, unsigned long long* hwin, int hmask,
@@ -520,7 +548,8 @@ void graph_batch_classify(Ctx* c, int n) {
         RP_LAUNCH(c, k_expand_copy, std::min(n, c->n_sm * 4), T, 0, c->ups_dev, c->op_seq, c->ctl, c->side[0],
                   c->side[1], c->vjobs);
     }
-    RP_LAUNCH(c, k_classify, grid_ops, T, 0, c->ups_dev, c->op_seq, c->N, c->ctl, c->hkeys, c->hwin,
+    if (!c->front_one_block)
+        RP_LAUNCH(c, k_classify, grid_ops, T, 0, c->ups_dev, c->op_seq, c->N, c->ctl, c->hkeys, c->hwin,
               c->hsize - 1, c->op_slot, c->feat_last, c->vdel_seq, (int)(c->n_local > 0));
     int grid = std::min(n, c->n_sm * 8);
     RP_LAUNCH(c, k_resolve, grid, T, 0, c->ups_dev, c->op_seq, c->ctl, c->hwin, c->op_slot, c->feat_last,
@@ -730,6 +759,94 @@ __device__ __forceinline__ void d_commit_degrees(Ctl* ctl, const Rec* __restrict
     }
 }
 
+// What follows the row update of a batch that one block handles: the list A_0 (sorted in shared memory from the winning
+// feature operations: no sweep of the frontier bitmap), the feature rows with their old values or deltas, and the senders
+// of hop 1 with their out-degree prefix.
+struct SeedArgs {
+    float* H0;
+    int ld;
+    float* D;          // compact rows of A_0, or null: nobody reads them
+    int keep_old;      // D receives the old values instead of deltas
+    int src_norm;
+    int32_t* A0;
+    int build_senders; // C_0 = A_0 (max / min aggregation and out-degree coefficients list their own)
+    int32_t* posmap;
+    int64_t* coff;
+};
+
+template <int MAXN>
+__device__ __forceinline__ void d_seed_rows(Ctl* ctl, const ripple_update* __restrict__ ups, const int32_t* __restrict__ feat_last,
+                                            const float* __restrict__ feat, int d0, uint32_t* bitmap, const Side& out,
+                                            const int32_t* __restrict__ deg_out_old, const SeedArgs& a) {
+    __shared__ int s_raw[MAXN], s_ids[MAXN];
+    __shared__ int64_t scratch_l[33];
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int n = min(ctl->n_ops, MAXN);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const ripple_update op = ups[i];
+        if ((op.op == RIPPLE_OP_SET_FEATURE || op.op == RIPPLE_OP_DEL_VERTEX) && feat_last[op.u] == i) {
+            s_raw[atomicAdd(&s_n, 1)] = op.u;
+            atomicAnd(&bitmap[op.u >> 5], ~(1u << (op.u & 31)));   // (resolution marked it for the general chain's sweep)
+        }
+    }
+    __syncthreads();
+    const int na = s_n;
+    for (int i = threadIdx.x; i < na; i += blockDim.x) {   // ascending: the rank of an id is the number of smaller ones
+        const int mine = s_raw[i];
+        int rank = 0;
+        for (int k = 0; k < na; ++k) rank += s_raw[k] < mine;
+        s_ids[rank] = mine;
+        a.A0[rank] = mine;
+    }
+    if (threadIdx.x == 0) { ctl->nA[0] = na; if (a.build_senders) ctl->nC[0] = na; }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = warp; i < na; i += (int)(blockDim.x >> 5)) {   // one warp per row
+        const int v = s_ids[i];
+        const ripple_update last = ups[feat_last[v]];
+        // the last word on the row is either a payload row or the vertex's deletion (zeros)
+        const float* src = last.op == RIPPLE_OP_SET_FEATURE ? feat + (size_t)last.v * d0 : nullptr;
+        float cn = 1.f, co = 1.f;
+        if (a.src_norm) {
+            const int d_now = out.deg[v], d_old = deg_out_old[v];
+            cn = d_now > 0 ? 1.0f / sqrtf((float)d_now) : 0.0f;
+            co = d_old < 0 ? cn : d_old > 0 ? 1.0f / sqrtf((float)d_old) : 0.0f;
+        }
+        for (int k = lane; k < a.ld; k += 32) {
+            const float x = (src && k < d0) ? src[k] : 0.f;
+            if (a.D) {
+                const float o = a.H0[(size_t)v * a.ld + k];
+                a.D[(size_t)i * a.ld + k] = a.keep_old ? o : cn * x - co * o;
+            }
+            a.H0[(size_t)v * a.ld + k] = x;
+        }
+    }
+    if (!a.build_senders) return;
+    int64_t carry = 0;
+    for (int i0 = 0; i0 < na; i0 += (int)blockDim.x) {
+        const int i = i0 + (int)threadIdx.x;
+        int64_t d = 0, sum;
+        if (i < na) {
+            a.posmap[s_ids[i]] = i;
+            d = out.deg[s_ids[i]];
+        }
+        const int64_t ex = block_exclusive_scan<int64_t>(d, scratch_l, sum);
+        if (i < na) a.coff[i] = carry + ex;
+        carry += sum;
+    }
+    if (threadIdx.x == 0) {
+        a.coff[na] = carry;
+        ctl->E[1] = (unsigned long long)carry;
+    }
+}
+
+static SeedArgs seed_args(const Ctx* c) {
+    return SeedArgs{c->H[0], c->ld[0], c->pre[1] ? (float*)nullptr : c->D[0], (int)(c->attention || rp_monotonic(c->agg)), (int)c->src_norm,
+                    c->A[0], (int)(!rp_monotonic(c->agg) && !c->src_norm), c->posmap, c->coff};
+}
+
 // The kernels of the row update, one launch each ...
 __global__ void k_del_mark(Ctl* ctl, const Rec* __restrict__ rec, Side out, Side in) { pdl_enter(); d_del_mark(ctl, rec, out, in); }
 __global__ void k_del_tail_read(Ctl* ctl, Rec* rec, Side out, Side in) { pdl_enter(); d_del_tail_read(ctl, rec, out, in); }
@@ -755,7 +872,9 @@ __global__ void k_commit_degrees(Ctl* ctl, const Rec* __restrict__ rec, Side out
 __global__ void __launch_bounds__(1024)
 k_mutate_small(Ctl* ctl, Rec* rec, Side out, Side in, const int32_t* __restrict__ grow_out,
                const int32_t* __restrict__ grow_in, const int32_t* __restrict__ shrink_out,
-               const int32_t* __restrict__ shrink_in, int64_t* moved_start, int32_t* moved_cap, int32_t* deg_out_old) {
+               const int32_t* __restrict__ shrink_in, int64_t* moved_start, int32_t* moved_cap, int32_t* deg_out_old,
+               int seed, const ripple_update* __restrict__ ups, const int32_t* __restrict__ feat_last,
+               const float* __restrict__ feat, int d0, uint32_t* bitmap, const __grid_constant__ SeedArgs sa) {
     pdl_enter();
     d_del_mark(ctl, rec, out, in);
     __syncthreads();
@@ -770,6 +889,9 @@ k_mutate_small(Ctl* ctl, Rec* rec, Side out, Side in, const int32_t* __restrict_
     d_add_write(ctl, rec, out, in);
     __syncthreads();
     d_commit_degrees(ctl, rec, out, in, deg_out_old, moved_start, moved_cap);
+    if (!seed || ctl->abort) return;
+    __syncthreads();
+    d_seed_rows<RP_ONE_BLOCK_BATCH>(ctl, ups, feat_last, feat, d0, bitmap, out, deg_out_old, sa);
 }
 
 // A batch of a handful of updates, none of them a vertex deletion, for models whose hop-0 senders are exactly
@@ -791,24 +913,15 @@ struct ApplySmallArgs {
     int64_t* moved_start;
     int32_t* moved_cap;
     int32_t* deg_out_old;
-    float* H0;
-    int ld;
-    float* D;
-    int keep_old;
-    int32_t* A0;
-    int build_senders;
-    int32_t *senders, *posmap;
-    int64_t* coff;
+    SeedArgs seed;
 };
 
 __global__ void __launch_bounds__(1024)
 k_apply_small(const __grid_constant__ ApplySmallArgs a) {
     pdl_enter();
-    __shared__ int s_ids[RP_TINY_BATCH];
-    __shared__ int s_n;
     Ctl* ctl = a.st.ctl;
     const StageIn& src_in = a.st.in;
-    if (threadIdx.x == 0) { d_ctl_reset(ctl, src_in.n_ops, src_in.n_rows); s_n = 0; }
+    if (threadIdx.x == 0) { d_ctl_reset(ctl, src_in.n_ops, src_in.n_rows); }
     if (src_in.ups) {   // (the payload rows are read where they lie)
         if ((int)threadIdx.x < 3 * src_in.n_ops)
             reinterpret_cast<uint32_t*>(a.st.ups)[threadIdx.x] = reinterpret_cast<const uint32_t*>(src_in.ups)[threadIdx.x];
@@ -838,52 +951,7 @@ k_apply_small(const __grid_constant__ ApplySmallArgs a) {
     d_commit_degrees(ctl, a.rec, a.out, a.in, a.deg_out_old, a.moved_start, a.moved_cap);
     __syncthreads();
     if (ctl->abort) return;
-    // A_0: the vertices whose last feature operation this is, ascending
-    const int n = ctl->n_ops;
-    if ((int)threadIdx.x < n) {
-        const ripple_update op = ups[threadIdx.x];
-        if (op.op == RIPPLE_OP_SET_FEATURE && a.feat_last[op.u] == (int)threadIdx.x) {
-            s_ids[atomicAdd(&s_n, 1)] = op.u;
-            atomicAnd(&a.bitmap[op.u >> 5], ~(1u << (op.u & 31)));   // (resolution marked it for the general chain's sweep)
-        }
-    }
-    __syncthreads();
-    const int na = s_n;
-    int mine = -1, rank = 0;
-    if ((int)threadIdx.x < na) {
-        mine = s_ids[threadIdx.x];
-        for (int k = 0; k < na; ++k) rank += s_ids[k] < mine;
-    }
-    __syncthreads();
-    if (mine >= 0) { s_ids[rank] = mine; a.A0[rank] = mine; }
-    if (threadIdx.x == 0) { ctl->nA[0] = na; if (a.build_senders) ctl->nC[0] = na; }
-    __syncthreads();
-    // feature rows: one warp per vertex of A_0
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int i = warp; i < na; i += (int)(blockDim.x >> 5)) {
-        const int v = s_ids[i];
-        const float* src = feat + (size_t)ups[a.feat_last[v]].v * a.st.d0;
-        for (int k = lane; k < a.ld; k += 32) {
-            const float x = k < a.st.d0 ? src[k] : 0.f;
-            const float o = a.H0[(size_t)v * a.ld + k];
-            a.D[(size_t)i * a.ld + k] = a.keep_old ? o : x - o;
-            a.H0[(size_t)v * a.ld + k] = x;
-        }
-    }
-    // senders of hop 1 = A_0, with the prefix of their out-degrees (max / min aggregation lists its own: the rows
-    // of A_0 whose values really changed)
-    if (a.build_senders && threadIdx.x == 0) {
-        int64_t sum = 0;
-        for (int i = 0; i < na; ++i) {
-            const int v = s_ids[i];
-            a.senders[i] = v;
-            a.posmap[v] = i;
-            a.coff[i] = sum;
-            sum += a.out.deg[v];
-        }
-        a.coff[na] = sum;
-        ctl->E[1] = (unsigned long long)sum;
-    }
+    d_seed_rows<RP_TINY_APPLY>(ctl, ups, a.feat_last, feat, a.st.d0, a.bitmap, a.out, a.deg_out_old, a.seed);
 }
 
 static ApplySmallArgs apply_small_args(const Ctx* c) {
@@ -894,9 +962,7 @@ static ApplySmallArgs apply_small_args(const Ctx* c) {
     a.bitmap = c->bitmap;
     for (int s = 0; s < 2; ++s) { a.grow[s] = c->grow_list[s]; a.shrink[s] = c->shrink_list[s]; }
     a.moved_start = c->moved_start; a.moved_cap = c->moved_cap; a.deg_out_old = c->deg_out_old;
-    a.H0 = c->H[0]; a.ld = c->ld[0]; a.D = c->D[0]; a.keep_old = c->attention || rp_monotonic(c->agg);
-    a.A0 = c->A[0]; a.build_senders = !rp_monotonic(c->agg);
-    a.senders = c->Clist[0]; a.posmap = c->posmap; a.coff = c->coff;
+    a.seed = seed_args(c);
     return a;
 }
 
@@ -908,12 +974,20 @@ void graph_batch_apply_small(Ctx* c) { RP_LAUNCH(c, k_apply_small, 1, 1024, 0, a
 cudaError_t graph_batch_retarget(Ctx* c, int n, cudaGraphExec_t exec, cudaGraphNode_t root) {
     cudaKernelNodeParams p{};
     StageArgs st;
+    ClassifyArgs cl;
     ApplySmallArgs ap;
-    void* args[1];
+    void* args[2];
     if (batch_is_tiny(c, n)) {
         ap = apply_small_args(c);
         args[0] = &ap;
         p.func = reinterpret_cast<void*>(k_apply_small);
+        p.gridDim = dim3(1); p.blockDim = dim3(1024);
+    } else if (c->front_one_block) {
+        st = stage_args(c);
+        cl = classify_args(c);
+        args[0] = &st;
+        args[1] = &cl;
+        p.func = reinterpret_cast<void*>(k_stage_classify);
         p.gridDim = dim3(1); p.blockDim = dim3(1024);
     } else {
         st = stage_args(c);
@@ -925,7 +999,7 @@ cudaError_t graph_batch_retarget(Ctx* c, int n, cudaGraphExec_t exec, cudaGraphN
     return cudaGraphExecKernelNodeSetParams(exec, root, &p);
 }
 
-void graph_batch_mutate(Ctx* c, int n) {
+void graph_batch_mutate(Ctx* c, int n, bool seed) {
     if (n <= 0) return;
     const int T = 256;
     int grid = std::min(div_up(2 * n, T), c->n_sm * 8);
@@ -933,7 +1007,9 @@ void graph_batch_mutate(Ctx* c, int n) {
     Side& i = c->side[1];
     if (n <= RP_ONE_BLOCK_BATCH) {
         RP_LAUNCH(c, k_mutate_small, 1, 1024, 0, c->ctl, c->rec, o, i, c->grow_list[0], c->grow_list[1],
-                  c->shrink_list[0], c->shrink_list[1], c->moved_start, c->moved_cap, c->deg_out_old);
+                  c->shrink_list[0], c->shrink_list[1], c->moved_start, c->moved_cap, c->deg_out_old, (int)seed,
+                  (const ripple_update*)c->ups_dev, (const int32_t*)c->feat_last, (const float*)c->feat_dev, c->d[0], c->bitmap,
+                  seed_args(c));
         return;
     }
     RP_LAUNCH(c, k_del_mark, grid, T, 0, c->ctl, c->rec, o, i);

@@ -409,7 +409,8 @@ k_update_rows_elementwise(const Ctl* ctl, const __grid_constant__ UpdParams p) {
 
 // Launches every form that the row counts can call for; exactly one of them does the work of each problem (decided on
 // the device).
-static void launch_update(Ctx* c, UpdPair& u, const TcW* const (&tw)[2], const TcW* both = nullptr) {
+// `over`: the hop whose list (A_over or C_over) the rows come from.
+static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2], const TcW* both = nullptr) {
     if (u.p[0].K == 0) {
         RP_LAUNCH(c, k_update_rows_elementwise, c->n_sm * 8, 256, 0, c->ctl, u.p[0]);
         return;
@@ -421,10 +422,10 @@ static void launch_update(Ctx* c, UpdPair& u, const TcW* const (&tw)[2], const T
         p.narrow_min_rows = 0;
         // The forms for many rows are only put into the chain when the last batch's frontiers (or a whole-graph pass)
         // were large enough for them; without them the tiled SIMT form takes whatever comes.
-        if (!c->tc_armed && p.list) continue;
+        if (!c->tc_armed[over] && p.list) continue;
         if (tw[i]->w && c->gemm_mode != RIPPLE_GEMM_FP32) {
             p.tc_mode = c->gemm_mode == RIPPLE_GEMM_TF32 ? TC_TF32 : TC_TF32X3;
-            p.tc_min_rows = 1024;
+            p.tc_min_rows = RP_TC_MIN_ROWS;
             p.tc_withhold = c->debug_tc_withhold;
             p.tc_w = tw[i]->w; p.tc_groups = tw[i]->groups; p.tc_chunks = tw[i]->chunks;
             tc.p[tc.n++] = p;
@@ -434,7 +435,7 @@ static void launch_update(Ctx* c, UpdPair& u, const TcW* const (&tw)[2], const T
         }
     }
     if (c->few_rows_form && u.p[0].list) RP_LAUNCH(c, k_update_rows<true>, c->n_sm * 4, 256, 0, c->ctl, u);
-    else if (u.p[0].list || tc.n < u.n || c->N < 1024) RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, u);
+    else if (u.p[0].list || tc.n < u.n || c->N < RP_TC_MIN_ROWS) RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, u);
     for (int i = 0; i < u.n; ++i)
         if (u.p[i].narrow_min_rows) RP_LAUNCH(c, k_update_rows_narrow, c->n_sm * 2, 256, NARROW_SMEM, c->ctl, u.p[i]);
     if (both && tc.n == 2) {
@@ -444,18 +445,18 @@ static void launch_update(Ctx* c, UpdPair& u, const TcW* const (&tw)[2], const T
     if (tc.n) launch_update_tc(c, tc);
 }
 
-static void launch_update(Ctx* c, const UpdParams& p, const TcW& tw) {
+static void launch_update(Ctx* c, const UpdParams& p, int over, const TcW& tw) {
     UpdPair u{};
     u.p[0] = p;
     u.n = 1;
-    launch_update(c, u, {&tw, &tw});
+    launch_update(c, u, over, {&tw, &tw});
 }
 
 // P^l_u = W_n^T h^{l-1}_u (all rows if `full`)
 static UpdParams neighbour_problem(Ctx* c, int l, bool full) {
     const LayerDev& ly = c->layer[l];
     UpdParams p{};
-    p.list = full ? nullptr : c->Clist[(l - 1) & 1];
+    p.list = full ? nullptr : sender_list(c, l - 1);
     p.n_dev = full ? nullptr : &c->ctl->nC[l - 1];
     p.n_host = c->N;
     p.a_mode = A_SELF; p.epi_mode = EPI_COMMIT; p.alpha = 1.0f;
@@ -492,7 +493,7 @@ static void project(Ctx* c, int l, const UpdParams& nbr, bool full) {
     u.p[0] = nbr;
     u.n = 1;
     if (c->Z[l]) u.p[u.n++] = self_problem(c, l, full);   // the same rows: one launch for both products
-    launch_update(c, u, {&ly.tc_nbr, &ly.tc_self}, ly.tc_pair.w ? &ly.tc_pair : nullptr);
+    launch_update(c, u, l - 1, {&ly.tc_nbr, &ly.tc_self}, ly.tc_pair.w ? &ly.tc_pair : nullptr);
 }
 
 void project_full(Ctx* c, int l) { project(c, l, neighbour_problem(c, l, true), true); }
@@ -511,7 +512,7 @@ void sender_transform(Ctx* c, int l) {
 
 void self_project(Ctx* c, int l, bool full) {
     if (!c->Z[l] || c->pre[l]) return;   // (a layer that transforms first has done it with the neighbour projection)
-    launch_update(c, self_problem(c, l, full), c->layer[l].tc_self);
+    launch_update(c, self_problem(c, l, full), l - 1, c->layer[l].tc_self);
 }
 
 void update_rows(Ctx* c, int l, bool full) {
@@ -542,12 +543,12 @@ void update_rows(Ctx* c, int l, bool full) {
         p.a_mode = pre ? A_SELF : A_SUM; p.epi_mode = EPI_TEMP; p.alpha = 1.0f + ly.eps;
         p.K = ly.ld_in; p.W = ly.W1; p.ldw = ly.ld_hid; p.bias = ly.b1; p.n_cols = ly.ld_hid;
         p.act = RIPPLE_ACT_RELU; p.Hout = c->T; p.ld_o = ly.ld_hid; p.Dout = nullptr;
-        launch_update(c, p, ly.tc_main);
+        launch_update(c, p, l, ly.tc_main);
         p.a_mode = A_DENSE; p.epi_mode = EPI_COMMIT; p.addend = nullptr; p.addend_rw = nullptr; p.addend_delta = nullptr;
         p.Hprev = c->T; p.ld_h = ly.ld_hid;
         p.K = ly.ld_hid; p.W = ly.W2; p.ldw = ly.ld_out; p.bias = ly.b2; p.n_cols = ly.ld_out;
         p.act = ly.act; p.Hout = c->H[l]; p.ld_o = ly.ld_out; p.Dout = dout;
-        launch_update(c, p, ly.tc_2);
+        launch_update(c, p, l, ly.tc_2);
         return;
     }
     p.epi_mode = EPI_COMMIT;
@@ -563,7 +564,7 @@ void update_rows(Ctx* c, int l, bool full) {
     p.ldw = ly.ld_out; p.bias = ly.b1; p.n_cols = ly.ld_out;
     p.act = ly.act; p.Hout = c->H[l]; p.ld_o = ly.ld_out; p.Dout = dout;
     if (!pre) p.ld_add = ly.ld_out;   // leading dimension of the cached projection
-    launch_update(c, p, ly.tc_main);
+    launch_update(c, p, l, ly.tc_main);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -589,8 +590,10 @@ __global__ void k_feature_rows(Ctl* ctl, const ripple_update* __restrict__ ups, 
         }
         for (int k = lane_id(); k < ld; k += 32) {
             float x = (src && k < d0) ? src[k] : 0.f;
-            float o = H0[(size_t)v * ld + k];
-            D[(size_t)i * ld + k] = keep_old ? o : cn * x - co * o;
+            if (D) {
+                float o = H0[(size_t)v * ld + k];
+                D[(size_t)i * ld + k] = keep_old ? o : cn * x - co * o;
+            }
             H0[(size_t)v * ld + k] = x;
         }
     }
@@ -600,7 +603,7 @@ void feature_rows(Ctx* c, int n) {
     if (n <= 0) return;
     RP_LAUNCH(c, k_feature_rows, std::min(div_up(n, 8), c->n_sm * 8), 256, 0, c->ctl, c->ups_dev, c->feat_dev,
               c->d[0], c->A[0], c->feat_last, (int)c->src_norm, c->side[0].deg, c->deg_out_old, c->H[0],
-              c->ld[0], c->D[0], (int)(rp_monotonic(c->agg) || c->attention));
+              c->ld[0], c->pre[1] ? (float*)nullptr : c->D[0], (int)(rp_monotonic(c->agg) || c->attention));
 }
 
 // ---------------------------------------------------------------------------------------------

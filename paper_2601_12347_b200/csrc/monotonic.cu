@@ -516,7 +516,7 @@ __global__ void k_max_senders(Ctl* ctl, int l, const int32_t* __restrict__ A, co
 
 static void launch_long_rows(Ctx* c, int l, int mode, const float* M, int ld, float* S, int32_t* long_rows, int* n_long) {
     const int nv = div_up(ld, 128), is_min = (int)(c->agg == RIPPLE_AGG_MIN);
-    int2* items = reinterpret_cast<int2*>(c->coff);   // the senders' degree prefix is not needed at this point
+    int2* items = c->items;
     int* n_items = &c->ctl->max_items[l];
     float* saved = c->Dt;                              // compact scratch rows (no layer transforms before a max)
     RP_LAUNCH(c, k_max_long_begin, c->n_sm * 2, 256, 0, c->ctl, mode, long_rows, n_long, c->side[1], ld, S, saved,

@@ -75,7 +75,7 @@ static void destroy_ctx(Ctx* c) {
     cudaFree(c->halo_owner); cudaFree(c->halo_rid); cudaFree(c->silent_dev); cudaFree(c->rows_sent);
     free(c->halo_owner_h); free(c->halo_rid_h);
     for (int i = 0; i < c->n_ipc_opened; ++i) cudaIpcCloseMemHandle(c->ipc_opened[i]);
-    cudaFree(c->T); cudaFree(c->Dt); cudaFree(c->coff); cudaFree(c->bitmap); cudaFree(c->bitmap2); cudaFree(c->old_idx); cudaFree(c->invmask); cudaFree(c->posmap); cudaFree(c->deg_out_old);
+    cudaFree(c->T); cudaFree(c->Dt); cudaFree(c->coff); cudaFree(c->items); cudaFree(c->bitmap); cudaFree(c->bitmap2); cudaFree(c->old_idx); cudaFree(c->invmask); cudaFree(c->posmap); cudaFree(c->deg_out_old);
     cudaFree(c->feat_last); cudaFree(c->ups_dev); cudaFree(c->opw_dev); cudaFree(c->feat_dev); cudaFree(c->hkeys); cudaFree(c->hwin); cudaFree(c->op_seq); cudaFree(c->vdel_seq); cudaFree(c->vjobs);
     cudaFree(c->op_slot); cudaFree(c->rec); cudaFree(c->tile_sums); cudaFree(c->scan_done); cudaFree(c->ctl);
     cudaFree(c->moved_start); cudaFree(c->moved_cap);
@@ -126,7 +126,7 @@ static ripple_status run_full(Ctx* c) {
     return RIPPLE_OK;
 }
 
-static size_t coff_items(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / (RP_ANEW_CHUNK / 2)) + 64; }
+static size_t item_count(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / (RP_ANEW_CHUNK / 2)) + 64; }
 
 static std::vector<float> padded_matrix(const float* src, int rows, int cols, int rows_p, int cols_p) {
     std::vector<float> m((size_t)rows_p * cols_p, 0.f);
@@ -233,7 +233,7 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         memset(c->stage_host, 0, c->stage_bytes);
         k_touch_host<<<1, 256, 0, c->stream>>>(c->stage_host, c->stage_bytes, reinterpret_cast<volatile int*>(c->ctl_host));
         c->n_words = (N + 31) / 32;
-        c->n_tile_sums = std::max(div_up(N, 1024) + 2, div_up(c->n_words, 256) + 2);
+        c->n_tile_sums = std::max(div_up(N, 1024) + 2, 2 * div_up(c->n_words, 256) + 4);
         CK(dev_alloc(&c->tile_sums, (size_t)c->n_tile_sums, 0));
         CK(dev_alloc(&c->scan_done, 1, 0));
         for (auto& e : c->ev) CK(cudaEventCreate(&e));
@@ -387,10 +387,10 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         }
         CK(dev_alloc(&c->moved_start, (size_t)4 * o.max_batch));
         CK(dev_alloc(&c->moved_cap, (size_t)4 * o.max_batch));
-        // degree prefix of a sender list; also the (vertex, chunk) work items of long in-lists during a
-        // gather: a row of more than 256 entries gives at most 2 items per 256 of them, a row gathered anew by the
-        // fold one per RP_ANEW_CHUNK and one more
-        CK(dev_alloc(&c->coff, coff_items(c, (size_t)N), 0));
+        // (vertex, chunk) work items of long in-lists: a row of more than 256 entries gives at most 2 items per 256 of
+        // them, a row gathered anew by the fold one per RP_ANEW_CHUNK and one more
+        CK(dev_alloc(&c->items, item_count(c, (size_t)N)));
+        CK(dev_alloc(&c->coff, (size_t)N + 2, 0));   // degree prefix of a sender list
         CK(dev_alloc(&c->bitmap, (size_t)c->n_words + 256, 0));
         if (rp_monotonic(agg)) {
             CK(dev_alloc(&c->bitmap2, (size_t)c->n_words + 256, 0));
@@ -463,11 +463,14 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
         STAMP();  // 0
         // Apply (Sec. 3.3): normalise the batch, mutate both adjacency directions, replace features
         graph_batch_classify(c, nb);
-        graph_batch_mutate(c, nb);
-        frontier_seed_features(c, nb);
-        feature_rows(c, nb);
+        const bool seeded = nb <= RP_ONE_BLOCK_BATCH;   // the block that updates the rows goes on to A_0 and its senders
+        graph_batch_mutate(c, nb, seeded);
+        if (!seeded) {
+            frontier_seed_features(c, nb);
+            feature_rows(c, nb);
+        }
         if (rp_monotonic(c->agg)) max_senders_build(c, 0);
-        else senders_build(c, 0, nb);
+        else if (!seeded || c->src_norm) senders_build(c, 0, nb);
     }
     STAMP();  // 1
     if (rp_monotonic(c->agg)) {
@@ -492,7 +495,7 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
             att_hop(c, l, nb, small);
             STAMP();
             att_update(c, l, false);
-            if (l < L) { if (small) senders_build_small(c, l); else senders_build(c, l, nb); }
+            if (l < L) senders_build(c, l, nb);
             STAMP();
         }
     }
@@ -507,10 +510,12 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
         if (pull) frontier_compact(c, l);
         STAMP();
         scatter_layer(c, l, nb);
-        // tiny batches on graphs whose frontier bitmap one block can sweep: A_l, and later the next hop's senders,
-        // by one launch each instead of two
+        // tiny batches on graphs whose frontier bitmap one block can sweep: A_l by one launch instead of two
         const bool merged = tiny && !pull && c->n_words <= RP_TINY_WORDS;
-        if (merged) frontier_compact_small(c, l);
+        // the next hop's senders are listed along with the frontier where this hop's are done with by then
+        const bool senders_too = l < L && !pull && !c->src_norm && nb > 0;
+        if (merged) frontier_compact_small(c, l, senders_too);
+        else if (senders_too) frontier_compact_senders(c, l);
         else if (!pull) frontier_compact(c, l);
         if (nb <= 0) senders_release(c, l - 1);   // (otherwise the last kernel of the hop's delta form clears them)
         fold_deltas(c, l);
@@ -518,7 +523,7 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
         STAMP();
         self_project(c, l, false);
         update_rows(c, l, false);
-        if (l < L) { if (merged) senders_build_small(c, l); else senders_build(c, l, nb); }
+        if (l < L && !senders_too) senders_build(c, l, nb);
         STAMP();
     }
     graph_batch_cleanup(c, nb);
@@ -534,9 +539,10 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
 // if it turns out saturated: slower for that one batch, never wrong, and armed for the next.
 static void arm_rebuild(Ctx* c, int nb) {
     const bool no_history = c->batches_done == 0 || nb > 4 * std::max(c->last_nb, 1);
-    // the tensor-core update takes over from 1024 rows: in the chain if any frontier of the last batch came near
-    c->tc_armed = no_history;
-    for (int l = 0; l <= c->L; ++l) c->tc_armed |= c->stats.affected[l] >= 256 || c->stats.senders[l] >= 256;
+    // the tensor-core update takes over from a few hundred rows (see launch_update): in the chain of an update if the
+    // list it goes over came near that in the batch before
+    for (int l = 0; l <= c->L; ++l)
+        c->tc_armed[l] = no_history || c->stats.affected[l] >= RP_TC_MIN_ROWS / 4 || c->stats.senders[l] >= RP_TC_MIN_ROWS / 4;
     for (int l = 1; l <= c->L; ++l) {
         bool armed = false;
         if (rp_monotonic(c->agg) || c->attention) armed = false;
@@ -574,8 +580,10 @@ static int chain_size(const Ctx* c, int nb) {
 static bool launch_batch_graph(Ctx* c, int ng) {
     if (c->no_graphs || c->timing || ng < 1 || c->debug_tc_withhold) return false;
     // the captured chain differs with the expansion kernels and with the hops whose rebuilding form is enqueued
-    uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->tc_armed ? 4 : 0);
+    uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->few_rows_form ? 4 : 0);
+    key = 2 * key + (c->front_one_block ? 1 : 0);
     for (int l = 1; l <= c->L; ++l) key = 4 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0);
+    for (int l = 0; l <= c->L; ++l) key = 2 * key + (c->tc_armed[l] ? 1 : 0);
     int slot = -1;
     for (int i = 0; i < RP_GRAPH_SLOTS; ++i)
         if (c->graph_exec[i] && c->graph_key[i] == key) slot = i;
@@ -665,7 +673,10 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
     }
     arm_rebuild(c, nb);
     c->has_opw = c->weighted && edge_weights && nb;
-    c->few_rows_form = ng <= 128;
+    c->few_rows_form = nb <= 128;
+    // a batch of a few tens of kilobytes is staged and classified by one block (more would keep it waiting for the bus)
+    c->front_one_block = !c->may_expand && ng <= RP_ONE_BLOCK_BATCH &&
+                         sizeof(ripple_update) * (size_t)nb + sizeof(float) * (size_t)nr * c->d[0] <= (32u << 10);
     // The first kernel of the chain fetches the batch itself, from device memory or from pinned host memory: the caller's
     // if it is pinned, else a packed copy in the library's own staging area.  Pageable batches that do not fit there
     // are copied ahead of the chain.
@@ -905,7 +916,8 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
     CK(grow_array(&c->att_so, N0 + 32, N1 + 32, 0));
     if (c->att_items) CK(grow_array(&c->att_items, N0 + (size_t)(c->side[1].col_size / RP_ATT_CHUNK) + 64, N1 + (size_t)(c->side[1].col_size / RP_ATT_CHUNK) + 64, 0));
     {
-        CK(grow_array(&c->coff, coff_items(c, N0), coff_items(c, N1), 0));
+        CK(grow_array(&c->items, item_count(c, N0), item_count(c, N1), 0));
+        CK(grow_array(&c->coff, N0 + 2, N1 + 2, 0));
     }
     {
         const size_t w0 = (size_t)c->n_words + 256, w1 = (N1 + 31) / 32 + 256;
@@ -919,7 +931,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
     CK(grow_array(&c->feat_last, N0, N1, 0xFF));
     CK(grow_array(&c->vdel_seq, N0, N1, 0xFF));
     {
-        const int nt = std::max(div_up((int64_t)N1, 1024) + 2, div_up((int64_t)((N1 + 31) / 32), 256) + 2);
+        const int nt = std::max(div_up((int64_t)N1, 1024) + 2, 2 * div_up((int64_t)((N1 + 31) / 32), 256) + 4);
         CK(grow_array(&c->tile_sums, (size_t)c->n_tile_sums, (size_t)nt, 0));
         c->n_tile_sums = nt;
     }
@@ -938,7 +950,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
         CK(cudaMemcpy(lists_dev, lists.data(), sizeof(int32_t*) * lists.size(), cudaMemcpyHostToDevice));
         c->launches = 0;
         c->debug_tc_withhold = 0;
-        c->tc_armed = 1;
+        for (int l = 0; l <= c->L; ++l) c->tc_armed[l] = 1;
         c->few_rows_form = count <= 256;
         RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
         k_list_new_vertices<<<std::min(div_up(count, 256), c->n_sm * 4), 256, 0, c->stream>>>(c->ctl, L, first, count, lists_dev, (int)lists.size());
@@ -1171,7 +1183,7 @@ extern "C" ripple_status ripple_part_begin(ripple_ctx* ctx, const ripple_update*
     c->may_expand = 0;
     c->has_opw = c->weighted && edge_weights && nb;
     c->debug_tc_withhold = 0;
-    c->tc_armed = 1;
+    for (int l = 0; l <= c->L; ++l) c->tc_armed[l] = 1;
     c->few_rows_form = nb <= 128;
     for (int l = 0; l <= c->L; ++l) c->rebuild_armed[l] = 0;
     if (nb) cudaMemcpyAsync(c->ups_dev, ups, sizeof(ripple_update) * (size_t)nb, kind, c->stream);

@@ -23,6 +23,7 @@
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
 #define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold (sizes the item buffer)
+#define RP_TC_MIN_ROWS 512          // row count from which a layer update takes the tensor-core form
 #define RP_ATT_CHUNK 128            // attention: in-list entries per work item of a recomputation (sizes the item buffer)
 #define RP_TINY_BATCH 32            // batches up to this size list their frontiers and senders in one block each
 #define RP_TINY_APPLY 4             // ... and up to this size run the whole of Apply in one block (operations are resolved one after the other there)
@@ -191,7 +192,7 @@ struct Ctx {
     int64_t max_batch;
     int scatter_mode, gemm_mode, timing;
     int rebuild_armed[RP_MAXL + 1];   // per hop: the rebuilding form is enqueued for this batch (see arm_rebuild)
-    int tc_armed;                     // the tensor-core form of the layer update is enqueued for this batch
+    int tc_armed[RP_MAXL + 1];        // updates over the rows of A_l (or C_l) carry their tensor-core form in this batch
     int pull_hop[RP_MAXL + 1];        // per hop: the delta scatter of this batch gathers per sink instead of pushing (see arm_rebuild)
     int gather_min_width;             // narrowest message row (floats) whose hop may gather (environment RIPPLE_GATHER_MIN_WIDTH)
     long long gather_min_messages;    // ... if the hop delivered at least this many messages in the batch before
@@ -229,6 +230,7 @@ struct Ctx {
     int ws[RP_MAXL + 1];     // row width (floats, padded) of S^l and of hop-l messages
     int32_t* A[RP_MAXL + 1];   // affected lists
     int32_t* Clist[2];         // sender list, ping-pong (A_l followed by extra sources)
+    int2* items;               // (vertex, in-list chunk) work items of long rows
     int64_t* coff;             // exclusive prefix of out-degrees over the sender list (+1)
     uint32_t* bitmap;          // N bits
     int n_words;
@@ -257,6 +259,7 @@ struct Ctx {
     char* stage_host;  // pinned: operations, weights and payload rows of a batch that arrives in pageable memory
     size_t stage_bytes;
     StageIn stage_in;  // the batch being applied
+    int front_one_block;   // the batch being applied is staged and classified by one block
     int few_rows_form; // the batch being applied is small: its row updates carry the few-row form (see k_update_rows)
     int no_graphs;
     cudaGraph_t graph[RP_GRAPH_SLOTS];
@@ -277,6 +280,10 @@ struct Ctx {
     int64_t launches;
     char err[512];
 };
+
+// the senders C_l: the affected vertices themselves, unless a changed source coefficient adds vertices to them (or
+// max / min aggregation drops some)
+inline int32_t* sender_list(const Ctx* c, int l) { return c->src_norm || rp_monotonic(c->agg) ? c->Clist[l & 1] : c->A[l]; }
 
 // ---- helpers -----------------------------------------------------------------------------------
 inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
@@ -320,7 +327,7 @@ bool batch_is_tiny(const Ctx* c, int n);                // a handful of updates:
 void graph_batch_stage_in(Ctx* c);                      // first kernel of a chain: the batch into the library's buffers, control block reset
 void graph_batch_apply_small(Ctx* c);                   // first kernel of a tiny batch's chain: the same, all of Apply and the hop-0 senders, in one block
 cudaError_t graph_batch_retarget(Ctx* c, int n, cudaGraphExec_t exec, cudaGraphNode_t root);   // a captured chain reads this batch
-void graph_batch_mutate(Ctx* c, int n);                 // apply the net changes to both directions
+void graph_batch_mutate(Ctx* c, int n, bool seed = false);   // apply the net changes to both directions; seed: batches of one block's size list A_0, write its rows and the hop-1 senders on the way
 void graph_batch_cleanup(Ctx* c, int n);                // reset per-batch scratch
 cudaError_t graph_export(Ctx* c, int64_t* rowptr, int32_t* col, float* weight, int64_t col_capacity, int64_t* n_edges);
 
@@ -331,8 +338,8 @@ void frontier_seed_features(Ctx* c, int n);             // A_0 from the batch's 
 void frontier_mark(Ctx* c, int l, bool walk, int n);    // bitmap of A_l: (walk) edge-record sinks, A_{l-1} and Out(C_{l-1}); rebuilding hops: bottom-up
 void frontier_mark_extras(Ctx* c, int l);               // marks only what no walk finds (for hops whose message walk marks its sinks itself)
 void frontier_compact(Ctx* c, int l);                   // bitmap -> ascending list A_l
-void frontier_compact_small(Ctx* c, int l);              // the same in one block (tiny batches, small graphs)
-void senders_build_small(Ctx* c, int l);                // C_l = A_l with its degree prefix, in one block
+void frontier_compact_senders(Ctx* c, int l);           // the same, and C_l = A_l with its degree prefix
+void frontier_compact_small(Ctx* c, int l, bool senders);   // likewise in one block (tiny batches, small graphs)
 void senders_build(Ctx* c, int l, int n);               // C_l, posmap, coff, E_{l+1}
 void senders_release(Ctx* c, int l);                    // clear posmap entries of C_l
 

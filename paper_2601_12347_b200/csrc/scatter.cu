@@ -213,8 +213,7 @@ void spmm_full(Ctx* c, int l) {
         M = c->P[l];
     }
     const int grid = c->n_sm * 16, T = 256;
-    // work items of the long rows live in the degree-prefix buffer, which is idle during a full pass
-    int2* items = reinterpret_cast<int2*>(c->coff);
+    int2* items = c->items;
     int* n_items = &c->ctl->work_counter[(l - 1) & 7];
 #define SPMM(NV, LPR)                                                                                              \
     do {                                                                                                           \
@@ -228,6 +227,52 @@ void spmm_full(Ctx* c, int l) {
 }
 
 // ---------------------------------------------------------------------------------------------
+// edge-change records
+// ---------------------------------------------------------------------------------------------
+// Messages of the net edge changes: S_v += sign * w * M_r with M_r = c_old m_old of the record's
+// source (= c_new m_new - D_u if the source is a sender of this hop, c m otherwise) and w the edge's
+// stored weight (1 without stored weights).  One warp per record; rows have the inbox width.
+// A pushing hop delivers them along with the walk (both only add to the accumulator), from the far end of the grid; a
+// gathering hop, whose gather stores the rows it finishes, afterwards in a launch of their own.
+struct RecMsgs {
+    const Rec* rec;
+    int src_norm;
+    const int32_t* deg_out;
+    const int32_t* posmap;
+    const float* Mrows;
+};
+
+__device__ __forceinline__ void d_scatter_records(const Ctl* ctl, const RecMsgs& a, const float* __restrict__ D, int ld, float* S) {
+    const int n = ctl->n_rec;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5, warp = nwarps - 1 - (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = lane_id(), nq = ld >> 2;
+    for (int r = warp; r < n; r += nwarps) {
+        if (a.rec[r].silent) continue;   // partitioned execution: the source's worker sends for this edge
+        const int u = a.rec[r].u;
+        const int p = a.posmap[u];
+        const float4* hrow = reinterpret_cast<const float4*>(a.Mrows + (size_t)u * ld);
+        const float cn = a.src_norm ? coef_from_degree(a.deg_out[u]) : 1.0f;
+        const float sgn = (float)a.rec[r].sign * a.rec[r].w;
+        float* dst = S + (size_t)a.rec[r].v * ld;
+        for (int q = lane; q < nq; q += 32) {
+            float4 h = __ldg(hrow + q);
+            float4 m = make_float4(cn * h.x, cn * h.y, cn * h.z, cn * h.w);
+            if (p >= 0) {
+                float4 d = __ldg(reinterpret_cast<const float4*>(D + (size_t)p * ld) + q);
+                m.x -= d.x; m.y -= d.y; m.z -= d.z; m.w -= d.w;
+            }
+            red_add_v4(dst + 4 * q, make_float4(sgn * m.x, sgn * m.y, sgn * m.z, sgn * m.w));
+        }
+    }
+}
+
+__global__ void k_scatter_records(Ctl* ctl, int l, const RecMsgs recs, const float* __restrict__ D, int ld, float* S) {
+    pdl_enter();
+    if (ctl->abort || ctl->regather[l]) return;
+    d_scatter_records(ctl, recs, D, ld, S);
+}
+
+// ---------------------------------------------------------------------------------------------
 // push scatter
 // ---------------------------------------------------------------------------------------------
 constexpr int PUSH_CHUNK = 64, PUSH_CHUNK_LARGE = 256;  // edges per warp work item
@@ -235,9 +280,11 @@ constexpr int PUSH_CHUNK = 64, PUSH_CHUNK_LARGE = 256;  // edges per warp work i
 template <int NV, int LPR>
 __global__ void __launch_bounds__(256)
 k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff,
-               Side out, const float* __restrict__ D, int ld, float* S, uint32_t* bitmap) {
+               Side out, const float* __restrict__ D, int ld, float* S, uint32_t* bitmap,
+               const RecMsgs recs) {
     pdl_enter();
     if (ctl->abort || ctl->pull[l] || ctl->regather[l]) return;
+    d_scatter_records(ctl, recs, D, ld, S);
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
@@ -302,11 +349,13 @@ k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64
 template <int NQ, bool WEIGHTED>
 __global__ void __launch_bounds__(256)
 k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff,
-                      Side out, const float* __restrict__ D, float* S, uint32_t* bitmap) {
+                      Side out, const float* __restrict__ D, float* S, uint32_t* bitmap,
+                      const RecMsgs recs) {
     pdl_enter();
     constexpr int LCM = NQ == 12 ? 96 : NQ == 10 ? 160 : NQ * 32;
     constexpr int NI = LCM / 32, G = LCM / NQ, LD = NQ * 4;
     if (ctl->abort || ctl->pull[l] || ctl->regather[l]) return;
+    d_scatter_records(ctl, recs, D, LD, S);
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
@@ -607,40 +656,6 @@ k_scatter_gather_long(Ctl* ctl, int l, Side in, const int32_t* __restrict__ posm
 }
 
 // ---------------------------------------------------------------------------------------------
-// edge-change records
-// ---------------------------------------------------------------------------------------------
-// Messages of the net edge changes: S_v += sign * w * M_r with M_r = c_old m_old of the record's
-// source (= c_new m_new - D_u if the source is a sender of this hop, c m otherwise) and w the edge's
-// stored weight (1 without stored weights).  One warp per record; rows have the inbox width.
-__global__ void k_scatter_records(Ctl* ctl, int l, const Rec* __restrict__ rec, int src_norm,
-                                  const int32_t* __restrict__ deg_out, const int32_t* __restrict__ posmap,
-                                  const float* __restrict__ Mrows, const float* __restrict__ D, int ld, float* S) {
-    pdl_enter();
-    if (ctl->abort || ctl->regather[l]) return;
-    const int n = ctl->n_rec;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int lane = lane_id(), nq = ld >> 2;
-    for (int r = warp; r < n; r += nwarps) {
-        if (rec[r].silent) continue;   // partitioned execution: the source's worker sends for this edge
-        const int u = rec[r].u;
-        const int p = posmap[u];
-        const float4* hrow = reinterpret_cast<const float4*>(Mrows + (size_t)u * ld);
-        const float cn = src_norm ? coef_from_degree(deg_out[u]) : 1.0f;
-        const float sgn = (float)rec[r].sign * rec[r].w;
-        float* dst = S + (size_t)rec[r].v * ld;
-        for (int q = lane; q < nq; q += 32) {
-            float4 h = __ldg(hrow + q);
-            float4 m = make_float4(cn * h.x, cn * h.y, cn * h.z, cn * h.w);
-            if (p >= 0) {
-                float4 d = __ldg(reinterpret_cast<const float4*>(D + (size_t)p * ld) + q);
-                m.x -= d.x; m.y -= d.y; m.z -= d.z; m.w -= d.w;
-            }
-            red_add_v4(dst + 4 * q, make_float4(sgn * m.x, sgn * m.y, sgn * m.z, sgn * m.w));
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
 // rebuilding hop (scoped recomputation of the aggregates, the "RC" strategy of Sec. 3.2 applied to
 // one hop): S_v of every affected vertex is gathered again over In_new(v) from the current rows
 // ---------------------------------------------------------------------------------------------
@@ -847,7 +862,7 @@ k_fold_deltas(Ctl* ctl, int l, const int32_t* __restrict__ A, int ld, float* S, 
 void fold_deltas(Ctx* c, int l) {
     if (c->fused_fold[l]) return;   // folded inside the row update's epilogue
     const float* M = c->pre[l] ? c->P[l] : c->H[l - 1];
-    int2* items = reinterpret_cast<int2*>(c->coff);   // the degree prefix of the senders is no longer needed
+    int2* items = c->items;
     const int ld = c->ws[l];
     RP_LAUNCH(c, k_fold_deltas, c->n_sm * 8, 256, 0, c->ctl, l, c->A[l], ld, c->S[l], c->dS[l], c->Eb[l],
               c->rebuild_tau2, c->side[1].deg, items);
@@ -872,7 +887,7 @@ void choose_direction(Ctx* c, int l) {
 void scatter_layer(Ctx* c, int l, int n) {
     const int ld = c->ws[l];
     const float* D = c->D[(l - 1) & 1];
-    const int32_t* senders = c->Clist[(l - 1) & 1];
+    const int32_t* senders = sender_list(c, l - 1);
     const int T = 256;
     const int grid = c->n_sm * 8;
     // Edge records: M_r = c_old m_old of the record's source = c_new m_new - D_u for a sender.  A
@@ -886,8 +901,10 @@ void scatter_layer(Ctx* c, int l, int n) {
         Mrows = c->P[l];
     }
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l], c->stream);
-#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap)
-    int2* gather_items = reinterpret_cast<int2*>(c->coff);   // (the marking walk was the last reader of the degree prefix)
+#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap, recs)
+    int2* gather_items = c->items;
+    const RecMsgs recs{c->rec, (int)c->src_norm, c->side[0].deg, c->posmap, Mrows};
+    bool recs_done = false;
 #define PULL(NV, LPR)                                                                                                  \
     do {                                                                                                               \
         RP_LAUNCH(c, (k_scatter_gather<NV, LPR>), grid, T, 0, c->ctl, l, c->A[l], c->side[1], c->posmap, Dm, ld,      \
@@ -900,21 +917,22 @@ void scatter_layer(Ctx* c, int l, int n) {
         RP_LAUNCH(c, k_scatter_push_bulk, grid, T, (size_t)8 * 2 * ld * sizeof(float), c->ctl, l, senders, c->coff,
                   c->side[0], Dm, ld, c->dS[l], c->bitmap);
     } else if (!c->pull_hop[l] && c->scatter_mode != RIPPLE_SCATTER_REGATHER) {
-#define PACKED(NQ, WGT) RP_LAUNCH(c, (k_scatter_push_packed<NQ, WGT>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, c->dS[l], c->bitmap)
+#define PACKED(NQ, WGT) RP_LAUNCH(c, (k_scatter_push_packed<NQ, WGT>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, c->dS[l], c->bitmap, recs)
         if (ld == 48 && c->weighted) PACKED(12, true);
         else if (ld == 48) PACKED(12, false);
         else if (ld == 40 && c->weighted) PACKED(10, true);
         else if (ld == 40) PACKED(10, false);
 #undef PACKED
         else RP_WIDTH_DISPATCH(ld, PUSH);
+        recs_done = true;
     }
     if (c->pull_hop[l]) RP_WIDTH_DISPATCH(ld, PULL);
 #undef PUSH
 #undef PULL
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l + 1], c->stream);
     if (n > 0) {
-        RP_LAUNCH(c, k_scatter_records, std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, c->rec,
-                  (int)c->src_norm, c->side[0].deg, c->posmap, Mrows, Dm, ld, c->dS[l]);
+        if (!recs_done)
+            RP_LAUNCH(c, k_scatter_records, std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, recs, Dm, ld, c->dS[l]);
         const float* rows = c->pre[l] ? c->P[l] : c->H[l - 1];
 #define ROWS(NV, LPR) RP_LAUNCH(c, (k_regather_rows<NV, LPR>), std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, c->rec, c->side[1], c->side[0].deg, (int)c->src_norm, rows, ld, c->S[l], c->dS[l], c->Eb[l], senders, c->posmap, (int)(!c->pull_hop[l]), (int)c->self_term, c->A[l - 1], c->bitmap, (int)(c->n_local > 0))
         RP_WIDTH_DISPATCH(ld, ROWS);
@@ -928,7 +946,7 @@ void regather_layer(Ctx* c, int l) {
     const int ld = c->ws[l];
     const float* M = c->pre[l] ? c->P[l] : c->H[l - 1];   // P^l rows of the senders are already current
     const int grid = c->n_sm * 16, T = 256;
-    int2* items = reinterpret_cast<int2*>(c->coff);   // the degree prefix of the senders is no longer needed
+    int2* items = c->items;
     int* n_items = &c->ctl->work_counter[(l - 1) & 7];
     if (c->timing) cudaEventRecord(c->ev_rg[2 * l], c->stream);
 #define REGATHER(NV, LPR)                                                                                          \
