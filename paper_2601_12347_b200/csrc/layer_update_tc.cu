@@ -1,7 +1,7 @@
 // Tensor-core form of the affected-row layer update for sm_100a: tcgen05.mma (kind::tf32) with
 // the accumulator tile in tensor memory.
 //
-// One persistent CTA per SM takes tiles of R affected rows x one group of at most 128 output columns.  The product is
+// One persistent CTA per SM takes tiles of 128 affected rows x one group of at most 128 output columns.  The product is
 // formed transposed, weights times rows: the 128 lanes of the accumulator are output columns and its R columns are
 // affected rows, so that a warp reading it back holds 32 consecutive columns of one row per register -- whole lines
 // of the row's embedding, cached projection and delta, with no turn through shared memory.
@@ -10,9 +10,13 @@
 // memory, in the K-major 128-byte-swizzle layout the tensor core reads.  The tensor core takes the upper 19 bits of an
 // fp32 entry x (its tf32 part, hi); the loaders read the landed pieces back and store lo = x - hi, exact in fp32, as a
 // second operand.  The transposed weights lie in global memory already split, swizzled and cut into chunks, so that a
-// chunk is one bulk copy.  One thread issues hi * hi + lo * hi + hi * lo per 8-float K step, which reproduces the fp32
-// product to about 2^-21 relative (the product of the two low parts is left out).  With tc_mode = TC_TF32 only hi * hi
-// is issued (plain TF32, 2^-10).  Row factors (sink normalisation, GIN's self factor) are applied to the finished sums.
+// chunk is one bulk copy.  One thread issues, per 8-float K step, the weights' hi times [hi | lo] of the rows (256 columns)
+// and the weights' lo times the rows' hi: all but the product of the two low parts (2^-22 relative).  The small products
+// gather in accumulator columns of their own and meet the large ones in the epilogue: the tensor core rounds every
+// addition towards zero, and of a sum of 96 terms (K = 256) only 32 are then added at full size.  Error against fp64,
+// 2-norm: 3.6e-7 at K = 100, 7e-7 at K = 256, 1.5e-6 at K = 602 (one accumulator for all of it: 1.2e-6, 1.8e-6, 5e-6; fp32
+// sums on SIMT: 2.9e-7 at K = 256).  With tc_mode = TC_TF32 only hi * hi is issued (plain TF32, 2^-10).  Row factors (sink
+// normalisation, GIN's self factor) are applied to the finished sums.
 // Accumulators are double-buffered in tensor memory: the epilogue warps finish a tile (bias / cached terms /
 // activation / delta / commit) while the next tile's main loop is already running.
 //
@@ -20,10 +24,10 @@
 // about a microsecond per step whatever the bandwidth, so they overlap and each is kept free of chains: sixteen loader
 // warps with three chunks in flight, one warp that does nothing but issue (its operands in uniform registers), one that
 // fetches weights, eight epilogue warps whose loads travel ahead and whose stores are predicated.  The weights of a group
-// stay in shared memory for the life of the CTA while they fit (K <= 128: 128 KB, tiles of 128 rows); beyond that they
-// stream from L2 with every chunk, on tiles of 192 rows.  Groups of one row tile run on neighbouring CTAs at the same
-// time and find each other's rows in L2; two narrow products over the same rows (the neighbour and the self projection
-// of a layer's senders) share one group, side by side.
+// stay in shared memory for the life of the CTA while they fit (K <= 128: 128 KB); beyond that they stream from L2 with
+// every chunk.  Groups of one row tile run on neighbouring CTAs at the same time and find each other's rows in L2; two
+// narrow products over the same rows (the neighbour and the self projection of a layer's senders) share one group, side
+// by side.
 // Measured on 600 K rows (self and aggregate product of a layer, K = 100, 256 columns each: 1.18 -> 0.67 ms; neighbour
 // and self projection, K = 256, 48 columns each: 0.99 ms on SIMT -> 0.32; GIN's two products of 256 x 256: 2.02 -> 0.97 ms).
 //
@@ -40,23 +44,19 @@ namespace rp {
 
 constexpr int TC_COLS = 128;     // output columns per group (= TMEM lanes)
 constexpr int TC_KC = 32;        // floats per K chunk: one 128-byte swizzle row
-// Loader threads: sixteen warps on tiles of 192 rows, eight on tiles of 128 (whose epilogue, with a cached projection to
-// read for every row, needs the registers more).
+constexpr int TC_TILE = 128;     // affected rows per tile
+// Loader threads: sixteen warps where the weights stream, eight where they stay (whose epilogue, with a cached projection
+// to read for every row, needs the registers more).
 __host__ __device__ constexpr int tc_loaders(bool resident) { return resident ? 256 : 512; }
-__host__ __device__ constexpr int tc_tile(bool resident) { return resident ? 128 : 192; }
 constexpr int TC_EPI_WARPS = 8;  // two per tensor-memory lane quarter, half of the tile's rows each
 __host__ __device__ constexpr int tc_threads(bool resident) { return tc_loaders(resident) + 32 * TC_EPI_WARPS + 64; }   // and the warps that issue and that fetch the weights
 constexpr int TC_W_HALF = TC_COLS * 128;         // one half (hi or lo) of a chunk of weights
 constexpr int TC_W_BYTES = 2 * TC_W_HALF;
 constexpr int TC_RESIDENT_CHUNKS = 4;            // weights of up to this many chunks stay in shared memory
-constexpr int TC_W_STAGES = 2;                   // stages of weights that stream
-// Stages of rows as they come (the high operand) and of their remainders (the low one); blocks of 16 rows an epilogue
-// warp reads ahead.  What fits: 227 KB hold 64 or 128 KB of weights and
-//   weights stay:    3 x 16 KB + 2 x 16 KB of rows, 16 KB read ahead (alpha h + scale S: 2 x 16 KB twice)
-//   weights stream:  3 x 24 KB + 2 x 24 KB of rows, 32 KB read ahead (alpha h + scale S: 3 x 24 KB twice, 16 KB)
-__host__ __device__ constexpr int tc_hi(bool resident, bool sum) { return resident && sum ? 2 : 3; }
-__host__ __device__ constexpr int tc_lo(bool resident, bool sum) { return sum ? tc_hi(resident, sum) : 2; }
-__host__ __device__ constexpr int tc_ahead(bool resident, bool sum) { return resident || sum ? 1 : 2; }
+// What fits into 227 KB: stages of rows ([hi | lo], 32 KB each), weights, and the epilogue's rows in flight (32 KB).
+constexpr int TC_W_STAGES = 3;                   // stages of weights that stream
+__host__ __device__ constexpr int tc_stages(bool resident) { return resident ? 2 : 3; }
+constexpr int TC_AHEAD = 2;                      // blocks of 16 rows an epilogue warp reads ahead
 constexpr uint32_t TC_SPIN_LIMIT = 1u << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -181,16 +181,16 @@ __device__ __forceinline__ T tc_pick(const T (&own)[N], int k) {
 //   acc_empty[b]   8 arrivals (one per epilogue warp, accumulators read)             -> MMA warp may overwrite
 // The step counter runs on across tiles, so the loads of the next tile start while the last MMAs of this one are
 // still in flight.
-// RESIDENT: the weights stay in shared memory, tiles of 128 rows; else they stream, tiles of 256 rows.
+// RESIDENT: the weights stay in shared memory; else they stream.
 // SUM: the row operand is alpha h + scale S (GIN), two rows per entry.
 template <bool RESIDENT, bool SUM>
 __global__ void __launch_bounds__(tc_threads(RESIDENT), 1)
 k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     constexpr int TC_LOADERS = tc_loaders(RESIDENT);
-    constexpr int TILE = tc_tile(RESIDENT), RSTEP = TC_LOADERS / 8, ITS = TILE / RSTEP;
-    constexpr int X_HALF = TILE * 128, NH = tc_hi(RESIDENT, SUM), NL = tc_lo(RESIDENT, SUM);
+    constexpr int TILE = TC_TILE, RSTEP = TC_LOADERS / 8, ITS = TILE / RSTEP;
+    constexpr int X_HALF = TILE * 128, X_BYTES = 2 * X_HALF, NH = tc_stages(RESIDENT);
     constexpr int W_SLOTS = RESIDENT ? TC_RESIDENT_CHUNKS : TC_W_STAGES;
-    constexpr int BUF = TILE <= 128 ? 128 : 256;                 // tensor-memory columns from one accumulator to the other
+    constexpr int BUF = 2 * TILE;                                // tensor-memory columns of an accumulator: [hi hi | corrections]
     pdl_enter();
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_x[NH], full_w[W_SLOTS], empty[NH], acc_full[2], acc_empty[2], drained;
@@ -218,9 +218,8 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     const int nchunks = p.tc_chunks, K = p.K;
     const float* weights = p.tc_w + (size_t)grp * nchunks * (TC_W_BYTES / 4);
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint8_t* x_ring = smem;                                      // stages of rows
-    uint8_t* l_ring = smem + (size_t)NH * X_HALF;                // stages of their remainders
-    uint8_t* w_ring = l_ring + (size_t)NL * X_HALF;              // stages of [hi | lo] weights, or all chunks of them
+    uint8_t* x_ring = smem;                                      // stages of rows: [as they come | their remainders]
+    uint8_t* w_ring = smem + (size_t)NH * X_BYTES;               // stages of [hi | lo] weights, or all chunks of them
     constexpr uint32_t tmem_cols = 2 * BUF;
 
     if (tid == 0) {
@@ -257,7 +256,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         const float* const base = (from_s ? p.S : p.Hprev) + c * 4;
         const int ldr = from_s ? p.ld_s : p.ld_h, ldh = p.ld_h;
         const int32_t* const list = p.a_mode == A_DENSE ? nullptr : p.list;
-        const uint32_t x_mine = smem_u32(x_ring) + tc_swz(rb, c), l_mine = smem_u32(l_ring) + tc_swz(rb, c);
+        const uint32_t x_mine = smem_u32(x_ring) + tc_swz(rb, c);
         int rows_next[ITS];           // rows of the tile after the one being requested
         auto ids = [&](int lt) {
 #pragma unroll
@@ -299,10 +298,10 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
 #pragma unroll
             for (int it = 0; it < ITS; ++it) {
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                             ::"r"(x_mine + (uint32_t)(s_l * X_HALF + it * (RSTEP * 128))), "l"(ptr[it] + off), "r"(bytes) : "memory");
+                             ::"r"(x_mine + (uint32_t)(s_l * X_BYTES + it * (RSTEP * 128))), "l"(ptr[it] + off), "r"(bytes) : "memory");
                 if constexpr (SUM)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                                 ::"r"(l_mine + (uint32_t)(s_l * X_HALF + it * (RSTEP * 128))), "l"(ptr_h[it] + off), "r"(bytes) : "memory");
+                                 ::"r"(x_mine + (uint32_t)(s_l * X_BYTES + X_HALF + it * (RSTEP * 128))), "l"(ptr_h[it] + off), "r"(bytes) : "memory");
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
             if (++s_l == NH) s_l = 0;
@@ -328,12 +327,12 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         const float alpha = p.alpha;
 #pragma unroll
         for (int d = 0; d < NH - 1; ++d) { keep(d); request(d < total_steps); }
-        int s = 0, sl = 0, s_prev = NH - 1;
+        int s = 0, s_prev = NH - 1;
         uint32_t ph_prev = 1;         // phase of the stage that the step before used (a fresh barrier counts as completed)
         bool ok = true;
         for (int g = 0; g < total_steps && ok; ++g) {
             asm volatile("cp.async.wait_group %0;" ::"n"(NH - 2) : "memory");
-            const uint32_t hi = x_mine + (uint32_t)(s * X_HALF), lo = l_mine + (uint32_t)(sl * X_HALF);
+            const uint32_t hi = x_mine + (uint32_t)(s * X_BYTES), lo = hi + X_HALF;
             if (x3 || SUM) {
                 float4 x[ITS];
 #pragma unroll
@@ -356,8 +355,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&full_x[s]);
-            // the stage that the step before used takes the chunk NH - 1 steps ahead (and, with two stages of
-            // remainders, the next step's remainders go where those of the step before were)
+            // the stage that the step before used takes the chunk NH - 1 steps ahead
             ok = mbar_wait_bounded(&empty[s_prev], ph_prev, spin_limit);
             keep(s_prev);
             request(g + NH - 1 < total_steps);
@@ -365,7 +363,6 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             if (g == 0) ph_prev = 0;
             s_prev = s;
             if (++s == NH) s = 0;
-            if (++sl == NL) sl = 0;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         if (!ok) s_fail = 1;
@@ -411,7 +408,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         // Rows are worked on in blocks.  What is read ahead of a block was requested DEPTH blocks before, across the end of
         // the tile too, as asynchronous copies into shared memory, 16 bytes per lane and four rows per instruction:
         // loads into registers were waited for at the next barrier wait, whatever their distance to the first use.
-        constexpr int DEPTH = tc_ahead(RESIDENT, SUM), BLOCKS = HALF / BLK;
+        constexpr int DEPTH = TC_AHEAD, BLOCKS = HALF / BLK;
         float* const zbuf = reinterpret_cast<float*>(w_ring + (size_t)W_SLOTS * TC_W_BYTES) + (warp - TC_LOADERS / 32) * (DEPTH * BLK * 32);
         // the piece of the row that this lane copies: four columns, of the problem they belong to
         const float* piece;
@@ -455,6 +452,15 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 uint32_t x[BLK];
                 tc_load16(x, t_mine + (uint32_t)(blk * BLK));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                float h[BLK];
+#pragma unroll
+                for (int r = 0; r < BLK; ++r) h[r] = __uint_as_float(x[r]);
+                if (x3) {
+                    tc_load16(x, t_mine + (uint32_t)(TILE + blk * BLK));
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int r = 0; r < BLK; ++r) h[r] += __uint_as_float(x[r]);
+                }
                 if (plus_s) {   // (transformed aggregates with a self term of their own: GIN layers that narrow)
 #pragma unroll 1
                     for (int r = 0; r < BLK; ++r) {
@@ -462,7 +468,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                         const float sc = __shfl_sync(FULL, s_src, at + r);
                         float acc = 0.f;
 #pragma unroll
-                        for (int j = 0; j < BLK; ++j) acc = j == r ? __uint_as_float(x[j]) : acc;
+                        for (int j = 0; j < BLK; ++j) acc = j == r ? h[j] : acc;
                         if (i0 + r >= n || !col_ok) continue;
                         const size_t row = (size_t)v * ldo, sa = (size_t)v * p.ld_add + lc;
                         float t = p.addend_rw ? p.addend_rw[sa] : p.addend[sa];
@@ -471,10 +477,10 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                             p.addend_rw[sa] = t;
                             p.addend_delta[sa] = 0.f;
                         }
-                        float h = (p.a_mode == A_AGG ? sc : alpha) * acc + bias + sc * t;
-                        if (any_z) h += p.addend2[row + lc];
-                        if (relu) h = fmaxf(h, 0.f);
-                        if (temp) { hout[(size_t)(i0 + r) * ldo] = h; continue; }
+                        float y = (p.a_mode == A_AGG ? sc : alpha) * acc + bias + sc * t;
+                        if (any_z) y += p.addend2[row + lc];
+                        if (relu) y = fmaxf(y, 0.f);
+                        if (temp) { hout[(size_t)(i0 + r) * ldo] = y; continue; }
                         if (dout) {
                             const float o = hout[row];
                             float cn = 1.f, co = 1.f;
@@ -483,15 +489,12 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                                 cn = coef_deg(p.deg_out[v]);
                                 co = dold >= 0 ? coef_deg(dold) : cn;
                             }
-                            dout[(size_t)(i0 + r) * ldo] = keep_old ? o : cn * h - co * o;
+                            dout[(size_t)(i0 + r) * ldo] = keep_old ? o : cn * y - co * o;
                         }
-                        hout[row] = h;
+                        hout[row] = y;
                     }
                     return;
                 }
-                float h[BLK];
-#pragma unroll
-                for (int r = 0; r < BLK; ++r) h[r] = __uint_as_float(x[r]);
                 if (scaled) {
 #pragma unroll
                     for (int r = 0; r < BLK; ++r) h[r] = __shfl_sync(FULL, s_src, at + r) * h[r] + bias;
@@ -573,10 +576,10 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     } else if (warp == TC_LOADERS / 32 + TC_EPI_WARPS) {
         // ---------------- MMA issue ----------------
         const bool lead = tc_elect();
-        constexpr uint32_t idesc = tc_idesc(TILE);
-        const uint64_t dx0 = tc_smem_desc(smem_u32(x_ring)), dl0 = tc_smem_desc(smem_u32(l_ring)), dw0 = tc_smem_desc(smem_u32(w_ring));
+        constexpr uint32_t idesc = tc_idesc(TILE), idesc_wide = tc_idesc(2 * TILE);
+        const uint64_t dx0 = tc_smem_desc(smem_u32(x_ring)), dw0 = tc_smem_desc(smem_u32(w_ring));
         const bool withhold = p.tc_withhold != 0;
-        int s = 0, sl = 0, sw = 0;
+        int s = 0, sw = 0;
         uint32_t ph = 0, phw = 0;              // ring slots and phases of this step
         bool ok = true;
         for (int lt = 0; lt < my_tiles; ++lt) {
@@ -598,18 +601,15 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 // barrier: in the loaders the fence would wait for their row gathers in flight as well.
                 fence_async_smem();
                 tc_fence_after();
-                const uint64_t xh = dx0 + (uint64_t)((uint32_t)s * (X_HALF >> 4)), xl = dl0 + (uint64_t)((uint32_t)sl * (X_HALF >> 4));
+                const uint64_t xh = dx0 + (uint64_t)((uint32_t)s * (X_BYTES >> 4));
                 const uint64_t wh = dw0 + (uint64_t)((uint32_t)sw * (TC_W_BYTES >> 4)), wl = wh + (TC_W_HALF >> 4);
                 const bool last = kc == nchunks - 1;
                 if (lead) {
 #pragma unroll
                     for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
                         if (8 * j < left) {
-                            tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, idesc, (kc | j) != 0);
-                            if (x3) {
-                                tc_mma_tf32(d_addr, wl + 2 * j, xh + 2 * j, idesc, 1u);
-                                tc_mma_tf32(d_addr, wh + 2 * j, xl + 2 * j, idesc, 1u);
-                            }
+                            tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, x3 ? idesc_wide : idesc, (kc | j) != 0);
+                            if (x3) tc_mma_tf32(d_addr + TILE, wl + 2 * j, xh + 2 * j, idesc, 1u);
                         }
                     }
                     tc_commit(&empty[s]);
@@ -619,7 +619,6 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 }
                 __syncwarp();
                 if (++s == NH) { s = 0; ph ^= 1; }
-                if (++sl == NL) sl = 0;
                 if (!RESIDENT && ++sw == TC_W_STAGES) { sw = 0; phw ^= 1; }
             }
             if (!ok) break;
@@ -666,15 +665,15 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     }
 }
 
-static size_t tc_smem_bytes(bool resident, bool sum) {
-    return (size_t)(tc_hi(resident, sum) + tc_lo(resident, sum)) * tc_tile(resident) * 128 +
-           (size_t)(resident ? TC_RESIDENT_CHUNKS : TC_W_STAGES) * TC_W_BYTES + (size_t)TC_EPI_WARPS * tc_ahead(resident, sum) * 16 * 128 + 1024;
+static size_t tc_smem_bytes(bool resident) {
+    return (size_t)tc_stages(resident) * TC_TILE * 256 + (size_t)(resident ? TC_RESIDENT_CHUNKS : TC_W_STAGES) * TC_W_BYTES +
+           (size_t)TC_EPI_WARPS * TC_AHEAD * 16 * 128 + 1024;
 }
 
 void launch_update_tc(Ctx* c, const UpdPair& pair) {
     const bool resident = pair.p[0].tc_chunks <= TC_RESIDENT_CHUNKS, sum = pair.p[0].a_mode == A_SUM;
     // one persistent CTA per SM: operands and weights fill its shared memory
-#define TC_GO(RES, SUM) RP_LAUNCH(c, (k_update_rows_tc<RES, SUM>), c->n_sm, tc_threads(RES), tc_smem_bytes(RES, SUM), c->ctl, pair)
+#define TC_GO(RES, SUM) RP_LAUNCH(c, (k_update_rows_tc<RES, SUM>), c->n_sm, tc_threads(RES), tc_smem_bytes(RES), c->ctl, pair)
     if (resident && sum) TC_GO(true, true);
     else if (resident) TC_GO(true, false);
     else if (sum) TC_GO(false, true);
@@ -683,7 +682,7 @@ void launch_update_tc(Ctx* c, const UpdPair& pair) {
 }
 
 void tc_prepare() {
-#define TC_SET(RES, SUM) cudaFuncSetAttribute(k_update_rows_tc<RES, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(RES, SUM))
+#define TC_SET(RES, SUM) cudaFuncSetAttribute(k_update_rows_tc<RES, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(RES))
     TC_SET(true, true);
     TC_SET(true, false);
     TC_SET(false, true);
