@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256)
 k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff, Side out,
            const int32_t* __restrict__ posmap, const float* __restrict__ Hprev, const float* __restrict__ Old, int ld_h,
            const float* __restrict__ s_old, const float* __restrict__ att_s, const float* __restrict__ att_t,
-           float slope, int d, int ld, float* dS, uint32_t* bitmap, const Rec* __restrict__ rec) {
+           float slope, int d, int ld, float* dS, uint32_t* bitmap, const Rec* __restrict__ rec, int rows) {
     pdl_enter();
     if (ctl->abort) return;
     {   // the members of A_l that the walk does not find: sinks of edge changes, and A_{l-1} (the senders)
@@ -113,7 +113,9 @@ k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* 
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
     const int qden = d >> 2, cden = d & 3;   // the denominator's place in the row
-    TicketWalk walk(&ctl->walk_ticket[l], E, ATT_CHUNK, 4 * ATT_CHUNK);
+    __shared__ int2 s_queue[8][WALK_QUEUE];
+    int2* queue = s_queue[threadIdx.x >> 5];
+    TicketWalk walk(&ctl->walk_ticket[l], E, ATT_CHUNK, 4 * ATT_CHUNK, rows, ld);
     for (; walk.has(); walk.advance()) {
         const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
         walk.take();
@@ -134,12 +136,10 @@ k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* 
             }
             const float sn = att_s[u], so = s_old[i];
             const int cnt_total = (int)(seg_end - e);
-            for (int j0 = 0; j0 < cnt_total; j0 += 32) {
-                const bool have = j0 + lane < cnt_total;
-                const int mine = have ? out.col[base + j0 + lane] : 0;
+            walk_entries<false>(out.col, nullptr, base, cnt_total, walk, queue, [&](int mine, float, int cnt) {
+                const bool have = lane < cnt;
                 const float mine_t = have ? att_t[mine] : 0.f;
                 const int mine_skip = have ? (posmap[mine] >= 0) : 1;
-                const int cnt = min(32, cnt_total - j0);
                 if (have) {   // every sink joins the hop's frontier: the same walk as the frontier's own
                     const uint32_t m = 1u << (mine & 31);
                     if (!(bitmap[mine >> 5] & m)) atomicOr(&bitmap[mine >> 5], m);
@@ -164,7 +164,7 @@ k_att_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* 
                         }
                     }
                 }
-            }
+            });
             e = seg_end;
             ++i;
         }
@@ -441,7 +441,7 @@ static void launch_gather(Ctx* c, int l) {
 void att_update(Ctx* c, int l, bool full) {
     const LayerDev& ly = c->layer[l];
     float* old_rows = (full || l == c->L) ? nullptr : c->D[l & 1];   // the last hop sends nothing
-    RP_LAUNCH(c, k_att_update, c->n_sm * 8, 256, 0, c->ctl, full ? (const int32_t*)nullptr : c->A[l],
+    RP_LAUNCH(c, k_att_update, RP_RESIDENT(c, k_att_update, 256), 256, 0, c->ctl, full ? (const int32_t*)nullptr : c->A[l],
               full ? (const int*)nullptr : &c->ctl->nA[l], c->N, c->S[l], c->ws[l], ly.d_in, c->side[1].deg, ly.act,
               c->H[l], c->ld[l], old_rows, full ? (uint32_t*)nullptr : c->bitmap,
               full ? (const int32_t*)nullptr : sender_list(c, l - 1), full ? (const int*)nullptr : &c->ctl->nC[l - 1], c->posmap);
@@ -452,7 +452,7 @@ void att_full(Ctx* c, int l) {
     const LayerDev& ly = c->layer[l];
     RP_LAUNCH(c, k_att_scalars, c->n_sm * 8, 256, 0, c->ctl, (const int32_t*)nullptr, (const int*)nullptr, c->N,
               c->H[l - 1], c->ld[l - 1], ly.W1, c->att_s[l], c->att_t[l], (float*)nullptr);
-    RP_LAUNCH(c, k_att_fold, c->n_sm * 8, 256, 0, c->ctl, l, (const int32_t*)nullptr, (const int*)nullptr, c->N, 1,
+    RP_LAUNCH(c, k_att_fold, RP_RESIDENT(c, k_att_fold, 256), 256, 0, c->ctl, l, (const int32_t*)nullptr, (const int*)nullptr, c->N, 1,
               c->ws[l], c->S[l], c->dS[l], c->Eb[l], c->rebuild_tau2, c->side[1].deg, c->posmap, c->att_items, ly.d_in,
               ly.act, c->H[l], c->ld[l], (float*)nullptr, (uint32_t*)nullptr);
     launch_gather(c, l);
@@ -468,7 +468,7 @@ void att_hop(Ctx* c, int l, int n, bool small) {
     RP_LAUNCH(c, k_att_scalars, c->n_sm * 4, T, 0, c->ctl, senders, (const int*)&c->ctl->nC[l - 1], 0, c->H[l - 1],
               c->ld[l - 1], ly.W1, c->att_s[l], c->att_t[l], c->att_so);
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l], c->stream);
-#define PUSH(NV, LPR) RP_LAUNCH(c, (k_att_push<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, senders, c->coff, c->side[0], c->posmap, c->H[l - 1], Old, c->ld[l - 1], c->att_so, c->att_s[l], c->att_t[l], ly.eps, ly.d_in, ld, c->dS[l], c->bitmap, (const Rec*)c->rec)
+#define PUSH(NV, LPR) RP_LAUNCH(c, (k_att_push<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, senders, c->coff, c->side[0], c->posmap, c->H[l - 1], Old, c->ld[l - 1], c->att_so, c->att_s[l], c->att_t[l], ly.eps, ly.d_in, ld, c->dS[l], c->bitmap, (const Rec*)c->rec, c->N)
     RP_WIDTH_DISPATCH(ld, PUSH);
 #undef PUSH
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l + 1], c->stream);
@@ -476,7 +476,7 @@ void att_hop(Ctx* c, int l, int n, bool small) {
     // the list A_l: the message walk has marked it
     if (small) frontier_compact_small(c, l, false);   // (a handful of updates on a graph whose bitmap one block can sweep)
     else frontier_compact(c, l);
-    RP_LAUNCH(c, k_att_fold, c->n_sm * 8, T, 0, c->ctl, l, c->A[l], (const int*)&c->ctl->nA[l], 0, 0, ld, c->S[l],
+    RP_LAUNCH(c, k_att_fold, RP_RESIDENT(c, k_att_fold, 256), T, 0, c->ctl, l, c->A[l], (const int*)&c->ctl->nA[l], 0, 0, ld, c->S[l],
               c->dS[l], c->Eb[l], c->rebuild_tau2, c->side[1].deg, c->posmap, c->att_items, ly.d_in, ly.act, c->H[l],
               c->ld[l], l == c->L ? (float*)nullptr : c->D[l & 1], c->bitmap);   // (the bitmap is free between two hops' markings)
     launch_gather(c, l);

@@ -246,7 +246,7 @@ __device__ __forceinline__ void set_bit(uint32_t* bitmap, int v) {
 
 constexpr int WALK_CHUNK = 256;  // edges per warp work item
 
-__global__ void k_mark_frontier(Ctl* ctl, int l, int self_term, int walk, const int32_t* __restrict__ senders,
+__global__ void k_mark_frontier(Ctl* ctl, int l, int self_term, const int32_t* __restrict__ senders,
                                 const int64_t* __restrict__ coff, Side out, const Rec* __restrict__ rec,
                                 const int32_t* __restrict__ A_prev, uint32_t* bitmap) {
     pdl_enter();
@@ -257,13 +257,17 @@ __global__ void k_mark_frontier(Ctl* ctl, int l, int self_term, int walk, const 
     if (self_term)
         for (int i = gtid; i < ctl->nA[l - 1]; i += gsize) set_bit(bitmap, A_prev[i]);
     // out-neighbours of the senders of the previous hop (the push scatter marks them itself)
-    if (!walk || ctl->regather[l]) return;   // (a rebuilding hop marks bottom-up)
+    if (ctl->regather[l]) return;   // (a rebuilding hop marks bottom-up)
     const int nC = ctl->nC[l - 1];
     if (nC == 0) return;
     const int64_t E = coff[nC];
-    const int warp = gtid >> 5, nwarps = gsize >> 5, lane = lane_id();
-    for (int64_t e0 = (int64_t)warp * WALK_CHUNK; e0 < E; e0 += (int64_t)nwarps * WALK_CHUNK) {
-        int64_t e1 = min(e0 + WALK_CHUNK, E);
+    const int lane = lane_id();
+    // (by ticket: the fixed split's slowest warp took three times the mean; a hop that walks here does not push, so the
+    // counter is free)
+    TicketWalk deal(&ctl->walk_ticket[l], E, WALK_CHUNK / 4, WALK_CHUNK);
+    for (; deal.has(); deal.advance()) {
+        const int64_t e0 = deal.at, e1 = min(e0 + deal.chunk, E);
+        deal.take();
         int i = upper_row(coff, nC, e0);
         int64_t e = e0;
         while (e < e1) {
@@ -350,18 +354,16 @@ void frontier_seed_features(Ctx* c, int n) {
     bitmap_to_list(c, c->A[0], &c->ctl->nA[0], nullptr);
 }
 
-// Marks the members of A_l that do not come from walking the senders' out-lists (sinks of edge
-// changes, A_{l-1} for models with a self term) and, if `walk`, those that do.
-void frontier_mark(Ctx* c, int l, bool walk, int n) {
-    // without a walk of its own (the push scatter marks the sinks it reaches) the rest of the marking rides
-    // along with the last kernel of the hop's delta form; an empty batch has nothing to mark
+// Marks the members of A_l on hops that gather (`walk`): sinks of edge changes, A_{l-1} for models with a self term, and
+// what a walk of the senders' out-lists reaches (a push marks all of these itself); and, where a rebuild is possible,
+// bottom-up.
+void frontier_mark(Ctx* c, int l, bool walk) {
     if (walk)
-        RP_LAUNCH(c, k_mark_frontier, c->n_sm * 8, 256, 0, c->ctl, l, (int)c->self_term,
-                  (int)walk, sender_list(c, l - 1), c->coff, c->side[0], c->rec, c->A[l - 1], c->bitmap);
-    (void)n;
+        RP_LAUNCH(c, k_mark_frontier, RP_RESIDENT(c, k_mark_frontier, 256), 256, 0, c->ctl, l, (int)c->self_term,
+                  sender_list(c, l - 1), c->coff, c->side[0], c->rec, c->A[l - 1], c->bitmap);
     if (!c->rebuild_armed[l]) return;
     // the list A_l is not built yet: its buffer holds the queue of undecided long rows
-    RP_LAUNCH(c, k_mark_bottom_up, c->n_sm * 8, 256, 0, c->ctl, l, c->N, c->side[1], c->posmap, c->bitmap, c->A[l],
+    RP_LAUNCH(c, k_mark_bottom_up, RP_RESIDENT(c, k_mark_bottom_up, 256), 256, 0, c->ctl, l, c->N, c->side[1], c->posmap, c->bitmap, c->A[l],
               &c->ctl->n_long[l]);
     RP_LAUNCH(c, k_mark_bottom_up_long, c->n_sm * 4, 256, 0, c->ctl, l, c->side[1], c->posmap, c->bitmap, c->A[l],
               &c->ctl->n_long[l]);
@@ -423,12 +425,6 @@ k_frontier_small(Ctl* ctl, int l, uint32_t* bitmap, int n_words, int32_t* list, 
             coff[total] = deg_total;
         }
     }
-}
-
-// the members of A_l that no walk of out-lists finds: sinks of edge changes, A_{l-1} for models with a self term
-void frontier_mark_extras(Ctx* c, int l) {
-    RP_LAUNCH(c, k_mark_frontier, c->n_sm * 2, 256, 0, c->ctl, l, (int)c->self_term, 0, sender_list(c, l - 1), c->coff,
-              c->side[0], c->rec, c->A[l - 1], c->bitmap);
 }
 
 void frontier_compact_small(Ctx* c, int l, bool senders) {

@@ -506,7 +506,7 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
         // (decided per hop on the device for the rebuilding form).
         const bool pull = c->pull_hop[l] != 0;
         choose_direction(c, l);
-        frontier_mark(c, l, pull, nb);
+        frontier_mark(c, l, pull);
         if (pull) frontier_compact(c, l);
         STAMP();
         scatter_layer(c, l, nb);

@@ -66,6 +66,7 @@ struct Ctl {
     int rebuild_items[RP_MAXL + 1];   // (vertex, chunk) work items of the long rows among them
     int max_items[RP_MAXL + 1];       // max / min: (long row, chunk) work items of hop l's recomputation
     int walk_ticket[RP_MAXL + 1];     // walk of the senders' out-lists: next unassigned chunk (see OutWalk)
+    int ew_ticket[RP_MAXL + 1];       // elementwise update: next unassigned run of pieces
     int hub_ticket[RP_MAXL + 1];      // chunks of long in-lists: next unassigned work item
     int regather_ticket[RP_MAXL + 1]; // rebuilding form: next unassigned position of A_l
     int gather_ticket[RP_MAXL + 1];   // gathering form of the delta scatter: next unassigned position of A_l
@@ -289,6 +290,15 @@ inline int32_t* sender_list(const Ctx* c, int l) { return c->src_norm || rp_mono
 inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 inline int pad4(int x) { return (x + 3) & ~3; }
 
+// Blocks of a kernel that are resident together: the grid of a kernel whose blocks split rows of equal cost evenly.  (A
+// grid of eight blocks per SM of which registers admit six ran its last quarter alone, on a quarter of the threads.)
+template <typename K>
+inline int occupancy(K kernel, int block) {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, 0) == cudaSuccess && n > 0 ? n : 1;
+}
+#define RP_RESIDENT(ctx, kernel, block) ([&] { static const int per_sm_ = rp::occupancy(kernel, block); return (ctx)->n_sm * per_sm_; }())
+
 // Every kernel of the library goes through this: programmatic stream serialisation (see pdl_enter)
 // unless switched off for the context.
 #define RP_LAUNCH(ctx, kernel, grid, block, smem, ...)                                            \
@@ -335,8 +345,7 @@ cudaError_t graph_export(Ctx* c, int64_t* rowptr, int32_t* col, float* weight, i
 void scan_degrees(Ctx* c, const int32_t* list, const int* n_dev, int n_host, const int32_t* deg,
                   int64_t* out, unsigned long long* total_dev);
 void frontier_seed_features(Ctx* c, int n);             // A_0 from the batch's feature updates
-void frontier_mark(Ctx* c, int l, bool walk, int n);    // bitmap of A_l: (walk) edge-record sinks, A_{l-1} and Out(C_{l-1}); rebuilding hops: bottom-up
-void frontier_mark_extras(Ctx* c, int l);               // marks only what no walk finds (for hops whose message walk marks its sinks itself)
+void frontier_mark(Ctx* c, int l, bool walk);           // bitmap of A_l: (walk) edge-record sinks, A_{l-1} and Out(C_{l-1}); rebuilding hops: bottom-up
 void frontier_compact(Ctx* c, int l);                   // bitmap -> ascending list A_l
 void frontier_compact_senders(Ctx* c, int l);           // the same, and C_l = A_l with its degree prefix
 void frontier_compact_small(Ctx* c, int l, bool senders);   // likewise in one block (tiny batches, small graphs)

@@ -41,7 +41,7 @@ __device__ __forceinline__ void add4(float4& a, const float4& x, float c) {
 constexpr int SPMM_HUB_DEGREE = 256;
 constexpr int SPMM_HUB_CHUNK = 256;
 // acc += sum over in-list entries [j_begin, j_end) of row v of c_u * M_u; LPR lanes hold one row
-// (NV float4 slots each), a warp works on 32 / LPR neighbours per step, four steps in flight.
+// (NV float4 slots each), a warp works on 32 / LPR neighbours per step, several steps in flight.
 template <int NV, int LPR>
 __device__ __forceinline__ void spmm_accumulate(float4 (&acc)[NV], const Side& in, int v, int j_begin, int j_end,
                                                 const int32_t* __restrict__ deg_out, int src_norm,
@@ -55,7 +55,7 @@ __device__ __forceinline__ void spmm_accumulate(float4 (&acc)[NV], const Side& i
         // stored edge weights (weighted sum with per-edge weights): the entry's weight is its coefficient
         float mine_w = (in.w && j0 + lane < j_end) ? in.w[base + j0 + lane] : 1.0f;
         int cnt = min(32, j_end - j0);
-        constexpr int UNR = 4;
+        constexpr int UNR = NV == 1 ? 8 : 4;   // rows in flight per lane group (48 floats, rebuilt hop of 123 M entries: 8 is 0.3 ms faster than 4)
         for (int j = 0; j < cnt; j += UNR * EPI) {
             int u[UNR];
             float cu[UNR];
@@ -281,7 +281,7 @@ template <int NV, int LPR>
 __global__ void __launch_bounds__(256)
 k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff,
                Side out, const float* __restrict__ D, int ld, float* S, uint32_t* bitmap,
-               const RecMsgs recs) {
+               const RecMsgs recs, int rows) {
     pdl_enter();
     if (ctl->abort || ctl->pull[l] || ctl->regather[l]) return;
     d_scatter_records(ctl, recs, D, ld, S);
@@ -291,7 +291,9 @@ k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64
     const int lane = lane_id(), nq = ld >> 2;
     constexpr int EPI = 32 / LPR;
     const int sub = lane / LPR, ql = lane % LPR;
-    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE);
+    __shared__ int2 s_queue[8][WALK_QUEUE];
+    int2* queue = s_queue[threadIdx.x >> 5];
+    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE, rows, ld);
     for (; walk.has(); walk.advance()) {
         const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
         walk.take();
@@ -310,11 +312,8 @@ k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64
                 d[k] = q < nq ? __ldg(drow + q) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
             const int cnt_total = (int)(seg_end - e);
-            for (int j0 = 0; j0 < cnt_total; j0 += 32) {
-                int mine = j0 + lane < cnt_total ? out.col[base + j0 + lane] : 0;
-                // stored edge weights: the message along an edge is the sender's delta row times the edge's weight
-                float mine_w = (out.w && j0 + lane < cnt_total) ? out.w[base + j0 + lane] : 1.0f;
-                int cnt = min(32, cnt_total - j0);
+            walk_entries<true>(out.col, out.w, base, cnt_total, walk, queue, [&](int mine, float mine_w, int cnt) {
+                // (stored edge weights: the message along an edge is the sender's delta row times the edge's weight)
                 // every sink joins the hop's affected set (same walk as the frontier's): one lane per
                 // edge, 32 edges per instruction
                 if (lane < cnt) {
@@ -334,7 +333,7 @@ k_scatter_push(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64
                         }
                     }
                 }
-            }
+            });
             e = seg_end;
             ++i;
         }
@@ -350,7 +349,7 @@ template <int NQ, bool WEIGHTED>
 __global__ void __launch_bounds__(256)
 k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, const int64_t* __restrict__ coff,
                       Side out, const float* __restrict__ D, float* S, uint32_t* bitmap,
-                      const RecMsgs recs) {
+                      const RecMsgs recs, int rows) {
     pdl_enter();
     constexpr int LCM = NQ == 12 ? 96 : NQ == 10 ? 160 : NQ * 32;
     constexpr int NI = LCM / 32, G = LCM / NQ, LD = NQ * 4;
@@ -363,7 +362,9 @@ k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, cons
     int msg_of[NI], slot_of[NI];
 #pragma unroll
     for (int i = 0; i < NI; ++i) { msg_of[i] = (32 * i + lane) / NQ; slot_of[i] = (32 * i + lane) % NQ; }
-    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE);
+    __shared__ int2 s_queue[8][WALK_QUEUE];
+    int2* queue = s_queue[threadIdx.x >> 5];
+    TicketWalk walk(&ctl->walk_ticket[l], E, PUSH_CHUNK, PUSH_CHUNK_LARGE, rows, LD);
     for (; walk.has(); walk.advance()) {
         const int64_t e0 = walk.at, e1 = min(e0 + walk.chunk, E);
         walk.take();
@@ -379,11 +380,7 @@ k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, cons
 #pragma unroll
             for (int k = 0; k < NI; ++k) d[k] = __ldg(drow + slot_of[k]);
             const int cnt_total = (int)(seg_end - e);
-            for (int j0 = 0; j0 < cnt_total; j0 += 32) {
-                int mine = j0 + lane < cnt_total ? out.col[base + j0 + lane] : 0;
-                float mine_w = 1.0f;
-                if (WEIGHTED && j0 + lane < cnt_total) mine_w = out.w[base + j0 + lane];
-                int cnt = min(32, cnt_total - j0);
+            walk_entries<WEIGHTED>(out.col, out.w, base, cnt_total, walk, queue, [&](int mine, float mine_w, int cnt) {
                 if (lane < cnt) {
                     const uint32_t m = 1u << (mine & 31);
                     if (!(bitmap[mine >> 5] & m)) atomicOr(&bitmap[mine >> 5], m);
@@ -401,7 +398,7 @@ k_scatter_push_packed(Ctl* ctl, int l, const int32_t* __restrict__ senders, cons
                         if (idx < cnt) red_add_v4(S + (size_t)v * LD + 4 * slot_of[k], m4);
                     }
                 }
-            }
+            });
             e = seg_end;
             ++i;
         }
@@ -864,7 +861,7 @@ void fold_deltas(Ctx* c, int l) {
     const float* M = c->pre[l] ? c->P[l] : c->H[l - 1];
     int2* items = c->items;
     const int ld = c->ws[l];
-    RP_LAUNCH(c, k_fold_deltas, c->n_sm * 8, 256, 0, c->ctl, l, c->A[l], ld, c->S[l], c->dS[l], c->Eb[l],
+    RP_LAUNCH(c, k_fold_deltas, RP_RESIDENT(c, k_fold_deltas, 256), 256, 0, c->ctl, l, c->A[l], ld, c->S[l], c->dS[l], c->Eb[l],
               c->rebuild_tau2, c->side[1].deg, items);
     if (!c->Eb[l]) return;
 #define HUBS(NV, LPR)                                                                                              \
@@ -901,7 +898,7 @@ void scatter_layer(Ctx* c, int l, int n) {
         Mrows = c->P[l];
     }
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l], c->stream);
-#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap, recs)
+#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap, recs, c->N)
     int2* gather_items = c->items;
     const RecMsgs recs{c->rec, (int)c->src_norm, c->side[0].deg, c->posmap, Mrows};
     bool recs_done = false;
@@ -917,7 +914,7 @@ void scatter_layer(Ctx* c, int l, int n) {
         RP_LAUNCH(c, k_scatter_push_bulk, grid, T, (size_t)8 * 2 * ld * sizeof(float), c->ctl, l, senders, c->coff,
                   c->side[0], Dm, ld, c->dS[l], c->bitmap);
     } else if (!c->pull_hop[l] && c->scatter_mode != RIPPLE_SCATTER_REGATHER) {
-#define PACKED(NQ, WGT) RP_LAUNCH(c, (k_scatter_push_packed<NQ, WGT>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, c->dS[l], c->bitmap, recs)
+#define PACKED(NQ, WGT) RP_LAUNCH(c, (k_scatter_push_packed<NQ, WGT>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, c->dS[l], c->bitmap, recs, c->N)
         if (ld == 48 && c->weighted) PACKED(12, true);
         else if (ld == 48) PACKED(12, false);
         else if (ld == 40 && c->weighted) PACKED(10, true);
