@@ -38,6 +38,7 @@ struct UpdParams {
     const float* addend2;           // rows by id added as they are, same leading dimension (may be null)
     float* addend_rw;               // if set: addend with its pending per-batch sums folded in on the way
     float* addend_delta;            //   (addend_rw += addend_delta, addend_delta = 0); replaces addend
+    int* ticket;                    // elementwise form: next unassigned run of pieces
     const int* rebuilt;             // if set and not zero: the aggregate was gathered anew, nothing is pending (elementwise form)
     int dout_old;                   // Dout receives the row's previous value instead of a delta (monotonic aggregation)
     int src_norm;
@@ -101,14 +102,8 @@ __device__ __forceinline__ float4 upd_load_old(const UpdParams& p, int v, int co
     return *reinterpret_cast<const float4*>(p.Hout + (size_t)v * p.ld_o + col);
 }
 
-// bias, optional addend, activation, then either a compact temp row or commit + delta row;
-// `old` / `zpre` are the previously stored value and the addend2 value if the caller has
-// prefetched them (has_old / has_z)
-__device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, int col, float4 h, float sc,
-                                              bool has_old = false,
-                                              float4 old = make_float4(0.f, 0.f, 0.f, 0.f),
-                                              bool has_z = false,
-                                              float4 zpre = make_float4(0.f, 0.f, 0.f, 0.f)) {
+// bias, optional addend, activation, then either a compact temp row or commit + delta row
+__device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, int col, float4 h, float sc) {
     if (p.bias) {
         float4 b = __ldg(reinterpret_cast<const float4*>(p.bias + col));
         h.x += b.x; h.y += b.y; h.z += b.z; h.w += b.w;
@@ -128,7 +123,7 @@ __device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, 
         h.x += sc * s.x; h.y += sc * s.y; h.z += sc * s.z; h.w += sc * s.w;
     }
     if (p.addend2) {
-        float4 z = has_z ? zpre : *reinterpret_cast<const float4*>(p.addend2 + (size_t)v * p.ld_add + col);
+        float4 z = *reinterpret_cast<const float4*>(p.addend2 + (size_t)v * p.ld_add + col);
         h.x += z.x; h.y += z.y; h.z += z.z; h.w += z.w;
     }
     if (p.act == RIPPLE_ACT_RELU) {
@@ -140,7 +135,7 @@ __device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, 
     }
     float4* dst = reinterpret_cast<float4*>(p.Hout + (size_t)v * p.ld_o + col);
     if (p.Dout) {
-        float4 o = has_old ? old : *dst;
+        float4 o = *dst;
         float cn = 1.f, co = 1.f;
         if (p.src_norm) {
             int dold = p.deg_out_old[v];

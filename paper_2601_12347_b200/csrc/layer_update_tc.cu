@@ -13,9 +13,10 @@
 // chunk is one bulk copy.  One thread issues, per 8-float K step, the weights' hi times [hi | lo] of the rows (256 columns)
 // and the weights' lo times the rows' hi: all but the product of the two low parts (2^-22 relative).  The small products
 // gather in accumulator columns of their own and meet the large ones in the epilogue: the tensor core rounds every
-// addition towards zero, and of a sum of 96 terms (K = 256) only 32 are then added at full size.  Error against fp64,
-// 2-norm: 3.6e-7 at K = 100, 7e-7 at K = 256, 1.5e-6 at K = 602 (one accumulator for all of it: 1.2e-6, 1.8e-6, 5e-6; fp32
-// sums on SIMT: 2.9e-7 at K = 256).  With tc_mode = TC_TF32 only hi * hi is issued (plain TF32, 2^-10).  Row factors (sink
+// addition towards zero, and of a sum of 96 terms (K = 256) only 32 are then added at full size.  (More than 128 output
+// columns: only the product with the rows' lo has columns of its own, the one with the weights' lo joins the large ones.)
+// Error against fp64, 2-norm, one group: 3.6e-7 at K = 100, 7e-7 at K = 256, 1.5e-6 at K = 602 (one accumulator for all of
+// it: 1.2e-6, 1.8e-6, 5e-6; fp32 sums on SIMT: 2.9e-7 at K = 256).  With tc_mode = TC_TF32 only hi * hi is issued (plain TF32, 2^-10).  Row factors (sink
 // normalisation, GIN's self factor) are applied to the finished sums.
 // Accumulators are double-buffered in tensor memory: the epilogue warps finish a tile (bias / cached terms /
 // activation / delta / commit) while the next tile's main loop is already running.
@@ -588,7 +589,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             if (ub > 0) ok = __all_sync(FULL, mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit));
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF);
+            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF), d_corr = d_addr + (G == 1 ? TILE : 0);
             int left = K;
             for (int kc = 0; kc < nchunks; ++kc, left -= TC_KC) {
                 if (RESIDENT) sw = kc;
@@ -609,7 +610,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                     for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
                         if (8 * j < left) {
                             tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, x3 ? idesc_wide : idesc, (kc | j) != 0);
-                            if (x3) tc_mma_tf32(d_addr + TILE, wl + 2 * j, xh + 2 * j, idesc, 1u);
+                            if (x3) tc_mma_tf32(d_corr, wl + 2 * j, xh + 2 * j, idesc, 1u);
                         }
                     }
                     tc_commit(&empty[s]);
