@@ -1,0 +1,125 @@
+"""The edges of the kernels' tiles and of the dispatch between their forms, against the oracle: graph, affected sets and
+counters exact, embeddings within 1e-4 (1 + |ref|) and cached aggregates within the same bound scaled by sqrt(in-degree)
+(GIN stacks: plus GIN_ROW_SLACK of the row's largest entry), as in test_gpu_parity."""
+import numpy as np
+import pytest
+
+from paper_2601_12347_b200 import inputs as I
+from tolerances import GIN_ROW_SLACK
+
+import test_gpu_parity as G
+
+pytestmark = pytest.mark.gpu
+
+env = G.env
+
+
+def feature_batch(n, ids, dim, seed):
+    ups = G.ups_array([(I.OP_SET_FEATURE, int(u), i) for i, u in enumerate(ids)])
+    return ups, I.features(len(ids), dim, seed)
+
+
+def apply_and_check(rp, orc, ups, rows, L, slack=0.0):
+    rp.apply_batch(ups, rows)
+    assert orc.apply_incremental(ups, rows) == 0
+    G.check_graph(rp, orc)
+    G.check_frontiers(rp, orc, L)
+    G.check_values(rp, orc.full(), L, [None] + [orc.full_S(l) for l in range(1, L + 1)], row_slack=slack)
+
+
+# Tensor-core form of the layer update: K chunks of 32 (31, 32, 33, and four / five of them: the weights stay in shared
+# memory up to 128), column groups of 128 (5 ... 257 columns, two narrow products side by side), row tiles of 128 and
+# the 512 rows from which the form is taken (n - 1, n and n + 1 of both), normalised sources, GIN's summed operand.
+TC_MODELS = {
+    "sage_31_5_47": lambda: I.sage_model([31, 5, 47], I.AGG_MEAN),
+    "sage_33_129_256": lambda: I.sage_model([33, 129, 256], I.AGG_SUM),
+    "sage_602_41_257": lambda: I.sage_model([602, 41, 257], I.AGG_MEAN),
+    "sage_300_128_48": lambda: I.sage_model([300, 128, 48], I.AGG_MEAN),
+    "gcn_32_48_128": lambda: I.graphconv_model([32, 48, 128], I.AGG_WSUM_GCN),
+    "gcn_129_100_130": lambda: I.graphconv_model([129, 100, 130], I.AGG_WSUM_GCN),
+    "gin_33_129": lambda: I.gin_model(33, 129, 2, eps=0.25),
+    "gin_128_128": lambda: I.gin_model(128, 128, 2, eps=0.25),
+    "gin_100_256": lambda: I.gin_model(100, 256, 2, eps=0.25),
+}
+
+
+@pytest.mark.parametrize("name", list(TC_MODELS.keys()))
+def test_row_updates_at_the_edges_of_their_tiles(env, name):
+    ripple, Oracle = env
+    model = TC_MODELS[name]()
+    L = len(model.layers)
+    slack = GIN_ROW_SLACK if name.startswith("gin") else 0.0
+    for n in (511, 512, 513, 641):
+        src, dst = I.er_graph(n, 4 * n, 3)
+        X = I.features(n, model.dims[0], 3)
+        W = I.make_weights(model, 3, zero_bias=False)
+        rp = ripple.Ripple(n, src, dst, X, model, W, max_batch=1024)
+        orc = Oracle(n, src, dst, X, model, W)
+        G.check_values(rp, orc.full(), L, row_slack=slack)
+        for b in range(2):      # every row changes; then an ordinary batch on the launch geometry of the large one
+            apply_and_check(rp, orc, *feature_batch(n, range(n), model.dims[0], 70 + b), L, slack)
+        apply_and_check(rp, orc, *feature_batch(n, range(0, n, n // 7), model.dims[0], 80), L, slack)
+        rp.recompute_full()
+        G.check_values(rp, orc.full(), L, row_slack=slack)
+        rp.close()
+
+
+# A walk that adds into rows of half a gigabyte is made twice, over the lower and the upper half of the ids (330 K rows of
+# 256 floats and three messages per row are past the line); the pulled hop marks its sinks by ticket.
+@pytest.mark.parametrize("kind", ["sage-push", "sage-pull", "weighted-push", "attention"])
+def test_walks_over_rows_that_outgrow_the_cache(env, kind):
+    ripple, Oracle = env
+    n, hubs, per_hub, d = 330_001, 64, 16_001, 256
+    rng = np.random.default_rng(5)
+    src = np.repeat(np.arange(hubs, dtype=np.int32) * 5003, per_hub)
+    dst = np.concatenate([rng.choice(n, per_hub, replace=False) for _ in range(hubs)]).astype(np.int32)
+    keep = src != dst
+    src, dst = src[keep], dst[keep]
+    kw = {"edge_weights": I.edge_weights(src.size, 5)} if kind == "weighted-push" else {}
+    model = {"sage": I.sage_model([d, d], I.AGG_SUM), "weighted": I.graphconv_model([d, d], I.AGG_WSUM_EDGE),
+             "attention": I.gat_model(d, 1, d_att=8, slope=0.2)}[kind.split("-")[0]]
+    X = I.features(n, d, 5)
+    W = I.make_weights(model, 5)
+    mode = ripple.SCATTER_PULL if kind == "sage-pull" else ripple.SCATTER_PUSH
+    rp = ripple.Ripple(n, src, dst, X, model, W, scatter_mode=ripple.SCATTER_AUTO if kind == "attention" else mode, **kw)
+    orc = Oracle(n, src, dst, X, model, W, **kw)
+    ups, rows = feature_batch(n, np.arange(hubs) * 5003, d, 6)
+    rp.apply_batch(ups, rows)
+    assert orc.apply_incremental(ups, rows) == 0
+    G.check_frontiers(rp, orc, 1)
+    assert rp.stats()["active_edges"][1] >= 2 * n
+    G.check_values(rp, orc.full(), 1)
+    rp.close()
+
+
+# How a batch reaches the device: one block up to 4 updates, up to 512 updates and 32 KB staged by one block, pinned copies
+# up to 64 KB read where they lie, larger ones through the staging area or by separate copies.
+@pytest.mark.parametrize("mem", ["host", "pinned", "device"])
+@pytest.mark.parametrize("d", [8, 602])
+def test_batches_at_the_edges_of_the_staging_forms(env, mem, d):
+    import torch
+    ripple, Oracle = env
+    model = I.sage_model([d, 24, 10], I.AGG_MEAN)
+    n = 1500
+    src, dst = I.er_graph(n, 6000, 11)
+    X = I.features(n, d, 11)
+    W = I.make_weights(model, 11, zero_bias=False)
+    rp = ripple.Ripple(n, src, dst, X, model, W)
+    orc = Oracle(n, src, dst, X, model, W)
+    stream = I.UpdateStream(n, src, dst, d, 11)
+    for b, bs in enumerate([1, 4, 5, 13, 14, 26, 28, 511, 512, 513, 700, 512]):
+        if b % 2:
+            ups, rows = feature_batch(n, (np.arange(bs) * 7 + b) % n, d, 300 + b)
+        else:
+            ups, rows = stream.next_batch(bs)
+        a, r = ups, rows
+        if mem != "host":
+            a = torch.from_numpy(np.stack([ups["op"], ups["u"], ups["v"]], axis=1).astype(np.int32))
+            r = torch.from_numpy(rows)
+            a, r = (a.cuda(), r.cuda()) if mem == "device" else (a.pin_memory(), r.pin_memory())
+        rp.apply_batch(a, r)
+        assert orc.apply_incremental(ups, rows) == 0
+        G.check_graph(rp, orc)
+        G.check_frontiers(rp, orc, 2)
+        G.check_values(rp, orc.full(), 2)
+    rp.close()
