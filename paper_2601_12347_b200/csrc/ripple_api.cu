@@ -101,6 +101,19 @@ static ripple_status sync_and_fetch_ctl(Ctx* c) {
     return RIPPLE_OK;
 }
 
+// the control block of work that can only fail by a bounded wait that gave up, as a status
+static ripple_status finished(Ctx* c) {
+    if (!c->ctl_host->err) return RIPPLE_OK;
+    set_err(c, "a bounded device-side wait gave up; the embeddings are no longer consistent: destroy the context");
+    return (ripple_status)c->ctl_host->err;
+}
+
+// diagnostic: a wait that nothing ends, to exercise the time-out path without faulting the device
+static int debug_tc_withhold() {
+    const char* e = getenv("RIPPLE_DEBUG_TC_WITHHOLD");
+    return e && e[0] == '1';
+}
+
 // layer l of the full inference: cached aggregates and embeddings of every vertex
 static void full_layer(Ctx* c, int l) {
     if (c->attention) { att_full(c, l); return; }
@@ -114,12 +127,13 @@ static void full_layer(Ctx* c, int l) {
 // full layer-wise inference over the current graph (Eq. 1-2): bootstrap and recompute-all
 static ripple_status run_full(Ctx* c) {
     c->launches = 0;
-    c->debug_tc_withhold = 0;
+    c->debug_tc_withhold = debug_tc_withhold();
     RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
     if (c->timing) cudaEventRecord(c->ev[0], c->stream);
     for (int l = 1; l <= c->L; ++l) full_layer(c, l);
     if (c->timing) cudaEventRecord(c->ev[1], c->stream);
     ripple_status st = sync_and_fetch_ctl(c);
+    if (!st) st = finished(c);
     if (st) return st;
     if (c->timing) cudaEventElapsedTime(&c->stats.ms_bootstrap, c->ev[0], c->ev[1]);
     c->stats.gpu_launches = c->launches;
@@ -667,10 +681,7 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
         for (int i = 0; i < nb && !wide; ++i) wide = ups[i].op == RIPPLE_OP_DEL_VERTEX;
     const int ng = wide ? (int)c->max_batch : chain_size(c, nb);
     c->may_expand = wide || mem != RIPPLE_MEM_HOST;
-    {   // diagnostic: a wait that nothing ends, to exercise the time-out path without faulting the device
-        const char* e = getenv("RIPPLE_DEBUG_TC_WITHHOLD");
-        c->debug_tc_withhold = e && e[0] == '1';
-    }
+    c->debug_tc_withhold = debug_tc_withhold();
     arm_rebuild(c, nb);
     c->has_opw = c->weighted && edge_weights && nb;
     c->few_rows_form = nb <= 128;
@@ -949,7 +960,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
         CK(cudaMalloc(&lists_dev, sizeof(int32_t*) * lists.size()));
         CK(cudaMemcpy(lists_dev, lists.data(), sizeof(int32_t*) * lists.size(), cudaMemcpyHostToDevice));
         c->launches = 0;
-        c->debug_tc_withhold = 0;
+        c->debug_tc_withhold = debug_tc_withhold();
         for (int l = 0; l <= c->L; ++l) c->tc_armed[l] = 1;
         c->few_rows_form = count <= 256;
         RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
@@ -959,9 +970,9 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
             self_project(c, l, false);
             update_rows(c, l, false);
         }
-        RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
         st = sync_and_fetch_ctl(c);
         cudaFree(lists_dev);
+        if (!st) st = finished(c);
         if (st) return st;
     }
     return RIPPLE_OK;
@@ -1154,10 +1165,12 @@ extern "C" ripple_status ripple_part_bootstrap_layer(ripple_ctx* ctx, int32_t l)
     cudaSetDevice(c->device);
     c->launches = 0;
     RP_LAUNCH(c, k_ctl_reset, 1, 1, 0, c->ctl, 0, 0);
+    c->debug_tc_withhold = debug_tc_withhold();
     part_fetch_halo_rows(c, l - 1);
     full_layer(c, l);
     c->stats.num_layers = c->L;
-    return finish_phase(c);
+    ripple_status st = sync_and_fetch_ctl(c);
+    return st ? st : finished(c);
 }
 
 extern "C" ripple_status ripple_part_begin(ripple_ctx* ctx, const ripple_update* ups, int64_t n, const float* feat_rows,
@@ -1182,7 +1195,7 @@ extern "C" ripple_status ripple_part_begin(ripple_ctx* ctx, const ripple_update*
     c->launches = 0;
     c->may_expand = 0;
     c->has_opw = c->weighted && edge_weights && nb;
-    c->debug_tc_withhold = 0;
+    c->debug_tc_withhold = debug_tc_withhold();
     for (int l = 0; l <= c->L; ++l) c->tc_armed[l] = 1;
     c->few_rows_form = nb <= 128;
     for (int l = 0; l <= c->L; ++l) c->rebuild_armed[l] = 0;
@@ -1241,6 +1254,7 @@ extern "C" ripple_status ripple_part_end(ripple_ctx* ctx) {
     cudaSetDevice(c->device);
     graph_batch_cleanup(c, c->part_nb);
     ripple_status st = sync_and_fetch_ctl(c);
+    if (!st) st = finished(c);   // (a rejected batch ends in ripple_part_begin)
     if (st) return st;
     const Ctl& h = *c->ctl_host;
     ripple_stats& s = c->stats;

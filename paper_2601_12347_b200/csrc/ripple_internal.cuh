@@ -199,7 +199,7 @@ struct Ctx {
     long long gather_min_messages;    // ... if the hop delivered at least this many messages in the batch before
     long long batches_done;
     int last_nb;
-    int debug_tc_withhold;   // diagnostic (environment RIPPLE_DEBUG_TC_WITHHOLD=1): see ripple_create
+    int debug_tc_withhold;   // diagnostic (environment RIPPLE_DEBUG_TC_WITHHOLD=1, read by every call that updates rows)
     int pdl;                 // launch with programmatic stream serialisation (off: environment RIPPLE_NO_PDL=1)
     int may_expand;   // the batch being enqueued may hold vertex deletions (always assumed for device batches)
     long long regather_min_messages;   // default threshold only: hops with fewer messages always push
