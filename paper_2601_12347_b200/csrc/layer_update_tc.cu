@@ -624,12 +624,13 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             }
             if (!ok) break;
         }
-        if (!ok) {   // no product of this CTA may be in flight when it leaves
-            if (lead) {
-                s_fail = 1;
-                tc_commit(&drained);
-                mbar_wait_bounded(&drained, 0, TC_SPIN_LIMIT);
-            }
+        // No product of this CTA may be in flight when it frees its tensor memory, however the other roles end: an epilogue
+        // that gave up waiting leaves while this warp still issues.  (In a pass that ends well the epilogue waits for the
+        // same products: nothing is lost by it.)
+        if (lead) {
+            if (!ok) s_fail = 1;
+            tc_commit(&drained);
+            mbar_wait_bounded(&drained, 0, TC_SPIN_LIMIT);
         }
     } else {
         // ---------------- weights: bulk copies, one thread ----------------
