@@ -637,6 +637,27 @@ static bool launch_batch_graph(Ctx* c, int ng) {
     return cudaGraphLaunch(c->graph_exec[slot], c->stream) == cudaSuccess;
 }
 
+static size_t pad16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// The address under which this device's kernels read all of [p, p + bytes), bytes > 0, or null if they cannot, or not in
+// words: pinned host memory whose pages are registered to the end of the range, or this device's own memory.  (Pageable
+// memory, a buffer registered only in part, another device's memory and odd addresses are for the copy engine.)
+static const void* device_reads(const Ctx* c, const void* p, size_t bytes, int32_t mem) {
+    cudaPointerAttributes first, last;
+    if (cudaPointerGetAttributes(&first, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&last, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool here = first.type == cudaMemoryTypeHost ||
+                      (mem == RIPPLE_MEM_DEVICE && (first.type == cudaMemoryTypeManaged || (first.type == cudaMemoryTypeDevice && first.device == c->device)));
+    if (!here || last.type != first.type || last.device != first.device || !first.devicePointer ||
+        static_cast<char*>(last.devicePointer) - static_cast<char*>(first.devicePointer) != (ptrdiff_t)(bytes - 1) ||
+        (reinterpret_cast<uintptr_t>(first.devicePointer) & 3))
+        return nullptr;
+    return first.devicePointer;
+}
+
 extern "C" ripple_status ripple_apply_batch(ripple_ctx* ctx, const ripple_update* ups, int64_t n,
                                             const float* feat_rows, int64_t n_rows, int32_t mem) {
     return ripple_apply_batch_weighted(ctx, ups, n, feat_rows, n_rows, nullptr, mem);
@@ -688,38 +709,35 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
     // a batch of a few tens of kilobytes is staged and classified by one block (more would keep it waiting for the bus)
     c->front_one_block = !c->may_expand && ng <= RP_ONE_BLOCK_BATCH &&
                          sizeof(ripple_update) * (size_t)nb + sizeof(float) * (size_t)nr * c->d[0] <= (32u << 10);
-    // The first kernel of the chain fetches the batch itself, from device memory or from pinned host memory: the caller's
-    // if it is pinned, else a packed copy in the library's own staging area.  Pageable batches that do not fit there
-    // are copied ahead of the chain.
+    // The first kernel of the chain fetches the batch itself, from device memory or from pinned host memory: from where
+    // the caller has it if kernels can read that, else from a packed copy in the library's own staging area.  Pageable
+    // batches that do not fit there, and device batches that kernels cannot read, are copied ahead of the chain.
     c->stage_in = StageIn{ups, c->has_opw ? edge_weights : nullptr, feat_rows, nb, nr};
-    if (mem == RIPPLE_MEM_HOST) {
-        auto pad16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    {
         const size_t b_ups = sizeof(ripple_update) * (size_t)nb, b_w = c->has_opw ? sizeof(float) * (size_t)nb : 0;
         const size_t b_rows = sizeof(float) * (size_t)nr * c->d[0];
-        auto on_device = [](const void* p) -> const void* {   // the device's address of pinned host memory, or null
-            cudaPointerAttributes at;
-            if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-            return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
-        };
-        // (packing this much takes less time than the look-up and the device's first sight of pages it has not read before)
-        const bool small = pad16(b_ups) + pad16(b_w) + b_rows <= (64u << 10);
+        const size_t at_w = pad16(b_ups), at_rows = at_w + pad16(b_w), packed = at_rows + b_rows;
         const void *pu = nullptr, *pw = nullptr, *pr = nullptr;
-        if (!small && (pu = on_device(ups)) && (!nr || (pr = on_device(feat_rows))) && (!b_w || (pw = on_device(edge_weights)))) {
+        // (packing 64 KB takes less time than the look-up and the device's first sight of pages it has not read before)
+        const bool look = mem == RIPPLE_MEM_DEVICE || packed > (64u << 10);
+        if (look && (pu = device_reads(c, ups, b_ups, mem)) && (!nr || (pr = device_reads(c, feat_rows, b_rows, mem))) &&
+            (!b_w || (pw = device_reads(c, edge_weights, b_w, mem)))) {
             c->stage_in.ups = static_cast<const ripple_update*>(pu);
             c->stage_in.opw = static_cast<const float*>(pw);
             c->stage_in.rows = static_cast<const float*>(pr);
-        } else if (pad16(b_ups) + pad16(b_w) + b_rows <= c->stage_bytes) {
+        } else if (mem == RIPPLE_MEM_HOST && packed <= c->stage_bytes) {
             char* at = c->stage_host;
             memcpy(at, ups, b_ups);
+            if (b_w) memcpy(at + at_w, edge_weights, b_w);
+            if (nr) memcpy(at + at_rows, feat_rows, b_rows);
             c->stage_in.ups = reinterpret_cast<const ripple_update*>(at);
-            at += pad16(b_ups);
-            if (b_w) { memcpy(at, edge_weights, b_w); c->stage_in.opw = reinterpret_cast<const float*>(at); }
-            at += pad16(b_w);
-            if (nr) { memcpy(at, feat_rows, b_rows); c->stage_in.rows = reinterpret_cast<const float*>(at); }
+            c->stage_in.opw = b_w ? reinterpret_cast<const float*>(at + at_w) : nullptr;
+            c->stage_in.rows = reinterpret_cast<const float*>(at + at_rows);
         } else {
-            CK(cudaMemcpyAsync(c->ups_dev, ups, b_ups, cudaMemcpyHostToDevice, c->stream));
-            if (b_w) CK(cudaMemcpyAsync(c->opw_dev, edge_weights, b_w, cudaMemcpyHostToDevice, c->stream));
-            if (nr) CK(cudaMemcpyAsync(c->feat_dev, feat_rows, b_rows, cudaMemcpyHostToDevice, c->stream));
+            const cudaMemcpyKind kind = mem == RIPPLE_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+            CK(cudaMemcpyAsync(c->ups_dev, ups, b_ups, kind, c->stream));
+            if (b_w) CK(cudaMemcpyAsync(c->opw_dev, edge_weights, b_w, kind, c->stream));
+            if (nr) CK(cudaMemcpyAsync(c->feat_dev, feat_rows, b_rows, kind, c->stream));
             c->stage_in.ups = nullptr;
         }
     }
@@ -783,6 +801,7 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
     }
     return RIPPLE_OK;
 fail:
+    cudaGetLastError();   // (a refused copy is this call's error, not the next one's)
     return st;
 }
 
