@@ -7,6 +7,7 @@ for the stream.  There is no fallback: if the library has not been built, loadin
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 from typing import Dict, List, Optional, Sequence, Tuple
 
@@ -323,40 +324,57 @@ class Ripple:
         feat_rows: [n_rows, d0] fp32 in the same memory space; op_weights: [n] fp32 in the same
         memory space, the weight of every ADD_EDGE (graphs with stored edge weights only)."""
         if _is_torch_cuda(ups):
-            ups = ups.contiguous()
-            n, uptr, mem = ups.shape[0], ups.data_ptr(), MEM_DEVICE
-            if feat_rows is None:
-                nr, fptr = 0, None
-            else:
-                feat_rows = feat_rows.contiguous()
-                nr, fptr = feat_rows.shape[0], feat_rows.data_ptr()
+            mem = MEM_DEVICE
+            ups, uptr = self._tensor(ups, "int32", "ups")
+            n = ups.shape[0]
+            if feat_rows is not None:
+                feat_rows, fptr = self._tensor(feat_rows, "float32", "feat_rows")
+            if op_weights is not None:
+                op_weights, wptr = self._tensor(op_weights, "float32", "op_weights")
         else:
+            mem = MEM_HOST
             if hasattr(ups, "numpy"):      # pinned host tensor [n, 3] int32
-                n, uptr = ups.shape[0], ups.data_ptr()
+                ups, uptr = self._tensor(ups, "int32", "ups")
+                n = ups.shape[0]
             else:
                 ups = np.ascontiguousarray(ups, dtype=UPDATE_DTYPE)
                 n, uptr = ups.size, _addr(ups)
-            mem = MEM_HOST
-            if feat_rows is None:
-                nr, fptr = 0, None
-            elif hasattr(feat_rows, "numpy"):
-                nr, fptr = feat_rows.shape[0], feat_rows.data_ptr()
-            else:
-                feat_rows = np.ascontiguousarray(feat_rows, dtype=np.float32)
-                nr, fptr = feat_rows.shape[0], _addr(feat_rows)
+            if feat_rows is not None:
+                feat_rows, fptr = self._host_array(feat_rows, "feat_rows")
+            if op_weights is not None:
+                op_weights, wptr = self._host_array(op_weights, "op_weights")
+        # (the library goes by these counts: an array of another shape would be read past its end)
+        if hasattr(ups, "numpy") and ups.numel() != 3 * n:
+            raise ValueError(f"ups: [n, 3] expected, got {tuple(ups.shape)}")
+        if feat_rows is None:
+            nr, fptr = 0, None
+        else:
+            nr = feat_rows.shape[0]
+            if math.prod(feat_rows.shape) != nr * self.dims[0]:
+                raise ValueError(f"feat_rows: [rows, {self.dims[0]}] expected, got {tuple(feat_rows.shape)}")
         if op_weights is None:
             self._check(self.lib.ripple_apply_batch(self.h, uptr, n, fptr, nr, mem))
             return
-        if mem == MEM_DEVICE:
-            op_weights = op_weights.contiguous()
-            wptr = op_weights.data_ptr()
-        elif hasattr(op_weights, "numpy"):
-            wptr = op_weights.data_ptr()
-        else:
-            op_weights = np.ascontiguousarray(op_weights, dtype=np.float32)
-            wptr = _addr(op_weights)
         assert op_weights.shape[0] == n
+        if math.prod(op_weights.shape) != n:
+            raise ValueError(f"op_weights: [n] expected, got {tuple(op_weights.shape)}")
         self._check(self.lib.ripple_apply_batch_weighted(self.h, uptr, n, fptr, nr, wptr, mem))
+
+    @staticmethod
+    def _tensor(x, dtype: str, name: str):
+        """A tensor of a batch, contiguous and of the type that the library reads, and its address."""
+        if str(x.dtype) != "torch." + dtype:
+            raise TypeError(f"{name}: torch.{dtype} expected, got {x.dtype}")
+        x = x.contiguous()
+        return x, x.data_ptr()
+
+    def _host_array(self, x, name: str):
+        if _is_torch_cuda(x):
+            raise ValueError(f"{name} is in device memory, ups in host memory")
+        if hasattr(x, "numpy"):
+            return self._tensor(x, "float32", name)
+        x = np.ascontiguousarray(x, dtype=np.float32)
+        return x, _addr(x)
 
     def set_timing(self, on: bool) -> None:
         self._check(self.lib.ripple_set_timing(self.h, int(bool(on))))
