@@ -294,6 +294,7 @@ class Ripple:
         opt.rebuild_budget = float(rebuild_budget)
         opt.n_local = int(n_local)     # > 0: one worker of a partitioned execution (see partitioned.py)
         opt.device = torch.cuda.current_device()
+        self._device = torch.device("cuda", opt.device)
         self._stream = stream if stream is not None else torch.cuda.Stream()
         opt.stream = self._stream.cuda_stream
         self._handle.stream = self._stream
@@ -391,11 +392,19 @@ class Ripple:
 
     # ---- read-out (borrowed device memory, valid until the next apply / recompute / close) ----
     # Wrapping device memory as a tensor takes several microseconds, a good part of the smallest batches' time, so
-    # each buffer is wrapped once; callers get aliases.
+    # each buffer is wrapped once; callers get aliases.  The wrapped tensor lies on the context's device whatever the
+    # current one (as a tensor of another device it would be a copy, and go stale), and is an ordinary tensor whatever
+    # mode it is first asked for in.
+    def _wrap(self, arr):
+        with self._torch.inference_mode(False):
+            return self._torch.as_tensor(arr, device=self._device)
+
     def _view(self, key, make):
         t = self._views.get(key)
         if t is None:
-            t = self._views[key] = self._torch.as_tensor(make(), device="cuda")
+            t = self._wrap(make())
+            if type(t) is self._torch.Tensor:   # (a tracing mode's stand-in is that caller's alone)
+                self._views[key] = t
         return t.detach()
 
     def _make_matrix(self, fn, layer: int, width: int):
@@ -404,7 +413,8 @@ class Ripple:
         return _DevArray(ptr.value, (self.n, width), "<f4", strides=(4 * ld.value, 4), owner=self._handle)
 
     def embeddings(self, layer: int):
-        return self._view(("H", layer), lambda: self._make_matrix(self.lib.ripple_get_embeddings, layer, self.dims[layer]))
+        width = self.dims[layer]
+        return self._view(("H", layer), lambda: self._make_matrix(self.lib.ripple_get_embeddings, layer, width))
 
     def aggregate(self, layer: int):
         """(tensor view N x width, transformed): the cached aggregate of `layer`; if transformed,
@@ -414,7 +424,7 @@ class Ripple:
         self._check(self.lib.ripple_get_aggregate(self.h, layer, ctypes.byref(ptr), ctypes.byref(ld),
                                                   ctypes.byref(width), ctypes.byref(tr)))
         arr = _DevArray(ptr.value, (self.n, width.value), "<f4", strides=(4 * ld.value, 4), owner=self._handle)
-        return self._torch.as_tensor(arr, device="cuda"), bool(tr.value)
+        return self._wrap(arr), bool(tr.value)
 
     def affected(self, layer: int):
         ptr, cnt = ctypes.c_void_p(), ctypes.c_int64()
