@@ -418,7 +418,7 @@ k_update_rows_elementwise(const Ctl* ctl, const __grid_constant__ UpdParams p) {
 // Launches every form that the row counts can call for; exactly one of them does the work of each problem (decided on
 // the device).
 // `over`: the hop whose list (A_over or C_over) the rows come from.
-static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2], const TcW* both = nullptr) {
+static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2]) {
     if (u.p[0].K == 0) {
         RP_LAUNCH(c, k_update_rows_elementwise, RP_RESIDENT(c, k_update_rows_elementwise, 256), 256, 0, c->ctl, u.p[0]);
         return;
@@ -438,7 +438,7 @@ static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2
             p.tc_w = tw[i]->w; p.tc_groups = tw[i]->groups; p.tc_chunks = tw[i]->chunks;
             tc.p[tc.n++] = p;
         } else if (p.n_cols <= NBN && p.a_mode != A_SUM) {
-            // plain fp32 arithmetic was asked for: narrow outputs over many rows have a form of their own
+            // narrow outputs over many rows have a form of their own
             p.narrow_min_rows = NARROW_MIN_ROWS;
         }
     }
@@ -446,10 +446,6 @@ static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2
     else if (u.p[0].list || tc.n < u.n || c->N < RP_TC_MIN_ROWS) RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, u);
     for (int i = 0; i < u.n; ++i)
         if (u.p[i].narrow_min_rows) RP_LAUNCH(c, k_update_rows_narrow, c->n_sm * 2, 256, NARROW_SMEM, c->ctl, u.p[i]);
-    if (both && tc.n == 2) {
-        tc.stacked = 1;
-        tc.p[0].tc_w = both->w; tc.p[0].tc_groups = both->groups;
-    }
     if (tc.n) launch_update_tc(c, tc);
 }
 
@@ -501,7 +497,7 @@ static void project(Ctx* c, int l, const UpdParams& nbr, bool full) {
     u.p[0] = nbr;
     u.n = 1;
     if (c->Z[l]) u.p[u.n++] = self_problem(c, l, full);   // the same rows: one launch for both products
-    launch_update(c, u, l - 1, {&ly.tc_nbr, &ly.tc_self}, ly.tc_pair.w ? &ly.tc_pair : nullptr);
+    launch_update(c, u, l - 1, {&ly.tc_nbr, &ly.tc_self});
 }
 
 void project_full(Ctx* c, int l) { project(c, l, neighbour_problem(c, l, true), true); }

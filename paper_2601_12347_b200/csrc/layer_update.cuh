@@ -55,7 +55,6 @@ struct UpdParams {
 struct UpdPair {
     UpdParams p[2];
     int n;
-    int stacked;   // tensor-core form: both problems, over the very same rows, in one column group
 };
 
 __device__ __forceinline__ float coef_deg(int deg) { return deg > 0 ? 1.0f / sqrtf((float)deg) : 0.0f; }

@@ -13,24 +13,23 @@
 // chunk is one bulk copy.  One thread issues, per 8-float K step, the weights' hi times [hi | lo] of the rows (256 columns)
 // and the weights' lo times the rows' hi: all but the product of the two low parts (2^-22 relative).  The small products
 // gather in accumulator columns of their own and meet the large ones in the epilogue: the tensor core rounds every
-// addition towards zero, and of a sum of 96 terms (K = 256) only 32 are then added at full size.  (More than 128 output
-// columns: only the product with the rows' lo has columns of its own, the one with the weights' lo joins the large ones.)
-// Error against fp64, 2-norm, one group: 3.6e-7 at K = 100, 7e-7 at K = 256, 1.5e-6 at K = 602 (one accumulator for all of
-// it: 1.2e-6, 1.8e-6, 5e-6; fp32 sums on SIMT: 2.9e-7 at K = 256).  With tc_mode = TC_TF32 only hi * hi is issued (plain TF32, 2^-10).  Row factors (sink
+// addition towards zero, and of a sum of 96 terms (K = 256) only 32 are then added at full size.
+// Error against fp64, 2-norm, 116 to 256 columns alike: 2.1e-7 at K = 32, 3.6e-7 at 100, 7e-7 at 256, 1.5e-6 at 602; GIN's
+// two products of 256 x 256 1.3e-6 (one accumulator for all of it: 6.8e-7, 1.2e-6, 2.4e-6, 5e-6; 4.4e-6; fp32 sums on SIMT: 1.1e-7,
+// 1.8e-7, 2.9e-7, 4.4e-7; 3.5e-7).  With tc_mode = TC_TF32 only hi * hi is issued (plain TF32, 2^-10).  Row factors (sink
 // normalisation, GIN's self factor) are applied to the finished sums.
 // Accumulators are double-buffered in tensor memory: the epilogue warps finish a tile (bias / cached terms /
 // activation / delta / commit) while the next tile's main loop is already running.
 //
 // What bounds it and why it is cut this way.  Each of the three pipelines -- gather and split, products, epilogue -- needs
 // about a microsecond per step whatever the bandwidth, so they overlap and each is kept free of chains: sixteen loader
-// warps with three chunks in flight, one warp that does nothing but issue (its operands in uniform registers), one that
-// fetches weights, eight epilogue warps whose loads travel ahead and whose stores are predicated.  The weights of a group
-// stay in shared memory for the life of the CTA while they fit (K <= 128: 128 KB); beyond that they stream from L2 with
-// every chunk.  Groups of one row tile run on neighbouring CTAs at the same time and find each other's rows in L2; two
-// narrow products over the same rows (the neighbour and the self projection of a layer's senders) share one group, side
-// by side.
-// Measured on 600 K rows (self and aggregate product of a layer, K = 100, 256 columns each: 1.18 -> 0.67 ms; neighbour
-// and self projection, K = 256, 48 columns each: 0.99 ms on SIMT -> 0.32; GIN's two products of 256 x 256: 2.02 -> 0.97 ms).
+// warps with three stages of rows where the weights stream, eight with two where they stay, one warp that does nothing but
+// issue (its operands in uniform registers), one that fetches weights, eight epilogue warps whose loads travel ahead and
+// whose stores are predicated.  The weights of a group stay in shared memory for the life of the CTA while they fit
+// (K <= 128: 128 KB); beyond that they stream from L2 with every chunk.  Groups of one row tile run on neighbouring CTAs
+// at the same time and find each other's rows in L2.
+// Measured on 600 K rows (self and aggregate product of a layer, K = 100, 256 columns each: 1.18 -> 0.67 ms; GIN's two
+// products of 256 x 256: 2.02 -> 0.97 ms).
 //
 // Every wait is bounded: if an mbarrier does not complete within the spin limit the CTA records
 // RIPPLE_ERR_TIMEOUT in the control block, waits (again bounded) for its own copies and products in flight, frees its
@@ -199,9 +198,8 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     __shared__ volatile int s_fail;
 
     if (ctl->abort) return;
-    // This CTA's column group: those of the first problem, then those of the second; or one group for both.
-    const bool stacked = pair.stacked != 0;
-    const int g0 = pair.p[0].tc_groups, G = g0 + (pair.n > 1 && !stacked ? pair.p[1].tc_groups : 0);
+    // This CTA's column group: those of the first problem, then those of the second.
+    const int g0 = pair.p[0].tc_groups, G = g0 + (pair.n > 1 ? pair.p[1].tc_groups : 0);
     const int my_g = (int)blockIdx.x % G, member = (int)blockIdx.x / G, members = ((int)gridDim.x - my_g + G - 1) / G;
     const UpdParams& p = pair.p[my_g < g0 ? 0 : 1];
     const int grp = my_g < g0 ? my_g : my_g - g0;
@@ -373,20 +371,16 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         // group, one per lane; the two warps of a quarter take half of the tile's rows each, BLK rows at a time.
         constexpr int BLK = 16, HALF = TILE / 2, OWN = HALF / 32;
         const int q = warp & 3, half = (warp - TC_LOADERS / 32) >> 2;
-        // what this lane's column belongs to
-        int lc = grp * TC_COLS + 32 * q + lane;
-        const UpdParams* mine = &p;
-        if (stacked && lc >= pair.p[0].n_cols) { lc -= pair.p[0].n_cols; mine = &pair.p[1]; }
-        const bool col_ok = lc < mine->n_cols;
-        if (!col_ok) { lc = 0; mine = &p; }
-        float* const hout = mine->Hout + lc;
-        float* const dout = mine->epi_mode == EPI_COMMIT && mine->Dout ? mine->Dout + lc : nullptr;
-        const float bias = mine->bias ? mine->bias[lc] : 0.f;
-        const int ldo = mine->ld_o;
+        int lc = grp * TC_COLS + 32 * q + lane;   // this lane's column
+        const bool col_ok = lc < p.n_cols;
+        if (!col_ok) lc = 0;
+        float* const hout = p.Hout + lc;
+        float* const dout = p.epi_mode == EPI_COMMIT && p.Dout ? p.Dout + lc : nullptr;
+        const float bias = p.bias ? p.bias[lc] : 0.f;
+        const int ldo = p.ld_o;
         const uint32_t ld_bytes = 4u * (uint32_t)ldo;
-        const bool relu = mine->act == RIPPLE_ACT_RELU, keep_old = mine->dout_old != 0;
-        // (the same for every lane of the launch)
-        const bool any_z = p.addend2 != nullptr, any_old = upd_needs_old(p) || (stacked && upd_needs_old(pair.p[1]));
+        const bool relu = p.act == RIPPLE_ACT_RELU, keep_old = p.dout_old != 0;
+        const bool any_z = p.addend2 != nullptr, any_old = upd_needs_old(p);
         const bool plus_s = p.addend || p.addend_rw, temp = p.epi_mode == EPI_TEMP;
         const bool coefs = p.src_norm && any_old;
         const bool scaled = p.a_mode == A_AGG || plus_s;
@@ -411,15 +405,9 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         // loads into registers were waited for at the next barrier wait, whatever their distance to the first use.
         constexpr int DEPTH = TC_AHEAD, BLOCKS = HALF / BLK;
         float* const zbuf = reinterpret_cast<float*>(w_ring + (size_t)W_SLOTS * TC_W_BYTES) + (warp - TC_LOADERS / 32) * (DEPTH * BLK * 32);
-        // the piece of the row that this lane copies: four columns, of the problem they belong to
-        const float* piece;
-        {
-            int pc = grp * TC_COLS + 32 * q + 4 * (lane & 7);
-            const UpdParams* of = &p;
-            if (stacked && pc >= pair.p[0].n_cols) { pc -= pair.p[0].n_cols; of = &pair.p[1]; }
-            if (pc >= of->n_cols) { pc = 0; of = &p; }
-            piece = (any_z ? of->addend2 : of->Hout) + pc;
-        }
+        // the piece of the row that this lane copies: four columns
+        const int pc = grp * TC_COLS + 32 * q + 4 * (lane & 7);
+        const float* const piece = (any_z ? p.addend2 : p.Hout) + (pc < p.n_cols ? pc : 0);
         auto fetch = [&](int slot, int v_src, int at) {
 #pragma unroll
             for (int i = 0; i < BLK / 4; ++i) {
@@ -589,7 +577,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             if (ub > 0) ok = __all_sync(FULL, mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit));
             if (!ok) break;
             tc_fence_after();
-            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF), d_corr = d_addr + (G == 1 ? TILE : 0);
+            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF), d_corr = d_addr + TILE;
             int left = K;
             for (int kc = 0; kc < nchunks; ++kc, left -= TC_KC) {
                 if (RESIDENT) sw = kc;
@@ -692,12 +680,17 @@ void tc_prepare() {
 #undef TC_SET
 }
 
-// The weights (row-major K x ldw; W2, if given, K x ldw2 beside them) as the kernel copies them: per column group and K
-// chunk, the group's 128 columns as rows of 32 K entries, first rounded to tf32, then the remainders (likewise
-// rounded), in the swizzled layout of the operand.
-cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const float* W2, int ldw2) {
+// The weights (row-major K x ldw) as the kernel copies them: per column group and K chunk, the group's 128 columns as rows
+// of 32 K entries, first rounded to tf32, then the remainders (likewise rounded), in the swizzled layout of the operand.
+//
+// Which outputs have them, and from how many rows the form is taken (RP_TC_MIN_ROWS), is a line of precision.  The form is
+// the faster one from 512 rows on, also for narrow outputs (whole-graph pass of one layer, K = 256, 256 columns: 512 rows
+// 39 us, fp32 sums 46; 1024: 39 / 52; 32 768: 94 / 321; 48 columns: 39 / 47, 39 / 48 and 51 / 114), but two to three times
+// less exact than fp32 sums (see the top of the file).  Outputs of 113 to 256 columns over 1024 and more rows have always
+// been split products, and less exact ones than these; all others are fp32 sums and stay so.
+cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw) {
     *out = TcW{};
-    if (K <= 0 || ldw <= 0) return cudaSuccess;
+    if (K <= 0 || ldw < RP_TC_MIN_COLS || ldw > RP_TC_MAX_COLS) return cudaSuccess;
     auto round_tf32 = [](float v) {
         uint32_t bits;
         memcpy(&bits, &v, 4);
@@ -705,15 +698,13 @@ cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const flo
         memcpy(&v, &bits, 4);
         return v;
     };
-    const int cols = ldw + (W2 ? ldw2 : 0);
-    out->groups = (cols + TC_COLS - 1) / TC_COLS;
+    out->groups = (ldw + TC_COLS - 1) / TC_COLS;
     out->chunks = (K + TC_KC - 1) / TC_KC;
     const size_t block = TC_W_BYTES / 4;
     std::vector<float> pack(block * out->chunks * out->groups, 0.f);
     for (int k = 0; k < K; ++k)
-        for (int j = 0; j < cols; ++j) {
-            const float x = j < ldw ? W[(size_t)k * ldw + j] : W2[(size_t)k * ldw2 + (j - ldw)];
-            const float h = round_tf32(x);
+        for (int j = 0; j < ldw; ++j) {
+            const float x = W[(size_t)k * ldw + j], h = round_tf32(x);
             const int g = j / TC_COLS, r = j - g * TC_COLS, kc = k / TC_KC, kk = k - kc * TC_KC;
             float* blk = pack.data() + ((size_t)g * out->chunks + kc) * block;
             const uint32_t at = tc_swz(r, kk >> 2) / 4 + (kk & 3);

@@ -23,7 +23,9 @@
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
 #define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold (sizes the item buffer)
-#define RP_TC_MIN_ROWS 512          // row count from which a layer update takes the tensor-core form
+#define RP_TC_MIN_ROWS 1024         // row count from which a layer update takes the tensor-core form,
+#define RP_TC_MIN_COLS 113          // for outputs of RP_TC_MIN_COLS .. RP_TC_MAX_COLS columns (see tc_weights_build)
+#define RP_TC_MAX_COLS 256
 #define RP_ATT_CHUNK 128            // attention: in-list entries per work item of a recomputation (sizes the item buffer)
 #define RP_TINY_BATCH 32            // batches up to this size list their frontiers and senders in one block each
 #define RP_TINY_APPLY 4             // ... and up to this size run the whole of Apply in one block (operations are resolved one after the other there)
@@ -155,7 +157,6 @@ struct LayerDev {
     TcW tc_nbr;  // neighbour matrix, for layers that transform before the scatter
     TcW tc_2;    // GIN: second matrix
     TcW tc_self; // SAGE: self matrix, for the cached self projection
-    TcW tc_pair; // neighbour and self matrix side by side, where both together have at most 128 columns
 };
 
 struct Ctx {
@@ -383,7 +384,7 @@ void feature_rows(Ctx* c, int n);                       // hop 0: overwrite feat
 void extra_sender_rows(Ctx* c, int l, int n);           // deltas of senders whose row did not change
 
 // layer_update_tc.cu
-cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw, const float* W2_host = nullptr, int ldw2 = 0);
+cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw);
 void tc_prepare();   // one-time kernel attributes (not allowed inside a stream capture)
 void narrow_prepare();   // likewise, for the update form for narrow outputs
 

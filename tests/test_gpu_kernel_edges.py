@@ -28,8 +28,9 @@ def apply_and_check(rp, orc, ups, rows, L, slack=0.0):
 
 
 # Tensor-core form of the layer update: K chunks of 32 (31, 32, 33, and four / five of them: the weights stay in shared
-# memory up to 128), column groups of 128 (5 ... 257 columns, two narrow products side by side), row tiles of 128 and
-# the 512 rows from which the form is taken (n - 1, n and n + 1 of both), normalised sources, GIN's summed operand.
+# memory up to 128), column groups of 128, the widths for which it is taken (113 to 256; narrower and wider ones are fp32
+# sums), row tiles of 128 and the 1024 rows from which it is taken (n - 1, n and n + 1 of both), normalised sources, GIN's
+# summed operand.
 TC_MODELS = {
     "sage_31_5_47": lambda: I.sage_model([31, 5, 47], I.AGG_MEAN),
     "sage_33_129_256": lambda: I.sage_model([33, 129, 256], I.AGG_SUM),
@@ -49,11 +50,11 @@ def test_row_updates_at_the_edges_of_their_tiles(env, name):
     model = TC_MODELS[name]()
     L = len(model.layers)
     slack = GIN_ROW_SLACK if name.startswith("gin") else 0.0
-    for n in (511, 512, 513, 641):
+    for n in (1023, 1024, 1025, 1153):
         src, dst = I.er_graph(n, 4 * n, 3)
         X = I.features(n, model.dims[0], 3)
         W = I.make_weights(model, 3, zero_bias=False)
-        rp = ripple.Ripple(n, src, dst, X, model, W, max_batch=1024)
+        rp = ripple.Ripple(n, src, dst, X, model, W, max_batch=2048)
         orc = Oracle(n, src, dst, X, model, W)
         G.check_values(rp, orc.full(), L, row_slack=slack)
         for b in range(2):      # every row changes; then an ordinary batch on the launch geometry of the large one
@@ -123,3 +124,25 @@ def test_batches_at_the_edges_of_the_staging_forms(env, mem, d):
         G.check_frontiers(rp, orc, 2)
         G.check_values(rp, orc.full(), 2)
     rp.close()
+
+
+# The default arithmetic is fp32 sums outside the tensor-core form's lines and the split product inside: a layer's product
+# over rows without in-neighbours, against fp64, on both sides of the lines.  u = 2^-24.  A sequential fp32 sum of K terms of
+# random sign: one rounding per term, 0.58 u / x rms for a partial sum of mantissa x (0.41 u over a binade), and partial sums
+# that grow like sqrt(k): 0.41 u sqrt(K / 2).  The tensor core truncates one addition per eight terms (0.31 u each, by measurement
+# at K = 32 to 602) and its operands' remainders are rounded (2.2 u).  Half as much again is allowed of either.
+@pytest.mark.parametrize("rows", [600, 1022, 1024, 4000])
+@pytest.mark.parametrize("K", [32, 100, 256, 602])
+def test_products_are_as_exact_as_their_arithmetic(env, K, rows):
+    ripple, _ = env
+    for d in (24, 48, 96, 112, 113, 128, 256, 257):
+        model = I.sage_model([K, d], I.AGG_MEAN)
+        X, W = I.features(rows, K, d), I.make_weights(model, 3, zero_bias=False)
+        rp = ripple.Ripple(rows, np.array([0], dtype=np.int32), np.array([1], dtype=np.int32), X, model, W)
+        got = rp.embeddings(1).cpu().numpy().astype(np.float64)[2:]
+        rp.close()
+        ref = X.astype(np.float64)[2:] @ W[0]["Wa"].astype(np.float64) + W[0]["ba"]
+        tensor = 113 <= d <= 256 and rows >= 1024
+        bound = 1.5 * 2.0 ** -24 * (2.2 + 0.31 * K / 8 if tensor else 0.41 * np.sqrt(K / 2))
+        err = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
+        assert err <= bound, (d, err, bound)
