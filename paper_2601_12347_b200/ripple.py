@@ -305,6 +305,7 @@ class Ripple:
             msg = self.lib.ripple_last_error(None).decode()
             self.h.value = None
             raise RippleError(st, msg)
+        self._wrap_buffers()
 
     # ---- lifetime ------------------------------------------------------------------------
     def close(self):
@@ -386,13 +387,15 @@ class Ripple:
         self._views.clear()
         self._check(self.lib.ripple_reserve_vertices(self.h, int(n)))
         self.n = int(n)
+        self._wrap_buffers()
 
     def recompute_full(self) -> None:
         self._check(self.lib.ripple_recompute_full(self.h))
 
     # ---- read-out (borrowed device memory, valid until the next apply / recompute / close) ----
-    # Wrapping device memory as a tensor takes several microseconds, a good part of the smallest batches' time, so
-    # each buffer is wrapped once; callers get aliases.  The wrapped tensor lies on the context's device whatever the
+    # Wrapping device memory as a tensor takes several microseconds (the first time tens), a good part of the smallest
+    # batches' time, so each buffer is wrapped once, when it is allocated (first pass of a context, one update on the
+    # sparse graph: 70 to 80 us less); callers get aliases.  The wrapped tensor lies on the context's device whatever the
     # current one (as a tensor of another device it would be a copy, and go stale), and is an ordinary tensor whatever
     # mode it is first asked for in.
     def _wrap(self, arr):
@@ -406,6 +409,11 @@ class Ripple:
             if type(t) is self._torch.Tensor:   # (a tracing mode's stand-in is that caller's alone)
                 self._views[key] = t
         return t.detach()
+
+    def _wrap_buffers(self):
+        for layer in range(self.L + 1):
+            self.embeddings(layer), self.affected(layer)
+        self.degrees()
 
     def _make_matrix(self, fn, layer: int, width: int):
         ptr, ld = ctypes.c_void_p(), ctypes.c_int64()

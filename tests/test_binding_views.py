@@ -56,3 +56,21 @@ def test_views_read_in_inference_mode_serve_training_too(env):
     assert torch.allclose(w.grad[:, 0], rp.embeddings(2).sum(0), rtol=1e-4)
     assert not rp.affected(2).is_inference() and not rp.degrees()[0].is_inference()
     rp.close()
+
+
+@pytest.mark.gpu
+def test_buffers_are_wrapped_when_they_are_allocated(env, monkeypatch):
+    ripple_, _ = env
+    model = I.sage_model([18, 36, 10], I.AGG_MEAN)
+    src, dst = I.er_graph(300, 2000, 3)
+    rp = ripple_.Ripple(300, src, dst, I.features(300, 18, 3), model, I.make_weights(model, 3))
+    old = rp.embeddings(1)
+    for n in (300, 400):
+        if n == 400:
+            rp.reserve_vertices(n)
+        with monkeypatch.context() as m:
+            m.setattr(torch, "as_tensor", None)
+            assert [rp.embeddings(l).shape for l in range(3)] == [(n, 18), (n, 36), (n, 10)]
+            assert rp.degrees()[0].shape == (n,) and rp.affected(0).numel() == 0
+    assert rp.embeddings(1).data_ptr() != old.data_ptr()
+    rp.close()
