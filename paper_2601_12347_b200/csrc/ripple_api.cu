@@ -588,51 +588,56 @@ static int chain_size(const Ctx* c, int nb) {
 
 // The chain (twenty to fifty mostly short kernels) is captured once per launch geometry into a CUDA graph and replayed:
 // a launch of its own costs the host 2.3 us, more than many of the kernels take, a node of a replayed chain 0.9 us
-// (both measured on empty kernels).  Returns false if this batch must take the direct path.
-static bool launch_batch_graph(Ctx* c, int ng) {
-    if (c->no_graphs || c->timing || ng < 1 || c->debug_tc_withhold) return false;
-    // the captured chain differs with the expansion kernels and with the hops whose rebuilding form is enqueued
+// (both measured on empty kernels).  The captured chain differs with the expansion kernels and with the hops whose
+// rebuilding form is enqueued.
+static uint64_t chain_key(const Ctx* c, int ng) {
     uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->few_rows_form ? 4 : 0);
     key = 2 * key + (c->front_one_block ? 1 : 0);
     for (int l = 1; l <= c->L; ++l) key = 4 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0);
     for (int l = 0; l <= c->L; ++l) key = 2 * key + (c->tc_armed[l] ? 1 : 0);
-    int slot = -1;
-    for (int i = 0; i < RP_GRAPH_SLOTS; ++i)
-        if (c->graph_exec[i] && c->graph_key[i] == key) slot = i;
-    if (slot < 0) {
-        // Capturing costs a millisecond or more: only a chain that keeps coming back is worth it.  A
-        // stream whose batch sizes never repeat is launched kernel by kernel.
-        int seen = -1;
-        for (int i = 0; i < RP_GRAPH_SEEN; ++i)
-            if (c->seen_key[i] == key) seen = i;
-        if (seen < 0) {
-            seen = c->seen_next++ % RP_GRAPH_SEEN;
-            c->seen_key[seen] = key;
-            c->seen_count[seen] = 0;
-        }
-        if (++c->seen_count[seen] < 2) return false;
-        slot = c->graph_next++ % RP_GRAPH_SLOTS;
-        if (c->graph_exec[slot]) { cudaGraphExecDestroy(c->graph_exec[slot]); c->graph_exec[slot] = nullptr; }
-        cudaGraph_t g = nullptr;
-        if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { c->no_graphs = 1; return false; }
-        c->launches = 0;
-        enqueue_batch(c, ng, false);
-        cudaError_t e = cudaStreamEndCapture(c->stream, &g);
-        size_t roots = 1;
-        if (e == cudaSuccess) e = cudaGraphGetRootNodes(g, &c->graph_root[slot], &roots);
-        if (e == cudaSuccess && roots != 1) e = cudaErrorUnknown;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_exec[slot], g, 0);
-        if (c->graph[slot]) cudaGraphDestroy(c->graph[slot]);
-        c->graph[slot] = g;   // (its root node names the node of the executable chain)
-        if (e != cudaSuccess) { cudaGetLastError(); c->graph_exec[slot] = nullptr; c->no_graphs = 1; return false; }
-        c->graph_key[slot] = key;
-        c->graph_launches[slot] = c->launches;
-    } else if (graph_batch_retarget(c, ng, c->graph_exec[slot], c->graph_root[slot]) != cudaSuccess) {
+    return key;
+}
+
+static bool replay_chain(Ctx* c, int ng, int slot) {
+    if (graph_batch_retarget(c, ng, c->graph_exec[slot], c->graph_root[slot]) != cudaSuccess ||
+        cudaGraphLaunch(c->graph_exec[slot], c->stream) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     c->launches = c->graph_launches[slot];
-    return cudaGraphLaunch(c->graph_exec[slot], c->stream) == cudaSuccess;
+    return true;
+}
+
+// Called with the batch already launched kernel by kernel, so that the device works while the host captures and
+// instantiates (a quarter of a millisecond for the shortest chains, twice that for the longest).
+static void capture_chain(Ctx* c, int ng, uint64_t key, int slot) {
+    const int64_t launched = c->launches;
+    if (c->graph_exec[slot]) { cudaGraphExecDestroy(c->graph_exec[slot]); c->graph_exec[slot] = nullptr; }
+    if (c->graph[slot]) { cudaGraphDestroy(c->graph[slot]); c->graph[slot] = nullptr; }
+    c->chains.drop(slot);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        c->launches = 0;
+        enqueue_batch(c, ng, false);
+        e = cudaStreamEndCapture(c->stream, &g);
+    }
+    size_t roots = 0;
+    if (e == cudaSuccess) e = cudaGraphGetRootNodes(g, nullptr, &roots);
+    if (e == cudaSuccess && roots != 1) e = cudaErrorUnknown;   // (its one root is told where a batch lies)
+    if (e == cudaSuccess) e = cudaGraphGetRootNodes(g, &c->graph_root[slot], &roots);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_exec[slot], g, 0);
+    if (e == cudaSuccess) {
+        c->graph[slot] = g;   // (its root node names the node of the executable chain)
+        c->graph_launches[slot] = c->launches;
+        c->chains.put(slot, key);
+    } else {
+        cudaGetLastError();
+        if (g) cudaGraphDestroy(g);
+        c->graph_exec[slot] = nullptr;
+        c->no_graphs = 1;
+    }
+    c->launches = launched;
 }
 
 static size_t pad16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -739,9 +744,16 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
             c->stage_in.ups = nullptr;
         }
     }
-    if (!launch_batch_graph(c, ng)) {
-        c->launches = 0;
-        evi = enqueue_batch(c, ng, c->timing != 0);
+    {
+        const bool chains = !c->no_graphs && !c->timing && !c->debug_tc_withhold;
+        const uint64_t key = chain_key(c, ng);
+        int slot = chains ? c->chains.find(key) : -1;
+        if (slot < 0 || !replay_chain(c, ng, slot)) {
+            const bool unknown = chains && slot < 0;
+            c->launches = 0;
+            evi = enqueue_batch(c, ng, c->timing != 0);
+            if (unknown && (slot = c->chains.place(key)) >= 0) capture_chain(c, ng, key, slot);
+        }
     }
     {   // (the chain's last kernel has put the control block into ctl_host)
         cudaError_t e = cudaStreamSynchronize(c->stream);
@@ -917,9 +929,7 @@ extern "C" ripple_status ripple_reserve_vertices(ripple_ctx* ctx, int64_t num_ve
     for (int l = 1; l <= L; ++l) if (c->layer[l].kind == RIPPLE_LAYER_GIN) max_hid = std::max(max_hid, c->layer[l].ld_hid);
     CK(cudaStreamSynchronize(c->stream));
     for (auto& g : c->graph_exec) if (g) { cudaGraphExecDestroy(g); g = nullptr; }   // captured chains hold the old addresses
-    memset(c->graph_key, 0, sizeof(c->graph_key));
-    memset(c->seen_key, 0, sizeof(c->seen_key));
-    memset(c->seen_count, 0, sizeof(c->seen_count));
+    c->chains.clear();
     for (int l = 0; l <= L; ++l) {
         CK(grow_array(&c->H[l], N0 * c->ld[l], N1 * c->ld[l], 0));
         CK(grow_array(&c->A[l], N0 + 32, N1 + 32, 0));

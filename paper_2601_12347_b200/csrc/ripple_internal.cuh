@@ -17,8 +17,6 @@
 #define RP_MAXL RIPPLE_MAX_LAYERS
 #define RP_TOMB (-1)
 #define RP_ONE_BLOCK_BATCH 512   // batches up to this size have their row updates done by one block
-#define RP_GRAPH_SLOTS 16
-#define RP_GRAPH_SEEN 32    // recently seen chain keys: a chain is captured at its second appearance
 #define RP_POOL_CLASSES 32          // block size classes of the adjacency store: class k holds blocks of 2^k entries
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
@@ -30,6 +28,8 @@
 #define RP_TINY_BATCH 32            // batches up to this size list their frontiers and senders in one block each
 #define RP_TINY_APPLY 4             // ... and up to this size run the whole of Apply in one block (operations are resolved one after the other there)
 #define RP_TINY_WORDS 16384         // ... and list a hop's frontier in one block if its bitmap has at most this many words
+
+#include "chain_store.h"
 
 namespace rp {
 
@@ -264,15 +264,11 @@ struct Ctx {
     int front_one_block;   // the batch being applied is staged and classified by one block
     int few_rows_form; // the batch being applied is small: its row updates carry the few-row form (see k_update_rows)
     int no_graphs;
-    cudaGraph_t graph[RP_GRAPH_SLOTS];
-    cudaGraphExec_t graph_exec[RP_GRAPH_SLOTS];
-    cudaGraphNode_t graph_root[RP_GRAPH_SLOTS];   // the chain's first kernel: its argument says where the batch lies
-    uint64_t graph_key[RP_GRAPH_SLOTS];
-    int64_t graph_launches[RP_GRAPH_SLOTS];
-    int graph_next;
-    uint64_t seen_key[RP_GRAPH_SEEN];
-    int seen_count[RP_GRAPH_SEEN];
-    int seen_next;
+    ChainStore chains;
+    cudaGraph_t graph[ChainStore::SLOTS];
+    cudaGraphExec_t graph_exec[ChainStore::SLOTS];
+    cudaGraphNode_t graph_root[ChainStore::SLOTS];   // the chain's first kernel: its argument says where the batch lies
+    int64_t graph_launches[ChainStore::SLOTS];
     Ctl* ctl;        // device
     Ctl* ctl_host;   // pinned
     ripple_stats stats;

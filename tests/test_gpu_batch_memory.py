@@ -7,6 +7,8 @@ import pytest
 
 from paper_2601_12347_b200 import inputs as I
 
+from tolerances import GIN_ROW_SLACK
+
 import test_gpu_parity as G
 
 pytestmark = pytest.mark.gpu
@@ -128,4 +130,35 @@ def test_operation_weights_arrive_from_every_memory_space(env, mem):
             rp.apply_batch(*t)
         _check(rp, orc, ups, rows, op_weights=w)
         assert np.array_equal(rp.export_graph_weighted()[2], orc.export_weights())
+    rp.close()
+
+
+def test_more_launch_geometries_than_captured_chains_are_kept(env):
+    """Sizes and memory spaces mixed on one context: twenty and more geometries go round, so chains are captured while a
+    batch is in flight, replayed, given up and captured again."""
+    import torch
+    rp, orc, src, dst = _pair(env, weighted=True)
+    stream = I.UpdateStream(N, src, dst, D, 12)
+    rng = np.random.default_rng(4)
+    sizes = [1, 3, 5, 12, 17, 33, 65, 128, 129, 300, 600, 1025]
+    todo = [(s, m) for s in sizes for m in ("host", "pinned", "device")]
+    for rnd in range(4):
+        order = rng.permutation(len(todo)) if rnd < 3 else np.repeat(rng.permutation(len(todo))[:8], 3)
+        for k in order:
+            count, mem = todo[k]
+            ups, rows = stream.next_batch(count)
+            w = I.edge_weights(count, 900 + rnd) if count % 2 else None
+            a = [_raw(ups), rows] + ([w] if w is not None else [])
+            t = [torch.from_numpy(x) for x in a]
+            if mem == "host":
+                rp.apply_batch(ups, *a[1:])
+            else:
+                t = [x.cuda() if mem == "device" else x.pin_memory() for x in t]
+                torch.cuda.synchronize()
+                rp.apply_batch(*t)
+            assert orc.apply_incremental(ups, rows, op_weights=w) == 0
+            G.check_frontiers(rp, orc, 2)
+        G.check_graph(rp, orc)
+        assert np.array_equal(rp.export_graph_weighted()[2], orc.export_weights())
+        G.check_values(rp, orc.full(), 2, row_slack=GIN_ROW_SLACK)
     rp.close()
