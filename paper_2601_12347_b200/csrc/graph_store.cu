@@ -866,9 +866,10 @@ __global__ void k_commit_degrees(Ctl* ctl, const Rec* __restrict__ rec, Side out
     d_commit_degrees(ctl, rec, out, in, deg_out_old, moved_start, moved_cap);
 }
 
-// ... and all of them in one block, a barrier between the phases, for the batches that are replayed
-// from a captured chain (up to RP_ONE_BLOCK_BATCH operations: a few hundred records at most, which one
-// block handles in a single sweep per phase).  Small batches are bound by the number of launches.
+// ... and all of them in one block, a barrier between the phases, for batches of up to RP_ONE_BLOCK_BATCH operations: as
+// many records at most, which one block handles in a single sweep per phase.  (A batch in device memory is not inspected
+// and may hold vertex deletions; the records these expand to take the block further sweeps.)  Small batches are bound by
+// the number of launches.
 __global__ void __launch_bounds__(1024)
 k_mutate_small(Ctl* ctl, Rec* rec, Side out, Side in, const int32_t* __restrict__ grow_out,
                const int32_t* __restrict__ grow_in, const int32_t* __restrict__ shrink_out,

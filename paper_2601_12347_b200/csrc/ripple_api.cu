@@ -399,8 +399,9 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         }
         CK(dev_alloc(&c->moved_start, (size_t)4 * o.max_batch));
         CK(dev_alloc(&c->moved_cap, (size_t)4 * o.max_batch));
-        // (vertex, chunk) work items of long in-lists: a row of more than 256 entries gives at most 2 items per 256 of
-        // them, a row gathered anew by the fold one per RP_ANEW_CHUNK and one more
+        // (vertex, chunk) work items: a list of more than RP_ANEW_CHUNK entries gives at most 2 items per RP_ANEW_CHUNK of
+        // them, a row gathered anew by the fold one per RP_ANEW_CHUNK and one more; no kernel that fills the buffer cuts
+        // its lists shorter (each asserts it)
         CK(dev_alloc(&c->items, item_count(c, (size_t)N)));
         CK(dev_alloc(&c->coff, (size_t)N + 2, 0));   // degree prefix of a sender list
         CK(dev_alloc(&c->bitmap, (size_t)c->n_words + 256, 0));
@@ -525,11 +526,10 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
         // tiny batches on graphs whose frontier bitmap one block can sweep: A_l by one launch instead of two
         const bool merged = tiny && !pull && c->n_words <= RP_TINY_WORDS;
         // the next hop's senders are listed along with the frontier where this hop's are done with by then
-        const bool senders_too = l < L && !pull && !c->src_norm && nb > 0;
+        const bool senders_too = l < L && !pull && !c->src_norm;
         if (merged) frontier_compact_small(c, l, senders_too);
         else if (senders_too) frontier_compact_senders(c, l);
         else if (!pull) frontier_compact(c, l);
-        if (nb <= 0) senders_release(c, l - 1);   // (otherwise the last kernel of the hop's delta form clears them)
         fold_deltas(c, l);
         regather_layer(c, l);
         STAMP();

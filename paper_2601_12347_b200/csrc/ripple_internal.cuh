@@ -20,7 +20,7 @@
 #define RP_POOL_CLASSES 32          // block size classes of the adjacency store: class k holds blocks of 2^k entries
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
-#define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold (sizes the item buffer)
+#define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold; the smallest of the chunks whose items share a buffer, which it sizes
 #define RP_TC_MIN_ROWS 1024         // row count from which a layer update takes the tensor-core form,
 #define RP_TC_MIN_COLS 113          // for outputs of RP_TC_MIN_COLS .. RP_TC_MAX_COLS columns (see tc_weights_build)
 #define RP_TC_MAX_COLS 256
@@ -67,7 +67,7 @@ struct Ctl {
     int n_rebuilt[RP_MAXL + 1];       // aggregate rows of hop l gathered anew because their rounding budget ran out
     int rebuild_items[RP_MAXL + 1];   // (vertex, chunk) work items of the long rows among them
     int max_items[RP_MAXL + 1];       // max / min: (long row, chunk) work items of hop l's recomputation
-    int walk_ticket[RP_MAXL + 1];     // walk of the senders' out-lists: next unassigned chunk (see OutWalk)
+    int walk_ticket[RP_MAXL + 1];     // walk of the senders' out-lists: next unassigned chunk (see TicketWalk)
     int ew_ticket[RP_MAXL + 1];       // elementwise update: next unassigned run of pieces
     int hub_ticket[RP_MAXL + 1];      // chunks of long in-lists: next unassigned work item
     int regather_ticket[RP_MAXL + 1]; // rebuilding form: next unassigned position of A_l

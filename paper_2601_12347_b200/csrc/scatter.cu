@@ -40,6 +40,8 @@ __device__ __forceinline__ void add4(float4& a, const float4& x, float c) {
 // single warp busy for 0.7 ms, longer than everything else of a hop on the sparse graph.
 constexpr int SPMM_HUB_DEGREE = 256;
 constexpr int SPMM_HUB_CHUNK = 256;
+static_assert(SPMM_HUB_CHUNK >= RP_ANEW_CHUNK && SPMM_HUB_DEGREE >= RP_ANEW_CHUNK, "the item buffer is sized by RP_ANEW_CHUNK");
+
 // acc += sum over in-list entries [j_begin, j_end) of row v of c_u * M_u; LPR lanes hold one row
 // (NV float4 slots each), a warp works on 32 / LPR neighbours per step, several steps in flight.
 template <int NV, int LPR>
@@ -232,8 +234,10 @@ void spmm_full(Ctx* c, int l) {
 // Messages of the net edge changes: S_v += sign * w * M_r with M_r = c_old m_old of the record's
 // source (= c_new m_new - D_u if the source is a sender of this hop, c m otherwise) and w the edge's
 // stored weight (1 without stored weights).  One warp per record; rows have the inbox width.
-// A pushing hop delivers them along with the walk (both only add to the accumulator), from the far end of the grid; a
-// gathering hop, whose gather stores the rows it finishes, afterwards in a launch of their own.
+// A pushing hop delivers them in the walk's launch (both only add to the accumulator), by the last blocks of the grid:
+// the pushes launch eight blocks per SM, of which registers admit three to five at a time, so on a large walk these
+// blocks begin when others run out of tickets.  A gathering hop, whose gather stores the rows it finishes, delivers them
+// afterwards in a launch of their own.
 struct RecMsgs {
     const Rec* rec;
     int src_norm;
@@ -487,6 +491,7 @@ k_scatter_push_bulk(Ctl* ctl, int l, const int32_t* __restrict__ senders, const 
 constexpr int GATHER_WINDOW = 128;
 constexpr int GATHER_LONG = 512;     // longer in-lists are cut into work items of GATHER_ITEM entries
 constexpr int GATHER_ITEM = 256;
+static_assert(GATHER_ITEM >= RP_ANEW_CHUNK && GATHER_LONG >= RP_ANEW_CHUNK, "the item buffer is sized by RP_ANEW_CHUNK");
 constexpr int GATHER_TAKE = 8;       // sinks per ticket
 
 template <int NV, int LPR>
