@@ -1246,6 +1246,7 @@ extern "C" ripple_status ripple_part_begin(ripple_ctx* ctx, const ripple_update*
     if (c->ctl_host->err) {
         st = (ripple_status)c->ctl_host->err;
         set_err(c, "batch rejected by a worker (status %d)", (int)st);
+        senders_release(c, 0);   // (no hop follows that would take its senders out of the position map)
         graph_batch_cleanup(c, c->part_nb);
         finish_phase(c);
         return st;
