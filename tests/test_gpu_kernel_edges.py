@@ -93,8 +93,9 @@ def test_walks_over_rows_that_outgrow_the_cache(env, kind):
     rp.close()
 
 
-# How a batch reaches the device: one block up to 4 updates, up to 512 updates and 32 KB staged by one block, pinned copies
-# up to 64 KB read where they lie, larger ones through the staging area or by separate copies.
+# How a batch reaches the device: one block up to 4 updates, up to 512 updates and 32 KB staged by one block, more by a grid;
+# host batches of up to 64 KB packed into the staging area, larger ones read where they lie if they are pinned and packed
+# if not.  (Batches beyond the staging area: test_gpu_batch_memory.py.)
 @pytest.mark.parametrize("mem", ["host", "pinned", "device"])
 @pytest.mark.parametrize("d", [8, 602])
 def test_batches_at_the_edges_of_the_staging_forms(env, mem, d):
