@@ -7,7 +7,6 @@ for the stream.  There is no fallback: if the library has not been built, loadin
 from __future__ import annotations
 
 import ctypes
-import math
 import os
 from typing import Dict, List, Optional, Sequence, Tuple
 
@@ -193,10 +192,6 @@ class _DevArray:
         self._owner = owner
 
 
-def _addr(a: np.ndarray) -> int:
-    return a.__array_interface__["data"][0]   # (a.ctypes.data builds an object first)
-
-
 def _is_torch_cuda(x) -> bool:
     return hasattr(x, "is_cuda") and bool(x.is_cuda)
 
@@ -325,58 +320,46 @@ class Ripple:
         """ups: numpy array of UPDATE_DTYPE (host) or CUDA int32 tensor [n, 3] (device);
         feat_rows: [n_rows, d0] fp32 in the same memory space; op_weights: [n] fp32 in the same
         memory space, the weight of every ADD_EDGE (graphs with stored edge weights only)."""
-        if _is_torch_cuda(ups):
-            mem = MEM_DEVICE
-            ups, uptr = self._tensor(ups, "int32", "ups")
-            n = ups.shape[0]
-            if feat_rows is not None:
-                feat_rows, fptr = self._tensor(feat_rows, "float32", "feat_rows")
-            if op_weights is not None:
-                op_weights, wptr = self._tensor(op_weights, "float32", "op_weights")
+        nr, fptr, d0 = 0, None, self.dims[0]
+        if hasattr(ups, "numpy"):          # tensor [n, 3] int32, on the device or pinned
+            mem = MEM_DEVICE if ups.is_cuda else MEM_HOST
+            ups, uptr, n, size = self._tensor(ups, "torch.int32", "ups")
+            if size != 3 * n:
+                raise ValueError(f"ups: [n, 3] expected, got {tuple(ups.shape)}")
         else:
             mem = MEM_HOST
-            if hasattr(ups, "numpy"):      # pinned host tensor [n, 3] int32
-                ups, uptr = self._tensor(ups, "int32", "ups")
-                n = ups.shape[0]
-            else:
-                ups = np.ascontiguousarray(ups, dtype=UPDATE_DTYPE)
-                n, uptr = ups.size, _addr(ups)
-            if feat_rows is not None:
-                feat_rows, fptr = self._host_array(feat_rows, "feat_rows")
-            if op_weights is not None:
-                op_weights, wptr = self._host_array(op_weights, "op_weights")
+            ups = np.ascontiguousarray(ups, dtype=UPDATE_DTYPE)
+            n, uptr = ups.size, ups.ctypes.data
         # (the library goes by these counts: an array of another shape would be read past its end)
-        if hasattr(ups, "numpy") and ups.numel() != 3 * n:
-            raise ValueError(f"ups: [n, 3] expected, got {tuple(ups.shape)}")
-        if feat_rows is None:
-            nr, fptr = 0, None
-        else:
-            nr = feat_rows.shape[0]
-            if math.prod(feat_rows.shape) != nr * self.dims[0]:
-                raise ValueError(f"feat_rows: [rows, {self.dims[0]}] expected, got {tuple(feat_rows.shape)}")
+        if feat_rows is not None:
+            feat_rows, fptr, nr, size = self._array(feat_rows, mem, "feat_rows")
+            if size != nr * d0:
+                raise ValueError(f"feat_rows: [rows, {d0}] expected, got {tuple(feat_rows.shape)}")
         if op_weights is None:
             self._check(self.lib.ripple_apply_batch(self.h, uptr, n, fptr, nr, mem))
             return
-        assert op_weights.shape[0] == n
-        if math.prod(op_weights.shape) != n:
+        op_weights, wptr, nw, size = self._array(op_weights, mem, "op_weights")
+        assert nw == n
+        if size != n:
             raise ValueError(f"op_weights: [n] expected, got {tuple(op_weights.shape)}")
         self._check(self.lib.ripple_apply_batch_weighted(self.h, uptr, n, fptr, nr, wptr, mem))
 
+    # An array of a batch, contiguous and of the type that the library reads: itself (to be kept until the call is over),
+    # its address, its first extent and its size.
     @staticmethod
     def _tensor(x, dtype: str, name: str):
-        """A tensor of a batch, contiguous and of the type that the library reads, and its address."""
-        if str(x.dtype) != "torch." + dtype:
-            raise TypeError(f"{name}: torch.{dtype} expected, got {x.dtype}")
+        if str(x.dtype) != dtype:
+            raise TypeError(f"{name}: {dtype} expected, got {x.dtype}")
         x = x.contiguous()
-        return x, x.data_ptr()
+        return x, x.data_ptr(), x.shape[0], x.numel()
 
-    def _host_array(self, x, name: str):
-        if _is_torch_cuda(x):
-            raise ValueError(f"{name} is in device memory, ups in host memory")
-        if hasattr(x, "numpy"):
-            return self._tensor(x, "float32", name)
+    def _array(self, x, mem: int, name: str):
+        if mem == MEM_DEVICE or hasattr(x, "numpy"):
+            if mem == MEM_HOST and x.is_cuda:
+                raise ValueError(f"{name} is in device memory, ups in host memory")
+            return self._tensor(x, "torch.float32", name)
         x = np.ascontiguousarray(x, dtype=np.float32)
-        return x, _addr(x)
+        return x, x.ctypes.data, x.shape[0], x.size
 
     def set_timing(self, on: bool) -> None:
         self._check(self.lib.ripple_set_timing(self.h, int(bool(on))))
