@@ -19,7 +19,7 @@ namespace rp {
 
 constexpr int MAX_HUB_DEGREE = 256;    // longer in-lists are recomputed in chunks, one warp per chunk
 constexpr int MAX_HUB_CHUNK = 256;     // in-list entries per chunk
-static_assert(MAX_HUB_CHUNK >= RP_ANEW_CHUNK && MAX_HUB_DEGREE >= RP_ANEW_CHUNK, "the item buffer is sized by RP_ANEW_CHUNK");
+static_assert(MAX_HUB_CHUNK >= RP_ITEM_MIN, "the item buffer is sized by it");
 constexpr int MAX_FULL_PASS_DEGREE = 4096;   // a full pass has rows enough to keep every warp busy: only longer lists are chunked
 constexpr int MAX_CHUNK = 64;          // edges per warp work item of the message walk
 

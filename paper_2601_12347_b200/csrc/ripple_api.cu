@@ -140,7 +140,9 @@ static ripple_status run_full(Ctx* c) {
     return RIPPLE_OK;
 }
 
-static size_t item_count(const Ctx* c, size_t n) { return n + (size_t)(c->side[1].col_size / (RP_ANEW_CHUNK / 2)) + 64; }
+// (sink or tile, piece) work items: at most one that is not a full piece per sink with a long list and one per tile of
+// eight or more sinks; no kernel that fills the buffer cuts its lists shorter (each asserts it)
+static size_t item_count(const Ctx* c, size_t n) { return 2 * n + (size_t)(c->side[1].col_size / RP_ITEM_MIN) + 64; }
 
 static std::vector<float> padded_matrix(const float* src, int rows, int cols, int rows_p, int cols_p) {
     std::vector<float> m((size_t)rows_p * cols_p, 0.f);
@@ -241,6 +243,7 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         }
         tc_prepare();
         narrow_prepare();
+        sweep_prepare();
         max_prepare();
         CK(cudaMallocHost(&c->ctl_host, sizeof(Ctl)));
         memset(c->ctl_host, 0, sizeof(Ctl));
@@ -399,9 +402,6 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         }
         CK(dev_alloc(&c->moved_start, (size_t)4 * o.max_batch));
         CK(dev_alloc(&c->moved_cap, (size_t)4 * o.max_batch));
-        // (vertex, chunk) work items: a list of more than RP_ANEW_CHUNK entries gives at most 2 items per RP_ANEW_CHUNK of
-        // them, a row gathered anew by the fold one per RP_ANEW_CHUNK and one more; no kernel that fills the buffer cuts
-        // its lists shorter (each asserts it)
         CK(dev_alloc(&c->items, item_count(c, (size_t)N)));
         CK(dev_alloc(&c->coff, (size_t)N + 2, 0));   // degree prefix of a sender list
         CK(dev_alloc(&c->bitmap, (size_t)c->n_words + 256, 0));
@@ -443,12 +443,12 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
             const long long e0 = (long long)E;
             CK(cudaMemcpy(&c->ctl->num_edges, &e0, sizeof(e0), cudaMemcpyHostToDevice));
         }
+        c->stats.num_edges = E;
         if (c->n_local == 0) {   // (a partitioned context is bootstrapped layer by layer, in step with its peers)
             st = run_full(c);
             if (st) { memcpy(g_create_err, c->err, sizeof(g_create_err)); goto fail_keep_msg; }
         }
         c->stats.num_layers = L;
-        c->stats.num_edges = E;
         *out = reinterpret_cast<ripple_ctx*>(c);
         return RIPPLE_OK;
     }
@@ -514,22 +514,18 @@ static int enqueue_batch(Ctx* c, int nb, bool stamps) {
     }
     // one superstep per hop (Sec. 3.3.1): frontier, send + aggregate, compute + prepare
     for (int l = 1; l <= L && !rp_monotonic(c->agg) && !c->attention; ++l) {
-        // The push scatter walks the same out-lists as the frontier and marks the sinks itself; the
-        // gathering forms need the list A_l first, so the frontier walk is a pass of its own for them
-        // (decided per hop on the device for the rebuilding form).
-        const bool pull = c->pull_hop[l] != 0;
+        // What delivers the messages (push or sweep) marks their sinks itself.
         choose_direction(c, l);
-        frontier_mark(c, l, pull);
-        if (pull) frontier_compact(c, l);
+        frontier_mark(c, l);
         STAMP();
         scatter_layer(c, l, nb);
         // tiny batches on graphs whose frontier bitmap one block can sweep: A_l by one launch instead of two
-        const bool merged = tiny && !pull && c->n_words <= RP_TINY_WORDS;
-        // the next hop's senders are listed along with the frontier where this hop's are done with by then
-        const bool senders_too = l < L && !pull && !c->src_norm;
+        const bool merged = tiny && c->n_words <= RP_TINY_WORDS;
+        // the next hop's senders are listed along with the frontier
+        const bool senders_too = l < L && !c->src_norm;
         if (merged) frontier_compact_small(c, l, senders_too);
         else if (senders_too) frontier_compact_senders(c, l);
-        else if (!pull) frontier_compact(c, l);
+        else frontier_compact(c, l);
         fold_deltas(c, l);
         regather_layer(c, l);
         STAMP();
@@ -574,6 +570,10 @@ static void arm_rebuild(Ctx* c, int nb) {
                      (double)c->stats.senders[l - 1] * c->ws[l] * sizeof(float) <= 32.0 * (1 << 20) &&
                      c->stats.active_edges[l] >= 8 * c->stats.affected[l];
         c->pull_hop[l] = gather;
+        // The sweeping form goes into the chain beside the push where the hop may carry enough messages for it (the device
+        // then chooses by what it does carry).
+        c->sweep_armed[l] = !gather && c->scatter_mode == RIPPLE_SCATTER_AUTO && !rp_monotonic(c->agg) && !c->attention && c->n_local == 0 &&
+                            sweep_may_pay(c, l, no_history);
     }
 }
 
@@ -593,7 +593,7 @@ static int chain_size(const Ctx* c, int nb) {
 static uint64_t chain_key(const Ctx* c, int ng) {
     uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->few_rows_form ? 4 : 0);
     key = 2 * key + (c->front_one_block ? 1 : 0);
-    for (int l = 1; l <= c->L; ++l) key = 4 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0);
+    for (int l = 1; l <= c->L; ++l) key = 8 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0) + (c->sweep_armed[l] ? 4 : 0);
     for (int l = 0; l <= c->L; ++l) key = 2 * key + (c->tc_armed[l] ? 1 : 0);
     return key;
 }
@@ -786,7 +786,7 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
             s.affected[l] = h.nA[l];
             s.senders[l] = h.nC[l];
             s.active_edges[l] = l ? (int64_t)h.E[l] + h.n_rec : 0;
-            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l];
+            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l] == 1;   // (a sweep that the device chose delivers deltas like the push)
             s.in_edges[l] = (int64_t)h.pull_work[l];
             s.message_width[l] = l ? c->ws[l] : 0;
             s.rows_rebuilt[l] = h.n_rebuilt[l];

@@ -20,7 +20,8 @@
 #define RP_POOL_CLASSES 32          // block size classes of the adjacency store: class k holds blocks of 2^k entries
 #define RP_POOL_MIN_CLASS 3         // smallest block that is kept for reuse: 8 entries
 #define RP_POOL_LIST_CAP 16384      // blocks a class's free list can hold
-#define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold; the smallest of the chunks whose items share a buffer, which it sizes
+#define RP_ANEW_CHUNK 256           // in-list entries per work item of a row gathered anew by the fold
+#define RP_ITEM_MIN 64              // smallest piece into which long in-lists, and the lists of many sinks, are cut: it sizes the item buffer
 #define RP_TC_MIN_ROWS 1024         // row count from which a layer update takes the tensor-core form,
 #define RP_TC_MIN_COLS 113          // for outputs of RP_TC_MIN_COLS .. RP_TC_MAX_COLS columns (see tc_weights_build)
 #define RP_TC_MAX_COLS 256
@@ -71,9 +72,9 @@ struct Ctl {
     int ew_ticket[RP_MAXL + 1];       // elementwise update: next unassigned run of pieces
     int hub_ticket[RP_MAXL + 1];      // chunks of long in-lists: next unassigned work item
     int regather_ticket[RP_MAXL + 1]; // rebuilding form: next unassigned position of A_l
-    int gather_ticket[RP_MAXL + 1];   // gathering form of the delta scatter: next unassigned position of A_l
-    int gather_long_ticket[RP_MAXL + 1];  // ... and next unassigned work item of the long in-lists
-    int gather_items[RP_MAXL + 1];    // gathering form of the delta scatter: (sink, chunk) work items of the long in-lists
+    int gather_ticket[RP_MAXL + 1];   // sweeping form of the delta scatter: next unassigned run of vertices
+    int gather_long_ticket[RP_MAXL + 1];  // ... and next unassigned work item
+    int gather_items[RP_MAXL + 1];    // sweeping form of the delta scatter: (sink, piece) work items of the long in-lists
     long long num_edges;              // current edge count (kept across batches)
     int work_counter[8];              // dynamic work distribution tickets (reset by the consumer)
 };
@@ -196,6 +197,7 @@ struct Ctx {
     int rebuild_armed[RP_MAXL + 1];   // per hop: the rebuilding form is enqueued for this batch (see arm_rebuild)
     int tc_armed[RP_MAXL + 1];        // updates over the rows of A_l (or C_l) carry their tensor-core form in this batch
     int pull_hop[RP_MAXL + 1];        // per hop: the delta scatter of this batch gathers per sink instead of pushing (see arm_rebuild)
+    int sweep_armed[RP_MAXL + 1];     // per hop: the sweeping form is enqueued beside the push, the device chooses
     int gather_min_width;             // narrowest message row (floats) whose hop may gather (environment RIPPLE_GATHER_MIN_WIDTH)
     long long gather_min_messages;    // ... if the hop delivered at least this many messages in the batch before
     long long batches_done;
@@ -326,6 +328,23 @@ inline int occupancy(K kernel, int block) {
         else { CALL(8, 32); }                             \
     } while (0)
 
+// dispatch on the 16-byte pieces of a row per lane, and on whether entries carry a factor
+#define RP_PIECES_DISPATCH(ld, WGT, CALL)                                              \
+    do {                                                                               \
+        const int nv_ = div_up((ld), 128);                                             \
+        if (WGT) {                                                                     \
+            if (nv_ <= 1) { CALL(1, true); }                                           \
+            else if (nv_ <= 2) { CALL(2, true); }                                      \
+            else if (nv_ <= 4) { CALL(4, true); }                                      \
+            else { CALL(8, true); }                                                    \
+        } else {                                                                       \
+            if (nv_ <= 1) { CALL(1, false); }                                          \
+            else if (nv_ <= 2) { CALL(2, false); }                                     \
+            else if (nv_ <= 4) { CALL(4, false); }                                     \
+            else { CALL(8, false); }                                                   \
+        }                                                                              \
+    } while (0)
+
 // graph_store.cu
 cudaError_t graph_build(Ctx* c, const int32_t* src_dev, const int32_t* dst_dev, const float* w_dev, int64_t E,
                         double slack, int64_t pool_edges);
@@ -342,7 +361,7 @@ cudaError_t graph_export(Ctx* c, int64_t* rowptr, int32_t* col, float* weight, i
 void scan_degrees(Ctx* c, const int32_t* list, const int* n_dev, int n_host, const int32_t* deg,
                   int64_t* out, unsigned long long* total_dev);
 void frontier_seed_features(Ctx* c, int n);             // A_0 from the batch's feature updates
-void frontier_mark(Ctx* c, int l, bool walk);           // bitmap of A_l: (walk) edge-record sinks, A_{l-1} and Out(C_{l-1}); rebuilding hops: bottom-up
+void frontier_mark(Ctx* c, int l);                      // bitmap of A_l of a rebuilding hop, bottom-up
 void frontier_compact(Ctx* c, int l);                   // bitmap -> ascending list A_l
 void frontier_compact_senders(Ctx* c, int l);           // the same, and C_l = A_l with its degree prefix
 void frontier_compact_small(Ctx* c, int l, bool senders);   // likewise in one block (tiny batches, small graphs)
@@ -351,6 +370,8 @@ void senders_release(Ctx* c, int l);                    // clear posmap entries 
 
 // scatter.cu
 void spmm_full(Ctx* c, int l);                          // S^l for every vertex (bootstrap)
+void sweep_prepare();                                   // one-time kernel attributes (not allowed inside a stream capture)
+bool sweep_may_pay(const Ctx* c, int l, bool no_history);   // the sweeping form belongs into the chain of hop l
 void bitmap_to_list_from(Ctx* c, uint32_t* bitmap, int32_t* list, int* count_dev, unsigned long long* pull_work);
 // monotonic.cu (max aggregation, Sec. 3.4.2)
 void max_full(Ctx* c, int l);                           // bootstrap: cached maxima of every vertex

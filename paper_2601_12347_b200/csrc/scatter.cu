@@ -14,10 +14,9 @@
 // push: the out-edges of the senders are cut into equal chunks; a warp keeps the sender's delta
 //       row in registers and issues one 16-byte vector reduction per lane and edge (narrow rows:
 //       several edges per warp instruction).
-// pull: a warp per affected sink walks its in-list, keeps only sources that are senders
-//       (position map), sums their delta rows in registers and touches S_v once.
-#include "device_utils.cuh"
-#include "ripple_internal.cuh"
+// sweep: the in-lists of all vertices are read, sources that are senders kept (a filter, then the position map),
+//       their delta rows summed in registers, and a sink's accumulator touched once.
+#include "row_gather.cuh"
 
 #include <algorithm>
 
@@ -35,13 +34,6 @@ __device__ __forceinline__ void add4(float4& a, const float4& x, float c) {
 // bootstrap: S_v for every vertex by gathering over in-edges (Eq. 1)
 // LPR lanes hold one row (NV float4 slots each); a warp works on 32 / LPR in-neighbours at a time.
 // ---------------------------------------------------------------------------------------------
-// In-lists longer than this are cut into chunks handled by separate warps.  A warp gathers about
-// three neighbours per microsecond at 256 floats per row, so one 2048-neighbour row used to keep a
-// single warp busy for 0.7 ms, longer than everything else of a hop on the sparse graph.
-constexpr int SPMM_HUB_DEGREE = 256;
-constexpr int SPMM_HUB_CHUNK = 256;
-static_assert(SPMM_HUB_CHUNK >= RP_ANEW_CHUNK && SPMM_HUB_DEGREE >= RP_ANEW_CHUNK, "the item buffer is sized by RP_ANEW_CHUNK");
-
 // acc += sum over in-list entries [j_begin, j_end) of row v of c_u * M_u; LPR lanes hold one row
 // (NV float4 slots each), a warp works on 32 / LPR neighbours per step, several steps in flight.
 template <int NV, int LPR>
@@ -98,76 +90,145 @@ __device__ __forceinline__ void spmm_accumulate(float4 (&acc)[NV], const Side& i
     }
 }
 
-// One warp per vertex.  A vertex with a long in-list only zeroes its row here and queues
-// (vertex, chunk) work items for k_spmm_hubs, so that no single warp walks thousands of neighbours.
-template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
-k_spmm_pull(int N, Side in, const int32_t* __restrict__ deg_out, int src_norm,
-            const float* __restrict__ M, int ld, float* __restrict__ S, int2* items, int* n_items, int* ticket) {
-    pdl_enter();
-    const int lane = lane_id(), nq = ld >> 2;
-    const int sub = lane / LPR, ql = lane % LPR;
-    // vertices are handed out in runs of eight by ticket: in-lists differ in length
-    for (;;) {
-        int v0 = 0;
-        if (lane == 0) v0 = atomicAdd(ticket, 8);
-        v0 = __shfl_sync(FULL, v0, 0);
-        if (v0 >= N) break;
-    for (int v = v0; v < min(v0 + 8, N); ++v) {
-        const int deg = in.deg[v];
-        float4 acc[NV];
+// S_v = sum over In(v) of c_u M_u for a list of sinks (or for every vertex): the bootstrap's aggregation and the
+// rebuilding form of a hop.  A warp takes the lists of 32 sinks at a time, laid end to end (see row_gather.cuh), zeroes
+// their rows and adds to them; a list too long for that is queued in pieces for the kernel below, a warp per piece.
+// All 124 M in-edges of the graph of 2.4 M vertices, 48 floats per row: 2.99 -> 2.24 to 2.46 ms (a warp per sink and a trip to
+// memory for every step of a list -> this); 100 floats: 4.9 -> 4.3 to 4.75 ms.
+struct RowSums {
+    Side in;
+    const int32_t* list;        // sinks (null: every vertex)
+    const int* n_dev;           // their number on the device (null: n_host)
+    int n_host;
+    const int32_t* deg_out;
+    int src_norm;
+    const float* M;
+    int ld;
+    float* S;
+    int2* items;                // (sink, piece) of the long lists
+    int* n_items;
+    int* ticket;
+    int take;                   // sinks per tile
+    int long_list, item, piece; // lists of more than long_list entries go in pieces of `item`, tiles of more than `piece` in such
+    float* budget;              // a row gathered anew has spent nothing
+};
+
+template <int NV, bool WGT, typename RUN>
+__device__ __forceinline__ void sum_rows(const RowLanes& g, const RUN& run, const RowSums& a, const RowQueue<WGT>& q, float4 (&acc)[NV], int begin = 0) {
+    const int lane = lane_id();
+    IdWindow<WGT, RUN> nx;
+    nx.request(run, a.in, begin);
+    for (int f0 = begin; f0 < run.total; f0 += RG_WINDOW) {
+        const int n = min(RG_WINDOW, run.total - f0);
+        int last = -1;
+        __syncwarp();   // the window before has been walked
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (deg > SPMM_HUB_DEGREE) {
-            const int nch = (deg + SPMM_HUB_CHUNK - 1) / SPMM_HUB_CHUNK;
-            int first = 0;
-            if (lane == 0) first = atomicAdd(n_items, nch);
-            first = __shfl_sync(FULL, first, 0);
-            for (int ch = lane; ch < nch; ch += 32) items[first + ch] = make_int2(v, ch);
-        } else {
-            spmm_accumulate<NV, LPR>(acc, in, v, 0, deg, deg_out, src_norm, M, ld);
+        for (int k = 0; k < 4; ++k) {
+            const int u = nx.u[k], v = nx.sink(k), at = 32 * k + lane;
+            const int flag = RUN::ONE ? 0 : rg_new_sink(__ballot_sync(FULL, u >= 0), v, last);
+            if (u >= 0) q.put(at, u | flag, v, WGT && a.src_norm ? coef_from_degree(a.deg_out[u]) : nx.weight(k));
         }
-        if (sub == 0) {
-            float4* dst = reinterpret_cast<float4*>(S + (size_t)v * ld);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                int q = ql + LPR * k;
-                if (q < nq) dst[q] = acc[k];
-            }
-        }
-    }
+        __syncwarp();
+        nx.request(run, a.in, f0 + RG_WINDOW);
+        rg_walk<NV, WGT, RUN::ONE>(g, q, n, a.M, a.ld, a.S, acc);
     }
 }
 
-// The chunks of the long in-lists, one warp per 256-entry chunk; chunk sums are added to the row,
-// which the kernel that queued the chunks has zeroed.
-template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
-k_spmm_hubs(Side in, const int32_t* __restrict__ deg_out, int src_norm, const float* __restrict__ M, int ld,
-            float* S, const int2* __restrict__ items, const int* __restrict__ n_items, int* ticket) {
+constexpr int SUM_T = 256;
+
+template <int NV, bool WGT>
+__global__ void __launch_bounds__(SUM_T, NV == 1 ? 3 : 1)
+k_sum_rows(const Ctl* ctl, int l, int only_if_rebuilding, const __grid_constant__ RowSums a) {
     pdl_enter();
-    const int lane = lane_id(), nq = ld >> 2;
-    const int sub = lane / LPR, ql = lane % LPR;
-    const int n = *n_items;
-    if (n == 0) return;
-    TicketWalk walk(ticket, n, 1, 1);
-    for (; walk.has(); walk.advance()) {
-        const int2 w = items[walk.at];
-        walk.take();
-        const int deg = in.deg[w.x];
-        float4 acc[NV];
+    if (only_if_rebuilding && (ctl->abort || !ctl->regather[l])) return;
+    __shared__ __align__(16) char s_q[SUM_T / 32][RowQueue<WGT>::bytes(RG_WINDOW)];
+    const int n = a.n_dev ? *a.n_dev : a.n_host, lane = lane_id();
+    const RowQueue<WGT> q(s_q[threadIdx.x >> 5], RG_WINDOW);
+    const RowLanes g(a.ld);
+    float4 acc[NV];
+    rg_zero<NV>(acc);
+    TileDeal deal(a.take == 32 ? a.ticket : nullptr);
+    for (int tile = deal.first();; tile = deal.next()) {
+        const long long i0 = (long long)a.take * tile;
+        if (i0 >= n) break;
+        const int cnt = (int)min((long long)a.take, n - i0);
+        const TileLists t(a.in, a.list, i0, cnt);
+        if (a.budget && lane < cnt) a.budget[t.v] = 0.f;
+        TileRun run = t.run(a.long_list);
+        for (int r0 = 0; r0 < cnt; r0 += g.G) {   // the rows start from zero
+            const int r = r0 + g.sub, row = __shfl_sync(FULL, t.v, r & 31);
+            if (g.sub < g.G && r < cnt) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        spmm_accumulate<NV, LPR>(acc, in, w.x, w.y * SPMM_HUB_CHUNK, min(deg, (w.y + 1) * SPMM_HUB_CHUNK), deg_out,
-                                 src_norm, M, ld);
-        if (sub == 0) {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                int q = ql + LPR * k;
-                if (q < nq) red_add_v4(S + (size_t)w.x * ld + 4 * q, acc[k]);
+                for (int k = 0; k < NV; ++k) {
+                    const int p = g.ql + 32 * k;
+                    if (p < g.nq) *reinterpret_cast<float4*>(a.S + (size_t)row * a.ld + 4 * p) = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
             }
         }
+        rg_queue_rest(t, tile, run.total, a.long_list, a.item, a.piece, a.items, a.n_items);
+        run.total = min(run.total, a.piece);
+        sum_rows<NV, WGT>(g, run, a, q, acc);
     }
+}
+
+template <int NV, bool WGT>
+__global__ void __launch_bounds__(SUM_T, NV == 1 ? 3 : 1)
+k_sum_rows_long(const Ctl* ctl, int l, int only_if_rebuilding, const __grid_constant__ RowSums a, int* ticket) {
+    pdl_enter();
+    if (only_if_rebuilding && (ctl->abort || !ctl->regather[l])) return;
+    __shared__ __align__(16) char s_q[SUM_T / 32][RowQueue<WGT>::bytes(RG_WINDOW)];
+    const int n = *a.n_items;
+    if (n == 0) return;
+    const RowQueue<WGT> q(s_q[threadIdx.x >> 5], RG_WINDOW);
+    const RowLanes g(a.ld);
+    float4 acc[NV];
+    rg_zero<NV>(acc);
+    TicketWalk walk(ticket, n, 1, 4);
+    for (; walk.has(); walk.advance()) {
+        const int from = (int)walk.at, to = min(n, from + walk.chunk);
+        walk.take();
+        for (int it = from; it < to; ++it) {
+        const int2 w = a.items[it];
+        if (w.x < 0) {
+            const int tile = -1 - w.x;
+            const long long i0 = (long long)a.take * tile;
+            TileRun run = TileLists(a.in, a.list, i0, (int)min((long long)a.take, (a.n_dev ? *a.n_dev : a.n_host) - i0)).run(a.long_list);
+            run.total = min(run.total, (w.y + 1) * a.piece);
+            sum_rows<NV, WGT>(g, run, a, q, acc, w.y * a.piece);
+            continue;
+        }
+        const int deg = a.in.deg[w.x];
+        const ListRun run(w.x, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item));
+        sum_rows<NV, WGT>(g, run, a, q, acc);
+        rg_finish_one<NV>(g, a.S + (size_t)w.x * a.ld, acc);
+        }
+    }
+}
+
+static_assert(RP_ANEW_CHUNK >= RP_ITEM_MIN, "the item buffer is sized by it");
+
+// How the lists are cut: pieces of which every warp of the device gets a few, so that none is still at one when the others
+// have run out.
+template <typename A>
+static void cut_lists(const Ctx* c, A& a) {
+    const long long per_warp = (long long)c->stats.num_edges / (c->n_sm * 64);
+    a.item = RP_ITEM_MIN;
+    while (a.item < 1024 && 2 * a.item <= per_warp) a.item *= 2;
+    a.piece = std::min(a.item, 512);
+    a.long_list = std::min(a.item, 256);
+    a.take = c->N >= 32 * 64 * c->n_sm ? 32 : 8;   // (32 sinks from two tiles per warp)
+}
+
+static void launch_row_sums(Ctx* c, int l, RowSums a, bool only_if_rebuilding) {
+    cut_lists(c, a);
+    const bool wgt = c->weighted || a.src_norm;
+#define SUMS(NV, WGT)                                                                                                     \
+    do {                                                                                                                  \
+        RP_LAUNCH(c, (k_sum_rows<NV, WGT>), RP_RESIDENT(c, (k_sum_rows<NV, WGT>), SUM_T), SUM_T, 0, (const Ctl*)c->ctl, l, (int)only_if_rebuilding, a); \
+        RP_LAUNCH(c, (k_sum_rows_long<NV, WGT>), RP_RESIDENT(c, (k_sum_rows_long<NV, WGT>), SUM_T), SUM_T, 0, (const Ctl*)c->ctl, l, (int)only_if_rebuilding, a, &c->ctl->hub_ticket[l]); \
+    } while (0)
+    RP_PIECES_DISPATCH(a.ld, wgt, SUMS);
+#undef SUMS
 }
 
 // The few rows that the fold sends back to be gathered anew.  The chain waits for the longest chunk, so a whole block takes
@@ -207,25 +268,25 @@ k_spmm_anew(Side in, const int32_t* __restrict__ deg_out, int src_norm, const fl
     }
 }
 
+static RowSums row_sums(Ctx* c, int l) {
+    RowSums a{};
+    a.in = c->side[1];
+    a.deg_out = c->side[0].deg;
+    a.src_norm = c->src_norm;
+    a.M = c->pre[l] ? c->P[l] : c->H[l - 1];
+    a.ld = c->ws[l];
+    a.S = c->S[l];
+    a.items = c->items;
+    a.n_items = &c->ctl->work_counter[(l - 1) & 7];
+    a.ticket = &c->ctl->regather_ticket[l];
+    return a;
+}
+
 void spmm_full(Ctx* c, int l) {
-    const int ld = c->ws[l];
-    const float* M = c->H[l - 1];
-    if (c->pre[l]) {
-        project_full(c, l);
-        M = c->P[l];
-    }
-    const int grid = c->n_sm * 16, T = 256;
-    int2* items = c->items;
-    int* n_items = &c->ctl->work_counter[(l - 1) & 7];
-#define SPMM(NV, LPR)                                                                                              \
-    do {                                                                                                           \
-        RP_LAUNCH(c, (k_spmm_pull<NV, LPR>), grid, T, 0, c->N, c->side[1], c->side[0].deg, (int)c->src_norm, M,   \
-                  ld, c->S[l], items, n_items, &c->ctl->regather_ticket[l]);                                      \
-        RP_LAUNCH(c, (k_spmm_hubs<NV, LPR>), grid, T, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld,     \
-                  c->S[l], items, n_items, &c->ctl->hub_ticket[l]);                                                \
-    } while (0)
-    RP_WIDTH_DISPATCH(ld, SPMM);
-#undef SPMM
+    if (c->pre[l]) project_full(c, l);
+    RowSums a = row_sums(c, l);
+    a.n_host = c->N;
+    launch_row_sums(c, l, a, false);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -477,232 +538,281 @@ k_scatter_push_bulk(Ctl* ctl, int l, const int32_t* __restrict__ senders, const 
 }
 
 // ---------------------------------------------------------------------------------------------
-// gathering form of the delta scatter: per affected sink, the delta rows of the senders among its
-// in-neighbours are summed in registers and reach the accumulator row as ONE addition.  The sender
-// delta rows are few (they stay in L2) and are read with plain loads; no
-// accumulator row is touched more than once.  It pays where a message is wide: 256-float
-// messages cost the push one kilobyte of read-modify-write each in the L2 slices and evict each
-// other's accumulator rows in between.
+// sweeping form of the delta scatter: every in-list is read once and the delta rows of the senders in it are summed in
+// registers, so that a sink's accumulator row takes one addition where the push makes one per message.
 //
-// A warp examines GATHER_WINDOW in-list entries at a time (four per lane, their position-map
-// lookups in flight together), compacts the hits into shared memory and then gathers them like
-// the bootstrap gather does: LPR lanes per row, 32 / LPR rows per step, several steps in flight.
+// Whether an id is a sender's is first asked of a filter in shared memory, which every block fills from the sender list:
+// one bit per vertex on graphs of up to 2^20 of them, else one of 2^20 bits per id by a multiplicative hash; the position
+// map, one trip to L2, is asked about the few that pass.  The delta rows are few and stay in L2.
+//
+// What bounds it: the requests that an SM's L1 takes (a bit of the filter per entry, a word of the position map per row,
+// two or three lines per row) and the trips to memory of a window, at half of the issue slots; 4.5 ps per entry without a row.
 // ---------------------------------------------------------------------------------------------
-constexpr int GATHER_WINDOW = 128;
-constexpr int GATHER_LONG = 512;     // longer in-lists are cut into work items of GATHER_ITEM entries
-constexpr int GATHER_ITEM = 256;
-static_assert(GATHER_ITEM >= RP_ANEW_CHUNK && GATHER_LONG >= RP_ANEW_CHUNK, "the item buffer is sized by RP_ANEW_CHUNK");
-constexpr int GATHER_TAKE = 8;       // sinks per ticket
+constexpr int SWEEP_BITS = 19;
+// one block per SM: threads by the registers that the rows on their way take
+template <int NV>
+__host__ __device__ constexpr int sweep_threads() { return NV == 1 ? 1024 : NV == 2 ? 768 : 512; }
 
-template <int NV, int LPR>
-__device__ __forceinline__ bool gather_accumulate(float4 (&acc)[NV], const Side& in, int v, int j_begin, int j_end,
-                                                  const int32_t* __restrict__ posmap, const float* __restrict__ D,
-                                                  int ld, int2* hits) {
-    const int lane = lane_id(), nq = ld >> 2;
-    constexpr int EPI = 32 / LPR;
-    constexpr int UNR = NV <= 2 ? 4 : 2;
-    constexpr int PER_LANE = GATHER_WINDOW / 32;
-    const int sub = lane / LPR, ql = lane % LPR;
-    const int64_t base = in.start[v];
+struct Sweep {
+    Side in;
+    const int32_t* senders;
+    const int32_t* posmap;
+    const float* D;
+    int ld;
+    float* dS;
+    uint32_t* bitmap;
+    int2* items;
+    int N, filter_words;
+    int take, long_list, item, piece;   // see RowSums
+};
+
+struct SenderFilter {
+    const uint32_t* bits;
+    bool on;
+    uint32_t mul;
+    int shift;               // the word of an id: (id * mul) >> shift; its bit: the id's lowest five
+    __device__ __forceinline__ uint32_t hit(int id) const { return bits[(uint32_t)id * mul >> shift] >> (id & 31) & 1u; }
+    // (filling the filter costs a cycle per sender, a look-up that it spares 0.005 of one; and hashed it lets a quarter of
+    // the others through at 2^17 senders)
+    __device__ __forceinline__ SenderFilter(const Ctl* ctl, int l, const Sweep& a, uint32_t* smem) : bits(smem) {
+        const int nC = ctl->nC[l - 1];
+        const bool exact = a.N <= 1 << SWEEP_BITS;
+        mul = exact ? 1u : 2654435761u;
+        shift = exact ? 5 : 32 - (SWEEP_BITS - 5);
+        on = 192ll * nC <= ctl->num_edges && (exact || nC <= 1 << (SWEEP_BITS - 2));
+        if (!on) return;
+        for (int i = threadIdx.x; i < a.filter_words; i += blockDim.x) smem[i] = 0u;
+        __syncthreads();
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nC; i += blockDim.x) {
+            const int id = a.senders[i];
+            atomicOr(&smem[(uint32_t)id * mul >> shift], 1u << (id & 31));
+        }
+        __syncthreads();
+    }
+};
+
+// The queue's first `held` ids become rows of D by the position map, which has the last word: what it does not know leaves
+// the queue.  Returns how many stay; `reached` takes, per lane, bits of the sinks reached.
+template <bool WGT, bool ONE>
+__device__ __forceinline__ int sweep_resolve(const RowQueue<WGT>& q, int held, const int32_t* __restrict__ posmap, unsigned& reached) {
+    const int lane = lane_id();
     const unsigned lt = (1u << lane) - 1u;
-    bool any = false;
-    for (int j0 = j_begin; j0 < j_end; j0 += GATHER_WINDOW) {
-        int u[PER_LANE], p[PER_LANE];
-        float w[PER_LANE];
+    int p[RG_CAP / 32];
 #pragma unroll
-        for (int k = 0; k < PER_LANE; ++k) {
-            const int j = j0 + 32 * k + lane;
-            u[k] = j < j_end ? in.col[base + j] : -1;
-            w[k] = (in.w && j < j_end) ? in.w[base + j] : 1.0f;
+    for (int k = 0; k < RG_CAP / 32; ++k) p[k] = 32 * k + lane < held ? posmap[q.row[32 * k + lane]] : -1;
+    int n = 0, last = -1;
+#pragma unroll
+    for (int k = 0; k < RG_CAP / 32; ++k) {
+        if (32 * k >= held) break;
+        const unsigned m = __ballot_sync(FULL, p[k] >= 0);
+        if (m == 0) continue;
+        const int v = ONE ? 0 : q.sink[32 * k + lane];
+        const float w = WGT ? q.w[32 * k + lane] : 1.0f;
+        const int flag = ONE ? 0 : rg_new_sink(m, v, last), at = n + __popc(m & lt);
+        if (WGT || !ONE) __syncwarp();
+        if (p[k] >= 0) {
+            q.row[at] = p[k] | flag;
+            if (!ONE) q.sink[at] = v;
+            if (WGT) q.w[at] = w;
+            reached |= ONE ? 1u : 1u << (v & 31);
         }
+        n += __popc(m);
+    }
+    __syncwarp();
+    return n;
+}
+
+// Adds the delta rows of the senders in a piece of one list to acc; returns, per lane, whether there were any.  The ids are
+// read four to a lane from the aligned place before the piece, two windows ahead.
+template <int NV, bool WGT>
+__device__ __forceinline__ unsigned sweep_list(const RowLanes& g, int64_t first, int n, const Sweep& a, const SenderFilter& filter,
+                                               const RowQueue<WGT>& q, float4 (&acc)[NV]) {
+    const int lane = lane_id(), lead = (int)(first & 3), total = lead + n;
+    const int32_t* const from = a.in.col + (first - lead);
+    auto ids = [&](int f) { return f < total ? *reinterpret_cast<const int4*>(from + f) : make_int4(0, 0, 0, 0); };   // (a list's last piece may reach into its slack)
+    unsigned reached = 0;
+    int held = 0;
+    int4 x0 = ids(4 * lane), x1 = ids(RG_WINDOW + 4 * lane);
+    for (int f0 = 0; f0 < total; f0 += RG_WINDOW) {
+        int u[4] = {x0.x, x0.y, x0.z, x0.w};
+        x0 = x1;
+        x1 = ids(f0 + 2 * RG_WINDOW + 4 * lane);
+        unsigned m = 0xfu;
+        if (f0 < lead || f0 + RG_WINDOW > total) {
 #pragma unroll
-        for (int k = 0; k < PER_LANE; ++k) p[k] = u[k] >= 0 ? posmap[u[k]] : -1;
-        int cnt = 0;
-        __syncwarp();   // the hits of the window before have all been read
-#pragma unroll
-        for (int k = 0; k < PER_LANE; ++k) {
-            const unsigned m = __ballot_sync(FULL, p[k] >= 0);
-            if (p[k] >= 0) hits[cnt + __popc(m & lt)] = make_int2(p[k], __float_as_int(w[k]));
-            cnt += __popc(m);
+            for (int k = 0; k < 4; ++k) {
+                const int f = f0 + 4 * lane + k;
+                if (f < lead || f >= total) {
+                    u[k] = 0;
+                    m &= ~(1u << k);
+                }
+            }
         }
+        if (filter.on) m &= filter.hit(u[0]) | filter.hit(u[1]) << 1 | filter.hit(u[2]) << 2 | filter.hit(u[3]) << 3;
+        if (__any_sync(FULL, m)) {
+            const int c = __popc(m), inc = warp_inclusive_scan(c);
+            int at = held + inc - c;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (m >> k & 1u) {
+                    q.row[at] = u[k];
+                    if (WGT) q.w[at] = a.in.w ? a.in.w[first - lead + f0 + 4 * lane + k] : 1.0f;
+                    ++at;
+                }
+            held += __shfl_sync(FULL, inc, 31);
+        }
+        if (held == 0 || (held < RG_DRAIN && f0 + RG_WINDOW < total)) continue;
         __syncwarp();
-        if (cnt == 0) continue;
-        any = true;
-        for (int j = 0; j < cnt; j += UNR * EPI) {
-            int pj[UNR];
-            float a[UNR];
-            float4 x[UNR][NV];
-#pragma unroll
-            for (int t = 0; t < UNR; ++t) {
-                const int jj = j + t * EPI + sub;
-                pj[t] = -1;
-                a[t] = 0.f;
-                if (jj < cnt) {
-                    const int2 h = hits[jj];
-                    pj[t] = h.x;
-                    a[t] = __int_as_float(h.y);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < UNR; ++t) {
-                const float4* row = reinterpret_cast<const float4*>(D + (size_t)max(pj[t], 0) * ld);
-#pragma unroll
-                for (int k = 0; k < NV; ++k) {
-                    const int q = ql + LPR * k;
-                    x[t][k] = (pj[t] >= 0 && q < nq) ? __ldg(row + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < UNR; ++t)
-#pragma unroll
-                for (int k = 0; k < NV; ++k) add4(acc[k], x[t][k], a[t]);
-        }
+        const int rows = sweep_resolve<WGT, true>(q, held, a.posmap, reached);
+        if (rows) rg_walk<NV, WGT, true>(g, q, rows, a.D, a.ld, a.dS, acc);
+        __syncwarp();
+        held = 0;
     }
-    if (any) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-#pragma unroll
-            for (int o = LPR; o < 32; o <<= 1) {
-                acc[k].x += __shfl_xor_sync(FULL, acc[k].x, o);
-                acc[k].y += __shfl_xor_sync(FULL, acc[k].y, o);
-                acc[k].z += __shfl_xor_sync(FULL, acc[k].z, o);
-                acc[k].w += __shfl_xor_sync(FULL, acc[k].w, o);
-            }
-        }
-    }
-    return any;
+    return reached;
 }
 
-// One warp per affected sink; a sink with a long in-list only queues (sink, chunk) work items.
-template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
-k_scatter_gather(Ctl* ctl, int l, const int32_t* __restrict__ A, Side in, const int32_t* __restrict__ posmap,
-                 const float* __restrict__ D, int ld, float* dS, int2* items) {
-    pdl_enter();
-    __shared__ int2 s_hits[8][GATHER_WINDOW];
-    if (ctl->abort || !ctl->pull[l] || ctl->regather[l]) return;
-    const int nA = ctl->nA[l];
-    const int lane = lane_id(), nq = ld >> 2;
-    const int sub = lane / LPR, ql = lane % LPR;
-    int2* hits = s_hits[threadIdx.x >> 5];
-    // sinks are handed out in runs of GATHER_TAKE by ticket: in-lists differ in length by orders of magnitude,
-    // and the grid need not match the number of resident blocks
-    for (;;) {
-        int i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&ctl->gather_ticket[l], GATHER_TAKE);
-        i0 = __shfl_sync(FULL, i0, 0);
-        if (i0 >= nA) break;
-    for (int i = i0; i < min(i0 + GATHER_TAKE, nA); ++i) {
-        const int v = A[i];
-        const int deg = in.deg[v];
-        if (deg > GATHER_LONG) {
-            const int nch = (deg + GATHER_ITEM - 1) / GATHER_ITEM;
-            int first = 0;
-            if (lane == 0) first = atomicAdd(&ctl->gather_items[l], nch);
-            first = __shfl_sync(FULL, first, 0);
-            for (int ch = lane; ch < nch; ch += 32) items[first + ch] = make_int2(v, ch);
-            continue;
-        }
-        float4 acc[NV];
+// Adds the delta rows of the senders in a tile's run to their sinks' accumulator rows; returns, per lane, bits of the sinks
+// reached.
+template <int NV, bool WGT>
+__device__ __forceinline__ unsigned sweep_tile(const RowLanes& g, const TileRun& run, const Sweep& a, const SenderFilter& filter,
+                                               const RowQueue<WGT>& q, float4 (&acc)[NV], int begin) {
+    const int lane = lane_id();
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned reached = 0;
+    int held = 0;
+    IdWindow<WGT, TileRun> nx;
+    nx.request(run, a.in, begin);
+    for (int f0 = begin; f0 < run.total; f0 += RG_WINDOW) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!gather_accumulate<NV, LPR>(acc, in, v, 0, deg, posmap, D, ld, hits)) continue;
-        if (sub == 0) {
-            // the accumulator is zero outside a batch and this is the hop's first kernel to touch the row
-            // (edge records are added after it): a plain store
-            float4* dst = reinterpret_cast<float4*>(dS + (size_t)v * ld);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                const int q = ql + LPR * k;
-                if (q < nq) dst[q] = acc[k];
-            }
+        for (int k = 0; k < 4; ++k) {
+            const bool in = nx.u[k] >= 0 && (!filter.on || filter.hit(max(nx.u[k], 0)));
+            const unsigned m = __ballot_sync(FULL, in);
+            if (in) q.put(held + __popc(m & lt), nx.u[k], nx.sink(k), nx.weight(k));
+            held += __popc(m);
         }
+        nx.request(run, a.in, f0 + RG_WINDOW);
+        if (held == 0 || (held < RG_DRAIN && f0 + RG_WINDOW < run.total)) continue;
+        __syncwarp();
+        const int rows = sweep_resolve<WGT, false>(q, held, a.posmap, reached);
+        if (rows) rg_walk<NV, WGT, false>(g, q, rows, a.D, a.ld, a.dS, acc);
+        __syncwarp();
+        held = 0;
     }
+    return reached;
+}
+
+// Steps of `take` consecutive vertices per warp; longer lists are queued for the kernel below.
+template <int NV, bool WGT>
+__global__ void __launch_bounds__(sweep_threads<NV>(), 1)
+k_sweep(Ctl* ctl, int l, const __grid_constant__ Sweep a, const RecMsgs recs) {
+    pdl_enter();
+    if (ctl->abort || !ctl->pull[l] || ctl->regather[l]) return;
+    extern __shared__ __align__(16) uint32_t s_dyn[];
+    d_scatter_records(ctl, recs, a.D, a.ld, a.dS);
+    if (ctl->nC[l - 1] == 0) return;
+    const SenderFilter filter(ctl, l, a, s_dyn);
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const RowQueue<WGT> q(reinterpret_cast<char*>(s_dyn + a.filter_words) + warp * RowQueue<WGT>::bytes(RG_CAP), RG_CAP);
+    const RowLanes g(a.ld);
+    float4 acc[NV];
+    rg_zero<NV>(acc);
+    TileDeal deal(a.take == 32 ? &ctl->gather_ticket[l] : nullptr);
+    for (int tile = deal.first();; tile = deal.next()) {
+        const long long v0 = (long long)a.take * tile;
+        if (v0 >= a.N) break;
+        const TileLists t(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0));
+        TileRun run = t.run(a.long_list);
+        rg_queue_rest(t, tile, run.total, a.long_list, a.item, a.piece, a.items, &ctl->gather_items[l]);
+        run.total = min(run.total, a.piece);
+        const unsigned reached = __reduce_or_sync(FULL, sweep_tile<NV, WGT>(g, run, a, filter, q, acc, 0));
+        if (reached && lane == 0) atomicOr(&a.bitmap[v0 >> 5], reached);   // (a tile lies within a word)
     }
 }
 
-// the chunks of the long in-lists: several warps add into the same accumulator row
-template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
-k_scatter_gather_long(Ctl* ctl, int l, Side in, const int32_t* __restrict__ posmap, const float* __restrict__ D, int ld,
-                      float* dS, const int2* __restrict__ items) {
+template <int NV, bool WGT>
+__global__ void __launch_bounds__(sweep_threads<NV>(), 1)
+k_sweep_long(Ctl* ctl, int l, const __grid_constant__ Sweep a) {
     pdl_enter();
-    __shared__ int2 s_hits[8][GATHER_WINDOW];
     if (ctl->abort || !ctl->pull[l] || ctl->regather[l]) return;
+    extern __shared__ __align__(16) uint32_t s_dyn[];
     const int n = ctl->gather_items[l];
-    const int lane = lane_id(), nq = ld >> 2;
-    const int sub = lane / LPR, ql = lane % LPR;
-    int2* hits = s_hits[threadIdx.x >> 5];
-    // items by ticket: they are equally long, but the senders among their entries are not equally many
-    for (;;) {
-        int it = 0;
-        if (lane == 0) it = atomicAdd(&ctl->gather_long_ticket[l], 1);
-        it = __shfl_sync(FULL, it, 0);
-        if (it >= n) break;
-        const int2 w = items[it];
-        const int deg = in.deg[w.x];
-        float4 acc[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!gather_accumulate<NV, LPR>(acc, in, w.x, w.y * GATHER_ITEM, min(deg, (w.y + 1) * GATHER_ITEM), posmap, D, ld,
-                                        hits))
+    if (n == 0) return;
+    const SenderFilter filter(ctl, l, a, s_dyn);
+    const int warp = threadIdx.x >> 5;
+    const RowQueue<WGT> q(reinterpret_cast<char*>(s_dyn + a.filter_words) + warp * RowQueue<WGT>::bytes(RG_CAP), RG_CAP);
+    const RowLanes g(a.ld);
+    float4 acc[NV];
+    rg_zero<NV>(acc);
+    TicketWalk walk(&ctl->gather_long_ticket[l], n, 1, 4);
+    for (; walk.has(); walk.advance()) {
+        const int from = (int)walk.at, to = min(n, from + walk.chunk);
+        walk.take();
+        for (int it = from; it < to; ++it) {
+        const int2 w = a.items[it];
+        if (w.x < 0) {
+            const long long v0 = (long long)a.take * (-1 - w.x);
+            TileRun run = TileLists(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0)).run(a.long_list);
+            run.total = min(run.total, (w.y + 1) * a.piece);
+            const unsigned sinks = __reduce_or_sync(FULL, sweep_tile<NV, WGT>(g, run, a, filter, q, acc, w.y * a.piece));
+            if (sinks && lane_id() == 0) atomicOr(&a.bitmap[v0 >> 5], sinks);
             continue;
-        if (sub == 0) {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                const int q = ql + LPR * k;
-                if (q < nq) red_add_v4(dS + (size_t)w.x * ld + 4 * q, acc[k]);
-            }
+        }
+        const int deg = a.in.deg[w.x];
+        const bool reached = __any_sync(FULL, sweep_list<NV, WGT>(g, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item), a, filter, q, acc));
+        if (!reached) continue;
+        rg_finish_one<NV>(g, a.dS + (size_t)w.x * a.ld, acc);
+        const uint32_t m = 1u << (w.x & 31);
+        if (lane_id() == 0 && !(a.bitmap[w.x >> 5] & m)) atomicOr(&a.bitmap[w.x >> 5], m);
         }
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// rebuilding hop (scoped recomputation of the aggregates, the "RC" strategy of Sec. 3.2 applied to
-// one hop): S_v of every affected vertex is gathered again over In_new(v) from the current rows
-// ---------------------------------------------------------------------------------------------
-template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
-k_regather(Ctl* ctl, int l, const int32_t* __restrict__ A, Side in, const int32_t* __restrict__ deg_out,
-           int src_norm, const float* __restrict__ M, int ld, float* __restrict__ S, int2* items,
-           int* n_items, float* budget) {
-    pdl_enter();
-    if (ctl->abort || !ctl->regather[l]) return;
-    const int nA = ctl->nA[l];
-    const int lane = lane_id(), nq = ld >> 2;
-    const int sub = lane / LPR, ql = lane % LPR;
-    // rows are handed out in runs of eight by ticket (the grid need not match the number of resident blocks)
-    for (;;) {
-        int i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&ctl->regather_ticket[l], 8);
-        i0 = __shfl_sync(FULL, i0, 0);
-        if (i0 >= nA) break;
-    for (int i = i0; i < min(i0 + 8, nA); ++i) {
-        const int v = A[i];
-        const int deg = in.deg[v];
-        float4 acc[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (deg > SPMM_HUB_DEGREE) {   // zero the row here, chunks are added by k_spmm_hubs
-            const int nch = (deg + SPMM_HUB_CHUNK - 1) / SPMM_HUB_CHUNK;
-            int first = 0;
-            if (lane == 0) first = atomicAdd(n_items, nch);
-            first = __shfl_sync(FULL, first, 0);
-            for (int ch = lane; ch < nch; ch += 32) items[first + ch] = make_int2(v, ch);
-        } else {
-            spmm_accumulate<NV, LPR>(acc, in, v, 0, deg, deg_out, src_norm, M, ld);
-        }
-        if (sub == 0) {
-            float4* dst = reinterpret_cast<float4*>(S + (size_t)v * ld);
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                int q = ql + LPR * k;
-                if (q < nq) dst[q] = acc[k];
-            }
-        }
-        if (budget && lane == 0) budget[v] = 0.f;   // a freshly gathered row has spent nothing
-    }
-    }
+template <int NV>
+static size_t sweep_smem(int filter_words, bool wgt) {
+    return sizeof(uint32_t) * (size_t)filter_words + (size_t)(sweep_threads<NV>() / 32) * (size_t)(wgt ? RowQueue<true>::bytes(RG_CAP) : RowQueue<false>::bytes(RG_CAP));
+}
+
+void sweep_prepare() {
+#define PREP(NV, WGT)                                                                                                                              \
+    do {                                                                                                                                           \
+        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));        \
+        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));   \
+    } while (0)
+    PREP(1, false); PREP(2, false); PREP(4, false); PREP(8, false);
+    PREP(1, true); PREP(2, true); PREP(4, true); PREP(8, true);
+#undef PREP
+    // the rows that many lists name are served by L1, so these kernels ask for as much of it as their queues leave
+#define PREP(NV, WGT)                                                                                                            \
+    do {                                                                                                                         \
+        cudaFuncSetAttribute(k_sum_rows<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);                         \
+        cudaFuncSetAttribute(k_sum_rows_long<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);                    \
+    } while (0)
+    PREP(1, false); PREP(2, false); PREP(4, false); PREP(8, false);
+    PREP(1, true); PREP(2, true); PREP(4, true); PREP(8, true);
+#undef PREP
+}
+
+static void launch_sweep(Ctx* c, int l, const int32_t* senders, const float* D, const RecMsgs& recs) {
+    Sweep a{};
+    a.in = c->side[1];
+    a.senders = senders;
+    a.posmap = c->posmap;
+    a.D = D;
+    a.ld = c->ws[l];
+    a.dS = c->dS[l];
+    a.bitmap = c->bitmap;
+    a.items = c->items;
+    a.N = c->N;
+    a.filter_words = std::min(1 << (SWEEP_BITS - 5), (div_up(c->N, 32) + 3) & ~3);   // (the queues behind it are aligned)
+    cut_lists(c, a);
+#define SWEEP(NV, WGT)                                                                                                                      \
+    do {                                                                                                                                    \
+        RP_LAUNCH(c, (k_sweep<NV, WGT>), c->n_sm, sweep_threads<NV>(), sweep_smem<NV>(a.filter_words, WGT), c->ctl, l, a, recs);                          \
+        RP_LAUNCH(c, (k_sweep_long<NV, WGT>), c->n_sm, sweep_threads<NV>(), sweep_smem<NV>(a.filter_words, WGT), c->ctl, l, a);                           \
+    } while (0)
+    RP_PIECES_DISPATCH(a.ld, c->weighted, SWEEP);
+#undef SWEEP
 }
 
 // A sink that lost at least as many in-edges as it keeps is rebuilt from its in-list, whatever
@@ -714,18 +824,18 @@ template <int NV, int LPR>
 __global__ void __launch_bounds__(256)
 k_regather_rows(Ctl* ctl, int l, const Rec* __restrict__ rec, Side in, const int32_t* __restrict__ deg_out,
                 int src_norm, const float* __restrict__ M, int ld, float* __restrict__ S, float* __restrict__ dS,
-                float* budget, const int32_t* __restrict__ senders, int32_t* posmap, int mark, int self_term,
+                float* budget, const int32_t* __restrict__ senders, int32_t* posmap, int self_term,
                 const int32_t* __restrict__ A_prev, uint32_t* bitmap, int chores_only) {
     pdl_enter();
     // Two chores of the hop ride along with this kernel, the last of the hop's delta form, whatever form
     // the hop takes.  The hop's senders are no longer looked up by anyone: their entries of the position
-    // map are cleared.  And (mark) the members of A_l that no out-list walk finds are marked: the sinks of
+    // map are cleared.  And the members of A_l that no walk finds are marked: the sinks of
     // net edge changes, and A_{l-1} for models with a self term.
     {
         const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsize = gridDim.x * blockDim.x;
         const int nC = ctl->nC[l - 1];
         for (int i = gtid; i < nC; i += gsize) posmap[senders[i]] = -1;
-        if (mark && !ctl->abort) {
+        if (!ctl->abort) {
             for (int i = gtid; i < ctl->n_rec; i += gsize) {
                 const int v = rec[i].v;
                 atomicOr(&bitmap[v >> 5], 1u << (v & 31));
@@ -765,12 +875,30 @@ k_regather_rows(Ctl* ctl, int l, const Rec* __restrict__ rec, Side in, const int
     }
 }
 
+// Microseconds, fitted to whole hops: a push pays per float delivered (0.65 ps where the accumulator stays in L2, 0.79
+// where it does not) and per sender, whose list a warp takes up after the one before (0.8 ns); a sweep per edge of the graph
+// (5.5 ps) and per row added up (4 ps and 0.29 per float), and is taken where it saves a tenth: hops at the line lose the launch.  Measured, push / sweep: 0.99 M messages of 256 floats from 80 K
+// senders on a graph of 1.2 M edges 216 / 125 us, 1.1 M of 40 floats 120 / 62; 50 M of 44 floats from 10 K senders, 115 M
+// edges, 1436 / 1341; 26 M of 48 floats, 124 M edges, 1000 / 1110.
+__host__ __device__ inline bool sweep_pays(double msgs, double senders, double edges, double vertices, int width) {
+    const bool outgrows = vertices * width * 4.0 > (double)WALK_TWICE;
+    const double push = 5.0 + 1e-6 * msgs * width * (outgrows ? 0.79 : 0.65) + 0.8e-3 * senders;
+    const double sweep = 30.0 + 1e-6 * (5.5 * edges + msgs * (4.0 + 0.29 * width));
+    return sweep < 0.9 * push;
+}
+
+// (twice what the hop carried in the batch before: the chain holds both forms well before the line)
+bool sweep_may_pay(const Ctx* c, int l, bool no_history) {
+    const double edges = (double)c->stats.num_edges, vertices = (double)c->N;
+    if (no_history) return sweep_pays(edges, vertices, edges, vertices, c->ws[l]);
+    return sweep_pays(2.0 * (double)c->stats.active_edges[l], 2.0 * (double)c->stats.senders[l - 1], edges, vertices, c->ws[l]);
+}
+
 // Form of hop l, decided on the device once the senders and their out-degree sum are known.
 //
-// Delta form: the out-edges of the senders each carry one message, added to the sink's aggregate
-// by a vector reduction (push), or gathered per sink over the senders among its in-neighbours
-// (k_scatter_gather: chosen on the host, per hop, for wide messages from few senders; slower than
-// the push for narrow rows because of the per-edge membership lookup).
+// Delta form: the out-edges of the senders each carry one message, added to the sink's accumulator by vector reductions
+// (push), or every in-list is read and the senders' delta rows in it are summed in registers (sweep: chosen on the host, per
+// hop, for wide messages from few senders, or here where it costs less).
 //
 // Rebuilding form: once the senders' out-edges are most of the graph, reading every in-edge of
 // the affected sinks once and overwriting their aggregates costs less than one reduction per
@@ -780,18 +908,21 @@ k_regather_rows(Ctl* ctl, int l, const Rec* __restrict__ rec, Side in, const int
 // of fewer than min_messages messages pushes regardless: on a graph of a million edges neither
 // form is throughput-bound, and the edge-balanced push is the more parallel of the two (measured
 // on the sparse graph, 256 floats per row: 0.24 ms pushed, 0.26 to 0.47 ms rebuilt).
-__global__ void k_choose_direction(Ctl* ctl, int l, int mode, int gather, float threshold, long long min_messages) {
+//
+// Between push and sweep, where both are in the chain, the cheaper one is taken (see sweep_pays).
+__global__ void k_choose_direction(Ctl* ctl, int l, int mode, int gather, float threshold, long long min_messages, int sweep, int N,
+                                   int width) {
     pdl_enter();
     const int nC = ctl->nC[l - 1];
     int re = 0;
+    const unsigned long long msgs = ctl->E[l] + (unsigned long long)ctl->n_rec;
     if (mode == RIPPLE_SCATTER_REGATHER) re = 1;
     else if (mode == RIPPLE_SCATTER_AUTO && threshold > 0.f) {
-        const unsigned long long msgs = ctl->E[l] + (unsigned long long)ctl->n_rec;
         re = (double)msgs >= (double)threshold * (double)ctl->num_edges && ctl->num_edges > 0 &&
              msgs >= (unsigned long long)min_messages;
     }
     if (nC == 0 && ctl->n_rec == 0) re = 0;
-    ctl->pull[l] = gather;
+    ctl->pull[l] = gather ? 1 : sweep && sweep_pays((double)msgs, (double)nC, (double)ctl->num_edges, (double)N, width) ? 2 : 0;
     ctl->regather[l] = re;
 }
 
@@ -878,11 +1009,11 @@ void fold_deltas(Ctx* c, int l) {
 
 void choose_direction(Ctx* c, int l) {
     // nothing to decide for a pushing hop: the control block's flags are already zero after its reset
-    if (!c->rebuild_armed[l] && !c->pull_hop[l] &&
+    if (!c->rebuild_armed[l] && !c->pull_hop[l] && !c->sweep_armed[l] &&
         (c->scatter_mode == RIPPLE_SCATTER_AUTO || c->scatter_mode == RIPPLE_SCATTER_PUSH ||
          c->scatter_mode == RIPPLE_SCATTER_PUSH_BULK)) return;
     RP_LAUNCH(c, k_choose_direction, 1, 1, 0, c->ctl, l, c->scatter_mode, (int)c->pull_hop[l],
-              c->rebuild_armed[l] ? c->regather_threshold[l] : -1.f, c->regather_min_messages);
+              c->rebuild_armed[l] ? c->regather_threshold[l] : -1.f, c->regather_min_messages, c->sweep_armed[l], c->N, c->ws[l]);
 }
 
 // delta form of hop l (does nothing on the device if the hop rebuilds)
@@ -903,17 +1034,9 @@ void scatter_layer(Ctx* c, int l, int n) {
         Mrows = c->P[l];
     }
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l], c->stream);
-#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap, recs, c->N)
-    int2* gather_items = c->items;
     const RecMsgs recs{c->rec, (int)c->src_norm, c->side[0].deg, c->posmap, Mrows};
     bool recs_done = false;
-#define PULL(NV, LPR)                                                                                                  \
-    do {                                                                                                               \
-        RP_LAUNCH(c, (k_scatter_gather<NV, LPR>), grid, T, 0, c->ctl, l, c->A[l], c->side[1], c->posmap, Dm, ld,      \
-                  c->dS[l], gather_items);                                                                             \
-        RP_LAUNCH(c, (k_scatter_gather_long<NV, LPR>), grid, T, 0, c->ctl, l, c->side[1], c->posmap, Dm, ld, c->dS[l], \
-                  (const int2*)gather_items);                                                                          \
-    } while (0)
+#define PUSH(NV, LPR) RP_LAUNCH(c, (k_scatter_push<NV, LPR>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, ld, c->dS[l], c->bitmap, recs, c->N)
     // (rows too wide for two staging buffers per warp in the default shared-memory allowance take the ordinary form)
     if (c->scatter_mode == RIPPLE_SCATTER_PUSH_BULK && !c->weighted && (size_t)8 * 2 * ld * sizeof(float) <= (48u << 10)) {
         RP_LAUNCH(c, k_scatter_push_bulk, grid, T, (size_t)8 * 2 * ld * sizeof(float), c->ctl, l, senders, c->coff,
@@ -928,15 +1051,17 @@ void scatter_layer(Ctx* c, int l, int n) {
         else RP_WIDTH_DISPATCH(ld, PUSH);
         recs_done = true;
     }
-    if (c->pull_hop[l]) RP_WIDTH_DISPATCH(ld, PULL);
 #undef PUSH
-#undef PULL
+    if (c->pull_hop[l] || c->sweep_armed[l]) {
+        launch_sweep(c, l, senders, Dm, recs);
+        recs_done = true;
+    }
     if (c->timing) cudaEventRecord(c->ev_sc[2 * l + 1], c->stream);
     if (n > 0) {
         if (!recs_done)
             RP_LAUNCH(c, k_scatter_records, std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, recs, Dm, ld, c->dS[l]);
         const float* rows = c->pre[l] ? c->P[l] : c->H[l - 1];
-#define ROWS(NV, LPR) RP_LAUNCH(c, (k_regather_rows<NV, LPR>), std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, c->rec, c->side[1], c->side[0].deg, (int)c->src_norm, rows, ld, c->S[l], c->dS[l], c->Eb[l], senders, c->posmap, (int)(!c->pull_hop[l]), (int)c->self_term, c->A[l - 1], c->bitmap, (int)(c->n_local > 0))
+#define ROWS(NV, LPR) RP_LAUNCH(c, (k_regather_rows<NV, LPR>), std::min(div_up(n, T / 32), c->n_sm * 8), T, 0, c->ctl, l, c->rec, c->side[1], c->side[0].deg, (int)c->src_norm, rows, ld, c->S[l], c->dS[l], c->Eb[l], senders, c->posmap, (int)c->self_term, c->A[l - 1], c->bitmap, (int)(c->n_local > 0))
         RP_WIDTH_DISPATCH(ld, ROWS);
 #undef ROWS
     }
@@ -945,21 +1070,12 @@ void scatter_layer(Ctx* c, int l, int n) {
 // rebuilding form of hop l (does nothing on the device unless the hop rebuilds); needs the list A_l
 void regather_layer(Ctx* c, int l) {
     if (!c->rebuild_armed[l]) return;
-    const int ld = c->ws[l];
-    const float* M = c->pre[l] ? c->P[l] : c->H[l - 1];   // P^l rows of the senders are already current
-    const int grid = c->n_sm * 16, T = 256;
-    int2* items = c->items;
-    int* n_items = &c->ctl->work_counter[(l - 1) & 7];
     if (c->timing) cudaEventRecord(c->ev_rg[2 * l], c->stream);
-#define REGATHER(NV, LPR)                                                                                          \
-    do {                                                                                                           \
-        RP_LAUNCH(c, (k_regather<NV, LPR>), grid, T, 0, c->ctl, l, c->A[l], c->side[1], c->side[0].deg,           \
-                  (int)c->src_norm, M, ld, c->S[l], items, n_items, c->Eb[l]);                                     \
-        RP_LAUNCH(c, (k_spmm_hubs<NV, LPR>), grid, T, 0, c->side[1], c->side[0].deg, (int)c->src_norm, M, ld,     \
-                  c->S[l], items, n_items, &c->ctl->hub_ticket[l]);                                                \
-    } while (0)
-    RP_WIDTH_DISPATCH(ld, REGATHER);
-#undef REGATHER
+    RowSums a = row_sums(c, l);   // (P^l rows of the senders are already current)
+    a.list = c->A[l];
+    a.n_dev = &c->ctl->nA[l];
+    a.budget = c->Eb[l];
+    launch_row_sums(c, l, a, true);
     if (c->timing) cudaEventRecord(c->ev_rg[2 * l + 1], c->stream);
 }
 
