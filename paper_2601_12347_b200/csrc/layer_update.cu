@@ -418,12 +418,14 @@ k_update_rows_elementwise(const Ctl* ctl, const __grid_constant__ UpdParams p) {
 // Launches every form that the row counts can call for; exactly one of them does the work of each problem (decided on
 // the device).
 // `over`: the hop whose list (A_over or C_over) the rows come from.
-static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2]) {
+// `both`: the weights of two problems over the same rows, side by side.
+static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2], const TcW* both = nullptr) {
     if (u.p[0].K == 0) {
         RP_LAUNCH(c, k_update_rows_elementwise, RP_RESIDENT(c, k_update_rows_elementwise, 256), 256, 0, c->ctl, u.p[0]);
         return;
     }
     UpdPair tc{};      // the problems that have a tensor-core twin
+    bool apart = false;   // narrow ones: each alone, unless their weights lie side by side
     for (int i = 0; i < u.n; ++i) {
         UpdParams& p = u.p[i];
         p.tc_mode = TC_OFF;
@@ -431,12 +433,13 @@ static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2
         // The forms for many rows are only put into the chain when the last batch's frontiers (or a whole-graph pass)
         // were large enough for them; without them the tiled SIMT form takes whatever comes.
         if (!c->tc_armed[over] && p.list) continue;
-        if (tw[i]->w && c->gemm_mode != RIPPLE_GEMM_FP32) {
-            p.tc_mode = c->gemm_mode == RIPPLE_GEMM_TF32 ? TC_TF32 : TC_TF32X3;
+        if (tw[i]->w && !(tw[i]->pieces && p.a_mode == A_SUM) && c->gemm_mode != RIPPLE_GEMM_FP32) {
+            p.tc_mode = c->gemm_mode == RIPPLE_GEMM_TF32 && !tw[i]->pieces ? TC_TF32 : TC_TF32X3;
             p.tc_min_rows = RP_TC_MIN_ROWS;
             p.tc_withhold = c->debug_tc_withhold;
             p.tc_w = tw[i]->w; p.tc_groups = tw[i]->groups; p.tc_chunks = tw[i]->chunks;
             tc.p[tc.n++] = p;
+            apart |= tw[i]->pieces;
         } else if (p.n_cols <= NBN && p.a_mode != A_SUM) {
             // narrow outputs over many rows have a form of their own
             p.narrow_min_rows = NARROW_MIN_ROWS;
@@ -446,7 +449,14 @@ static void launch_update(Ctx* c, UpdPair& u, int over, const TcW* const (&tw)[2
     else if (u.p[0].list || tc.n < u.n || c->N < RP_TC_MIN_ROWS) RP_LAUNCH(c, k_update_rows<false>, c->n_sm * 4, 256, 0, c->ctl, u);
     for (int i = 0; i < u.n; ++i)
         if (u.p[i].narrow_min_rows) RP_LAUNCH(c, k_update_rows_narrow, c->n_sm * 2, 256, NARROW_SMEM, c->ctl, u.p[i]);
-    if (tc.n) launch_update_tc(c, tc);
+    if (tc.n == 2 && apart && both && both->w && tc.p[0].list == tc.p[1].list) tc.p[0].tc_w = both->w;
+    else if (tc.n == 2 && apart) {
+        UpdPair second{};
+        second.p[second.n++] = tc.p[1];
+        tc.n = 1;
+        launch_update_tc(c, second, true);
+    }
+    if (tc.n) launch_update_tc(c, tc, apart);
 }
 
 static void launch_update(Ctx* c, const UpdParams& p, int over, const TcW& tw) {
@@ -497,7 +507,7 @@ static void project(Ctx* c, int l, const UpdParams& nbr, bool full) {
     u.p[0] = nbr;
     u.n = 1;
     if (c->Z[l]) u.p[u.n++] = self_problem(c, l, full);   // the same rows: one launch for both products
-    launch_update(c, u, l - 1, {&ly.tc_nbr, &ly.tc_self});
+    launch_update(c, u, l - 1, {&ly.tc_nbr, &ly.tc_self}, &ly.tc_both);
 }
 
 void project_full(Ctx* c, int l) { project(c, l, neighbour_problem(c, l, true), true); }

@@ -149,6 +149,6 @@ __device__ __forceinline__ void upd_epilogue4(const UpdParams& p, int v, int i, 
 }
 
 // layer_update_tc.cu
-void launch_update_tc(Ctx* c, const UpdPair& pair);
+void launch_update_tc(Ctx* c, const UpdPair& pair, bool pieces);
 
 }  // namespace rp

@@ -45,11 +45,12 @@ namespace rp {
 constexpr int TC_COLS = 128;     // output columns per group (= TMEM lanes)
 constexpr int TC_KC = 32;        // floats per K chunk: one 128-byte swizzle row
 constexpr int TC_TILE = 128;     // affected rows per tile
+constexpr int TC_PIECE = 16;     // entries of K whose large products the form for narrow outputs adds up in tensor memory
 // Loader threads: sixteen warps where the weights stream, eight where they stay (whose epilogue, with a cached projection
 // to read for every row, needs the registers more).
-__host__ __device__ constexpr int tc_loaders(bool resident) { return resident ? 256 : 512; }
+__host__ __device__ constexpr int tc_loaders(bool resident, bool pieces) { return pieces ? 128 : resident ? 256 : 512; }
 constexpr int TC_EPI_WARPS = 8;  // two per tensor-memory lane quarter, half of the tile's rows each
-__host__ __device__ constexpr int tc_threads(bool resident) { return tc_loaders(resident) + 32 * TC_EPI_WARPS + 64; }   // and the warps that issue and that fetch the weights
+__host__ __device__ constexpr int tc_threads(bool resident, bool pieces) { return tc_loaders(resident, pieces) + 32 * TC_EPI_WARPS + 64; }   // and the warps that issue and that fetch the weights
 constexpr int TC_W_HALF = TC_COLS * 128;         // one half (hi or lo) of a chunk of weights
 constexpr int TC_W_BYTES = 2 * TC_W_HALF;
 constexpr int TC_RESIDENT_CHUNKS = 4;            // weights of up to this many chunks stay in shared memory
@@ -163,6 +164,17 @@ __device__ __forceinline__ void tc_load16(uint32_t (&x)[16], uint32_t taddr) {
         : "r"(taddr) : "memory");
 }
 
+__device__ __forceinline__ void tc_load32(uint32_t (&x)[32], uint32_t taddr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]), "=r"(x[8]),
+          "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15]), "=r"(x[16]),
+          "=r"(x[17]), "=r"(x[18]), "=r"(x[19]), "=r"(x[20]), "=r"(x[21]), "=r"(x[22]), "=r"(x[23]), "=r"(x[24]),
+          "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]), "=r"(x[29]), "=r"(x[30]), "=r"(x[31])
+        : "r"(taddr) : "memory");
+}
 
 // own[k] without an index register
 template <int N, typename T>
@@ -183,14 +195,20 @@ __device__ __forceinline__ T tc_pick(const T (&own)[N], int k) {
 // still in flight.
 // RESIDENT: the weights stay in shared memory; else they stream.
 // SUM: the row operand is alpha h + scale S (GIN), two rows per entry.
-template <bool RESIDENT, bool SUM>
-__global__ void __launch_bounds__(tc_threads(RESIDENT), 1)
+// PIECES: narrow outputs, whose products were fp32 sums before and are no less exact here (see tc_weights_build).  What the
+// tensor core adds up at full size is 16 entries of K (two additions): the accumulator of the large products is handed over
+// that often, and its pieces meet in the epilogue's registers, in fp32; the small products gather over the whole tile.
+// Lanes 0..63 are the columns of the first problem, lanes 64..127 those of the second, which reads the same rows.  (The
+// epilogue's 64 sums per thread leave registers for four loader warps.)
+template <bool RESIDENT, bool SUM, bool PIECES>
+__global__ void __launch_bounds__(tc_threads(RESIDENT, PIECES), 1)
 k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
-    constexpr int TC_LOADERS = tc_loaders(RESIDENT);
+    constexpr int TC_LOADERS = tc_loaders(RESIDENT, PIECES);
     constexpr int TILE = TC_TILE, RSTEP = TC_LOADERS / 8, ITS = TILE / RSTEP;
     constexpr int X_HALF = TILE * 128, X_BYTES = 2 * X_HALF, NH = tc_stages(RESIDENT);
     constexpr int W_SLOTS = RESIDENT ? TC_RESIDENT_CHUNKS : TC_W_STAGES;
-    constexpr int BUF = 2 * TILE;                                // tensor-memory columns of an accumulator: [hi hi | corrections]
+    // Tensor-memory columns: two accumulators of [hi hi | corrections]; with PIECES two of the former, two of the latter.
+    constexpr int BUF = PIECES ? TILE : 2 * TILE;
     pdl_enter();
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_x[NH], full_w[W_SLOTS], empty[NH], acc_full[2], acc_empty[2], drained;
@@ -199,7 +217,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
 
     if (ctl->abort) return;
     // This CTA's column group: those of the first problem, then those of the second.
-    const int g0 = pair.p[0].tc_groups, G = g0 + (pair.n > 1 ? pair.p[1].tc_groups : 0);
+    const int g0 = pair.p[0].tc_groups, G = g0 + (!PIECES && pair.n > 1 ? pair.p[1].tc_groups : 0);
     const int my_g = (int)blockIdx.x % G, member = (int)blockIdx.x / G, members = ((int)gridDim.x - my_g + G - 1) / G;
     const UpdParams& p = pair.p[my_g < g0 ? 0 : 1];
     const int grp = my_g < g0 ? my_g : my_g - g0;
@@ -219,7 +237,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* x_ring = smem;                                      // stages of rows: [as they come | their remainders]
     uint8_t* w_ring = smem + (size_t)NH * X_BYTES;               // stages of [hi | lo] weights, or all chunks of them
-    constexpr uint32_t tmem_cols = 2 * BUF;
+    constexpr uint32_t tmem_cols = 4 * TILE;
 
     if (tid == 0) {
         for (int s = 0; s < NH; ++s) { mbar_init(&full_x[s], TC_LOADERS / 32); mbar_init(&empty[s], 1); }
@@ -371,8 +389,10 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         // group, one per lane; the two warps of a quarter take half of the tile's rows each, BLK rows at a time.
         constexpr int BLK = 16, HALF = TILE / 2, OWN = HALF / 32;
         const int q = warp & 3, half = (warp - TC_LOADERS / 32) >> 2;
-        int lc = grp * TC_COLS + 32 * q + lane;   // this lane's column
-        const bool col_ok = lc < p.n_cols;
+        const int col0 = PIECES ? 32 * (q & 1) : grp * TC_COLS + 32 * q;   // the first of this warp's columns
+        const UpdParams& p = PIECES && q >= 2 ? pair.p[1] : pair.p[my_g < g0 ? 0 : 1];
+        int lc = col0 + lane;                     // this lane's column
+        const bool col_ok = lc < p.n_cols && (!PIECES || q < 2 || pair.n > 1);
         if (!col_ok) lc = 0;
         float* const hout = p.Hout + lc;
         float* const dout = p.epi_mode == EPI_COMMIT && p.Dout ? p.Dout + lc : nullptr;
@@ -406,7 +426,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         constexpr int DEPTH = TC_AHEAD, BLOCKS = HALF / BLK;
         float* const zbuf = reinterpret_cast<float*>(w_ring + (size_t)W_SLOTS * TC_W_BYTES) + (warp - TC_LOADERS / 32) * (DEPTH * BLK * 32);
         // the piece of the row that this lane copies: four columns
-        const int pc = grp * TC_COLS + 32 * q + 4 * (lane & 7);
+        const int pc = col0 + 4 * (lane & 7);
         const float* const piece = (any_z ? p.addend2 : p.Hout) + (pc < p.n_cols ? pc : 0);
         auto fetch = [&](int slot, int v_src, int at) {
 #pragma unroll
@@ -422,8 +442,9 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
 #pragma unroll
             for (int d = 0; d < DEPTH; ++d) fetch(d, tc_pick<OWN>(v_next, d * BLK / 32), (d * BLK) & 31);
         }
-        for (int lt = 0; lt < my_tiles; ++lt) {
-            const int b = lt & 1, ub = lt >> 1;
+        bool ok = true;
+        int sg = 0;                         // accumulators handed over so far: one per tile, with PIECES one per piece of K
+        for (int lt = 0; lt < my_tiles && ok; ++lt) {
             const int r0 = tile_row(lt) + HALF * half;
 #pragma unroll
             for (int k = 0; k < OWN; ++k) {
@@ -431,25 +452,24 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 sc_own[k] = sc_next[k];
             }
             ids(lt + 1);
-            if (!mbar_wait_bounded(&acc_full[b], ub & 1, spin_limit)) { s_fail = 1; break; }
-            tc_fence_after();
-            const uint32_t t_mine = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * BUF + HALF * half);
-            auto block = [&](int blk) {
-                const int at = (blk * BLK) & 31, i0 = r0 + blk * BLK;
-                const int v_src = tc_pick<OWN>(v_own, blk * BLK / 32);
-                const float s_src = tc_pick<OWN>(sc_own, blk * BLK / 32);
+            auto take = [&](float (&h)[BLK], int blk, int buf) {   // BLK rows of the accumulator, its small products added
+                const uint32_t t_mine = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BUF + HALF * half + blk * BLK);
                 uint32_t x[BLK];
-                tc_load16(x, t_mine + (uint32_t)(blk * BLK));
+                tc_load16(x, t_mine);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                float h[BLK];
 #pragma unroll
                 for (int r = 0; r < BLK; ++r) h[r] = __uint_as_float(x[r]);
                 if (x3) {
-                    tc_load16(x, t_mine + (uint32_t)(TILE + blk * BLK));
+                    tc_load16(x, t_mine + (uint32_t)TILE);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                     for (int r = 0; r < BLK; ++r) h[r] += __uint_as_float(x[r]);
                 }
+            };
+            auto block = [&](int blk, float (&h)[BLK]) {
+                const int at = (blk * BLK) & 31, i0 = r0 + blk * BLK;
+                const int v_src = tc_pick<OWN>(v_own, blk * BLK / 32);
+                const float s_src = tc_pick<OWN>(sc_own, blk * BLK / 32);
                 if (plus_s) {   // (transformed aggregates with a self term of their own: GIN layers that narrow)
 #pragma unroll 1
                     for (int r = 0; r < BLK; ++r) {
@@ -553,13 +573,51 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 for (int r = 0; r < BLK; ++r)
                     tc_store_if(r < live, reinterpret_cast<float*>(reinterpret_cast<char*>(hout) + (uint64_t)v[r] * ld_bytes), h[r]);
             };
-            if (warp_busy) {
+            const int parts = PIECES ? (K + TC_PIECE - 1) / TC_PIECE : 1;
+            float sum[PIECES ? BLOCKS : 1][BLK];
+            for (int part = 0; part < parts; ++part, ++sg) {
+                const int b = sg & 1;
+                ok = mbar_wait_bounded(&acc_full[b], (sg >> 1) & 1, spin_limit);
+                if (!ok) { s_fail = 1; break; }
+                tc_fence_after();
+                if (warp_busy) {
+                    if constexpr (PIECES) {
+                        const uint32_t t_row = tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(HALF * half);
+                        if (part == 0) {
+#pragma unroll
+                            for (int r = 0; r < HALF; ++r) sum[r / BLK][r % BLK] = 0.f;
+                        }
+                        auto add = [&](uint32_t from) {
+#pragma unroll
+                            for (int r0_ = 0; r0_ < HALF; r0_ += 32) {
+                                uint32_t x[32];
+                                tc_load32(x, from + (uint32_t)r0_);
+                                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                                for (int r = 0; r < 32; ++r) sum[(r0_ + r) / BLK][(r0_ + r) % BLK] += __uint_as_float(x[r]);
+                            }
+                        };
+                        add(t_row + (uint32_t)(b * BUF));
+                        if (part == parts - 1) add(t_row + (uint32_t)(2 * TILE + (lt & 1) * TILE));
+                    } else {
 #pragma unroll 1
-                for (int blk = 0; blk < BLOCKS; ++blk) block(blk);
+                        for (int blk = 0; blk < BLOCKS; ++blk) {
+                            float h[BLK];
+                            take(h, blk, b);
+                            block(blk, h);
+                        }
+                    }
+                }
+                tc_fence_before();   // accumulators consumed: the MMA warp may overwrite them after this arrival
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[b]);
             }
-            tc_fence_before();   // accumulators consumed: the MMA warp may overwrite them after this arrival
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[b]);
+            if constexpr (PIECES) {
+                if (ok && warp_busy) {
+#pragma unroll
+                    for (int blk = 0; blk < BLOCKS; ++blk) block(blk, sum[blk]);
+                }
+            }
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     } else if (warp == TC_LOADERS / 32 + TC_EPI_WARPS) {
@@ -571,15 +629,24 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         int s = 0, sw = 0;
         uint32_t ph = 0, phw = 0;              // ring slots and phases of this step
         bool ok = true;
+        int sg = 0;                            // accumulators begun so far
         for (int lt = 0; lt < my_tiles; ++lt) {
-            const int b = lt & 1, ub = lt >> 1;
-            // the epilogue must have drained this accumulator buffer (tile lt - 2)
-            if (ub > 0) ok = __all_sync(FULL, mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit));
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t d_addr = tmem_base + (uint32_t)(b * BUF), d_corr = d_addr + TILE;
-            int left = K;
+            uint32_t d_addr = 0, d_corr = 0;
+            int left = K, b = 0;
             for (int kc = 0; kc < nchunks; ++kc, left -= TC_KC) {
+                auto begin = [&]() {
+                    // the epilogue must have drained this accumulator buffer (the one before the last)
+                    b = sg & 1;
+                    const int ub = sg >> 1;
+                    ++sg;
+                    if (ub > 0) ok = __all_sync(FULL, mbar_wait_bounded(&acc_empty[b], (ub - 1) & 1, spin_limit));
+                    if (!ok) return;
+                    tc_fence_after();
+                    d_addr = tmem_base + (uint32_t)(b * BUF);
+                    d_corr = PIECES ? tmem_base + (uint32_t)(2 * TILE + (lt & 1) * TILE) : d_addr + TILE;
+                };
+                if (!PIECES && kc == 0) begin();
+                if (!ok) break;
                 if (RESIDENT) sw = kc;
                 bool there = true;
                 if (!RESIDENT || lt == 0) there = mbar_wait_bounded(&full_w[sw], phw, spin_limit);
@@ -592,6 +659,29 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 tc_fence_after();
                 const uint64_t xh = dx0 + (uint64_t)((uint32_t)s * (X_BYTES >> 4));
                 const uint64_t wh = dw0 + (uint64_t)((uint32_t)sw * (TC_W_BYTES >> 4)), wl = wh + (TC_W_HALF >> 4);
+                if constexpr (PIECES) {
+                    // (a tile's small products may go where the tile before the last had them: its last piece has been drained)
+#pragma unroll 1
+                    for (int j0 = 0; j0 < TC_KC / 8 && 8 * j0 < left; j0 += TC_PIECE / 8) {
+                        begin();
+                        if (!ok) break;
+                        if (lead) {
+#pragma unroll
+                            for (int i = 0; i < TC_PIECE / 8; ++i) {
+                                const int j = j0 + i;
+                                if (8 * j < left) {
+                                    tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, idesc, i != 0);
+                                    tc_mma_tf32(d_corr, wh + 2 * j, xh + (X_HALF >> 4) + 2 * j, idesc, (kc | j) != 0);
+                                    tc_mma_tf32(d_corr, wl + 2 * j, xh + 2 * j, idesc, 1u);
+                                }
+                            }
+                            if (j0 + TC_PIECE / 8 >= TC_KC / 8 || 8 * (j0 + TC_PIECE / 8) >= left) tc_commit(&empty[s]);
+                            if (!(withhold && lt == 0)) tc_commit(&acc_full[b]);
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) break;
+                } else {
                 const bool last = kc == nchunks - 1;
                 if (lead) {
 #pragma unroll
@@ -605,6 +695,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                     // (diagnostic: with tc_withhold the first tile is never reported finished, so that
                     // the epilogue's bounded wait runs out and the status path can be exercised)
                     if (last && !(withhold && lt == 0)) tc_commit(&acc_full[b]);
+                }
                 }
                 __syncwarp();
                 if (++s == NH) { s = 0; ph ^= 1; }
@@ -660,23 +751,25 @@ static size_t tc_smem_bytes(bool resident) {
            (size_t)TC_EPI_WARPS * TC_AHEAD * 16 * 128 + 1024;
 }
 
-void launch_update_tc(Ctx* c, const UpdPair& pair) {
+void launch_update_tc(Ctx* c, const UpdPair& pair, bool pieces) {
     const bool resident = pair.p[0].tc_chunks <= TC_RESIDENT_CHUNKS, sum = pair.p[0].a_mode == A_SUM;
     // one persistent CTA per SM: operands and weights fill its shared memory
-#define TC_GO(RES, SUM) RP_LAUNCH(c, (k_update_rows_tc<RES, SUM>), c->n_sm, tc_threads(RES), tc_smem_bytes(RES), c->ctl, pair)
-    if (resident && sum) TC_GO(true, true);
-    else if (resident) TC_GO(true, false);
-    else if (sum) TC_GO(false, true);
-    else TC_GO(false, false);
+#define TC_GO(RES, SUM, PIECES) RP_LAUNCH(c, (k_update_rows_tc<RES, SUM, PIECES>), c->n_sm, tc_threads(RES, PIECES), tc_smem_bytes(RES), c->ctl, pair)
+    if (pieces) TC_GO(false, false, true);
+    else if (resident && sum) TC_GO(true, true, false);
+    else if (resident) TC_GO(true, false, false);
+    else if (sum) TC_GO(false, true, false);
+    else TC_GO(false, false, false);
 #undef TC_GO
 }
 
 void tc_prepare() {
-#define TC_SET(RES, SUM) cudaFuncSetAttribute(k_update_rows_tc<RES, SUM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(RES))
-    TC_SET(true, true);
-    TC_SET(true, false);
-    TC_SET(false, true);
-    TC_SET(false, false);
+#define TC_SET(RES, SUM, PIECES) cudaFuncSetAttribute(k_update_rows_tc<RES, SUM, PIECES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem_bytes(RES))
+    TC_SET(true, true, false);
+    TC_SET(true, false, false);
+    TC_SET(false, true, false);
+    TC_SET(false, false, false);
+    TC_SET(false, false, true);
 #undef TC_SET
 }
 
@@ -685,12 +778,20 @@ void tc_prepare() {
 //
 // Which outputs have them, and from how many rows the form is taken (RP_TC_MIN_ROWS), is a line of precision.  The form is
 // the faster one from 512 rows on, also for narrow outputs (whole-graph pass of one layer, K = 256, 256 columns: 512 rows
-// 39 us, fp32 sums 46; 1024: 39 / 52; 32 768: 94 / 321; 48 columns: 39 / 47, 39 / 48 and 51 / 114), but two to three times
-// less exact than fp32 sums (see the top of the file).  Outputs of 113 to 256 columns over 1024 and more rows have always
-// been split products, and less exact ones than these; all others are fp32 sums and stay so.
-cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw) {
+// 39 us, fp32 sums 46; 1024: 39 / 52; 32 768: 94 / 321), but two to three times less exact than fp32 sums (see the top of the
+// file).  Outputs of 113 to 256 columns over 1024 and more rows have always been split products, and less exact ones than
+// these; all others were fp32 sums and lose nothing: up to 64 columns the large products are summed in pieces, where K is
+// long enough for the fp32 sum to be the less exact one.  Error against fp64, 2-norm, rows ~ N(0, 1) / rectified, pieces and
+// fp32 sums: K = 192 1.9e-7 / 1.9e-7 and 2.5e-7 / 1.8e-7, K = 256 2.0e-7 / 1.9e-7 and 2.9e-7 / 2.0e-7, K = 602 2.1e-7 / 2.1e-7
+// and 4.4e-7 / 3.1e-7 (in pieces of 32 entries 2.2e-7 / 2.1e-7 at K = 256).  2.4 M rows, K = 256, two products of 48 columns:
+// 3.43 -> 1.29 ms; one of 40 columns over 80 K rows 125 -> 93 us.  Bound by shared memory: a chunk's weights and rows are
+// written, split and read by three products, twelve times the bytes of its rows.
+// W2: a second matrix over the same rows, for the form in pieces.
+cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const float* W2) {
     *out = TcW{};
-    if (K <= 0 || ldw < RP_TC_MIN_COLS || ldw > RP_TC_MAX_COLS) return cudaSuccess;
+    const bool pieces = ldw <= RP_TC_PIECES_MAX_COLS && K >= RP_TC_PIECES_MIN_K;
+    if (K <= 0 || !(pieces || (!W2 && ldw >= RP_TC_MIN_COLS && ldw <= RP_TC_MAX_COLS))) return cudaSuccess;
+    out->pieces = pieces;
     auto round_tf32 = [](float v) {
         uint32_t bits;
         memcpy(&bits, &v, 4);
@@ -702,15 +803,17 @@ cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw) {
     out->chunks = (K + TC_KC - 1) / TC_KC;
     const size_t block = TC_W_BYTES / 4;
     std::vector<float> pack(block * out->chunks * out->groups, 0.f);
-    for (int k = 0; k < K; ++k)
-        for (int j = 0; j < ldw; ++j) {
-            const float x = W[(size_t)k * ldw + j], h = round_tf32(x);
-            const int g = j / TC_COLS, r = j - g * TC_COLS, kc = k / TC_KC, kk = k - kc * TC_KC;
-            float* blk = pack.data() + ((size_t)g * out->chunks + kc) * block;
-            const uint32_t at = tc_swz(r, kk >> 2) / 4 + (kk & 3);
-            blk[at] = h;
-            blk[TC_W_HALF / 4 + at] = round_tf32(x - h);
-        }
+    for (int m = 0; m < (W2 ? 2 : 1); ++m)
+        for (int k = 0; k < K; ++k)
+            for (int j = 0; j < ldw; ++j) {
+                const float x = (m ? W2 : W)[(size_t)k * ldw + j], h = round_tf32(x);
+                const int col = j + m * (TC_COLS / 2);
+                const int g = col / TC_COLS, r = col - g * TC_COLS, kc = k / TC_KC, kk = k - kc * TC_KC;
+                float* blk = pack.data() + ((size_t)g * out->chunks + kc) * block;
+                const uint32_t at = tc_swz(r, kk >> 2) / 4 + (kk & 3);
+                blk[at] = h;
+                blk[TC_W_HALF / 4 + at] = round_tf32(x - h);
+            }
     cudaError_t e = cudaMalloc(&out->w, sizeof(float) * pack.size());
     if (!e) e = cudaMemcpy(out->w, pack.data(), sizeof(float) * pack.size(), cudaMemcpyHostToDevice);
     return e;

@@ -69,7 +69,7 @@ static void destroy_ctx(Ctx* c) {
         cudaFree(c->att_s[l]); cudaFree(c->att_t[l]);
         cudaFree(c->H[l]); cudaFree(c->S[l]); cudaFree(c->dS[l]); cudaFree(c->Eb[l]); cudaFree(c->Z[l]); cudaFree(c->P[l]); cudaFree(c->A[l]);
         cudaFree(c->layer[l].W1); cudaFree(c->layer[l].b1); cudaFree(c->layer[l].W2); cudaFree(c->layer[l].b2);
-        for (TcW* t : {&c->layer[l].tc_main, &c->layer[l].tc_nbr, &c->layer[l].tc_2, &c->layer[l].tc_self}) cudaFree(t->w);
+        for (TcW* t : {&c->layer[l].tc_main, &c->layer[l].tc_nbr, &c->layer[l].tc_2, &c->layer[l].tc_self, &c->layer[l].tc_both}) cudaFree(t->w);
     }
     cudaFree(c->att_so); cudaFree(c->att_items);
     cudaFree(c->halo_owner); cudaFree(c->halo_rid); cudaFree(c->silent_dev); cudaFree(c->rows_sent);
@@ -359,6 +359,7 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
                     else if (!c->pre[l])
                         CK(tc_weights_build(&ly.tc_main, w1.data(), ly.ld_in, ly.ld_out));
                     if (c->pre[l]) CK(tc_weights_build(&ly.tc_nbr, wn, ly.ld_in, c->ws[l]));
+                    if (c->pre[l] && y.kind == RIPPLE_LAYER_SAGE && ly.tc_nbr.pieces) CK(tc_weights_build(&ly.tc_both, wn, ly.ld_in, c->ws[l], w1.data()));
                     if (y.kind == RIPPLE_LAYER_GIN) CK(tc_weights_build(&ly.tc_2, w2.data(), ly.ld_hid, ly.ld_out));
                 }
             }

@@ -25,6 +25,8 @@
 #define RP_TC_MIN_ROWS 1024         // row count from which a layer update takes the tensor-core form,
 #define RP_TC_MIN_COLS 113          // for outputs of RP_TC_MIN_COLS .. RP_TC_MAX_COLS columns (see tc_weights_build)
 #define RP_TC_MAX_COLS 256
+#define RP_TC_PIECES_MAX_COLS 64    // ... and, in pieces of K, of up to RP_TC_PIECES_MAX_COLS columns
+#define RP_TC_PIECES_MIN_K 256      // over at least this many entries
 #define RP_ATT_CHUNK 128            // attention: in-list entries per work item of a recomputation (sizes the item buffer)
 #define RP_TINY_BATCH 32            // batches up to this size list their frontiers and senders in one block each
 #define RP_TINY_APPLY 4             // ... and up to this size run the whole of Apply in one block (operations are resolved one after the other there)
@@ -135,6 +137,7 @@ struct Rec {
 struct TcW {
     float* w;
     int groups, chunks;        // groups of 128 columns, K chunks of 32
+    bool pieces;               // narrow outputs: chunks are summed apart (see k_update_rows_tc)
 };
 
 // Where a batch lies: pinned host memory or device memory, in either case read by the first kernel of its chain.
@@ -157,6 +160,7 @@ struct LayerDev {
     TcW tc_main; // weights of the affected-row GEMM (GIN: first matrix)
     TcW tc_nbr;  // neighbour matrix, for layers that transform before the scatter
     TcW tc_2;    // GIN: second matrix
+    TcW tc_both; // the two of a SAGE layer that transforms before the scatter, side by side (narrow outputs)
     TcW tc_self; // SAGE: self matrix, for the cached self projection
 };
 
@@ -401,7 +405,7 @@ void feature_rows(Ctx* c, int n);                       // hop 0: overwrite feat
 void extra_sender_rows(Ctx* c, int l, int n);           // deltas of senders whose row did not change
 
 // layer_update_tc.cu
-cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw);
+cudaError_t tc_weights_build(TcW* out, const float* W_host, int K, int ldw, const float* W2_host = nullptr);
 void tc_prepare();   // one-time kernel attributes (not allowed inside a stream capture)
 void narrow_prepare();   // likewise, for the update form for narrow outputs
 
