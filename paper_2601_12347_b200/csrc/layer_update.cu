@@ -20,22 +20,27 @@ namespace rp {
 constexpr int BM = 64, BN = 64, BK = 64, TM = 4, TN = 4;
 
 // A frontier of a few rows (a batch of a few updates at the first hops) is nothing but latency: the tiled form
-// walks K in chunks, each a round trip to L2 behind the last.  For up to FEW_MAX rows and K up to FEW_K the same
-// kernel takes another route: a block owns FEW_ROWS rows and 32 output columns, stages its A rows in shared
-// memory once, its eight warps each take an eighth of K with every weight load independent of the others (one
-// round trip in all), the partial sums meet in shared memory and the ordinary epilogue finishes the rows.
-constexpr int FEW_ROWS = 16, FEW_K = 256, FEW_COLS = 32, FEW_MAX = 256;
+// walks K in chunks, each a round trip to L2 behind the last, and gives the device a tile per 64 rows.  While all items of
+// 16 rows and 32 output columns fit on the device at once the same kernel takes another route: a block stages the rows of
+// its item in shared memory (256 entries of K at a time), its eight warps each take an eighth of them with every weight
+// load independent of the others (one round trip in all), the partial sums meet in shared memory and the ordinary epilogue
+// finishes the rows.  (Two projections of some 900 rows, K = 256, 40 columns: 31 -> 13 us; 20 rows, K = 602, 256
+// columns: 49 -> 18.)
+constexpr int FEW_ROWS = 16, FEW_K = 256, FEW_COLS = 32;
+
+__device__ __forceinline__ int upd_few_items(const UpdParams& p, int n) {
+    return ((p.n_cols + FEW_COLS - 1) / FEW_COLS) * ((n + FEW_ROWS - 1) / FEW_ROWS);
+}
 
 __device__ __forceinline__ bool upd_few(const UpdParams& p, int n) {
-    return n > 0 && n <= FEW_MAX && p.K > 0 && p.K <= FEW_K;
+    return n > 0 && p.K > 0 && upd_few_items(p, n) <= (int)gridDim.x;
 }
 
 __device__ __forceinline__ void update_few_rows(const UpdParams& p, int n_all, int first, float* A_s, float* red, int* row_id,
                                                 float* row_scale) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int kq = p.K >> 2;
-    const int groups = (p.n_cols + FEW_COLS - 1) / FEW_COLS, row_groups = (n_all + FEW_ROWS - 1) / FEW_ROWS;
-    for (int item = first; item < groups * row_groups; item += gridDim.x) {
+    const int groups = (p.n_cols + FEW_COLS - 1) / FEW_COLS, items = upd_few_items(p, n_all);
+    for (int item = first; item < items; item += gridDim.x) {
         const int g = item % groups, r0 = (item / groups) * FEW_ROWS;
         const int n = min(FEW_ROWS, n_all - r0);   // rows of this block: compact indices r0 .. r0 + n - 1
         __syncthreads();
@@ -44,23 +49,26 @@ __device__ __forceinline__ void update_few_rows(const UpdParams& p, int n_all, i
             row_id[tid] = v;
             row_scale[tid] = upd_row_scale(p, v);
         }
-        __syncthreads();
-        for (int it = tid; it < n * kq; it += blockDim.x) {
-            const int r = it / kq, k = 4 * (it - r * kq);
-            *reinterpret_cast<float4*>(A_s + r * FEW_K + k) = upd_load_a(p, row_id[r], r0 + r, k, row_scale[r]);
-        }
-        __syncthreads();
         const int c = g * FEW_COLS + lane;
-        const int kper = (p.K + 7) >> 3, k_begin = warp * kper, k_end = min(p.K, k_begin + kper);
         float acc[FEW_ROWS];
 #pragma unroll
         for (int r = 0; r < FEW_ROWS; ++r) acc[r] = 0.f;
+        for (int k0 = 0; k0 < p.K; k0 += FEW_K) {
+            const int kn = min(FEW_K, p.K - k0), kq = kn >> 2;
+            __syncthreads();
+            for (int it = tid; it < n * kq; it += blockDim.x) {
+                const int r = it / kq, k = 4 * (it - r * kq);
+                *reinterpret_cast<float4*>(A_s + r * FEW_K + k) = upd_load_a(p, row_id[r], r0 + r, k0 + k, row_scale[r]);
+            }
+            __syncthreads();
+            const int kper = (kn + 7) >> 3, k_begin = warp * kper, k_end = min(kn, k_begin + kper);
 #pragma unroll 8
-        for (int k = k_begin; k < k_end; ++k) {
-            const float wv = c < p.n_cols ? __ldg(p.W + (size_t)k * p.ldw + c) : 0.f;
+            for (int k = k_begin; k < k_end; ++k) {
+                const float wv = c < p.n_cols ? __ldg(p.W + (size_t)(k0 + k) * p.ldw + c) : 0.f;
 #pragma unroll
-            for (int r = 0; r < FEW_ROWS; ++r)
-                if (r < n) acc[r] = fmaf(A_s[r * FEW_K + k], wv, acc[r]);
+                for (int r = 0; r < FEW_ROWS; ++r)
+                    if (r < n) acc[r] = fmaf(A_s[r * FEW_K + k], wv, acc[r]);
+            }
         }
 #pragma unroll
         for (int r = 0; r < FEW_ROWS; ++r) red[(warp * FEW_ROWS + r) * FEW_COLS + lane] = acc[r];
@@ -102,7 +110,7 @@ k_update_rows(const Ctl* ctl, const __grid_constant__ UpdPair pair) {
         static_assert(sizeof(As) >= sizeof(float) * FEW_ROWS * FEW_K && sizeof(Bs) >= sizeof(float) * 8 * FEW_ROWS * FEW_COLS,
                       "the few-row form borrows the tiles' shared memory");
         update_few_rows(p, n, first, &As[0][0], &Bs[0][0], row_id, row_scale);
-        used += ((p.n_cols + FEW_COLS - 1) / FEW_COLS) * ((n + FEW_ROWS - 1) / FEW_ROWS);
+        used += upd_few_items(p, n);
         continue;
     }
     const int row_tiles = (n + BM - 1) / BM, col_tiles = (p.n_cols + BN - 1) / BN;
