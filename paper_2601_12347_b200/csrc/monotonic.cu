@@ -17,9 +17,10 @@
 
 namespace rp {
 
-constexpr int MAX_HUB_DEGREE = 256;    // longer in-lists are recomputed in chunks, one warp per chunk
-constexpr int MAX_HUB_CHUNK = 256;     // in-list entries per chunk
-static_assert(MAX_HUB_CHUNK >= RP_ITEM_MIN, "the item buffer is sized by it");
+// A recomputation takes in-lists of more than `cut` entries in pieces of that size, one warp per piece: MAX_CUT_MIN to
+// MAX_CUT of them, by the graph's edges per warp of the device (see max_cut).  A full pass cuts by MAX_CUT.
+constexpr int MAX_CUT = 256, MAX_CUT_MIN = 128;
+static_assert(MAX_CUT_MIN >= RP_ITEM_MIN, "the item buffer is sized by it");
 constexpr int MAX_FULL_PASS_DEGREE = 4096;   // a full pass has rows enough to keep every warp busy: only longer lists are chunked
 constexpr int MAX_CHUNK = 64;          // edges per warp work item of the message walk
 
@@ -63,7 +64,7 @@ __device__ __forceinline__ void max_accumulate(float4 (&acc)[NV], const Side& in
     for (int j0 = j_begin; j0 < j_end; j0 += 32) {
         const int mine = j0 + lane < j_end ? in.col[base + j0 + lane] : 0;
         const int cnt = min(32, j_end - j0);
-        constexpr int UNR = 4;   // neighbour rows in flight per lane group
+        constexpr int UNR = NV == 1 ? 8 : 4;   // neighbour rows in flight per lane group
         for (int j = 0; j < cnt; j += UNR * EPI) {
             int u[UNR];
             float4 x[UNR][NV];
@@ -116,22 +117,53 @@ __device__ __forceinline__ void fill(float4 (&acc)[NV], float x) {
 // messages therefore record WHICH elements lost their maximiser (a bit mask per row); a row with
 // at most MAX_EL such elements re-reads only those, any other row is gathered in full.
 // ---------------------------------------------------------------------------------------------
-constexpr int MAX_EL = 16;
+constexpr int MAX_EL = 32;
 
-// set elements of a row's mask -> ascending indices; returns their number, or -1 if there are more
-// than MAX_EL (or the whole row was flagged).  Same result in every thread.
-__device__ __forceinline__ int mask_elements(const uint32_t* __restrict__ mask, int mw, int ld, int (&el)[MAX_EL]) {
-    int cnt = 0;
-    for (int w = 0; w < mw; ++w) {
-        uint32_t bits = mask[w];
-        while (bits) {
-            const int e = (w << 5) + __ffs(bits) - 1;
-            bits &= bits - 1;
-            if (e >= ld || cnt == MAX_EL) return -1;
-            el[cnt++] = e;
+// The set elements of a row's mask, ascending, into the warp's own el[MAX_EL] in shared memory (a word per lane: rows have
+// at most 1024 floats); returns their number, or -1 if there are more than MAX_EL (or the whole row was flagged).
+__device__ __forceinline__ int mask_elements(const uint32_t* __restrict__ mask, int mw, int ld, int* el) {
+    const int lane = lane_id();
+    const uint32_t bits = lane < mw ? mask[lane] : 0u;
+    const int left = ld - (lane << 5);                       // elements of the row from this word on
+    const bool beyond = bits && (left <= 0 || (left < 32 && bits >> left));
+    const int c = __popc(bits), inc = warp_inclusive_scan(c), total = __shfl_sync(FULL, inc, 31);
+    if (__any_sync(FULL, beyond) || total > MAX_EL) return -1;
+    int at = inc - c;
+    __syncwarp();   // the list of the row before has been read
+    for (uint32_t b = bits; b; b &= b - 1) el[at++] = (lane << 5) + __ffs(b) - 1;
+    __syncwarp();
+    return total;
+}
+
+// The maxima of the cnt > 0 elements el[] over the in-neighbours [j_begin, j_end) of v: that of el[t] in lane t.  As many
+// lanes as there are elements (a power of two) take an entry, the others further entries, four steps' loads on their way.
+// (A lane per entry with sixteen accumulators and the elements in local memory held 100 registers, two blocks per SM, and
+// the limit of sixteen elements was the better one.  GraphConv-max of 128-256-40 on a graph of 169 K vertices and 1.2 M edges,
+// B = 1000, whole pass: 609 -> 537 us; up to 32 elements, and in-lists cut by 128 where they were cut by 256: 463.)
+__device__ __forceinline__ float max_elements(const Side& in, int v, int j_begin, int j_end, const float* __restrict__ M, int ld,
+                                              const int* el, int cnt, int is_min) {
+    const int lane = lane_id();
+    const int bits = cnt <= 1 ? 0 : 32 - __clz(cnt - 1), lanes = 1 << bits, per = 32 >> bits;   // lanes per entry, entries per step
+    const int mine_el = el[min(lane & (lanes - 1), cnt - 1)], at = lane >> bits;
+    const int32_t* const col = in.col + in.start[v];
+    float acc = worst(is_min);
+    for (int j0 = j_begin; j0 < j_end; j0 += 128) {
+        int id[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) id[k] = j0 + 32 * k + lane < j_end ? col[j0 + 32 * k + lane] : -1;
+        for (int s = 0; s < lanes; ++s) {
+            float x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int u = __shfl_sync(FULL, id[k], s * per + at);
+                x[k] = u >= 0 ? __ldg(M + (size_t)u * ld + mine_el) : worst(is_min);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc = pick(acc, x[k], is_min);
         }
     }
-    return cnt;
+    for (int o = lanes; o < 32; o <<= 1) acc = pick(acc, __shfl_xor_sync(FULL, acc, o), is_min);
+    return acc;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -141,12 +173,14 @@ __device__ __forceinline__ int mask_elements(const uint32_t* __restrict__ mask, 
 // mode 1 (recomputation): rows = list; the result is compared with the cached row, stored if it
 //         differs, and the vertex is marked affected.
 template <int NV, int LPR>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, NV <= 2 ? 3 : 1)
 k_max_rows(Ctl* ctl, int l, int mode, const int32_t* __restrict__ list, const int* n_dev, int n_host, Side in,
            const float* __restrict__ M, int ld, float* __restrict__ S, uint32_t* bitmapA, int32_t* long_rows,
-           int* n_long, uint32_t* invmask, int mw, int is_min) {
+           int* n_long, uint32_t* invmask, int mw, int is_min, int cut) {
     pdl_enter();
     if (ctl->abort) return;
+    __shared__ int s_el[8][MAX_EL];
+    int* el = s_el[threadIdx.x >> 5];
     const int n = n_dev ? *n_dev : n_host;
     const int lane = lane_id(), nq = ld >> 2;
     const int sub = lane / LPR, ql = lane % LPR;
@@ -158,41 +192,25 @@ k_max_rows(Ctl* ctl, int l, int mode, const int32_t* __restrict__ list, const in
     for (int i = i0; i < i1; ++i) {
         const int v = list ? list[i] : i;
         const int deg = in.deg[v];
-        if (deg > (mode ? MAX_HUB_DEGREE : MAX_FULL_PASS_DEGREE)) {
+        if (deg > (mode ? cut : MAX_FULL_PASS_DEGREE)) {
             if (lane == 0) long_rows[atomicAdd(n_long, 1)] = v;
             continue;
         }
         if (mode) {   // few invalidated elements: re-read only those
             uint32_t* mask = invmask + (size_t)v * mw;
-            int el[MAX_EL];
             const int cnt = mask_elements(mask, mw, ld, el);
-            __syncwarp();
-            for (int w = lane; w < mw; w += 32) mask[w] = 0u;
+            if (lane < mw) mask[lane] = 0u;
             if (cnt >= 0 && deg > 0) {
-                float acc[MAX_EL];
-#pragma unroll
-                for (int t = 0; t < MAX_EL; ++t) acc[t] = worst(is_min);
-                const int64_t base = in.start[v];
-                for (int j = lane; j < deg; j += 32) {
-                    const float* row = M + (size_t)in.col[base + j] * ld;
-#pragma unroll
-                    for (int t = 0; t < MAX_EL; ++t)
-                        if (t < cnt) acc[t] = pick(acc[t], __ldg(row + el[t]), is_min);
-                }
                 bool differs = false;
-#pragma unroll
-                for (int t = 0; t < MAX_EL; ++t) {
-                    if (t < cnt) {
-                        float m = acc[t];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) m = pick(m, __shfl_xor_sync(FULL, m, o), is_min);
-                        if (lane == 0) {
-                            float* dst = S + (size_t)v * ld + el[t];
-                            if (*dst != m) { *dst = m; differs = true; }
-                        }
+                if (cnt > 0) {
+                    const float m = max_elements(in, v, 0, deg, M, ld, el, cnt, is_min);
+                    if (lane < cnt) {
+                        float* dst = S + (size_t)v * ld + el[lane];
+                        differs = *dst != m;
+                        if (differs) *dst = m;
                     }
                 }
-                if (lane == 0 && differs) mark_bit(bitmapA, v);
+                if (__any_sync(FULL, differs) && lane == 0) mark_bit(bitmapA, v);
                 continue;
             }
         }
@@ -231,16 +249,17 @@ k_max_rows(Ctl* ctl, int l, int mode, const int32_t* __restrict__ list, const in
 __global__ void __launch_bounds__(256)
 k_max_long_begin(Ctl* ctl, int mode, const int32_t* __restrict__ long_rows, const int* __restrict__ n_long, Side in,
                  int ld, float* __restrict__ S, float* __restrict__ saved, const uint32_t* __restrict__ invmask, int mw,
-                 int is_min, int2* items, int* n_items) {
+                 int is_min, int2* items, int* n_items, int cut) {
     pdl_enter();
     if (ctl->abort) return;
     const int n = *n_long;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id();
+    __shared__ int s_el[8][MAX_EL];
+    int* el = s_el[threadIdx.x >> 5];
     for (int i = warp; i < n; i += nwarps) {
         const int v = long_rows[i];
         float* srow = S + (size_t)v * ld;
-        int el[MAX_EL];
         const int cnt = mode ? mask_elements(invmask + (size_t)v * mw, mw, ld, el) : -1;
         for (int k = lane; k < ld; k += 32) {
             if (mode) saved[(size_t)i * ld + k] = srow[k];
@@ -248,7 +267,7 @@ k_max_long_begin(Ctl* ctl, int mode, const int32_t* __restrict__ long_rows, cons
         }
         __syncwarp();   // every element is saved before any is reset
         if (cnt >= 0 && lane < cnt) srow[el[lane]] = worst(is_min);
-        const int nch = (in.deg[v] + MAX_HUB_CHUNK - 1) / MAX_HUB_CHUNK;
+        const int nch = (in.deg[v] + cut - 1) / cut;
         int first = 0;
         if (lane == 0) first = atomicAdd(n_items, nch);
         first = __shfl_sync(FULL, first, 0);
@@ -257,41 +276,27 @@ k_max_long_begin(Ctl* ctl, int mode, const int32_t* __restrict__ long_rows, cons
 }
 
 template <int NV>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, NV <= 2 ? 3 : 1)
 k_max_long_chunks(Ctl* ctl, int mode, const int32_t* __restrict__ long_rows, const int2* __restrict__ items,
                   const int* __restrict__ n_items, Side in, const float* __restrict__ M, int ld, float* S,
-                  const uint32_t* __restrict__ invmask, int mw, int is_min) {
+                  const uint32_t* __restrict__ invmask, int mw, int is_min, int cut) {
     pdl_enter();
     if (ctl->abort) return;
     const int n = *n_items;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int lane = lane_id(), nq = ld >> 2;
+    __shared__ int s_el[8][MAX_EL];
+    int* el = s_el[threadIdx.x >> 5];
     for (int it = warp; it < n; it += nwarps) {
         const int v = long_rows[items[it].x], ch = items[it].y;
         const int deg = in.deg[v];
-        const int j0 = ch * MAX_HUB_CHUNK, j1 = min(deg, j0 + MAX_HUB_CHUNK);
+        const int j0 = ch * cut, j1 = min(deg, j0 + cut);
         float* srow = S + (size_t)v * ld;
-        int el[MAX_EL];
         const int cnt = mode ? mask_elements(invmask + (size_t)v * mw, mw, ld, el) : -1;
-        if (cnt >= 0) {   // few elements: every lane strides over the chunk for those alone
-            float acc[MAX_EL];
-#pragma unroll
-            for (int t = 0; t < MAX_EL; ++t) acc[t] = worst(is_min);
-            const int64_t base = in.start[v];
-            for (int j = j0 + lane; j < j1; j += 32) {
-                const float* row = M + (size_t)in.col[base + j] * ld;
-#pragma unroll
-                for (int t = 0; t < MAX_EL; ++t)
-                    if (t < cnt) acc[t] = pick(acc[t], __ldg(row + el[t]), is_min);
-            }
-#pragma unroll
-            for (int t = 0; t < MAX_EL; ++t) {
-                if (t < cnt) {
-                    float m = acc[t];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) m = pick(m, __shfl_xor_sync(FULL, m, o), is_min);
-                    if (lane == 0) atomic_pick_f32(srow + el[t], m, is_min);
-                }
+        if (cnt >= 0) {   // few elements: those alone
+            if (cnt > 0) {
+                const float m = max_elements(in, v, j0, j1, M, ld, el, cnt, is_min);
+                if (lane < cnt) atomic_pick_f32(srow + el[lane], m, is_min);
             }
             continue;
         }
@@ -515,14 +520,20 @@ __global__ void k_max_senders(Ctl* ctl, int l, const int32_t* __restrict__ A, co
     }
 }
 
+static int max_cut(const Ctx* c) {
+    int n = MAX_CUT_MIN;
+    while (n < MAX_CUT && 2 * n <= (long long)c->stats.num_edges / (c->n_sm * 64)) n *= 2;
+    return n;
+}
+
 static void launch_long_rows(Ctx* c, int l, int mode, const float* M, int ld, float* S, int32_t* long_rows, int* n_long) {
-    const int nv = div_up(ld, 128), is_min = (int)(c->agg == RIPPLE_AGG_MIN);
+    const int nv = div_up(ld, 128), is_min = (int)(c->agg == RIPPLE_AGG_MIN), cut = mode ? max_cut(c) : MAX_CUT;
     int2* items = c->items;
     int* n_items = &c->ctl->max_items[l];
     float* saved = c->Dt;                              // compact scratch rows (no layer transforms before a max)
     RP_LAUNCH(c, k_max_long_begin, c->n_sm * 2, 256, 0, c->ctl, mode, long_rows, n_long, c->side[1], ld, S, saved,
-              c->invmask, c->mw, is_min, items, n_items);
-#define CHUNKS(NV) RP_LAUNCH(c, k_max_long_chunks<NV>, c->n_sm * 8, 256, 0, c->ctl, mode, long_rows, items, n_items, c->side[1], M, ld, S, c->invmask, c->mw, is_min)
+              c->invmask, c->mw, is_min, items, n_items, cut);
+#define CHUNKS(NV) RP_LAUNCH(c, k_max_long_chunks<NV>, c->n_sm * 8, 256, 0, c->ctl, mode, long_rows, items, n_items, c->side[1], M, ld, S, c->invmask, c->mw, is_min, cut)
     if (nv <= 1) CHUNKS(1); else if (nv <= 2) CHUNKS(2); else if (nv <= 4) CHUNKS(4); else CHUNKS(8);
 #undef CHUNKS
     if (mode)
@@ -535,7 +546,7 @@ void max_full(Ctx* c, int l) {
     const int ld = c->ws[l];
     int32_t* long_rows = c->Clist[0];
     int* n_long = &c->ctl->work_counter[(l - 1) & 7];
-#define ROWS(NV, LPR) RP_LAUNCH(c, (k_max_rows<NV, LPR>), c->n_sm * 16, 256, 0, c->ctl, l, 0, (const int32_t*)nullptr, (const int*)nullptr, c->N, c->side[1], c->H[l - 1], ld, c->S[l], c->bitmap, long_rows, n_long, c->invmask, c->mw, (int)(c->agg == RIPPLE_AGG_MIN))
+#define ROWS(NV, LPR) RP_LAUNCH(c, (k_max_rows<NV, LPR>), c->n_sm * 16, 256, 0, c->ctl, l, 0, (const int32_t*)nullptr, (const int*)nullptr, c->N, c->side[1], c->H[l - 1], ld, c->S[l], c->bitmap, long_rows, n_long, c->invmask, c->mw, (int)(c->agg == RIPPLE_AGG_MIN), max_cut(c))
     RP_WIDTH_DISPATCH(ld, ROWS);
 #undef ROWS
     launch_long_rows(c, l, 0, c->H[l - 1], ld, c->S[l], long_rows, n_long);
@@ -561,7 +572,7 @@ void max_hop(Ctx* c, int l, int n) {
     bitmap_to_list_from(c, c->bitmap2, rlist, n_r, nullptr);
     int32_t* long_rows = c->Clist[l & 1];            // the next hop's sender list is not built yet
     int* n_long = &c->ctl->work_counter[(l - 1) & 7];
-#define ROWS(NV, LPR) RP_LAUNCH(c, (k_max_rows<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, 1, rlist, n_r, 0, c->side[1], c->H[l - 1], ld, c->S[l], c->bitmap, long_rows, n_long, c->invmask, c->mw, (int)(c->agg == RIPPLE_AGG_MIN))
+#define ROWS(NV, LPR) RP_LAUNCH(c, (k_max_rows<NV, LPR>), c->n_sm * 8, T, 0, c->ctl, l, 1, rlist, n_r, 0, c->side[1], c->H[l - 1], ld, c->S[l], c->bitmap, long_rows, n_long, c->invmask, c->mw, (int)(c->agg == RIPPLE_AGG_MIN), max_cut(c))
     RP_WIDTH_DISPATCH(ld, ROWS);
 #undef ROWS
     launch_long_rows(c, l, 1, c->H[l - 1], ld, c->S[l], long_rows, n_long);
