@@ -102,7 +102,7 @@ cudaError_t graph_build(Ctx* c, const int32_t* src, const int32_t* dst, const fl
         Side& sd = c->side[s];
         sd.base_end = (int64_t)c->ctl_host->pool_next[s];
         sd.col_size = sd.base_end + pool_edges;
-        if ((e = cudaMalloc(&sd.col, sizeof(int32_t) * (size_t)std::max<int64_t>(sd.col_size, 4) + 4))) return e;
+        if ((e = cudaMalloc(&sd.col, sizeof(int32_t) * (size_t)(std::max<int64_t>(sd.col_size, 4) + 4)))) return e;
         if (c->weighted && (e = cudaMalloc(&sd.w, sizeof(float) * (size_t)std::max<int64_t>(sd.col_size, 4)))) return e;
     }
     if (E > 0) RP_LAUNCH(c, k_fill_rows, grid_e, T, 0, src, dst, weight, E, N, out, in);

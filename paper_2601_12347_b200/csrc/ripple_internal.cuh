@@ -374,7 +374,7 @@ void senders_release(Ctx* c, int l);                    // clear posmap entries 
 
 // scatter.cu
 void spmm_full(Ctx* c, int l);                          // S^l for every vertex (bootstrap)
-void sweep_prepare();                                   // one-time kernel attributes (not allowed inside a stream capture)
+void sweep_prepare(const Ctx* c);                                   // one-time kernel attributes (not allowed inside a stream capture)
 bool sweep_may_pay(const Ctx* c, int l, bool no_history);   // the sweeping form belongs into the chain of hop l
 void bitmap_to_list_from(Ctx* c, uint32_t* bitmap, int32_t* list, int* count_dev, unsigned long long* pull_work);
 // monotonic.cu (max aggregation, Sec. 3.4.2)

@@ -773,24 +773,27 @@ static size_t sweep_smem(int filter_words, bool wgt) {
     return sizeof(uint32_t) * (size_t)filter_words + (size_t)(sweep_threads<NV>() / 32) * (size_t)(wgt ? RowQueue<true>::bytes(RG_CAP) : RowQueue<false>::bytes(RG_CAP));
 }
 
-void sweep_prepare() {
+// One-time attributes of the instances that this context's layers launch (setting them loads a kernel, half a millisecond).
+void sweep_prepare(const Ctx* c) {
+    for (int l = 1; l <= c->L; ++l) {
+        const bool sums = c->weighted || c->src_norm;
+        // the rows that many lists name are served by L1, so the sums ask for as much of it as their queues leave
+#define PREP(NV, WGT)                                                                                              \
+    do {                                                                                                           \
+        cudaFuncSetAttribute(k_sum_rows<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);           \
+        cudaFuncSetAttribute(k_sum_rows_long<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);      \
+    } while (0)
+        RP_PIECES_DISPATCH(c->ws[l], sums, PREP);
+#undef PREP
+        if (c->n_local > 0) continue;
 #define PREP(NV, WGT)                                                                                                                              \
     do {                                                                                                                                           \
-        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));        \
-        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));   \
+        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));      \
+        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT)); \
     } while (0)
-    PREP(1, false); PREP(2, false); PREP(4, false); PREP(8, false);
-    PREP(1, true); PREP(2, true); PREP(4, true); PREP(8, true);
+        RP_PIECES_DISPATCH(c->ws[l], c->weighted, PREP);
 #undef PREP
-    // the rows that many lists name are served by L1, so these kernels ask for as much of it as their queues leave
-#define PREP(NV, WGT)                                                                                                            \
-    do {                                                                                                                         \
-        cudaFuncSetAttribute(k_sum_rows<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);                         \
-        cudaFuncSetAttribute(k_sum_rows_long<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);                    \
-    } while (0)
-    PREP(1, false); PREP(2, false); PREP(4, false); PREP(8, false);
-    PREP(1, true); PREP(2, true); PREP(4, true); PREP(8, true);
-#undef PREP
+    }
 }
 
 static void launch_sweep(Ctx* c, int l, const int32_t* senders, const float* D, const RecMsgs& recs) {
