@@ -587,6 +587,22 @@ void max_senders_build(Ctx* c, int l) {
     scan_degrees(c, senders, &c->ctl->nC[l], 0, c->side[0].deg, c->coff, &c->ctl->E[l + 1]);
 }
 
-void max_prepare() {}
+// One-time attributes of the instances that this context's layers launch: behind a tensor-core update these kernels would
+// find 28 KB of L1 for the ids and rows that they share.
+void max_prepare(const Ctx* c) {
+    for (int l = 1; l <= c->L; ++l) {
+        const int ld = c->ws[l], nv = div_up(ld, 128);
+#define PREP(NV, LPR)                                                                                                      \
+    do {                                                                                                                   \
+        cudaFuncSetAttribute(k_max_messages<NV, LPR>, cudaFuncAttributePreferredSharedMemoryCarveout, 10);               \
+        cudaFuncSetAttribute(k_max_rows<NV, LPR>, cudaFuncAttributePreferredSharedMemoryCarveout, 10);                   \
+    } while (0)
+        RP_WIDTH_DISPATCH(ld, PREP);
+#undef PREP
+#define PREP(NV) cudaFuncSetAttribute(k_max_long_chunks<NV>, cudaFuncAttributePreferredSharedMemoryCarveout, 10)
+        if (nv <= 1) PREP(1); else if (nv <= 2) PREP(2); else if (nv <= 4) PREP(4); else PREP(8);
+#undef PREP
+    }
+}
 
 }  // namespace rp

@@ -243,7 +243,6 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
         }
         tc_prepare();
         narrow_prepare();
-        max_prepare();
         CK(cudaMallocHost(&c->ctl_host, sizeof(Ctl)));
         memset(c->ctl_host, 0, sizeof(Ctl));
         memset(c->stage_host, 0, c->stage_bytes);
@@ -373,7 +372,8 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
                 CK(cudaMemcpy(ly.b2, b2.data(), sizeof(float) * b2.size(), cudaMemcpyHostToDevice));
             }
         }
-        if (!c->attention && !rp_monotonic(agg)) sweep_prepare(c);
+        if (rp_monotonic(agg)) max_prepare(c);
+        else if (!c->attention) sweep_prepare(c);
         for (int l = 0; l <= L; ++l) {
             max_ld = std::max(max_ld, c->ld[l]);
             CK(dev_alloc(&c->H[l], (size_t)N * c->ld[l], 0));

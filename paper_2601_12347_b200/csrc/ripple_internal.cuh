@@ -381,7 +381,7 @@ void bitmap_to_list_from(Ctx* c, uint32_t* bitmap, int32_t* list, int* count_dev
 void max_full(Ctx* c, int l);                           // bootstrap: cached maxima of every vertex
 void max_hop(Ctx* c, int l, int n);                     // messages <old, new>, recomputation of invalidated sinks
 void max_senders_build(Ctx* c, int l);                  // rows of A_l whose embedding changed, with their out-degree prefix
-void max_prepare();
+void max_prepare(const Ctx* c);
 void choose_direction(Ctx* c, int l);                   // delta or rebuilding form of hop l (device-side decision)
 void scatter_layer(Ctx* c, int l, int n);               // delta messages of hop l into dS^l
 void regather_layer(Ctx* c, int l);                     // rebuilding form: S^l rows of A_l gathered anew
