@@ -32,7 +32,7 @@ from paper_2601_12347_b200 import inputs as I  # noqa: E402
 # captures of dram__bytes_read.sum + dram__bytes_write.sum; profiles/dram_traffic_dense_full_size_ncu.txt):
 #   last-hop push scatter of dense-2l (k_scatter_push_packed<12>, rows of 48 floats), three launches of
 #   18.6 M - 20.6 M messages: 79.4 - 79.9 bytes per message;
-#   rebuilding gather of dense-3l's last hop (k_regather + k_spmm_hubs, rows of 48 floats, 122 M in-edges):
+#   rebuilding gather of dense-3l's last hop (taken of the kernels before k_sum_rows, rows of 48 floats, 122 M in-edges):
 #   6.47 GB per pass = 53 bytes per in-edge.
 # A launch's traffic is the per-unit figure times the units it processed: same graph, same kernel, same
 # row width, so traffic grows in proportion to the messages (resp. in-edges).
@@ -393,7 +393,7 @@ def run_ours(args, rank, world, local_rank):
                 "traffic": traffic,
                 "frac_hbm": (traffic / 1e9 / (sc_ms / K / 1e3) / hbm_peak) if (traffic and sc_ms > 0) else None,
                 "hbm_peak": hbm_peak, "hbm_peak_source": f"of {peak_kind}",
-                "kernel": f"{'k_scatter_gather' if pulls * 2 > K else 'k_scatter_push'} (hop {L}, row width {ld_last} floats)",
+                "kernel": f"{'k_sweep' if pulls * 2 > K else 'k_scatter_push'} (hop {L}, row width {ld_last} floats)",
                 "pull_steps": int(pulls),
                 "ms_per_launch": sc_ms / K,
                 "messages_per_launch": msgs,
@@ -445,7 +445,7 @@ def run_ours(args, rank, world, local_rank):
             "bound": "l2-gather", "achieved": got, "peak": pk, "unit": "GB/s", "frac": got / pk, "traffic": traffic,
             "frac_hbm": (traffic / 1e9 / (ms / 1e3) / hbm_peak) if traffic else None,
             "hbm_peak": hbm_peak, "hbm_peak_source": f"of {peak_kind}",
-            "kernel": f"k_regather + k_spmm_hubs (hop {L}, row width {ld_last} floats)",
+            "kernel": f"k_sum_rows + k_sum_rows_long (hop {L}, row width {ld_last} floats)",
             "ms_per_launch": ms, "in_edges_per_launch": edges, "rebuilt_steps": int(rebuilt),
             "note": "the last hop rebuilds the affected aggregates from their in-lists; achieved = in-edges x row bytes / "
                     "time of the two gather kernels; peak = probe of L2 row gathers on a 64 MB window"}
@@ -551,7 +551,7 @@ def run_table(args):
                     "bootstrap_ms": boot, "full_recompute_ms": full_ms}
             if hop["rebuilt"][L] > 0:
                 # the dominant kernels of a rebuilding hop: the gather over the in-lists of the affected sinks
-                # (k_regather for short lists, k_spmm_hubs for the chunks of long ones).  It is bounded by the
+                # (k_sum_rows for tiles of short lists, k_sum_rows_long for the pieces of long ones).  It is bounded by the
                 # rate at which L2 serves row gathers: achieved = in-edges x row bytes per second, peak = the
                 # library's gather probe (same lane layout, no index traffic at all) on an L2-resident window
                 # of 64 MB; the same probe on a window of the source matrix's size (uniformly random rows, so
@@ -564,7 +564,7 @@ def run_table(args):
                 pk_big = edges * ldw * 4 / 1e9 / (ripple.probe_gather_rate(w.n, ldw, int(edges)) / 1e3)
                 per_edge = NCU_DRAM_BYTES_PER_IN_EDGE.get((name.split("-")[0], ldw))
                 line["last_hop_gather"] = {
-                    "bound": "l2-gather", "kernel": f"k_regather + k_spmm_hubs (hop {L}, row width {ldw} floats)",
+                    "bound": "l2-gather", "kernel": f"k_sum_rows + k_sum_rows_long (hop {L}, row width {ldw} floats)",
                     "ms": ms, "in_edges": edges, "achieved_GBps": got, "peak_GBps": pk, "frac": got / pk,
                     "probe_uniform_rows_matrix_sized_GBps": pk_big,
                     "traffic": per_edge * edges if per_edge else None,

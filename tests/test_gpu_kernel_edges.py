@@ -28,8 +28,8 @@ def apply_and_check(rp, orc, ups, rows, L, slack=0.0):
 
 
 # Tensor-core form of the layer update: K chunks of 32 (31, 32, 33, and four / five of them: the weights stay in shared
-# memory up to 128), column groups of 128, the widths for which it is taken (113 to 256; narrower and wider ones are fp32
-# sums), row tiles of 128 and the 1024 rows from which it is taken (n - 1, n and n + 1 of both), normalised sources, GIN's
+# memory up to 128), column groups of 128, the widths for which it is taken (113 to 256; up to 64 over 256 and more
+# entries there is a form in pieces, see test_gpu_narrow_products; others are fp32 sums), row tiles of 128 and the 1024 rows from which it is taken (n - 1, n and n + 1 of both), normalised sources, GIN's
 # summed operand.
 TC_MODELS = {
     "sage_31_5_47": lambda: I.sage_model([31, 5, 47], I.AGG_MEAN),
@@ -66,7 +66,7 @@ def test_row_updates_at_the_edges_of_their_tiles(env, name):
 
 
 # A walk that adds into rows of half a gigabyte is made twice, over the lower and the upper half of the ids (330 K rows of
-# 256 floats and three messages per row are past the line); the pulled hop marks its sinks by ticket.
+# 256 floats and three messages per row are past the line); the swept hop reads every in-list instead.
 @pytest.mark.parametrize("kind", ["sage-push", "sage-pull", "weighted-push", "attention"])
 def test_walks_over_rows_that_outgrow_the_cache(env, kind):
     ripple, Oracle = env
