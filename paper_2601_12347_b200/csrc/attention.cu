@@ -353,7 +353,14 @@ k_att_gather(Ctl* ctl, int l, const int2* __restrict__ items, int chunk, Side in
             nx.request(run, in, f0 + RG_WINDOW);
             rg_walk<NV, true, true>(g, q, min(RG_WINDOW, run.total - f0), Hprev, ld_h, S, acc);
         }
-        rg_finish_one<NV>(g, S + (size_t)v * ld, acc);   // (columns d .. ld_h - 1 of a row of h are zeros)
+        // columns d .. ld_h - 1 of a row of h are zeros, and what an overflowed weight makes of them belongs into no sum:
+        // the first of them is the denominator's
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int left = d - 4 * (g.ql + 32 * k);
+            if (left < 4) acc[k] = make_float4(left > 0 ? acc[k].x : 0.f, left > 1 ? acc[k].y : 0.f, left > 2 ? acc[k].z : 0.f, 0.f);
+        }
+        rg_finish_one<NV>(g, S + (size_t)v * ld, acc);
         den = warp_sum(den);
         if (lane == 0) atomicAdd(S + (size_t)v * ld + d, den);
     }

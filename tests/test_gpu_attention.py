@@ -180,3 +180,32 @@ def test_bad_attention_layers_are_refused(env):
     model.layers[1].d_out = 8
     with pytest.raises(Exception):
         ripple.Ripple(n, src, dst, X, model, I.make_weights(I.gat_model(12, 2, d_att=4), 1))
+
+
+@pytest.mark.parametrize("d", [44, 45, 46, 47, 48, 129, 131, 132])
+def test_overflowed_weights_stay_visible(env, d):
+    """A logit beyond the range of exp in fp32 gives an infinite weight and an infinite denominator: the rows it reaches are
+    NaN whatever the width, in a whole-graph pass and in rows recomputed by a batch, and all others are as ever."""
+    ripple, _ = env
+    n = 400
+    src, dst = I.er_graph(n, 2400, 9)
+    model = I.gat_model(d, 1)
+    W = I.make_weights(model, 9)
+    W[0]["bb"] = np.zeros_like(W[0]["bb"])                    # the source alone decides
+    q = W[0]["Wa"].astype(np.float64) @ W[0]["ba"].astype(np.float64)
+    X = I.features(n, d, 9)
+    huge = (300.0 * q / float(q @ q)).astype(np.float32)     # s_u = 300: exp overflows in fp32
+    X[5] = huge
+    rp = ripple.Ripple(n, src, dst, X, model, W)
+    reached = np.zeros(n, dtype=bool)
+    reached[dst[src == 5]] = True
+    assert reached.any() and not reached.all()
+    H = rp.embeddings(1).cpu().numpy()
+    assert np.isnan(H[reached]).all() and np.isfinite(H[~reached]).all()
+    ups = np.zeros(1, dtype=I.UPDATE_DTYPE)
+    ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, 6, 0
+    rp.apply_batch(ups, huge[None])
+    reached[dst[src == 6]] = True
+    H = rp.embeddings(1).cpu().numpy()
+    assert np.isnan(H[reached]).all() and np.isfinite(H[~reached]).all()
+    rp.close()
