@@ -164,8 +164,12 @@ typedef struct {
                              throughout.  AUTO: outputs of 113 to 256 columns over 1024 and more rows are
                              computed on the tensor cores as products of tf32-split operands (2-norm error
                              against fp64 3.6e-7 at 100 inputs, 7e-7 at 256, 1.5e-6 at 602; fp32 sums:
-                             1.8e-7, 2.9e-7, 4.4e-7), all others as fp32 sums.  TF32: the same outputs as plain tf32
-                             products (1e-3)                                                             */
+                             1.8e-7, 2.9e-7, 4.4e-7); outputs of up to 64 columns over 256 and more inputs
+                             and 1024 and more rows (GIN's first product excepted) on the tensor cores from
+                             operands in three bf16 parts, all 24 bits, with an error no larger than that
+                             of fp32 sums (7.4e-8 at 256 inputs, 1.0e-7 at 602); all others as fp32 sums.
+                             TF32: the outputs of 113 to 256 columns as plain tf32 products (1e-3), the
+                             others as in AUTO                                                           */
     int32_t timing;       /* non-zero: record per-stage CUDA-event times into ripple_stats                  */
     int32_t pre_transform;/* 0: a layer not wider than its input applies its neighbour matrix to the sender
                              rows before the scatter (messages and the cached aggregate then have the

@@ -45,7 +45,6 @@ namespace rp {
 constexpr int TC_COLS = 128;     // output columns per group (= TMEM lanes)
 constexpr int TC_KC = 32;        // floats per K chunk: one 128-byte swizzle row
 constexpr int TC_TILE = 128;     // affected rows per tile
-constexpr int TC_PIECE = 16;     // entries of K whose large products the form for narrow outputs adds up in tensor memory
 // Loader threads: sixteen warps where the weights stream, eight where they stay (whose epilogue, with a cached projection
 // to read for every row, needs the registers more).
 __host__ __device__ constexpr int tc_loaders(bool resident, bool pieces) { return pieces ? 128 : resident ? 256 : 512; }
@@ -116,14 +115,23 @@ __device__ __forceinline__ void tc_mma_tf32(uint32_t tmem_d, uint64_t adesc, uin
         ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
+__device__ __forceinline__ void tc_mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
                  ::"r"(smem_u32(bar)) : "memory");
 }
 
-// instruction descriptor: fp32 accumulate, tf32 x tf32, both K-major, N = rows, M = 128
-__host__ __device__ constexpr uint32_t tc_idesc(int rows) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(rows >> 3) << 17) | ((uint32_t)(TC_COLS >> 4) << 24);
+// instruction descriptor: fp32 accumulate, tf32 x tf32 (type 2) or bf16 x bf16 (type 1), both K-major, N = rows, M = 128
+__host__ __device__ constexpr uint32_t tc_idesc(int rows, uint32_t type = 2) {
+    return (1u << 4) | (type << 7) | (type << 10) | ((uint32_t)(rows >> 3) << 17) | ((uint32_t)(TC_COLS >> 4) << 24);
 }
 
 // byte offset of 16-byte chunk c (0..7) of row r inside a K-major SWIZZLE_128B tile
@@ -141,6 +149,28 @@ __device__ __forceinline__ float4 tc_lds(uint32_t a) {
 }
 __device__ __forceinline__ void tc_sts(uint32_t a, float4 v) {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+
+__device__ __forceinline__ void tc_sts2(uint32_t a, uint32_t x, uint32_t y) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+
+// x0 and x1 (in the upper half) as two parts in bf16, cut and rounded; both leave what the part lacks, exact in fp32.  (The
+// first part is cut: rounded, entries near the largest would become infinite.)
+__device__ __forceinline__ uint32_t bf16_left(float& x0, float& x1, uint32_t part) {
+    x0 -= __uint_as_float(part << 16);
+    x1 -= __uint_as_float(part & 0xffff0000u);
+    return part;
+}
+__device__ __forceinline__ uint32_t bf16_cut(float& x0, float& x1) {
+    uint32_t d;
+    asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(x1), "f"(x0));
+    return bf16_left(x0, x1, d);
+}
+__device__ __forceinline__ uint32_t bf16_round(float& x0, float& x1) {
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(x1), "f"(x0));
+    return bf16_left(x0, x1, d);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -195,11 +225,17 @@ __device__ __forceinline__ T tc_pick(const T (&own)[N], int k) {
 // still in flight.
 // RESIDENT: the weights stay in shared memory; else they stream.
 // SUM: the row operand is alpha h + scale S (GIN), two rows per entry.
-// PIECES: narrow outputs, whose products were fp32 sums before and are no less exact here (see tc_weights_build).  What the
-// tensor core adds up at full size is 16 entries of K (two additions): the accumulator of the large products is handed over
-// that often, and its pieces meet in the epilogue's registers, in fp32; the small products gather over the whole tile.
+// PIECES: narrow outputs, whose products are fp32 sums on SIMT and no less exact here, dense rows or sparse ones (see
+// tc_weights_build).  Rows and weights are cut into three parts in bf16, 8 bits each: all 24 bits of an entry.  One product
+// is large, that of the first parts, 16 bits wide, so that what the tensor core's rounding towards zero takes of a sum of
+// them is small; its accumulator is handed over with every chunk and the chunks meet in the epilogue's registers, in fp32.
+// The seven small products (all but that of the third parts, 2^-33 relative) gather over the whole tile.  In a stage, a
+// row's 128 bytes hold the first part and the second, the other half of the stage the third and 64 bytes of nothing.
 // Lanes 0..63 are the columns of the first problem, lanes 64..127 those of the second, which reads the same rows.  (The
 // epilogue's 64 sums per thread leave registers for four loader warps.)
+// Measured: 2.4 M rows, K = 256, two products of 48 columns 1.19 ms (fp32 sums 3.43).  Bound by the chain loaders, products,
+// epilogue with two accumulators between them: hand-overs every 16 entries 1.43 ms; the loaders' stores without bank
+// conflicts nothing.
 template <bool RESIDENT, bool SUM, bool PIECES>
 __global__ void __launch_bounds__(tc_threads(RESIDENT, PIECES), 1)
 k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
@@ -266,7 +302,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
         // thread: piece c of the rows rb + RSTEP it of every chunk.  A chunk travels as asynchronous copies straight into
         // its stage of the high operand, NH - 1 chunks ahead; when it has landed, the thread that asked for a piece reads
         // it back, takes what the tensor core will not see of it -- it reads the upper 19 bits of an entry -- and stores
-        // that as the low operand.  (Row pieces held in registers across the barrier waits took 1.9 us per chunk, most
+        // that as the low operand; with PIECES the three parts take the place of the piece and of its neighbours' in the row.  (Row pieces held in registers across the barrier waits took 1.9 us per chunk, most
         // of it one warp's chain of dependent instructions.)
         const int c = tid & 7, rb = tid >> 3;
         const bool from_s = p.a_mode == A_AGG || SUM;
@@ -354,6 +390,21 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 float4 x[ITS];
 #pragma unroll
                 for (int it = 0; it < ITS; ++it) x[it] = tc_lds(hi + it * (RSTEP * 128));
+                if constexpr (PIECES) {
+                    const uint32_t to = hi - tc_swz(rb, c) + tc_swz(rb, c >> 1) + 8 * (c & 1);
+                    __syncwarp();   // a row's pieces, with eight lanes of this warp, have been read
+#pragma unroll
+                    for (int it = 0; it < ITS; ++it) {
+                        const uint32_t at = to + it * (RSTEP * 128);
+                        float4& e = x[it];
+                        uint32_t lower = bf16_cut(e.x, e.y), upper = bf16_cut(e.z, e.w);
+                        tc_sts2(at, lower, upper);
+                        lower = bf16_round(e.x, e.y), upper = bf16_round(e.z, e.w);
+                        tc_sts2(at ^ 64, lower, upper);
+                        lower = bf16_round(e.x, e.y), upper = bf16_round(e.z, e.w);
+                        tc_sts2(at + X_HALF, lower, upper);
+                    }
+                } else {
                 if constexpr (SUM) {
 #pragma unroll
                     for (int it = 0; it < ITS; ++it) {
@@ -369,6 +420,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 for (int it = 0; it < ITS; ++it)
                     tc_sts(lo + it * (RSTEP * 128), make_float4(x[it].x - tf32_seen(x[it].x), x[it].y - tf32_seen(x[it].y),
                                                                 x[it].z - tf32_seen(x[it].z), x[it].w - tf32_seen(x[it].w)));
+                }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&full_x[s]);
@@ -443,7 +495,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
             for (int d = 0; d < DEPTH; ++d) fetch(d, tc_pick<OWN>(v_next, d * BLK / 32), (d * BLK) & 31);
         }
         bool ok = true;
-        int sg = 0;                         // accumulators handed over so far: one per tile, with PIECES one per piece of K
+        int sg = 0;                         // accumulators handed over so far: one per tile, with PIECES one per chunk
         for (int lt = 0; lt < my_tiles && ok; ++lt) {
             const int r0 = tile_row(lt) + HALF * half;
 #pragma unroll
@@ -573,7 +625,7 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 for (int r = 0; r < BLK; ++r)
                     tc_store_if(r < live, reinterpret_cast<float*>(reinterpret_cast<char*>(hout) + (uint64_t)v[r] * ld_bytes), h[r]);
             };
-            const int parts = PIECES ? (K + TC_PIECE - 1) / TC_PIECE : 1;
+            const int parts = PIECES ? nchunks : 1;
             float sum[PIECES ? BLOCKS : 1][BLK];
             for (int part = 0; part < parts; ++part, ++sg) {
                 const int b = sg & 1;
@@ -587,18 +639,21 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
 #pragma unroll
                             for (int r = 0; r < HALF; ++r) sum[r / BLK][r % BLK] = 0.f;
                         }
-                        auto add = [&](uint32_t from) {
+                        auto add = [&](uint32_t from, bool small) {   // (an infinite entry has no parts: its small products are NaN)
 #pragma unroll
                             for (int r0_ = 0; r0_ < HALF; r0_ += 32) {
                                 uint32_t x[32];
                                 tc_load32(x, from + (uint32_t)r0_);
                                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                                for (int r = 0; r < 32; ++r) sum[(r0_ + r) / BLK][(r0_ + r) % BLK] += __uint_as_float(x[r]);
+                                for (int r = 0; r < 32; ++r) {
+                                    float& h = sum[(r0_ + r) / BLK][(r0_ + r) % BLK];
+                                    if (!small || fabsf(h) < INFINITY) h += __uint_as_float(x[r]);
+                                }
                             }
                         };
-                        add(t_row + (uint32_t)(b * BUF));
-                        if (part == parts - 1) add(t_row + (uint32_t)(2 * TILE + (lt & 1) * TILE));
+                        add(t_row + (uint32_t)(b * BUF), false);
+                        if (part == parts - 1) add(t_row + (uint32_t)(2 * TILE + (lt & 1) * TILE), true);
                     } else {
 #pragma unroll 1
                         for (int blk = 0; blk < BLOCKS; ++blk) {
@@ -643,9 +698,10 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                     if (!ok) return;
                     tc_fence_after();
                     d_addr = tmem_base + (uint32_t)(b * BUF);
+                    // (a tile's small products may go where the tile before the last had them: its last chunk has been drained)
                     d_corr = PIECES ? tmem_base + (uint32_t)(2 * TILE + (lt & 1) * TILE) : d_addr + TILE;
                 };
-                if (!PIECES && kc == 0) begin();
+                if (PIECES || kc == 0) begin();
                 if (!ok) break;
                 if (RESIDENT) sw = kc;
                 bool there = true;
@@ -659,43 +715,38 @@ k_update_rows_tc(Ctl* ctl, const __grid_constant__ UpdPair pair) {
                 tc_fence_after();
                 const uint64_t xh = dx0 + (uint64_t)((uint32_t)s * (X_BYTES >> 4));
                 const uint64_t wh = dw0 + (uint64_t)((uint32_t)sw * (TC_W_BYTES >> 4)), wl = wh + (TC_W_HALF >> 4);
-                if constexpr (PIECES) {
-                    // (a tile's small products may go where the tile before the last had them: its last piece has been drained)
-#pragma unroll 1
-                    for (int j0 = 0; j0 < TC_KC / 8 && 8 * j0 < left; j0 += TC_PIECE / 8) {
-                        begin();
-                        if (!ok) break;
-                        if (lead) {
-#pragma unroll
-                            for (int i = 0; i < TC_PIECE / 8; ++i) {
-                                const int j = j0 + i;
-                                if (8 * j < left) {
-                                    tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, idesc, i != 0);
-                                    tc_mma_tf32(d_corr, wh + 2 * j, xh + (X_HALF >> 4) + 2 * j, idesc, (kc | j) != 0);
-                                    tc_mma_tf32(d_corr, wl + 2 * j, xh + 2 * j, idesc, 1u);
-                                }
-                            }
-                            if (j0 + TC_PIECE / 8 >= TC_KC / 8 || 8 * (j0 + TC_PIECE / 8) >= left) tc_commit(&empty[s]);
-                            if (!(withhold && lt == 0)) tc_commit(&acc_full[b]);
-                        }
-                        __syncwarp();
-                    }
-                    if (!ok) break;
-                } else {
-                const bool last = kc == nchunks - 1;
+                const bool last = PIECES || kc == nchunks - 1;   // of what this accumulator takes
                 if (lead) {
+                    if constexpr (PIECES) {
+                        constexpr uint32_t bf16 = tc_idesc(TILE, 1);
 #pragma unroll
-                    for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
-                        if (8 * j < left) {
-                            tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, x3 ? idesc_wide : idesc, (kc | j) != 0);
-                            if (x3) tc_mma_tf32(d_corr, wl + 2 * j, xh + 2 * j, idesc, 1u);
+                        for (int j = 0; j < TC_KC / 16; ++j) {     // one MMA K step = 16 entries = 32 bytes
+                            if (16 * j < left) {
+                                const uint64_t x1 = xh + 2 * j, x2 = x1 + 4, x_3 = x1 + (X_HALF >> 4);
+                                const uint64_t w1 = wh + 2 * j, w2 = w1 + 4, w3 = wl + 2 * j;
+                                tc_mma_bf16(d_addr, w1, x1, bf16, j != 0);
+                                tc_mma_bf16(d_corr, w1, x2, bf16, (kc | j) != 0);
+                                tc_mma_bf16(d_corr, w2, x1, bf16, 1u);
+                                tc_mma_bf16(d_corr, w2, x2, bf16, 1u);
+                                tc_mma_bf16(d_corr, w1, x_3, bf16, 1u);
+                                tc_mma_bf16(d_corr, w3, x1, bf16, 1u);
+                                tc_mma_bf16(d_corr, w2, x_3, bf16, 1u);
+                                tc_mma_bf16(d_corr, w3, x2, bf16, 1u);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < TC_KC / 8; ++j) {     // one MMA K step = 8 floats = 32 bytes
+                            if (8 * j < left) {
+                                tc_mma_tf32(d_addr, wh + 2 * j, xh + 2 * j, x3 ? idesc_wide : idesc, (kc | j) != 0);
+                                if (x3) tc_mma_tf32(d_corr, wl + 2 * j, xh + 2 * j, idesc, 1u);
+                            }
                         }
                     }
                     tc_commit(&empty[s]);
                     // (diagnostic: with tc_withhold the first tile is never reported finished, so that
                     // the epilogue's bounded wait runs out and the status path can be exercised)
                     if (last && !(withhold && lt == 0)) tc_commit(&acc_full[b]);
-                }
                 }
                 __syncwarp();
                 if (++s == NH) { s = 0; ph ^= 1; }
@@ -774,18 +825,18 @@ void tc_prepare() {
 }
 
 // The weights (row-major K x ldw) as the kernel copies them: per column group and K chunk, the group's 128 columns as rows
-// of 32 K entries, first rounded to tf32, then the remainders (likewise rounded), in the swizzled layout of the operand.
+// of 32 K entries, first rounded to tf32, then the remainders (likewise rounded), in the swizzled layout of the operand;
+// for the form in pieces as three parts in bf16, laid out as the rows' are.
 //
-// Which outputs have them, and from how many rows the form is taken (RP_TC_MIN_ROWS), is a line of precision.  The form is
-// the faster one from 512 rows on, also for narrow outputs (whole-graph pass of one layer, K = 256, 256 columns: 512 rows
-// 39 us, fp32 sums 46; 1024: 39 / 52; 32 768: 94 / 321), but two to three times less exact than fp32 sums (see the top of the
-// file).  Outputs of 113 to 256 columns over 1024 and more rows have always been split products, and less exact ones than
-// these; all others were fp32 sums and lose nothing: up to 64 columns the large products are summed in pieces, where K is
-// long enough for the fp32 sum to be the less exact one.  Error against fp64, 2-norm, rows ~ N(0, 1) / rectified, pieces and
-// fp32 sums: K = 192 1.9e-7 / 1.9e-7 and 2.5e-7 / 1.8e-7, K = 256 2.0e-7 / 1.9e-7 and 2.9e-7 / 2.0e-7, K = 602 2.1e-7 / 2.1e-7
-// and 4.4e-7 / 3.1e-7 (in pieces of 32 entries 2.2e-7 / 2.1e-7 at K = 256).  2.4 M rows, K = 256, two products of 48 columns:
-// 3.43 -> 1.29 ms; one of 40 columns over 80 K rows 125 -> 93 us.  Bound by shared memory: a chunk's weights and rows are
-// written, split and read by three products, twelve times the bytes of its rows.
+// Which outputs have them, and from how many rows the form is taken (RP_TC_MIN_ROWS), is a line of precision.  The tf32 form
+// is the faster one from 512 rows on (whole-graph pass of one layer, K = 256, 256 columns: 512 rows 39 us, fp32 sums 46;
+// 1024: 39 / 52; 32 768: 94 / 321), but two to three times less exact than fp32 sums (see the top of the file).  Outputs of
+// 113 to 256 columns over 1024 and more rows have always been split products, and less exact ones than these; all others
+// were fp32 sums and lose nothing: up to 64 columns the form in pieces takes them.  Its error against fp64, 2-norm, and that
+// of the fp32 sum, by the entries of a row that are not zero (N(0, 1); K = 256 and 602, 5 to 64 columns alike; neighbouring
+// entries or scattered ones): 1 entry 2.5e-8 / 2.5e-8, 2 2.6e-8 / 3.1e-8, 4 2.6e-8 / 4.0e-8, 16 3.3e-8 / 7.4e-8, 64 5.1e-8 / 1.4e-7,
+// all of 256 7.4e-8 / 2.9e-7, of 602 1.0e-7 / 4.4e-7; rectified rows 6.2e-8 / 2.1e-7 and 8.8e-8 / 3.0e-7.
+// One of 40 columns over 80 K rows: 89 us, fp32 sums 125.
 // W2: a second matrix over the same rows, for the form in pieces.
 cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const float* W2) {
     *out = TcW{};
@@ -799,6 +850,16 @@ cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const flo
         memcpy(&v, &bits, 4);
         return v;
     };
+    auto bf16_part = [](float& left, bool round) {   // (as bf16_cut and bf16_round)
+        uint32_t bits;
+        memcpy(&bits, &left, 4);
+        if (round) bits += 0x7fffu + (bits >> 16 & 1u);
+        bits &= 0xffff0000u;
+        float part;
+        memcpy(&part, &bits, 4);
+        left -= part;
+        return (uint16_t)(bits >> 16);
+    };
     out->groups = (ldw + TC_COLS - 1) / TC_COLS;
     out->chunks = (K + TC_KC - 1) / TC_KC;
     const size_t block = TC_W_BYTES / 4;
@@ -810,6 +871,15 @@ cudaError_t tc_weights_build(TcW* out, const float* W, int K, int ldw, const flo
                 const int col = j + m * (TC_COLS / 2);
                 const int g = col / TC_COLS, r = col - g * TC_COLS, kc = k / TC_KC, kk = k - kc * TC_KC;
                 float* blk = pack.data() + ((size_t)g * out->chunks + kc) * block;
+                if (pieces) {
+                    uint16_t* const to = reinterpret_cast<uint16_t*>(blk);
+                    const uint32_t first = tc_swz(r, kk >> 3) / 2 + (kk & 7);
+                    float left = x;
+                    to[first] = bf16_part(left, false);
+                    to[first ^ 32] = bf16_part(left, true);
+                    to[TC_W_HALF / 2 + first] = bf16_part(left, true);
+                    continue;
+                }
                 const uint32_t at = tc_swz(r, kk >> 2) / 4 + (kk & 3);
                 blk[at] = h;
                 blk[TC_W_HALF / 4 + at] = round_tf32(x - h);

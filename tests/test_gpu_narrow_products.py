@@ -1,6 +1,7 @@
-"""Products of at most 64 columns over 256 and more entries: the tensor-core form that sums pieces of 16 entries apart, at
-the edges of its rule (255 / 256 entries, 64 / 65 columns, 1023 / 1024 rows), of its pieces and chunks and of its tiles; two
-problems over the same rows side by side and single ones; and its error, which is no larger than that of fp32 sums."""
+"""Products of at most 64 columns over 256 and more entries: the tensor-core form that sums chunks of 32 entries apart, at
+the edges of its rule (255 / 256 entries, 64 / 65 columns, 1023 / 1024 rows), of its chunks and of its tiles; two
+problems over the same rows side by side and single ones; its error, which is no larger than that of fp32 sums, dense rows
+or sparse ones; and entries that have no parts."""
 import numpy as np
 import pytest
 
@@ -71,3 +72,60 @@ def test_no_less_exact_than_fp32_sums(env, K, cols):
         err.append(np.linalg.norm(got - ref) / np.linalg.norm(ref))
         rp.close()
     assert err[1] <= 1.1 * err[0], err
+
+
+def self_product(ripple, X, W, model, mode):
+    n = X.shape[0]
+    src = np.arange(n, dtype=np.int32)
+    rp = ripple.Ripple(n, src, (src + 1) % n, X, model, W, gemm_mode=mode)
+    got = rp.embeddings(1).cpu().numpy()
+    rp.close()
+    return got
+
+
+@pytest.mark.parametrize("K", [256, 602])
+@pytest.mark.parametrize("entries", [1, 2, 3, 4, 8, 16, 64])
+@pytest.mark.parametrize("near", [False, True])
+def test_sparse_rows_keep_the_bits_of_fp32(env, K, entries, near):
+    """Rows with a few entries that are not zero, scattered or side by side (across the middle of a chunk among them): a sum
+    of few terms has almost no rounding to hide behind, so operands held in fewer than 24 bits show (22 bits: 1.4e-7 where the
+    fp32 sum has 2.5e-8).  Both errors are at least that of one rounding and equal for one entry; a fiftieth for the luck of
+    the draw."""
+    ripple, _ = env
+    n, cols = 2048, 47
+    model = I.sage_model([K, cols])
+    W = I.make_weights(model, 5)
+    W[0]["Wb"] = np.zeros_like(W[0]["Wb"])
+    rng = np.random.default_rng(K + entries)
+    X = np.zeros((n, K), dtype=np.float32)
+    for i in range(n):
+        at = 32 * rng.integers(0, K // 32) + 16 - entries // 2 if near else 0
+        ids = np.arange(at, at + entries) % K if near else rng.choice(K, entries, replace=False)
+        X[i, ids] = rng.standard_normal(entries)
+    ref = X.astype(np.float64) @ W[0]["Wa"].astype(np.float64)
+    err = [np.linalg.norm(self_product(ripple, X, W, model, m) - ref) / np.linalg.norm(ref) for m in (ripple.GEMM_FP32, ripple.GEMM_AUTO)]
+    assert err[1] <= 1.02 * err[0], err
+
+
+def test_entries_without_parts(env):
+    """Infinite entries, NaN, and entries next to the largest: infinite, NaN and finite results where the fp32 sum has them."""
+    ripple, _ = env
+    n, K, cols = 2048, 300, 40
+    model = I.sage_model([K, cols])
+    W = I.make_weights(model, 6)
+    W[0]["Wb"] = np.zeros_like(W[0]["Wb"])
+    W[0]["Wa"][::3] = np.round(W[0]["Wa"][::3] * 64) / 64     # (weights with no second part, some of them zero)
+    rng = np.random.default_rng(1)
+    X = rng.standard_normal((n, K)).astype(np.float32)
+    at = rng.integers(0, K, n)
+    big = np.finfo(np.float32).max
+    for i in range(n):
+        X[i, at[i]] = (np.inf, -np.inf, np.nan, big, -big, 1.0)[i % 6]
+    X[6::12, 7] = -np.inf                                     # two infinite entries
+    a, b = (self_product(ripple, X, W, model, m) for m in (ripple.GEMM_FP32, ripple.GEMM_AUTO))
+    assert np.array_equal(np.isnan(a), np.isnan(b)) and np.isnan(a).any()
+    assert np.array_equal(np.isposinf(a), np.isposinf(b)) and np.isposinf(a).any()
+    assert np.array_equal(np.isneginf(a), np.isneginf(b)) and np.isneginf(a).any()
+    f = np.isfinite(a)
+    scale = 1.0 + np.abs(a[f].astype(np.float64))
+    assert np.max(np.abs(a[f].astype(np.float64) - b[f]) / scale) <= 1e-5
