@@ -233,7 +233,7 @@ __device__ __forceinline__ T tc_pick(const T (&own)[N], int k) {
 // row's 128 bytes hold the first part and the second, the other half of the stage the third and 64 bytes of nothing.
 // Lanes 0..63 are the columns of the first problem, lanes 64..127 those of the second, which reads the same rows.  (The
 // epilogue's 64 sums per thread leave registers for four loader warps.)
-// Measured: 2.4 M rows, K = 256, two products of 48 columns 1.19 ms (fp32 sums 3.43).  Bound by the chain loaders, products,
+// Measured: 2.4 M rows, K = 256, two products of 48 columns 1.31 -> 1.23 ms (fp32 sums 3.43).  Bound by the chain loaders, products,
 // epilogue with two accumulators between them: hand-overs every 16 entries 1.43 ms; the loaders' stores without bank
 // conflicts nothing.
 template <bool RESIDENT, bool SUM, bool PIECES>
