@@ -141,12 +141,11 @@ typedef struct {
 /* How hop l brings the cached aggregates S^l up to date.  PUSH / PULL: delta messages (Sec. 3.3.1),
  * scattered along the senders' out-edges or gathered per sink by a sweep over the in-lists.
  * REGATHER: the aggregates of the affected vertices are rebuilt from their in-lists (the scoped
- * recomputation of Sec. 3.2, for this hop only).  AUTO: PUSH or, where the hop's size makes it the
- * cheaper way, a sweep, except that a hop whose senders own at least regather_threshold of all edges
- * rebuilds, and that a hop of wide messages (128 floats or more) from few senders gathers per sink
- * (chosen per hop from what the hop carried in the batch before: at least 2^20 messages, eight or more
- * per affected sink, sender rows of at most 32 MiB in all; the environment variable
- * RIPPLE_GATHER_MIN_WIDTH, read by ripple_create, replaces the 128: 0 = never). */
+ * recomputation of Sec. 3.2, for this hop only).  AUTO: PUSH or, where the messages that the hop
+ * carries make it the cheaper way, a sweep (decided on the device; the environment variable
+ * RIPPLE_GATHER_MIN_WIDTH, read by ripple_create, is the narrowest message in floats for which a
+ * sweep is considered, 0 = never), except that a hop whose senders own at least regather_threshold of
+ * all edges rebuilds. */
 typedef enum {
     RIPPLE_SCATTER_AUTO = 0, RIPPLE_SCATTER_PUSH = 1, RIPPLE_SCATTER_PULL = 2, RIPPLE_SCATTER_REGATHER = 3,
     RIPPLE_SCATTER_PUSH_BULK = 4 /* PUSH with one bulk reduction of the copy engine per message (cp.reduce.async.bulk)
@@ -208,8 +207,8 @@ typedef struct {
     int64_t affected[RIPPLE_MAX_LAYERS + 1];      /* |A_l|, l = 0..L                                      */
     int64_t senders[RIPPLE_MAX_LAYERS + 1];       /* |C_l|: vertices whose outgoing message changed       */
     int64_t active_edges[RIPPLE_MAX_LAYERS + 1];  /* l = 1..L: edges carrying a message at hop l          */
-    int32_t scatter_pull[RIPPLE_MAX_LAYERS + 1];  /* l = 1..L: 0 deltas (pushed or, by the device's
-                                                     choice, swept), 1 gathered per sink, 2 rebuilt       */
+    int32_t scatter_pull[RIPPLE_MAX_LAYERS + 1];  /* l = 1..L: 0 pushed, 1 gathered per sink (swept),
+                                                     2 rebuilt                                            */
     int64_t in_edges[RIPPLE_MAX_LAYERS + 1];      /* l = 1..L: in-edges of A_l (what a gather walks)      */
     int32_t message_width[RIPPLE_MAX_LAYERS + 1]; /* l = 1..L: floats per message / aggregate row (padded) */
     int64_t pool_used, pool_size;                 /* overflow pool, out-direction, in edges: handed out so far

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "sweep_rule.h"
+
 namespace rp {
 
 constexpr unsigned FULL = 0xffffffffu;
@@ -97,7 +99,6 @@ __device__ __forceinline__ int upper_row(const int64_t* a, int n, int64_t x) {
 // and then over the upper half of the ids, in the order of the tickets: more of the rows are then still in L2 when their
 // next message arrives.  (2.4 M rows of 48 floats, 20 M messages: whole chain 1.56 -> 1.49 ms; of 104 floats: 4.12 ->
 // 3.74; three and four passes are no better, eight are slower than one: every pass reads and sorts out all ids again.)
-constexpr long long WALK_TWICE = 160ll << 20;   // bytes of rows from which a walk is made twice
 struct TicketWalk {
     long long total, at;
     int chunk, next, *ticket;

@@ -235,11 +235,9 @@ extern "C" ripple_status ripple_create(const ripple_graph* g, const float* featu
             c->pdl = !(e && e[0] == '1');
         }
         {
-            // Hops whose messages are at least this wide gather per sink once they carry a million messages
-            // (measured on the dense graph, 256 floats: see scatter.cu); 0 = never.
+            // AUTO: hops whose messages are at least this wide may be swept; 0 = never.
             const char* e = getenv("RIPPLE_GATHER_MIN_WIDTH");
-            c->gather_min_width = e ? atoi(e) : 128;
-            c->gather_min_messages = 1 << 20;
+            c->gather_min_width = e ? atoi(e) : 1;
         }
         tc_prepare();
         narrow_prepare();
@@ -561,20 +559,12 @@ static void arm_rebuild(Ctx* c, int nb) {
                                        0.5 * (double)c->regather_threshold[l] * (double)c->stats.num_edges) &&
                     c->stats.num_edges + c->max_batch >= c->regather_min_messages;
         c->rebuild_armed[l] = armed;
-        // The gathering form of the delta scatter is chosen here, from what the hop carried in the batch before
-        // (any choice is correct; a hop that turns out small gathers over a small frontier).
-        bool gather = c->scatter_mode == RIPPLE_SCATTER_PULL;
-        if (c->scatter_mode == RIPPLE_SCATTER_AUTO && !rp_monotonic(c->agg) && !c->attention && c->n_local == 0 &&
-            c->gather_min_width > 0 && c->ws[l] >= c->gather_min_width && !no_history)
-            gather = c->stats.active_edges[l] >= c->gather_min_messages && c->stats.scatter_pull[l] != 2 &&
-                     // the senders' delta rows stay in L2 with room to spare, and a sink's one addition replaces many
-                     (double)c->stats.senders[l - 1] * c->ws[l] * sizeof(float) <= 32.0 * (1 << 20) &&
-                     c->stats.active_edges[l] >= 8 * c->stats.affected[l];
-        c->pull_hop[l] = gather;
-        // The sweeping form goes into the chain beside the push where the hop may carry enough messages for it (the device
-        // then chooses by what it does carry).
-        c->sweep_armed[l] = !gather && c->scatter_mode == RIPPLE_SCATTER_AUTO && !rp_monotonic(c->agg) && !c->attention && c->n_local == 0 &&
-                            sweep_may_pay(c, l, no_history);
+        // Likewise the sweeping form, beside the push: the device chooses between them by what the hop does carry.
+        c->sweep_armed[l] = c->scatter_mode == RIPPLE_SCATTER_PULL ||
+                            (c->scatter_mode == RIPPLE_SCATTER_AUTO && !rp_monotonic(c->agg) && !c->attention && c->n_local == 0 &&
+                             c->gather_min_width > 0 && c->ws[l] >= c->gather_min_width &&
+                             sweep_may_pay(!no_history, (double)c->stats.active_edges[l], (double)c->stats.senders[l - 1],
+                                           (double)c->stats.num_edges, (double)c->N, c->ws[l]));
     }
 }
 
@@ -594,7 +584,7 @@ static int chain_size(const Ctx* c, int nb) {
 static uint64_t chain_key(const Ctx* c, int ng) {
     uint64_t key = ((uint64_t)ng << 3) | (c->may_expand ? 1 : 0) | (c->has_opw ? 2 : 0) | (c->few_rows_form ? 4 : 0);
     key = 2 * key + (c->front_one_block ? 1 : 0);
-    for (int l = 1; l <= c->L; ++l) key = 8 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->pull_hop[l] ? 2 : 0) + (c->sweep_armed[l] ? 4 : 0);
+    for (int l = 1; l <= c->L; ++l) key = 4 * key + (c->rebuild_armed[l] ? 1 : 0) + (c->sweep_armed[l] ? 2 : 0);
     for (int l = 0; l <= c->L; ++l) key = 2 * key + (c->tc_armed[l] ? 1 : 0);
     return key;
 }
@@ -787,7 +777,7 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
             s.affected[l] = h.nA[l];
             s.senders[l] = h.nC[l];
             s.active_edges[l] = l ? (int64_t)h.E[l] + h.n_rec : 0;
-            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l] == 1;   // (a sweep that the device chose delivers deltas like the push)
+            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l];
             s.in_edges[l] = (int64_t)h.pull_work[l];
             s.message_width[l] = l ? c->ws[l] : 0;
             s.rows_rebuilt[l] = h.n_rebuilt[l];

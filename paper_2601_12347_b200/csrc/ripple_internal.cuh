@@ -200,10 +200,8 @@ struct Ctx {
     int scatter_mode, gemm_mode, timing;
     int rebuild_armed[RP_MAXL + 1];   // per hop: the rebuilding form is enqueued for this batch (see arm_rebuild)
     int tc_armed[RP_MAXL + 1];        // updates over the rows of A_l (or C_l) carry their tensor-core form in this batch
-    int pull_hop[RP_MAXL + 1];        // per hop: the delta scatter of this batch gathers per sink instead of pushing (see arm_rebuild)
-    int sweep_armed[RP_MAXL + 1];     // per hop: the sweeping form is enqueued beside the push, the device chooses
-    int gather_min_width;             // narrowest message row (floats) whose hop may gather (environment RIPPLE_GATHER_MIN_WIDTH)
-    long long gather_min_messages;    // ... if the hop delivered at least this many messages in the batch before
+    int sweep_armed[RP_MAXL + 1];     // per hop: the sweeping form is enqueued, in AUTO beside the push (the device chooses)
+    int gather_min_width;             // narrowest message row (floats) whose hop may be swept in AUTO, 0 = none (environment RIPPLE_GATHER_MIN_WIDTH)
     long long batches_done;
     int last_nb;
     int debug_tc_withhold;   // diagnostic (environment RIPPLE_DEBUG_TC_WITHHOLD=1, read by every call that updates rows)
@@ -375,7 +373,6 @@ void senders_release(Ctx* c, int l);                    // clear posmap entries 
 // scatter.cu
 void spmm_full(Ctx* c, int l);                          // S^l for every vertex (bootstrap)
 void sweep_prepare(const Ctx* c);                                   // one-time kernel attributes (not allowed inside a stream capture)
-bool sweep_may_pay(const Ctx* c, int l, bool no_history);   // the sweeping form belongs into the chain of hop l
 void bitmap_to_list_from(Ctx* c, uint32_t* bitmap, int32_t* list, int* count_dev, unsigned long long* pull_work);
 // monotonic.cu (max aggregation, Sec. 3.4.2)
 void max_full(Ctx* c, int l);                           // bootstrap: cached maxima of every vertex

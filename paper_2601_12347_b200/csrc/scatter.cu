@@ -888,30 +888,10 @@ k_regather_rows(Ctl* ctl, int l, const Rec* __restrict__ rec, Side in, const int
     }
 }
 
-// Microseconds, fitted to whole hops: a push pays per float delivered (0.65 ps where the accumulator stays in L2, 0.79
-// where it does not) and per sender, whose list a warp takes up after the one before (0.8 ns); a sweep per edge of the graph
-// (5.5 ps) and per row added up (4 ps and 0.29 per float), and is taken where it saves a tenth: hops at the line lose the launch.  Measured, push / sweep: 0.99 M messages of 256 floats from 80 K
-// senders on a graph of 1.2 M edges 216 / 125 us, 1.1 M of 40 floats 120 / 62; 50 M of 44 floats from 10 K senders, 115 M
-// edges, 1436 / 1341; 26 M of 48 floats, 124 M edges, 1000 / 1110.
-__host__ __device__ inline bool sweep_pays(double msgs, double senders, double edges, double vertices, int width) {
-    const bool outgrows = vertices * width * 4.0 > (double)WALK_TWICE;
-    const double push = 5.0 + 1e-6 * msgs * width * (outgrows ? 0.79 : 0.65) + 0.8e-3 * senders;
-    const double sweep = 30.0 + 1e-6 * (5.5 * edges + msgs * (4.0 + 0.29 * width));
-    return sweep < 0.9 * push;
-}
-
-// (twice what the hop carried in the batch before: the chain holds both forms well before the line)
-bool sweep_may_pay(const Ctx* c, int l, bool no_history) {
-    const double edges = (double)c->stats.num_edges, vertices = (double)c->N;
-    if (no_history) return sweep_pays(edges, vertices, edges, vertices, c->ws[l]);
-    return sweep_pays(2.0 * (double)c->stats.active_edges[l], 2.0 * (double)c->stats.senders[l - 1], edges, vertices, c->ws[l]);
-}
-
 // Form of hop l, decided on the device once the senders and their out-degree sum are known.
 //
 // Delta form: the out-edges of the senders each carry one message, added to the sink's accumulator by vector reductions
-// (push), or every in-list is read and the senders' delta rows in it are summed in registers (sweep: chosen on the host, per
-// hop, for wide messages from few senders, or here where it costs less).
+// (push), or every in-list is read and the senders' delta rows in it are summed in registers (sweep).
 //
 // Rebuilding form: once the senders' out-edges are most of the graph, reading every in-edge of
 // the affected sinks once and overwriting their aggregates costs less than one reduction per
@@ -922,8 +902,10 @@ bool sweep_may_pay(const Ctx* c, int l, bool no_history) {
 // form is throughput-bound, and the edge-balanced push is the more parallel of the two (measured
 // on the sparse graph, 256 floats per row: 0.24 ms pushed, 0.26 to 0.47 ms rebuilt).
 //
-// Between push and sweep, where both are in the chain, the cheaper one is taken (see sweep_pays).
-__global__ void k_choose_direction(Ctl* ctl, int l, int mode, int gather, float threshold, long long min_messages, int sweep, int N,
+// Between push and sweep, where both are in the chain, the cheaper one is taken (see sweep_pays): what the batch before
+// carried says nothing about this one.  (Three layers on the graph of 124 M edges, one update after a thousand: hop 2 carries
+// 2 K messages of 256 floats, which a sweep chosen by the batch before took 0.5 ms for.)
+__global__ void k_choose_direction(Ctl* ctl, int l, int mode, float threshold, long long min_messages, int sweep, int N,
                                    int width) {
     pdl_enter();
     const int nC = ctl->nC[l - 1];
@@ -935,7 +917,7 @@ __global__ void k_choose_direction(Ctl* ctl, int l, int mode, int gather, float 
              msgs >= (unsigned long long)min_messages;
     }
     if (nC == 0 && ctl->n_rec == 0) re = 0;
-    ctl->pull[l] = gather ? 1 : sweep && sweep_pays((double)msgs, (double)nC, (double)ctl->num_edges, (double)N, width) ? 2 : 0;
+    ctl->pull[l] = mode == RIPPLE_SCATTER_PULL || (sweep && sweep_pays((double)msgs, (double)nC, (double)ctl->num_edges, (double)N, width));
     ctl->regather[l] = re;
 }
 
@@ -1022,11 +1004,10 @@ void fold_deltas(Ctx* c, int l) {
 
 void choose_direction(Ctx* c, int l) {
     // nothing to decide for a pushing hop: the control block's flags are already zero after its reset
-    if (!c->rebuild_armed[l] && !c->pull_hop[l] && !c->sweep_armed[l] &&
+    if (!c->rebuild_armed[l] && !c->sweep_armed[l] &&
         (c->scatter_mode == RIPPLE_SCATTER_AUTO || c->scatter_mode == RIPPLE_SCATTER_PUSH ||
          c->scatter_mode == RIPPLE_SCATTER_PUSH_BULK)) return;
-    RP_LAUNCH(c, k_choose_direction, 1, 1, 0, c->ctl, l, c->scatter_mode, (int)c->pull_hop[l],
-              c->rebuild_armed[l] ? c->regather_threshold[l] : -1.f, c->regather_min_messages, c->sweep_armed[l], c->N, c->ws[l]);
+    RP_LAUNCH(c, k_choose_direction, 1, 1, 0, c->ctl, l, c->scatter_mode, c->rebuild_armed[l] ? c->regather_threshold[l] : -1.f, c->regather_min_messages, c->sweep_armed[l], c->N, c->ws[l]);
 }
 
 // delta form of hop l (does nothing on the device if the hop rebuilds)
@@ -1054,7 +1035,7 @@ void scatter_layer(Ctx* c, int l, int n) {
     if (c->scatter_mode == RIPPLE_SCATTER_PUSH_BULK && !c->weighted && (size_t)8 * 2 * ld * sizeof(float) <= (48u << 10)) {
         RP_LAUNCH(c, k_scatter_push_bulk, grid, T, (size_t)8 * 2 * ld * sizeof(float), c->ctl, l, senders, c->coff,
                   c->side[0], Dm, ld, c->dS[l], c->bitmap);
-    } else if (!c->pull_hop[l] && c->scatter_mode != RIPPLE_SCATTER_REGATHER) {
+    } else if (c->scatter_mode != RIPPLE_SCATTER_PULL && c->scatter_mode != RIPPLE_SCATTER_REGATHER) {
 #define PACKED(NQ, WGT) RP_LAUNCH(c, (k_scatter_push_packed<NQ, WGT>), grid, T, 0, c->ctl, l, senders, c->coff, c->side[0], Dm, c->dS[l], c->bitmap, recs, c->N)
         if (ld == 48 && c->weighted) PACKED(12, true);
         else if (ld == 48) PACKED(12, false);
@@ -1065,7 +1046,7 @@ void scatter_layer(Ctx* c, int l, int n) {
         recs_done = true;
     }
 #undef PUSH
-    if (c->pull_hop[l] || c->sweep_armed[l]) {
+    if (c->sweep_armed[l]) {
         launch_sweep(c, l, senders, Dm, recs);
         recs_done = true;
     }

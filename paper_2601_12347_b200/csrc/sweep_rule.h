@@ -1,0 +1,36 @@
+// When a hop's messages are swept instead of pushed: plain C++, used on the host (is the sweep in the chain?) and on the
+// device (which of the two delivers?).
+//
+// Microseconds, fitted to whole hops: a push pays per float delivered (0.65 ps where the accumulator stays in L2, 0.79
+// where it does not) and per sender, whose list a warp takes up after the one before (0.8 ns); a sweep per edge of the graph
+// (5.5 ps) and per row added up (4 ps and 0.29 per float), and is taken where it saves a tenth: hops at the line lose the
+// launch.  Measured, push / sweep: 0.99 M messages of 256 floats from 80 K senders on a graph of 1.2 M edges 216 / 125 us,
+// 1.1 M of 40 floats 120 / 62; 50 M of 44 floats from 10 K senders, 115 M edges, 1436 / 1341; 26 M of 48 floats, 124 M edges,
+// 1000 / 1110.
+#pragma once
+
+#ifdef __CUDACC__
+#define RP_RULE __host__ __device__ inline
+#else
+#define RP_RULE inline
+#endif
+
+namespace rp {
+
+constexpr long long WALK_TWICE = 160ll << 20;   // bytes of rows from which a walk is made twice (see TicketWalk)
+
+// The device's choice, by what the hop does carry.
+RP_RULE bool sweep_pays(double msgs, double senders, double edges, double vertices, int width) {
+    const bool outgrows = vertices * width * 4.0 > (double)WALK_TWICE;
+    const double push = 5.0 + 1e-6 * msgs * width * (outgrows ? 0.79 : 0.65) + 0.8e-3 * senders;
+    const double sweep = 30.0 + 1e-6 * (5.5 * edges + msgs * (4.0 + 0.29 * width));
+    return sweep < 0.9 * push;
+}
+
+// The host's: both forms are in the chain if twice what the hop carried in the batch before would be swept (unknown: if all
+// edges from all vertices would).
+inline bool sweep_may_pay(bool known, double msgs, double senders, double edges, double vertices, int width) {
+    return known ? sweep_pays(2.0 * msgs, 2.0 * senders, edges, vertices, width) : sweep_pays(edges, vertices, edges, vertices, width);
+}
+
+}  // namespace rp

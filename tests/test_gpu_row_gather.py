@@ -110,3 +110,40 @@ def test_swept_and_pushed_hops_agree_where_the_device_chooses(env):
             assert np.max(np.abs(a - c) / (1 + np.abs(c))) <= 1e-4
     for rp in rps:
         rp.close()
+
+
+def feature_batch(rng, n, d, count):
+    vs = rng.choice(n, count, replace=False)
+    ups = np.zeros(count, dtype=I.UPDATE_DTYPE)
+    ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, vs, np.arange(count)
+    return ups, rng.standard_normal((count, d)).astype(np.float32)
+
+
+@pytest.mark.parametrize("min_width", [None, "0", "257"])
+def test_a_hop_is_swept_for_what_it_carries_not_for_the_batch_before(env, monkeypatch, min_width):
+    """Batches of 6000 and of one update in turn: hop 2 carries 1.5 M wide messages in the one, 2500 in the other, and is swept
+    in the one and pushed in the other; never swept where the least width excludes it."""
+    ripple, _ = env
+    if min_width is not None:
+        monkeypatch.setenv("RIPPLE_GATHER_MIN_WIDTH", min_width)
+    n, d = 30_000, 32
+    src, dst = I.er_graph(n, 1_500_000, 8)
+    model = I.sage_model([d, 256, 256])
+    X = I.features(n, d, 8)
+    W = I.make_weights(model, 8)
+    rps = [ripple.Ripple(n, src, dst, X, model, W, scatter_mode=m, regather_threshold=-1.0) for m in (ripple.SCATTER_AUTO, ripple.SCATTER_PUSH)]
+    rng = np.random.default_rng(8)
+    for count in (6000, 6000, 1, 6000, 1, 1, 6000):
+        ups, rows = feature_batch(rng, n, d, count)
+        for rp in rps:
+            rp.apply_batch(ups, rows)
+        st = rps[0].stats()
+        assert st["active_edges"][2] > (1 << 20) if count > 1 else st["active_edges"][2] < 10_000
+        assert list(st["scatter_pull"][1:3]) == [0, 1 if count > 1 and min_width is None else 0]
+        assert list(rps[1].stats()["scatter_pull"][1:3]) == [0, 0]
+        for l in range(3):
+            assert np.array_equal(rps[0].affected(l).cpu().numpy(), rps[1].affected(l).cpu().numpy())
+            a, c = (rp.embeddings(l).cpu().numpy() for rp in rps)
+            assert np.max(np.abs(a - c) / (1 + np.abs(c))) <= 1e-4
+    for rp in rps:
+        rp.close()

@@ -1,0 +1,56 @@
+"""When a hop is swept instead of pushed (csrc/sweep_rule.h, plain C++): the rule of the device and that of the host."""
+import os
+import subprocess
+
+import pytest
+
+from conftest import ROOT
+
+DRIVER = r"""
+#include <cstdio>
+#include "sweep_rule.h"
+// reads lines of: messages, senders, edges, vertices, width; prints for each 0/1 whether the device sweeps, and whether the
+// host has both forms in the chain of the batch after one that carried as much
+int main() {
+    double m, s, e, v;
+    int w;
+    while (std::scanf("%lf %lf %lf %lf %d", &m, &s, &e, &v, &w) == 5)
+        std::printf("%d%d\n", (int)rp::sweep_pays(m, s, e, v, w), (int)rp::sweep_may_pay(true, m, s, e, v, w));
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    d = tmp_path_factory.mktemp("sweep_rule")
+    (d / "driver.cpp").write_text(DRIVER)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", os.path.join(ROOT, "paper_2601_12347_b200", "csrc"),
+                           str(d / "driver.cpp"), "-o", str(d / "driver")])
+
+    def ask(hops):
+        out = subprocess.run([str(d / "driver")], input="\n".join(" ".join(map(str, h)) for h in hops), capture_output=True, text=True, check=True)
+        return [tuple(c == "1" for c in line) for line in out.stdout.split()]
+    return ask
+
+
+DENSE = (123_718_280, 2_449_029)
+
+
+def test_the_measured_hops_fall_on_their_side(rule):
+    swept = [(990_000, 80_000, 1_166_243, 169_343, 256), (1_100_000, 80_000, 1_166_243, 169_343, 40),
+             (20_000_000, 9_000, *DENSE, 256)]
+    pushed = [(26_000_000, 9_000, *DENSE, 48), (2_068, 3, *DENSE, 256), (1_500_000, 300, *DENSE, 256), (8_000, 200, *DENSE, 104)]
+    assert [r[0] for r in rule(swept)] == [True] * 3
+    assert [r[0] for r in rule(pushed)] == [False] * 4
+
+
+def test_what_the_device_may_sweep_is_in_the_chain(rule):
+    """A hop that is swept was in the chain if the batch before carried at least half as much, at every size."""
+    hops = [(m, m / k, e, v, w) for m in (1e4, 1e5, 1e6, 1e7, 1e8) for k in (10, 300, 10_000) for e, v in ((1.2e6, 1.7e5), DENSE)
+            for w in (16, 48, 104, 256, 1024) if m <= e]
+    half = [(m / 2, s / 2, e, v, w) for m, s, e, v, w in hops]
+    device = [r[0] for r in rule(hops)]
+    assert any(device) and not all(device)
+    for sweeps, before in zip(device, rule(half)):
+        assert not sweeps or before[1]
