@@ -796,10 +796,14 @@ void sweep_prepare(const Ctx* c) {
         else RP_WIDTH_DISPATCH(ld, PREP);
 #undef PREP
         if (c->n_local > 0) continue;
-#define PREP(NV, WGT)                                                                                                                              \
-    do {                                                                                                                                           \
-        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT));      \
-        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT)); \
+        // and the sweeps, for all but the filter and the queues of the one block
+#define PREP(NV, WGT)                                                                                                      \
+    do {                                                                                                                   \
+        const int smem = (int)sweep_smem<NV>(1 << (SWEEP_BITS - 5), WGT), share = div_up(100 * (smem + 1024), 228 << 10);  \
+        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);                         \
+        cudaFuncSetAttribute(k_sweep<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, share);                     \
+        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);                    \
+        cudaFuncSetAttribute(k_sweep_long<NV, WGT>, cudaFuncAttributePreferredSharedMemoryCarveout, share);                \
     } while (0)
         RP_PIECES_DISPATCH(c->ws[l], c->weighted, PREP);
 #undef PREP
