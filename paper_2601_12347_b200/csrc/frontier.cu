@@ -244,6 +244,43 @@ __device__ __forceinline__ void set_bit(uint32_t* bitmap, int v) {
     if (!(bitmap[v >> 5] & m)) atomicOr(&bitmap[v >> 5], m);
 }
 
+// A hop that sweeps only the lists of its frontier (see k_choose_direction) has it marked beforehand: sinks of net edge
+// changes, A_{l-1} for models with a self term, out-neighbours of the senders.
+constexpr int WALK_CHUNK = 256;  // edges per warp work item
+
+__global__ void k_mark_frontier(Ctl* ctl, int l, int self_term, const int32_t* __restrict__ senders,
+                                const int64_t* __restrict__ coff, Side out, const Rec* __restrict__ rec,
+                                const int32_t* __restrict__ A_prev, uint32_t* bitmap) {
+    pdl_enter();
+    if (ctl->abort || ctl->pull[l] != SWEEP_MARKED) return;
+    const int gtid = blockIdx.x * blockDim.x + threadIdx.x, gsize = gridDim.x * blockDim.x;
+    for (int i = gtid; i < ctl->n_rec; i += gsize) set_bit(bitmap, rec[i].v);
+    if (self_term)
+        for (int i = gtid; i < ctl->nA[l - 1]; i += gsize) set_bit(bitmap, A_prev[i]);
+    const int nC = ctl->nC[l - 1];
+    if (nC == 0) return;
+    const int64_t E = coff[nC];
+    const int lane = lane_id();
+    // (a hop that walks here does not push, so the push's counter is free)
+    TicketWalk deal(&ctl->walk_ticket[l], E, WALK_CHUNK / 4, WALK_CHUNK);
+    for (; deal.has(); deal.advance()) {
+        const int64_t e0 = deal.at, e1 = min(e0 + deal.chunk, E);
+        deal.take();
+        int i = upper_row(coff, nC, e0);
+        int64_t e = e0;
+        while (e < e1) {
+            const int64_t row_end = coff[i + 1];
+            if (row_end <= e) { ++i; continue; }
+            const int64_t seg_end = min(e1, row_end);
+            const int64_t base = out.start[senders[i]] + (e - coff[i]);
+            const int cnt = (int)(seg_end - e);
+            for (int j = lane; j < cnt; j += 32) set_bit(bitmap, out.col[base + j]);
+            e = seg_end;
+            ++i;
+        }
+    }
+}
+
 // Rebuilding hops mark bottom-up (the direction switch of a frontier search that has reached most
 // of the graph): v belongs to Out_new(C_{l-1}) iff one of its in-neighbours is a sender.  With the
 // senders owning most edges the first few probes of the position map settle almost every vertex,
@@ -304,9 +341,13 @@ void frontier_seed_features(Ctx* c, int n) {
     bitmap_to_list(c, c->A[0], &c->ctl->nA[0], nullptr);
 }
 
-// Where a rebuild is possible, marks the members of A_l bottom-up.  (Otherwise what delivers the messages marks their sinks,
-// and k_regather_rows the sinks of edge changes and A_{l-1} of models with a self term.)
+// Where a rebuild is possible, marks the members of A_l bottom-up, and where a sweep of their lists is, by a walk.  (Otherwise
+// what delivers the messages marks their sinks, and k_regather_rows the sinks of edge changes and A_{l-1} of models with a
+// self term.)
 void frontier_mark(Ctx* c, int l) {
+    if (c->scatter_mode == RIPPLE_SCATTER_PULL)
+        RP_LAUNCH(c, k_mark_frontier, RP_RESIDENT(c, k_mark_frontier, 256), 256, 0, c->ctl, l, (int)c->self_term,
+                  sender_list(c, l - 1), c->coff, c->side[0], c->rec, c->A[l - 1], c->bitmap);
     if (!c->rebuild_armed[l]) return;
     // the list A_l is not built yet: its buffer holds the queue of undecided long rows
     RP_LAUNCH(c, k_mark_bottom_up, RP_RESIDENT(c, k_mark_bottom_up, 256), 256, 0, c->ctl, l, c->N, c->side[1], c->posmap, c->bitmap, c->A[l],

@@ -777,7 +777,7 @@ extern "C" ripple_status ripple_apply_batch_weighted(ripple_ctx* ctx, const ripp
             s.affected[l] = h.nA[l];
             s.senders[l] = h.nC[l];
             s.active_edges[l] = l ? (int64_t)h.E[l] + h.n_rec : 0;
-            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l];
+            s.scatter_pull[l] = h.regather[l] ? 2 : h.pull[l] != PUSHED;
             s.in_edges[l] = (int64_t)h.pull_work[l];
             s.message_width[l] = l ? c->ws[l] : 0;
             s.rows_rebuilt[l] = h.n_rebuilt[l];

@@ -198,13 +198,16 @@ struct TileRun {
     }
 };
 
-// The lists of `cnt` sinks from position i0 of `list` (null: ids are positions), but for those of more than long_list entries.
+// The lists of `cnt` sinks from position i0 of `list` (null: ids are positions), but for those of more than long_list entries;
+// with `only`, those whose bit is set there.
 struct TileLists {
     int v, deg;
     int64_t start;
-    __device__ __forceinline__ TileLists(const Side& in, const int32_t* list, long long i0, int cnt) : v(0), deg(0), start(0) {
+    __device__ __forceinline__ TileLists(const Side& in, const int32_t* list, long long i0, int cnt, const uint32_t* only = nullptr)
+        : v(0), deg(0), start(0) {
         if (lane_id() < cnt) {
             v = list ? list[i0 + lane_id()] : (int)i0 + lane_id();
+            if (only && !(only[v >> 5] >> (v & 31) & 1u)) return;
             deg = in.deg[v];
             start = in.start[v];
         }

@@ -14,8 +14,8 @@
 // push: the out-edges of the senders are cut into equal chunks; a warp keeps the sender's delta
 //       row in registers and issues one 16-byte vector reduction per lane and edge (narrow rows:
 //       several edges per warp instruction).
-// sweep: the in-lists of all vertices are read, sources that are senders kept (a filter, then the position map),
-//       their delta rows summed in registers, and a sink's accumulator touched once.
+// sweep: the in-lists of all vertices, or of the marked ones, are read, sources that are senders kept (a filter, then the
+//       position map), their delta rows summed in registers, and a sink's accumulator touched once.
 #include "row_gather.cuh"
 
 #include <algorithm>
@@ -717,11 +717,14 @@ k_sweep(Ctl* ctl, int l, const __grid_constant__ Sweep a, const RecMsgs recs) {
     const RowLanes g(a.ld);
     float4 acc[NV];
     rg_zero<NV>(acc);
+    const uint32_t* const only = ctl->pull[l] == SWEEP_MARKED ? a.bitmap : nullptr;
     TileDeal deal(a.take == 32 ? &ctl->gather_ticket[l] : nullptr);
     for (int tile = deal.first();; tile = deal.next()) {
         const long long v0 = (long long)a.take * tile;
         if (v0 >= a.N) break;
-        const TileLists t(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0));
+        const int cnt = (int)min((long long)a.take, a.N - v0);
+        if (only && !(only[v0 >> 5] >> (v0 & 31) & (cnt < 32 ? (1u << cnt) - 1u : FULL))) continue;
+        const TileLists t(a.in, nullptr, v0, cnt, only);
         TileRun run = t.run(a.long_list);
         rg_queue_rest(t, tile, run.total, a.long_list, a.item, a.piece, a.items, &ctl->gather_items[l]);
         run.total = min(run.total, a.piece);
@@ -744,6 +747,7 @@ k_sweep_long(Ctl* ctl, int l, const __grid_constant__ Sweep a) {
     const RowLanes g(a.ld);
     float4 acc[NV];
     rg_zero<NV>(acc);
+    const uint32_t* const only = ctl->pull[l] == SWEEP_MARKED ? a.bitmap : nullptr;
     TicketWalk walk(&ctl->gather_long_ticket[l], n, 1, 4);
     for (; walk.has(); walk.advance()) {
         const int from = (int)walk.at, to = min(n, from + walk.chunk);
@@ -752,7 +756,7 @@ k_sweep_long(Ctl* ctl, int l, const __grid_constant__ Sweep a) {
         const int2 w = a.items[it];
         if (w.x < 0) {
             const long long v0 = (long long)a.take * (-1 - w.x);
-            TileRun run = TileLists(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0)).run(a.long_list);
+            TileRun run = TileLists(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0), only).run(a.long_list);
             run.total = min(run.total, (w.y + 1) * a.piece);
             const unsigned sinks = __reduce_or_sync(FULL, sweep_tile<NV, WGT>(g, run, a, filter, q, acc, w.y * a.piece));
             if (sinks && lane_id() == 0) atomicOr(&a.bitmap[v0 >> 5], sinks);
@@ -921,7 +925,9 @@ __global__ void k_choose_direction(Ctl* ctl, int l, int mode, float threshold, l
              msgs >= (unsigned long long)min_messages;
     }
     if (nC == 0 && ctl->n_rec == 0) re = 0;
-    ctl->pull[l] = mode == RIPPLE_SCATTER_PULL || (sweep && sweep_pays((double)msgs, (double)nC, (double)ctl->num_edges, (double)N, width));
+    if (mode == RIPPLE_SCATTER_PULL)
+        ctl->pull[l] = sweep_reads_all((double)msgs, (double)ctl->num_edges) ? SWEPT : SWEEP_MARKED;
+    else ctl->pull[l] = sweep && sweep_pays((double)msgs, (double)nC, (double)ctl->num_edges, (double)N, width) ? SWEPT : PUSHED;
     ctl->regather[l] = re;
 }
 

@@ -4,9 +4,9 @@
 // Microseconds, fitted to whole hops: a push pays per float delivered (0.65 ps where the accumulator stays in L2, 0.79
 // where it does not) and per sender, whose list a warp takes up after the one before (0.8 ns); a sweep per edge of the graph
 // (5.5 ps) and per row added up (4 ps and 0.29 per float), and is taken where it saves a tenth: hops at the line lose the
-// launch.  Measured, push / sweep: 0.99 M messages of 256 floats from 80 K senders on a graph of 1.2 M edges 216 / 125 us,
-// 1.1 M of 40 floats 120 / 62; 50 M of 44 floats from 10 K senders, 115 M edges, 1436 / 1341; 26 M of 48 floats, 124 M edges,
-// 1000 / 1110.
+// launch.  Measured, kernels of a hop, push / sweep: 1.0 M messages of 256 floats from 34 K senders on a graph of 1.2 M edges
+// 229 / 163 us, 1.1 M of 40 floats from 80 K senders 140 / 113; 49 M of 44 floats from 9 K senders, 115 M edges, 1455 / 1469;
+// 124 M edges: 24 M of 48 floats 956 / 1207 and of 256 5612 / 2141, 33 M of 128 floats 2134 / 1482.
 #pragma once
 
 #ifdef __CUDACC__
@@ -32,5 +32,14 @@ RP_RULE bool sweep_pays(double msgs, double senders, double edges, double vertic
 inline bool sweep_may_pay(bool known, double msgs, double senders, double edges, double vertices, int width) {
     return known ? sweep_pays(2.0 * msgs, 2.0 * senders, edges, vertices, width) : sweep_pays(edges, vertices, edges, vertices, width);
 }
+
+// What ctl->pull says of a hop.
+enum { PUSHED = 0, SWEPT = 1, SWEEP_MARKED = 2 };
+
+// Of a hop that is swept because the caller wants it (RIPPLE_SCATTER_PULL): every in-list of the graph, or only the lists of
+// its frontier, which a walk over the senders' out-lists marks first.  124 M edges, walk and sweep of the frontier / sweep of
+// everything: 9 messages of 100 floats 116 / 440 us, 22 K of 256 floats 250 / 480, 2.3 M 830 / 815, 19 M 1810 / 1630, 122 M of
+// 48 floats 4890 / 4170; 115 M edges: 0.4 M of 256 floats 1109 / 1070.
+RP_RULE bool sweep_reads_all(double msgs, double edges) { return 8.0 * msgs >= edges; }
 
 }  // namespace rp

@@ -147,3 +147,50 @@ def test_a_hop_is_swept_for_what_it_carries_not_for_the_batch_before(env, monkey
             assert np.max(np.abs(a - c) / (1 + np.abs(c))) <= 1e-4
     for rp in rps:
         rp.close()
+
+
+@pytest.mark.parametrize("agg", ["mean", "gcn", "weighted"])
+@pytest.mark.parametrize("n", [3000, 310_000, 600_001])     # tiles of 8 and of 32; ids that the filter holds and hashes
+def test_sweeps_of_the_frontiers_lists_and_of_all(env, n, agg):
+    """SCATTER_PULL: a hop that carries less than an eighth of the edges reads the lists of its frontier, marked beforehand;
+    with the hub among its senders (a third of the edges) all lists.  Feature updates, and edges that come and go."""
+    ripple, Oracle = env
+    d = 12
+    src, dst = lists_of_every_length(n, n % 1000)
+    have = set(zip(src.tolist(), dst.tolist()))
+    hub = n - 7
+    extra = [v for v in range(0, min(n, src.size // 2 + 200)) if v != hub and (hub, v) not in have]
+    src = np.concatenate([src, np.full(len(extra), hub, dtype=np.int32)])
+    dst = np.concatenate([dst, np.array(extra, dtype=np.int32)])
+    kw = {"edge_weights": I.edge_weights(src.size, 5)} if agg == "weighted" else {}
+    model = {"mean": I.sage_model([d, d, d, 8]), "gcn": I.graphconv_model([d, d, d, 8], I.AGG_WSUM_GCN),
+             "weighted": I.graphconv_model([d, d, d, 8], I.AGG_WSUM_EDGE)}[agg]
+    X = I.features(n, d, 3)
+    W = I.make_weights(model, 3)
+    rp = ripple.Ripple(n, src, dst, X, model, W, scatter_mode=ripple.SCATTER_PULL, pre_transform=False, **kw)
+    orc = Oracle(n, src, dst, X, model, W, **kw)
+    stream = I.UpdateStream(n, src, dst, d, 4)
+    rng = np.random.default_rng(n)
+    few = many = 0
+    for b in range(7):
+        if b in (2, 5):
+            ups = np.zeros(2, dtype=I.UPDATE_DTYPE)
+            ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, [hub, int(src[5])], [0, 1]
+            rows = rng.standard_normal((2, d)).astype(np.float32)
+        elif b in (0, 4):
+            vs = np.unique(rng.choice(src, 12 if b else 1))
+            ups = np.zeros(vs.size, dtype=I.UPDATE_DTYPE)
+            ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, vs, np.arange(vs.size)
+            rows = rng.standard_normal((vs.size, d)).astype(np.float32)
+        else:
+            ups, rows = stream.next_batch(30)
+        rp.apply_batch(ups, rows)
+        assert orc.apply_incremental(ups, rows) == 0
+        G.check_frontiers(rp, orc, 3)
+        st = rp.stats()
+        assert list(st["scatter_pull"][1:4]) == [1, 1, 1]
+        share = np.array(st["active_edges"][1:4]) * 8 >= st["num_edges"]
+        few, many = few + int((~share).sum()), many + int(share.sum())
+    assert few >= 3 and many >= 2, (few, many)
+    G.check_values(rp, orc.full(), 3, row_slack=GIN_ROW_SLACK if agg == "weighted" else 0.0)
+    rp.close()

@@ -9,13 +9,14 @@ from conftest import ROOT
 DRIVER = r"""
 #include <cstdio>
 #include "sweep_rule.h"
-// reads lines of: messages, senders, edges, vertices, width; prints for each 0/1 whether the device sweeps, and whether the
-// host has both forms in the chain of the batch after one that carried as much
+// reads lines of: messages, senders, edges, vertices, width; prints for each 0/1 whether the device sweeps, whether the
+// host has both forms in the chain of the batch after one that carried as much, and whether a sweep that the caller wants
+// reads every list
 int main() {
     double m, s, e, v;
     int w;
     while (std::scanf("%lf %lf %lf %lf %d", &m, &s, &e, &v, &w) == 5)
-        std::printf("%d%d\n", (int)rp::sweep_pays(m, s, e, v, w), (int)rp::sweep_may_pay(true, m, s, e, v, w));
+        std::printf("%d%d%d\n", (int)rp::sweep_pays(m, s, e, v, w), (int)rp::sweep_may_pay(true, m, s, e, v, w), (int)rp::sweep_reads_all(m, e));
     return 0;
 }
 """
@@ -54,3 +55,9 @@ def test_what_the_device_may_sweep_is_in_the_chain(rule):
     assert any(device) and not all(device)
     for sweeps, before in zip(device, rule(half)):
         assert not sweeps or before[1]
+
+
+def test_a_small_hop_does_not_read_the_whole_graph(rule):
+    small = [(m, 10, *DENSE, w) for m in (0, 9, 22_000, 2_300_000) for w in (48, 256)]
+    large = [(m, 10_000, *DENSE, w) for m in (20_000_000, 122_000_000) for w in (48, 256)]
+    assert not any(r[2] for r in rule(small)) and all(r[2] for r in rule(large))
