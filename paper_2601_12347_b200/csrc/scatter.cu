@@ -542,16 +542,19 @@ k_scatter_push_bulk(Ctl* ctl, int l, const int32_t* __restrict__ senders, const 
 // registers, so that a sink's accumulator row takes one addition where the push makes one per message.
 //
 // Whether an id is a sender's is first asked of a filter in shared memory, which every block fills from the sender list:
-// one bit per vertex on graphs of up to 2^20 of them, else one of 2^20 bits per id by a multiplicative hash; the position
+// one bit per vertex on graphs of up to 2^19 of them, else one of 2^19 bits per id by a multiplicative hash; the position
 // map, one trip to L2, is asked about the few that pass.  The delta rows are few and stay in L2.
 //
 // What bounds it: the requests that an SM's L1 takes (a bit of the filter per entry, a word of the position map per row,
 // two or three lines per row) and the trips to memory of a window, at half of the issue slots; 4.5 ps per entry without a row.
 // ---------------------------------------------------------------------------------------------
 constexpr int SWEEP_BITS = 19;
-// one block per SM: threads by the registers that the rows on their way take
+// One block per SM: as many threads as leave them the registers that the rows on their way and the ids of the next window
+// take, 102 where a lane has one or two pieces of a row (with 1024 and 768 threads 300 to 580 bytes a thread were spilled, now
+// 4 to 200, none at four pieces; eight spill 192 to 364, and 384 threads without are no faster).  49 M rows of 44 floats, 115 M
+// edges: 1469 -> 1269 us; 24 M of 256 floats, 124 M edges: 2141 -> 1988; 33 M of 128: 1482 -> 1261.
 template <int NV>
-__host__ __device__ constexpr int sweep_threads() { return NV == 1 ? 1024 : NV == 2 ? 768 : 512; }
+__host__ __device__ constexpr int sweep_threads() { return NV <= 2 ? 640 : 512; }
 
 struct Sweep {
     Side in;

@@ -5,8 +5,9 @@
 // where it does not) and per sender, whose list a warp takes up after the one before (0.8 ns); a sweep per edge of the graph
 // (5.5 ps) and per row added up (4 ps and 0.29 per float), and is taken where it saves a tenth: hops at the line lose the
 // launch.  Measured, kernels of a hop, push / sweep: 1.0 M messages of 256 floats from 34 K senders on a graph of 1.2 M edges
-// 229 / 163 us, 1.1 M of 40 floats from 80 K senders 140 / 113; 49 M of 44 floats from 9 K senders, 115 M edges, 1455 / 1469;
-// 124 M edges: 24 M of 48 floats 956 / 1207 and of 256 5612 / 2141, 33 M of 128 floats 2134 / 1482.
+// 230 / 164 us, 1.1 M of 40 floats from 80 K senders 135 / 110; 124 M edges: 24 M of 48 floats 968 / 1102 and of 256 5690 / 1990,
+// 33 M of 128 floats 2134 / 1261; 115 M edges: 39 M of 128 floats 4095 / 1728.  (Fitted before the sweep had its registers and
+// its L1: 49 M of 44 floats from 9 K senders, 115 M edges, 1451 / 1269, are still left to the push.)
 #pragma once
 
 #ifdef __CUDACC__
