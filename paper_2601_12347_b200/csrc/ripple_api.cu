@@ -563,8 +563,8 @@ static void arm_rebuild(Ctx* c, int nb) {
         c->sweep_armed[l] = c->scatter_mode == RIPPLE_SCATTER_PULL ||
                             (c->scatter_mode == RIPPLE_SCATTER_AUTO && !rp_monotonic(c->agg) && !c->attention && c->n_local == 0 &&
                              c->gather_min_width > 0 && c->ws[l] >= c->gather_min_width &&
-                             sweep_may_pay(!no_history, (double)c->stats.active_edges[l], (double)c->stats.senders[l - 1],
-                                           (double)c->stats.num_edges, (double)c->N, c->ws[l]));
+                             sweep_may_pay(!no_history, c->sweep_armed[l] != 0, (double)c->stats.active_edges[l],
+                                           (double)c->stats.senders[l - 1], (double)c->stats.num_edges, (double)c->N, c->ws[l]));
     }
 }
 

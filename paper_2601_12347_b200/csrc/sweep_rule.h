@@ -28,10 +28,13 @@ RP_RULE bool sweep_pays(double msgs, double senders, double edges, double vertic
     return sweep < 0.9 * push;
 }
 
-// The host's: both forms are in the chain if twice what the hop carried in the batch before would be swept (unknown: if all
-// edges from all vertices would).
-inline bool sweep_may_pay(bool known, double msgs, double senders, double edges, double vertices, int width) {
-    return known ? sweep_pays(2.0 * msgs, 2.0 * senders, edges, vertices, width) : sweep_pays(edges, vertices, edges, vertices, width);
+// The host's: both forms come into the chain if twice what the hop carried in the batch before would be swept (unknown: if all
+// edges from all vertices would), and stay in it while four times as much would: a stream of batches that differ by less than
+// a factor two keeps one chain, also near the line (each change of the chain costs a batch launched kernel by kernel and a
+// capture, a quarter to half a millisecond).
+inline bool sweep_may_pay(bool known, bool armed, double msgs, double senders, double edges, double vertices, int width) {
+    const double by = armed ? 4.0 : 2.0;
+    return known ? sweep_pays(by * msgs, by * senders, edges, vertices, width) : sweep_pays(edges, vertices, edges, vertices, width);
 }
 
 // What ctl->pull says of a hop.

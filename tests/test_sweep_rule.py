@@ -11,12 +11,16 @@ DRIVER = r"""
 #include "sweep_rule.h"
 // reads lines of: messages, senders, edges, vertices, width; prints for each 0/1 whether the device sweeps, whether the
 // host has both forms in the chain of the batch after one that carried as much, and whether a sweep that the caller wants
-// reads every list
-int main() {
+// reads every list; "stream" in the arguments: one stream of batches, what the host has in the chain lasts from line to line
+int main(int argc, char**) {
     double m, s, e, v;
     int w;
-    while (std::scanf("%lf %lf %lf %lf %d", &m, &s, &e, &v, &w) == 5)
-        std::printf("%d%d%d\n", (int)rp::sweep_pays(m, s, e, v, w), (int)rp::sweep_may_pay(true, m, s, e, v, w), (int)rp::sweep_reads_all(m, e));
+    bool armed = false;
+    while (std::scanf("%lf %lf %lf %lf %d", &m, &s, &e, &v, &w) == 5) {
+        const bool may = rp::sweep_may_pay(true, argc > 1 && armed, m, s, e, v, w);
+        std::printf("%d%d%d\n", (int)rp::sweep_pays(m, s, e, v, w), (int)may, (int)rp::sweep_reads_all(m, e));
+        armed = may;
+    }
     return 0;
 }
 """
@@ -29,8 +33,8 @@ def rule(tmp_path_factory):
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", os.path.join(ROOT, "paper_2601_12347_b200", "csrc"),
                            str(d / "driver.cpp"), "-o", str(d / "driver")])
 
-    def ask(hops):
-        out = subprocess.run([str(d / "driver")], input="\n".join(" ".join(map(str, h)) for h in hops), capture_output=True, text=True, check=True)
+    def ask(hops, *args):
+        out = subprocess.run([str(d / "driver"), *args], input="\n".join(" ".join(map(str, h)) for h in hops), capture_output=True, text=True, check=True)
         return [tuple(c == "1" for c in line) for line in out.stdout.split()]
     return ask
 
@@ -61,3 +65,18 @@ def test_a_small_hop_does_not_read_the_whole_graph(rule):
     small = [(m, 10, *DENSE, w) for m in (0, 9, 22_000, 2_300_000) for w in (48, 256)]
     large = [(m, 10_000, *DENSE, w) for m in (20_000_000, 122_000_000) for w in (48, 256)]
     assert not any(r[2] for r in rule(small)) and all(r[2] for r in rule(large))
+
+
+@pytest.mark.parametrize("width, edges, vertices, senders", [(256, *DENSE, 5_000), (128, 1_166_243, 169_343, 20_000), (40, 1_166_243, 169_343, 10_000)])
+def test_a_stream_near_the_line_keeps_its_chain(rule, width, edges, vertices, senders):
+    """Batches that carry between 0.75 and 1.3 times what a hop needs to bring the sweep into the chain."""
+    lo, hi = 1.0, float(edges)
+    for _ in range(60):     # the least number of messages after which both forms are in the chain
+        mid = (lo * hi) ** 0.5
+        lo, hi = (lo, mid) if rule([(mid, senders, edges, vertices, width)])[0][1] else (mid, hi)
+    assert 1.0 < hi < edges
+    sizes = [0.8, 1.3, 0.75, 1.1, 0.9, 1.25] * 8
+    chain = [r[1] for r in rule([(f * hi, f * senders, edges, vertices, width) for f in sizes], "stream")]
+    assert sum(a != b for a, b in zip(chain, chain[1:])) <= 1
+    gone = [r[1] for r in rule([(f * hi, f * senders, edges, vertices, width) for f in (1.3, 0.8, 0.2, 0.2)], "stream")]
+    assert gone == [True, True, False, False]     # and leaves it when the stream has become small
