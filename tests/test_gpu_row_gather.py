@@ -32,6 +32,13 @@ def lists_of_every_length(n, seed):
     return np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
 
 
+def feature_batch(rng, n, d, count):
+    vs = rng.choice(n, count, replace=False)
+    ups = np.zeros(count, dtype=I.UPDATE_DTYPE)
+    ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, vs, np.arange(count)
+    return ups, rng.standard_normal((count, d)).astype(np.float32)
+
+
 # widths: 1, 3, 5, 6, 10, 11, 12, 16, 25, 32, 33, 65 and 129 pieces of 16 bytes per row
 @pytest.mark.parametrize("d", [4, 12, 18, 24, 40, 44, 47, 64, 100, 128, 132, 260, 516])
 @pytest.mark.parametrize("agg", ["mean", "gcn", "weighted"])
@@ -88,7 +95,10 @@ def test_sweep_on_graphs_beyond_the_exact_filter(env, n):
 
 
 def test_swept_and_pushed_hops_agree_where_the_device_chooses(env):
-    """A small graph whose second hop carries most of the edges: AUTO sweeps it (dense frontier), PUSH does not."""
+    """Batches of 2100 feature updates (F), whose second hop carries nearly all edges from 18 K senders and is swept, and of 2100
+    edges deleted (D) and added (A), whose second hop carries a tenth and is pushed.  After an F both forms are in the chain:
+    D and A replay the chain captured for F and push on it.  After a D or an A the sweep is not in the chain, and F pushes
+    once.  900 feature updates (f) lie on the other side of the line, near enough to keep both.  PUSH pushes throughout."""
     ripple, _ = env
     n = 20_000
     src, dst = I.er_graph(n, 400_000, 4)
@@ -97,26 +107,27 @@ def test_swept_and_pushed_hops_agree_where_the_device_chooses(env):
     W = I.make_weights(model, 4)
     rps = [ripple.Ripple(n, src, dst, X, model, W, scatter_mode=m, regather_threshold=-1.0) for m in (ripple.SCATTER_AUTO, ripple.SCATTER_PUSH)]
     rng = np.random.default_rng(2)
-    for b in range(4):
-        vs = rng.choice(n, 900, replace=False)
-        ups = np.zeros(vs.size, dtype=I.UPDATE_DTYPE)
-        ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, vs, np.arange(vs.size)
-        rows = rng.standard_normal((vs.size, 64)).astype(np.float32)
+    edges = np.zeros(2100, dtype=I.UPDATE_DTYPE)
+    at = rng.choice(src.size, edges.size, replace=False)
+    edges["u"], edges["v"] = src[at], dst[at]
+    before = "F"      # (nothing known: both forms)
+    for kind in "FFFFDFFAFFDFfF":
+        if kind in "DA":
+            ups, rows = edges.copy(), None
+            ups["op"] = I.OP_DEL_EDGE if kind == "D" else I.OP_ADD_EDGE
+        else:
+            ups, rows = feature_batch(rng, n, 64, 2100 if kind == "F" else 900)
         for rp in rps:
             rp.apply_batch(ups, rows)
+        assert list(rps[0].stats()["scatter_pull"][1:3]) == [0, 1 if kind == "F" and before in "Ff" else 0], before + kind
+        before = kind
+        assert list(rps[1].stats()["scatter_pull"][1:3]) == [0, 0]
         for l in range(3):
             assert np.array_equal(rps[0].affected(l).cpu().numpy(), rps[1].affected(l).cpu().numpy())
             a, c = (rp.embeddings(l).cpu().numpy() for rp in rps)
             assert np.max(np.abs(a - c) / (1 + np.abs(c))) <= 1e-4
     for rp in rps:
         rp.close()
-
-
-def feature_batch(rng, n, d, count):
-    vs = rng.choice(n, count, replace=False)
-    ups = np.zeros(count, dtype=I.UPDATE_DTYPE)
-    ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, vs, np.arange(count)
-    return ups, rng.standard_normal((count, d)).astype(np.float32)
 
 
 @pytest.mark.parametrize("min_width", [None, "0", "257"])
