@@ -209,3 +209,38 @@ def test_overflowed_weights_stay_visible(env, d):
     H = rp.embeddings(1).cpu().numpy()
     assert np.isnan(H[reached]).all() and np.isfinite(H[~reached]).all()
     rp.close()
+
+
+@pytest.mark.parametrize("edges, d", [(0, 18), (2_500_000, 18), (4_900_000, 18), (4_900_000, 130)])   # pieces of 128, 256, 512 entries
+def test_rows_gathered_anew_at_the_edges_of_their_pieces(env, edges, d):
+    """In-lists around a window (128) and the piece of a recomputation, in a whole-graph pass and in batches whose rounding
+    budget is so tight that every row they reach comes due."""
+    ripple, Oracle = env
+    lengths = (1, 2, 31, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 1600)
+    rng = np.random.default_rng(7)
+    pool = 3200
+    n = pool + len(lengths)
+    src = [rng.choice(pool, k, replace=False) for k in lengths]
+    dst = [np.full(k, pool + i) for i, k in enumerate(lengths)]
+    if edges:       # among the pool: more edges make longer pieces
+        a, b = I.er_graph(pool, edges, 5)
+        src, dst = src + [a], dst + [b]
+    src, dst = np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+    model = I.gat_model(d, 1, d_att=8, slope=0.2)
+    size = np.float32(np.sqrt(18 / d))     # (logits of order one at either width: the sums' bound knows nothing of the weights' size)
+    X = size * I.features(n, d, 5)
+    W = I.make_weights(model, 5)
+    rp = ripple.Ripple(n, src, dst, X, model, W, rebuild_budget=1e-3)
+    orc = Oracle(n, src, dst, X, model, W)
+    G.check_values(rp, orc.full(), 1, cached_rows(orc, 1))
+    for b in range(2):
+        us = np.unique([s[rng.integers(s.size)] for s in np.split(src[:sum(lengths)], np.cumsum(lengths)[:-1])])
+        ups = np.zeros(us.size, dtype=I.UPDATE_DTYPE)
+        ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, us, np.arange(us.size)
+        rows = size * rng.standard_normal((us.size, d)).astype(np.float32)
+        rp.apply_batch(ups, rows)
+        assert orc.apply_incremental(ups, rows) == 0
+        assert rp.stats()["rows_rebuilt"][1] >= len(lengths)
+        G.check_frontiers(rp, orc, 1)
+        G.check_values(rp, orc.full(), 1, cached_rows(orc, 1))
+    rp.close()

@@ -147,3 +147,28 @@ def test_products_are_as_exact_as_their_arithmetic(env, K, rows):
         bound = 1.5 * 2.0 ** -24 * (2.2 + 0.31 * K / 8 if tensor else 0.41 * np.sqrt(K / 2))
         err = float(np.linalg.norm(got - ref) / np.linalg.norm(ref))
         assert err <= bound, (d, err, bound)
+
+
+@pytest.mark.parametrize("K", [8, 256, 260, 516, 602])
+@pytest.mark.parametrize("items", [1, 2, "all", "one row more"])
+def test_few_row_products_at_the_edge_of_the_device(env, K, items):
+    """The form of small batches for few rows takes items of 16 rows and 32 columns, 256 entries of K at a time, while all items
+    fit on the device at once (four per SM): one row group, two, all that fit (100 columns: four column groups), one row
+    beyond."""
+    import torch
+    ripple, Oracle = env
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = {1: 16, 2: 17, "all": 16 * sm, "one row more": 16 * sm + 1}[items]
+    n = rows + 50
+    ring = np.arange(1, n, dtype=np.int32)
+    src = np.concatenate([np.zeros(rows, dtype=np.int32), ring, ring])      # vertex 0 reaches `rows` sinks
+    dst = np.concatenate([1 + np.arange(rows, dtype=np.int32), 1 + ring % (n - 1), 1 + (ring + 6) % (n - 1)])
+    model = I.graphconv_model([K, 100], I.AGG_MEAN)
+    X = I.features(n, K, 3)
+    W = I.make_weights(model, 3, zero_bias=False)
+    rp = ripple.Ripple(n, src, dst, X, model, W, pre_transform=False)
+    orc = Oracle(n, src, dst, X, model, W)
+    for b in range(3):
+        apply_and_check(rp, orc, *feature_batch(n, [0], K, 90 + b), 1)
+        assert rp.stats()["affected"][1] == rows
+    rp.close()

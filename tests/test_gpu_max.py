@@ -147,3 +147,47 @@ def test_sparse_gcx_100_consecutive_batches(env, batch):
             G.check_values(rp, [orc.H(l) for l in range(L + 1)], L, [None] + [orc.S(l) for l in range(1, L + 1)])
     G.check_values(rp, orc.full(), L, [None] + [orc.full_S(l) for l in range(1, L + 1)])
     rp.close()
+
+
+# In-lists around a lane's share, the cut of a recomputation (128 entries, 256 from 2.4 M edges on) and twice that; elements
+# invalidated on both sides of a power of two (which sets the lanes per entry) and of the 32 that are re-read one by one.
+RECOMPUTED_LISTS = (1, 2, 31, 33, 64, 127, 128, 129, 255, 256, 257, 512, 513, 700)
+RECOMPUTED_ELEMENTS = (1, 2, 3, 8, 15, 16, 17, 31, 32, 33)
+
+
+@pytest.mark.parametrize("agg", [I.AGG_MAX, I.AGG_MIN], ids=["max", "min"])
+@pytest.mark.parametrize("d, filler", [(40, 0), (132, 0), (516, 0), (40, 2_600_000)])
+def test_recomputed_elements_and_lists_at_the_edges_of_their_forms(env, d, filler, agg):
+    """One sink per list length and number of elements: a neighbour of its own holds the extreme value in exactly that many
+    elements and gives them up in the batch."""
+    rng = np.random.default_rng(d)
+    pool = 2600
+    cases = [(k, e) for k in RECOMPUTED_LISTS for e in RECOMPUTED_ELEMENTS]
+    n = pool + 2 * len(cases)                     # the pool, the sinks, their neighbours
+    sinks, holders = pool + np.arange(len(cases)), pool + len(cases) + np.arange(len(cases))
+    src = [rng.choice(pool, k - 1, replace=False) for k, _ in cases] + [holders]
+    dst = [np.full(k - 1, v) for (k, _), v in zip(cases, sinks)] + [sinks]
+    if filler:                                    # edges among the pool: more of them cut lists into longer pieces
+        a, b = I.er_graph(pool, filler, 5)
+        src, dst = src + [a], dst + [b]
+    src, dst = np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+    sign = 1.0 if agg == I.AGG_MAX else -1.0
+    model = I.graphconv_model([d, 24], agg)
+    ripple, Oracle = env
+    X = I.features(n, d, d)
+    low = np.full((len(cases), d), -20.0 * sign, dtype=np.float32)
+    X[holders] = low
+    for i, (_, e) in enumerate(cases):
+        X[holders[i], rng.choice(d, min(e, d), replace=False)] = 10.0 * sign
+    W = I.make_weights(model, 3, zero_bias=False)
+    rp = ripple.Ripple(n, src, dst, X, model, W)
+    orc = Oracle(n, src, dst, X, model, W)
+    G.check_values(rp, orc.full(), 1, [None, orc.full_S(1)])
+    ups = np.zeros(len(cases), dtype=I.UPDATE_DTYPE)
+    ups["op"], ups["u"], ups["v"] = I.OP_SET_FEATURE, holders, np.arange(len(cases))
+    for rows in (low, X[holders], low - sign):    # given up, back (no recomputation), all elements at once
+        rp.apply_batch(ups, np.ascontiguousarray(rows))
+        assert orc.apply_incremental(ups, np.ascontiguousarray(rows)) == 0
+        G.check_frontiers(rp, orc, 1)
+        G.check_values(rp, [orc.H(l) for l in range(2)], 1, [None, orc.S(1)])
+    rp.close()
