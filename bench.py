@@ -148,13 +148,14 @@ def pct(xs, p):
 def scatter_bytes(stats, l, ld):
     """Algorithmic bytes of hop l's scatter in the form that ran (fp32, row width ld floats).
     push: each sender row read once, its out-list read once, one read + one write of an aggregate
-    row per message.  pull: in-lists of the affected sinks, one delta row per message, one read +
-    one write of each affected aggregate row."""
+    row per message.  swept: every in-list of the graph; rebuilt: in-lists of the affected sinks; either:
+    one row per sender, one read + one write of each affected aggregate row."""
     e = stats["active_edges"][l] - (stats["n_added"] + stats["n_deleted"])
     if stats["scatter_pull"][l]:
-        # in-list entry + position-map entry per in-edge of an affected sink; every sender's delta
+        # in-list entries, swept also a position-map entry per message (rebuilt: per in-edge); every sender's delta
         # row once (it is re-read from L2 after that); read + write of each affected aggregate row
-        return stats["in_edges"][l] * 8 + stats["senders"][l - 1] * 4 * ld + stats["affected"][l] * 8 * ld
+        ids = stats["num_edges"] * 4 + e * 4 if stats["scatter_pull"][l] == 1 else stats["in_edges"][l] * 8
+        return ids + stats["senders"][l - 1] * 4 * ld + stats["affected"][l] * 8 * ld
     return stats["senders"][l - 1] * (4 * ld + 8) + 4 * e + e * 8 * ld
 
 
@@ -732,7 +733,7 @@ def main():
     ap.add_argument("--workload", default="dense-2l")
     ap.add_argument("--batch", type=int, default=1000)
     ap.add_argument("--seed", type=int, default=0)
-    ap.add_argument("--scatter", type=int, default=0, help="0 auto, 1 push, 2 gather per sink")
+    ap.add_argument("--scatter", type=int, default=0, help="0 auto, 1 push, 2 sweep")
     ap.add_argument("--partitioned", type=int, default=0,
                     help="with --table: run the workloads as this many workers of the partitioned execution, all on one GPU")
     ap.add_argument("--partitioned-dist", action="store_true",

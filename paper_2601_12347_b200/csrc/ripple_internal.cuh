@@ -73,7 +73,7 @@ struct Ctl {
     int walk_ticket[RP_MAXL + 1];     // walk of the senders' out-lists: next unassigned chunk (see TicketWalk)
     int ew_ticket[RP_MAXL + 1];       // elementwise update: next unassigned run of pieces
     int hub_ticket[RP_MAXL + 1];      // chunks of long in-lists: next unassigned work item
-    int regather_ticket[RP_MAXL + 1]; // rebuilding form: next unassigned position of A_l
+    int regather_ticket[RP_MAXL + 1]; // sums over in-lists (max and min: recomputed rows): next unassigned tile of sinks
     int gather_ticket[RP_MAXL + 1];   // sweeping form of the delta scatter: next unassigned run of vertices
     int gather_long_ticket[RP_MAXL + 1];  // ... and next unassigned work item
     int gather_items[RP_MAXL + 1];    // sweeping form of the delta scatter: (sink, piece) work items of the long in-lists

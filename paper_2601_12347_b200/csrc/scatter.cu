@@ -188,19 +188,19 @@ k_sum_rows_long(const Ctl* ctl, int l, int only_if_rebuilding, const __grid_cons
         const int from = (int)walk.at, to = min(n, from + walk.chunk);
         walk.take();
         for (int it = from; it < to; ++it) {
-        const int2 w = a.items[it];
-        if (w.x < 0) {
-            const int tile = -1 - w.x;
-            const long long i0 = (long long)a.take * tile;
-            TileRun run = TileLists(a.in, a.list, i0, (int)min((long long)a.take, (a.n_dev ? *a.n_dev : a.n_host) - i0)).run(a.long_list);
-            run.total = min(run.total, (w.y + 1) * a.piece);
-            sum_rows<NV, WGT>(g, run, a, q, acc, w.y * a.piece);
-            continue;
-        }
-        const int deg = a.in.deg[w.x];
-        const ListRun run(w.x, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item));
-        sum_rows<NV, WGT>(g, run, a, q, acc);
-        rg_finish_one<NV>(g, a.S + (size_t)w.x * a.ld, acc);
+            const int2 w = a.items[it];
+            if (w.x < 0) {
+                const int tile = -1 - w.x;
+                const long long i0 = (long long)a.take * tile;
+                TileRun run = TileLists(a.in, a.list, i0, (int)min((long long)a.take, (a.n_dev ? *a.n_dev : a.n_host) - i0)).run(a.long_list);
+                run.total = min(run.total, (w.y + 1) * a.piece);
+                sum_rows<NV, WGT>(g, run, a, q, acc, w.y * a.piece);
+                continue;
+            }
+            const int deg = a.in.deg[w.x];
+            const ListRun run(w.x, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item));
+            sum_rows<NV, WGT>(g, run, a, q, acc);
+            rg_finish_one<NV>(g, a.S + (size_t)w.x * a.ld, acc);
         }
     }
 }
@@ -297,8 +297,8 @@ void spmm_full(Ctx* c, int l) {
 // stored weight (1 without stored weights).  One warp per record; rows have the inbox width.
 // A pushing hop delivers them in the walk's launch (both only add to the accumulator), by the last blocks of the grid:
 // the pushes launch eight blocks per SM, of which registers admit three to five at a time, so on a large walk these
-// blocks begin when others run out of tickets.  A gathering hop, whose gather stores the rows it finishes, delivers them
-// afterwards in a launch of their own.
+// blocks begin when others run out of tickets.  A swept hop delivers them in the sweep's first launch.  The bulk push and
+// hops that are always rebuilt have a launch of their own for them.
 struct RecMsgs {
     const Rec* rec;
     int src_norm;
@@ -545,8 +545,8 @@ k_scatter_push_bulk(Ctl* ctl, int l, const int32_t* __restrict__ senders, const 
 // one bit per vertex on graphs of up to 2^19 of them, else one of 2^19 bits per id by a multiplicative hash; the position
 // map, one trip to L2, is asked about the few that pass.  The delta rows are few and stay in L2.
 //
-// What bounds it: the requests that an SM's L1 takes (a bit of the filter per entry, a word of the position map per row,
-// two or three lines per row) and the trips to memory of a window, at half of the issue slots; 4.5 ps per entry without a row.
+// What bounds it: the trips to memory of a window and of the rows on their way with 20 warps per SM, at 59 to 65 % of L1TEX, 42
+// to 54 % of the issue slots and 37 to 55 % of L2 (30 M edges, 7.6 M rows of 256 floats: 0.59 ms, 12.3 TB/s out of L2).
 // ---------------------------------------------------------------------------------------------
 constexpr int SWEEP_BITS = 19;
 // One block per SM: as many threads as leave them the registers that the rows on their way and the ids of the next window
@@ -756,21 +756,21 @@ k_sweep_long(Ctl* ctl, int l, const __grid_constant__ Sweep a) {
         const int from = (int)walk.at, to = min(n, from + walk.chunk);
         walk.take();
         for (int it = from; it < to; ++it) {
-        const int2 w = a.items[it];
-        if (w.x < 0) {
-            const long long v0 = (long long)a.take * (-1 - w.x);
-            TileRun run = TileLists(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0), only).run(a.long_list);
-            run.total = min(run.total, (w.y + 1) * a.piece);
-            const unsigned sinks = __reduce_or_sync(FULL, sweep_tile<NV, WGT>(g, run, a, filter, q, acc, w.y * a.piece));
-            if (sinks && lane_id() == 0) atomicOr(&a.bitmap[v0 >> 5], sinks);
-            continue;
-        }
-        const int deg = a.in.deg[w.x];
-        const bool reached = __any_sync(FULL, sweep_list<NV, WGT>(g, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item), a, filter, q, acc));
-        if (!reached) continue;
-        rg_finish_one<NV>(g, a.dS + (size_t)w.x * a.ld, acc);
-        const uint32_t m = 1u << (w.x & 31);
-        if (lane_id() == 0 && !(a.bitmap[w.x >> 5] & m)) atomicOr(&a.bitmap[w.x >> 5], m);
+            const int2 w = a.items[it];
+            if (w.x < 0) {
+                const long long v0 = (long long)a.take * (-1 - w.x);
+                TileRun run = TileLists(a.in, nullptr, v0, (int)min((long long)a.take, a.N - v0), only).run(a.long_list);
+                run.total = min(run.total, (w.y + 1) * a.piece);
+                const unsigned sinks = __reduce_or_sync(FULL, sweep_tile<NV, WGT>(g, run, a, filter, q, acc, w.y * a.piece));
+                if (sinks && lane_id() == 0) atomicOr(&a.bitmap[v0 >> 5], sinks);
+                continue;
+            }
+            const int deg = a.in.deg[w.x];
+            const bool reached = __any_sync(FULL, sweep_list<NV, WGT>(g, a.in.start[w.x] + (int64_t)w.y * a.item, min(a.item, deg - w.y * a.item), a, filter, q, acc));
+            if (!reached) continue;
+            rg_finish_one<NV>(g, a.dS + (size_t)w.x * a.ld, acc);
+            const uint32_t m = 1u << (w.x & 31);
+            if (lane_id() == 0 && !(a.bitmap[w.x >> 5] & m)) atomicOr(&a.bitmap[w.x >> 5], m);
         }
     }
 }

@@ -29,8 +29,8 @@ def apply_and_check(rp, orc, ups, rows, L, slack=0.0):
 
 # Tensor-core form of the layer update: K chunks of 32 (31, 32, 33, and four / five of them: the weights stay in shared
 # memory up to 128), column groups of 128, the widths for which it is taken (113 to 256; up to 64 over 256 and more
-# entries there is a form in pieces, see test_gpu_narrow_products; others are fp32 sums), row tiles of 128 and the 1024 rows from which it is taken (n - 1, n and n + 1 of both), normalised sources, GIN's
-# summed operand.
+# entries there is a form in pieces, see test_gpu_narrow_products; others are fp32 sums), row tiles of 128 and the 1024 rows
+# from which it is taken (n - 1, n and n + 1 of both), normalised sources, GIN's summed operand.
 TC_MODELS = {
     "sage_31_5_47": lambda: I.sage_model([31, 5, 47], I.AGG_MEAN),
     "sage_33_129_256": lambda: I.sage_model([33, 129, 256], I.AGG_SUM),
@@ -127,7 +127,8 @@ def test_batches_at_the_edges_of_the_staging_forms(env, mem, d):
     rp.close()
 
 
-# The default arithmetic is fp32 sums outside the tensor-core form's lines and the split product inside: a layer's product
+# The default arithmetic is fp32 sums outside the lines of the tensor-core forms, tf32-split products from 113 columns on, and
+# up to 64 columns over 256 and more entries products of three bf16 parts, which have to be as exact as fp32 sums: a layer's product
 # over rows without in-neighbours, against fp64, on both sides of the lines.  u = 2^-24.  A sequential fp32 sum of K terms of
 # random sign: one rounding per term, 0.58 u / x rms for a partial sum of mantissa x (0.41 u over a binade), and partial sums
 # that grow like sqrt(k): 0.41 u sqrt(K / 2).  The tensor core truncates one addition per eight terms (0.31 u each, by measurement
